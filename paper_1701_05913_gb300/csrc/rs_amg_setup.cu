@@ -25,7 +25,6 @@
 namespace {
 
 constexpr int SG_CAP = 2048;     // candidate terms of one row of a product
-constexpr int SG_WARPS = 4;      // rows (warps) per block of the product
 
 // ---------------------------------------------------------------------------
 // exclusive prefix sums of int counts (out[n] = total)
@@ -301,90 +300,268 @@ __global__ void k_interp(int n, const int *__restrict__ ptr, const int *__restri
 
 // ---------------------------------------------------------------------------
 // 5. sparse products C = A B, a warp per row.  The row's candidate terms
-// (entry p of A's row, entry q of B's row p), numbered in that order, are
-// sorted by (column, number); a column's terms are then summed in number
-// order.  Count pass (cptr == nullptr): the distinct columns; fill pass:
-// columns and sums.  A row with more than SG_CAP terms sets *err.
+// (entry p of A's row, entry q of B's row p) are numbered in that order; a
+// column of the result is the sum of its terms in number order.  Rows are
+// taken by class of their number of terms, one launch per class that occurs,
+// so that a row's scratch is a few KB and not the largest row's: up to 32
+// terms stay in registers, one per lane; longer rows go through a hash table
+// of their columns in shared memory, 32 terms at a time.
+//
+// What bounds it: the chain of dependent loads of a row (A's entries, B's row
+// pointers, B's entries), so the rate is rows in flight.  With one sort of
+// 2048 slots (32 KB) per warp for every row, four rows in flight per SM, the
+// 14 products of a 128 x 128 x 64 hierarchy took 48 ms of the setup's 77.2;
+// the setup now takes 33.3 ms, most of it on the host.
 // ---------------------------------------------------------------------------
+constexpr int SG_CLASSES = 4;
+__host__ __device__ constexpr int sg_hi(int c) { return c == 0 ? 32 : c == 1 ? 128 : c == 2 ? 512 : SG_CAP; }
+// shared memory of one warp: table of 2 hi columns and sums, the distinct
+// columns and their slots
+constexpr size_t sg_warp_smem(int c)
+{
+    return c == 0 ? 0 : (size_t)sg_hi(c) * (2 * (sizeof(double) + sizeof(int)) + 2 * sizeof(int));
+}
+// 16 to 64 KB a block: up to 48 warps per SM for rows of up to 128 terms, 12
+// for up to 512, 3 beyond
+constexpr int sg_warps(int c) { return c < 2 ? 4 : c == 2 ? 2 : 1; }
+
+// terms of every row, the rows in each class (cls[0..3]) and those with more
+// than SG_CAP terms (cls[4])
+__global__ void k_sg_len(int n, const int *__restrict__ aptr, const int *__restrict__ acol,
+                         const int *__restrict__ bptr, int *__restrict__ len, int *__restrict__ cls)
+{
+    __shared__ int sc[SG_CLASSES + 1];
+    if (threadIdx.x <= SG_CLASSES) sc[threadIdx.x] = 0;
+    __syncthreads();
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        int64_t m = 0;
+        for (int p = aptr[i]; p < aptr[i + 1]; ++p) m += bptr[acol[p] + 1] - bptr[acol[p]];
+        const int c = m <= sg_hi(0) ? 0 : m <= sg_hi(1) ? 1 : m <= sg_hi(2) ? 2 : m <= sg_hi(3) ? 3 : 4;
+        len[i] = c < SG_CLASSES ? (int)m : SG_CAP + 1;
+        atomicAdd(&sc[c], 1);
+    }
+    __syncthreads();
+    if (threadIdx.x <= SG_CLASSES && sc[threadIdx.x]) atomicAdd(&cls[threadIdx.x], sc[threadIdx.x]);
+}
+
+// the number of lanes whose (non-decreasing) value is <= t, at most 31
+__device__ __forceinline__ int sg_find(int inc, int t)
+{
+    int pos = 0;
+#pragma unroll
+    for (int s = 16; s > 0; s >>= 1)
+        if (__shfl_sync(0xffffffffu, inc, pos + s - 1) <= t) pos += s;
+    return pos;
+}
+
+// 32 consecutive entries of A's row, one per lane: value, first entry of B's
+// row, and the inclusive scan of those rows' lengths
+struct SgChunk {
+    double a;
+    int q0, m, inc, total;
+};
 template <bool FILL>
-__global__ void __launch_bounds__(32 * SG_WARPS)
-k_spgemm(int n, const int *__restrict__ aptr, const int *__restrict__ acol, const double *__restrict__ aval,
-         const int *__restrict__ bptr, const int *__restrict__ bcol, const double *__restrict__ bval,
-         const int *__restrict__ cptr, int *__restrict__ out, double *__restrict__ cval, int *__restrict__ err)
+__device__ __forceinline__ SgChunk sg_chunk(int p, int pe, int lane, const int *__restrict__ acol,
+                                            const double *__restrict__ aval, const int *__restrict__ bptr)
+{
+    SgChunk k;
+    k.a = 0.0;
+    k.q0 = k.m = 0;
+    if (p + lane < pe) {
+        const int j = acol[p + lane];
+        if (FILL) k.a = aval[p + lane];
+        k.q0 = bptr[j];
+        k.m = bptr[j + 1] - k.q0;
+    }
+    k.inc = k.m;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, k.inc, o);
+        if (lane >= o) k.inc += y;
+    }
+    k.total = __shfl_sync(0xffffffffu, k.inc, 31);
+    return k;
+}
+
+// term t of a chunk (a lane's own t; every lane calls): its column and product
+template <bool FILL>
+__device__ __forceinline__ void sg_term(const SgChunk &k, int t, bool in, const int *__restrict__ bcol,
+                                        const double *__restrict__ bval, int &c, double &v)
+{
+    const int pos = sg_find(k.inc, t);
+    const int q = __shfl_sync(0xffffffffu, k.q0 + k.m - k.inc, pos) + t;
+    const double a = FILL ? __shfl_sync(0xffffffffu, k.a, pos) : 0.0;
+    if (in) {
+        c = bcol[q];
+        if (FILL) v = __dmul_rn(a, bval[q]);
+    }
+}
+
+// s plus the values v of the lanes in mask, in lane order (every lane calls;
+// mask 0: s as it is)
+__device__ __forceinline__ double sg_sum(double s, double v, unsigned mask, int lane)
+{
+    while (__any_sync(0xffffffffu, mask != 0)) {
+        const double x = __shfl_sync(0xffffffffu, v, mask ? __ffs(mask) - 1 : lane);
+        if (mask) {
+            s = __dadd_rn(s, x);
+            mask &= mask - 1;
+        }
+    }
+    return s;
+}
+
+// Count pass (FILL false): out[i] = the distinct columns of row i; fill pass:
+// columns (ascending) and sums from cptr[i].  A warp takes `chunk` (<= 32)
+// consecutive rows at a time and of these the rows of class cls.
+template <bool FILL>
+__global__ void __launch_bounds__(128)
+k_spgemm(int n, int cls, int chunk, const int *__restrict__ len, const int *__restrict__ aptr,
+         const int *__restrict__ acol, const double *__restrict__ aval, const int *__restrict__ bptr,
+         const int *__restrict__ bcol, const double *__restrict__ bval, const int *__restrict__ cptr,
+         int *__restrict__ out, double *__restrict__ cval)
 {
     extern __shared__ __align__(16) unsigned char sg_smem[];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    unsigned long long *key = (unsigned long long *)sg_smem + (size_t)wid * SG_CAP;
-    double *tv = (double *)(sg_smem + (size_t)SG_WARPS * SG_CAP * sizeof(unsigned long long)) + (size_t)wid * SG_CAP;
-    const int stride = gridDim.x * SG_WARPS;
-    for (int i = blockIdx.x * SG_WARPS + wid; i < n; i += stride) {
-        // the row's terms
-        int len = 0;
-        for (int p = aptr[i]; p < aptr[i + 1]; ++p) len += bptr[acol[p] + 1] - bptr[acol[p]];
-        if (len > SG_CAP) {
-            if (lane == 0) {
-                atomicOr(err, 1);
-                if (!FILL) out[i] = 0;
+    constexpr unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int hi = sg_hi(cls), lo = cls ? sg_hi(cls - 1) : -1;
+    // all warps' sums, then all tables, distinct columns and slots
+    double *tsum = (double *)sg_smem + (size_t)wid * 2 * hi;
+    int *ibase = (int *)(sg_smem + (size_t)nw * 2 * hi * sizeof(double));
+    int *tcol = ibase + (size_t)wid * 2 * hi;
+    int *dc = ibase + (size_t)nw * 2 * hi + (size_t)wid * hi;
+    int *dl = ibase + (size_t)nw * 3 * hi + (size_t)wid * hi;
+    const unsigned lt = (1u << lane) - 1;
+    for (int64_t b0 = ((int64_t)blockIdx.x * nw + wid) * chunk; b0 < n; b0 += (int64_t)gridDim.x * nw * chunk) {
+        const int myl = lane < chunk && b0 + lane < n ? len[b0 + lane] : SG_CAP + 2;
+        for (unsigned todo = __ballot_sync(FULL, myl > lo && myl <= hi); todo; todo &= todo - 1) {
+            const int r = __ffs(todo) - 1, i = (int)b0 + r;
+            const int rowlen = __shfl_sync(FULL, myl, r);
+            const int p0 = aptr[i], pe = aptr[i + 1];
+            const int o0 = FILL ? cptr[i] : 0;
+            if (cls == 0) {
+                // one term per lane
+                int c = -1, base = 0;
+                double v = 0.0;
+                for (int p = p0; p < pe; p += 32) {
+                    const SgChunk k = sg_chunk<FILL>(p, pe, lane, acol, aval, bptr);
+                    const int t = lane - base;
+                    sg_term<FILL>(k, t, t >= 0 && t < k.total, bcol, bval, c, v);
+                    base += k.total;
+                }
+                const bool in = lane < rowlen;
+                unsigned same = __match_any_sync(FULL, c);
+                const bool first = in && __ffs(same) - 1 == lane;
+                const unsigned firsts = __ballot_sync(FULL, first);
+                if (!FILL) {
+                    if (lane == 0) out[i] = __popc(firsts);
+                    continue;
+                }
+                const double s = sg_sum(0.0, v, first ? same : 0u, lane);
+                int rank = 0;
+                for (unsigned f = firsts; f; f &= f - 1) rank += __shfl_sync(FULL, c, __ffs(f) - 1) < c;
+                if (first) {
+                    out[o0 + rank] = c;
+                    cval[o0 + rank] = s;
+                }
+                continue;
             }
-            continue;
-        }
-        int base = 0;
-        for (int p = aptr[i]; p < aptr[i + 1]; ++p) {
-            const int j = acol[p];
-            const double a = aval[p];
-            const int q0 = bptr[j], m = bptr[j + 1] - q0;
-            for (int q = lane; q < m; q += 32) {
-                const int t = base + q;
-                key[t] = ((unsigned long long)(unsigned)bcol[q0 + q] << 32) | (unsigned)t;
-                if (FILL) tv[t] = __dmul_rn(a, bval[q0 + q]);
-            }
-            base += m;
-        }
-        int sz = 1;
-        while (sz < len) sz <<= 1;
-        for (int t = len + lane; t < sz; t += 32) key[t] = ~0ull;
-        __syncwarp();
-        // bitonic sort of (key, term) over sz entries
-        for (int k = 2; k <= sz; k <<= 1) {
-            for (int j = k >> 1; j > 0; j >>= 1) {
-                for (int t = lane; t < sz; t += 32) {
-                    const int u = t ^ j;
-                    if (u > t) {
-                        const bool up = (t & k) == 0;
-                        const unsigned long long kt = key[t], ku = key[u];
-                        if ((kt > ku) == up) {
-                            key[t] = ku;
-                            key[u] = kt;
-                            if (FILL) {
-                                const double x = tv[t];
-                                tv[t] = tv[u];
-                                tv[u] = x;
-                            }
+            // 32 terms at a time through the row's hash table of columns
+            const int lg = 32 - __clz(2 * rowlen - 1);      // table: the power of two >= 2 rowlen (<= 2 hi)
+            const int tsz = 1 << lg;
+            for (int k = lane; k < tsz; k += 32) tcol[k] = -1;
+            __syncwarp();
+            int nd = 0;
+            for (int p = p0; p < pe; p += 32) {
+                const SgChunk k = sg_chunk<FILL>(p, pe, lane, acol, aval, bptr);
+                for (int t0 = 0; t0 < k.total; t0 += 32) {
+                    const bool in = t0 + lane < k.total;
+                    int c = -1;
+                    double v = 0.0;
+                    sg_term<FILL>(k, t0 + lane, in, bcol, bval, c, v);
+                    // the first lane of each column finds or claims its slot;
+                    // the claiming lanes have different columns
+                    const unsigned same = __match_any_sync(FULL, c);
+                    const bool first = in && __ffs(same) - 1 == lane;
+                    bool fresh = false;
+                    int h = 0;
+                    if (first) {
+                        h = (int)(((unsigned)c * 2654435761u) >> (32 - lg));
+                        for (;;) {
+                            const int cur = atomicCAS(&tcol[h], -1, c);
+                            fresh = cur == -1;
+                            if (fresh || cur == c) break;
+                            h = (h + 1) & (tsz - 1);
                         }
                     }
+                    if (FILL) {
+                        const double s = sg_sum(first && !fresh ? tsum[h] : 0.0, v, first ? same : 0u, lane);
+                        if (first) tsum[h] = s;
+                    }
+                    const unsigned nm = __ballot_sync(FULL, fresh);
+                    if (FILL && fresh) {
+                        const int k2 = nd + __popc(nm & lt);
+                        dc[k2] = c;
+                        dl[k2] = h;
+                    }
+                    nd += __popc(nm);
+                    __syncwarp();
                 }
+            }
+            if (!FILL) {
+                if (lane == 0) out[i] = nd;
                 __syncwarp();
+                continue;
             }
-        }
-        // distinct columns: the first term of each column starts a segment
-        int nseg = 0;
-        const int o0 = FILL ? cptr[i] : 0;
-        for (int t0 = 0; t0 < len; t0 += 32) {
-            const int t = t0 + lane;
-            const bool first = t < len && (t == 0 || (key[t] >> 32) != (key[t - 1] >> 32));
-            const unsigned m = __ballot_sync(0xffffffffu, first);
-            if (FILL && first) {
-                const int o = o0 + nseg + __popc(m & ((1u << lane) - 1));
-                const unsigned c = (unsigned)(key[t] >> 32);
-                double s = 0.0;
-                for (int e = t; e < len && (unsigned)(key[e] >> 32) == c; ++e) s = __dadd_rn(s, tv[e]);
-                out[o] = (int)c;
-                cval[o] = s;
+            if (nd <= 128) {
+                // a column's place: the number of smaller ones
+                int ck[4], rk[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    ck[u] = lane + 32 * u < nd ? dc[lane + 32 * u] : 0x7fffffff;
+                    rk[u] = 0;
+                }
+                for (int j = 0; j < nd; ++j) {
+                    const int cj = dc[j];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) rk[u] += cj < ck[u];
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (lane + 32 * u < nd) {
+                        out[o0 + rk[u]] = ck[u];
+                        cval[o0 + rk[u]] = tsum[dl[lane + 32 * u]];
+                    }
+            } else {
+                // bitonic sort of (column, slot); a power of two >= nd fits (nd <= hi)
+                int sz = 256;
+                while (sz < nd) sz <<= 1;
+                for (int k = nd + lane; k < sz; k += 32) dc[k] = 0x7fffffff;
+                __syncwarp();
+                for (int k = 2; k <= sz; k <<= 1)
+                    for (int j = k >> 1; j > 0; j >>= 1) {
+                        for (int t = lane; t < sz; t += 32) {
+                            const int u = t ^ j;
+                            if (u > t) {
+                                const int ct = dc[t], cu = dc[u];
+                                if ((ct > cu) == ((t & k) == 0) && ct != cu) {
+                                    dc[t] = cu;
+                                    dc[u] = ct;
+                                    const int x = dl[t];
+                                    dl[t] = dl[u];
+                                    dl[u] = x;
+                                }
+                            }
+                        }
+                        __syncwarp();
+                    }
+                for (int k = lane; k < nd; k += 32) {
+                    out[o0 + k] = dc[k];
+                    cval[o0 + k] = tsum[dl[k]];
+                }
             }
-            nseg += __popc(m);
+            __syncwarp();
         }
-        if (!FILL && lane == 0) out[i] = nseg;
-        __syncwarp();
     }
 }
 
@@ -567,36 +744,56 @@ int transpose(rs_ctx *ctx, Dev &D, int n, int m, int64_t nnz, const int *ptr, co
     return rs_check_launch(ctx);
 }
 
+// one pass of the product: a launch per class of rows that occurs
+template <bool FILL>
+int spgemm_pass(rs_ctx *ctx, const int (&ncls)[SG_CLASSES + 1], int n, const int *len, const int *aptr,
+                const int *acol, const double *aval, const int *bptr, const int *bcol, const double *bval,
+                const int *cptr, int *out, double *cval)
+{
+    static unsigned long long raised = 0;      // one bit per device
+    const unsigned long long bit = 1ull << (ctx->device & 63);
+    if (!(raised & bit)) {
+        RS_CUDA_TRY(cudaFuncSetAttribute(k_spgemm<FILL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)(sg_warps(3) * sg_warp_smem(3))));
+        raised |= bit;
+    }
+    for (int c = 0; c < SG_CLASSES; ++c) {
+        if (!ncls[c]) continue;
+        const int w = sg_warps(c);
+        const int per_sm = c == 0 ? 12 : (int)std::min<size_t>(12, 220 * 1024 / (w * sg_warp_smem(c) + 1024));
+        // consecutive rows a warp looks through: few enough that every warp has some
+        const int64_t resident = (int64_t)ctx->num_sms * per_sm * w;
+        const int chunk = (int)std::max<int64_t>(1, std::min<int64_t>(32, n / resident));
+        const int64_t need = ((int64_t)n + (int64_t)chunk * w - 1) / ((int64_t)chunk * w);
+        const int gb = (int)std::max<int64_t>(1, std::min<int64_t>(need, (int64_t)ctx->num_sms * per_sm));
+        k_spgemm<FILL><<<gb, 32 * w, w * sg_warp_smem(c), ctx->stream>>>(n, c, chunk, len, aptr, acol, aval, bptr,
+                                                                         bcol, bval, cptr, out, cval);
+        RS_TRY(rs_check_launch(ctx));
+    }
+    return RS_OK;
+}
+
 // C = A B (n x k by k x m) into freshly allocated device arrays
 int spgemm(rs_ctx *ctx, Dev &D, int n, const int *aptr, const int *acol, const double *aval, const int *bptr,
            const int *bcol, const double *bval, int **cptr, int **ccol, double **cval, int64_t *cnnz)
 {
-    int *cnt, *err, tot = 0, herr = 0;
+    int *cnt, *len, *cls, tot = 0, ncls[SG_CLASSES + 1];
     RS_TRY(D.alloc(&cnt, n));
+    RS_TRY(D.alloc(&len, n));
     RS_TRY(D.alloc(cptr, n + 1));
-    RS_TRY(D.alloc(&err, 1));
-    RS_CUDA_TRY(cudaMemsetAsync(err, 0, sizeof(int), ctx->stream));
-    const size_t smem = (size_t)SG_WARPS * SG_CAP * (sizeof(unsigned long long) + sizeof(double));
-    static unsigned long long raised = 0;      // one bit per device
-    const unsigned long long bit = 1ull << (ctx->device & 63);
-    if (!(raised & bit)) {
-        RS_CUDA_TRY(cudaFuncSetAttribute(k_spgemm<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        RS_CUDA_TRY(cudaFuncSetAttribute(k_spgemm<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        raised |= bit;
-    }
-    const int gb = std::max(1, std::min((n + SG_WARPS - 1) / SG_WARPS, ctx->num_sms * 2));
-    k_spgemm<false><<<gb, 32 * SG_WARPS, smem, ctx->stream>>>(n, aptr, acol, aval, bptr, bcol, bval, nullptr, cnt,
-                                                               nullptr, err);
+    RS_TRY(D.alloc(&cls, SG_CLASSES + 1));
+    RS_CUDA_TRY(cudaMemsetAsync(cls, 0, sizeof(ncls), ctx->stream));
+    k_sg_len<<<grid_for(ctx, n, 128), 128, 0, ctx->stream>>>(n, aptr, acol, bptr, len, cls);
     RS_TRY(rs_check_launch(ctx));
-    RS_TRY(read_flag(ctx, err, &herr));
-    if (herr) return RS_ERR_INVALID_ARG;     // a row of the product has more than SG_CAP terms
+    RS_CUDA_TRY(cudaMemcpyAsync(ncls, cls, sizeof(ncls), cudaMemcpyDeviceToHost, ctx->stream));
+    RS_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
+    if (ncls[SG_CLASSES]) return RS_ERR_INVALID_ARG;     // a row of the product has more than SG_CAP terms
+    RS_TRY(spgemm_pass<false>(ctx, ncls, n, len, aptr, acol, aval, bptr, bcol, bval, nullptr, cnt, nullptr));
     RS_TRY(scan(ctx, D, cnt, *cptr, n, &tot));
     *cnnz = tot;
     RS_TRY(D.alloc(ccol, tot));
     RS_TRY(D.alloc(cval, tot));
-    k_spgemm<true><<<gb, 32 * SG_WARPS, smem, ctx->stream>>>(n, aptr, acol, aval, bptr, bcol, bval, *cptr, *ccol,
-                                                              *cval, err);
-    return rs_check_launch(ctx);
+    return spgemm_pass<true>(ctx, ncls, n, len, aptr, acol, aval, bptr, bcol, bval, *cptr, *ccol, *cval);
 }
 
 }  // namespace

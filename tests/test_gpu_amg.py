@@ -105,6 +105,41 @@ def test_amg_setup_at_full_size(rs, ctx, orc):
             assert all(np.array_equal(x, y) for x, y in zip(gl["P"], wp)), l
 
 
+def _scattered(n, w, reach, seed=5):
+    """Symmetric M-matrix: each row coupled to the next one and to w random
+    later rows at most `reach` away."""
+    rng = np.random.default_rng(seed)
+    D = np.zeros((n, n))
+    for i in range(n - 1):
+        D[i, i + 1] = 1.0 + rng.random()
+        D[i, rng.integers(i + 1, min(n, i + reach), size=w)] = 0.05 + rng.random()
+    D = np.maximum(D, D.T)
+    A = np.diag(D.sum(1) + 1e-2) - D
+    nz = A != 0
+    return dict(n=n, rowptr=np.concatenate([[0], np.cumsum(nz.sum(1))]).astype(np.int32),
+                col=np.nonzero(nz)[1].astype(np.int32), val=A[nz])
+
+
+# products with rows of 8 to 171 terms, and of 13 to 1934 terms with up to 266
+# distinct columns: every class of the sparse product and both column sorts
+@pytest.mark.parametrize("n,w,reach,coarse", [(300, 8, 18, 20), (1000, 8, 1000, 300)])
+def test_amg_products_of_long_rows(rs, ctx, orc, n, w, reach, coarse):
+    d = _scattered(n, w, reach)
+    got = rs.Precond(ctx, rs.Mat.csr(ctx, d), "amg", amg=dict(max_coarse=coarse)).amg_levels()
+    want = orc.Amg(orc.Mat.csr(d), max_coarse=coarse).levels()
+    assert len(got) == len(want) >= 2
+    for l, (g, (wa, wp)) in enumerate(zip(got, want)):
+        assert all(np.array_equal(x, y) for x, y in zip(g["A"], wa)), l
+
+
+def test_amg_product_row_limit(rs, ctx):
+    """A Galerkin row of more than 2048 candidate terms is refused."""
+    A = rs.Mat.csr(ctx, _scattered(1200, 12, 1200))
+    with pytest.raises(rs.RsError) as e:
+        rs.Precond(ctx, A, "amg", amg=dict(max_coarse=300))
+    assert e.value.status == rs.ERR_INVALID_ARG
+
+
 @pytest.mark.parametrize("smoother", [0, 1])
 @pytest.mark.parametrize("solver", ["cg", "gmres"])
 @pytest.mark.parametrize("shape,kz", [((32, 32, 32), 1.0), ((30, 22, 13), 0.1)])
