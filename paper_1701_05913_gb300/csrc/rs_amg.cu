@@ -176,7 +176,7 @@ void rs_amg_destroy(AmgData *M)
     delete M;
 }
 
-int rs_amg_create(rs_ctx *ctx, int n, const int *d_ptr, const int *d_col, const double *d_val, const rs_mat *A0,
+int rs_amg_create(rs_ctx *ctx, int n, int64_t nnz, const int *d_ptr, const int *d_col, const double *d_val, const rs_mat *A0,
                   double theta, int max_levels, int max_coarse, int nu, int smoother, AmgData **out)
 {
     *out = nullptr;
@@ -192,7 +192,7 @@ int rs_amg_create(rs_ctx *ctx, int n, const int *d_ptr, const int *d_col, const 
         M->A[0] = const_cast<rs_mat *>(A0);
     } else {
         M->own0 = true;
-        st = rs_mat_create_rect_dev(ctx, n, -1, d_ptr, d_col, d_val, &M->A[0]);
+        st = rs_mat_create_dev(ctx, n, nnz, d_ptr, d_col, d_val, &M->A[0]);
     }
     // the hierarchy (Alg. 3), smoother diagonals and the coarsest inverse
     if (!st) st = rs_amg_setup_device(M, theta, max_levels, max_coarse);

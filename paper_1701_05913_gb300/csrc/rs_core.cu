@@ -764,8 +764,7 @@ int rs_residual_launch(const rs_mat *A, const double *b, const double *x, double
 // ---------------------------------------------------------------------------
 // matrices
 // ---------------------------------------------------------------------------
-static int validate_pattern(int nrows, int ncols, const std::vector<int> &ptr,
-                            const std::vector<int> &col, bool need_diag = true)
+static int validate_pattern(int nrows, const std::vector<int> &ptr, const std::vector<int> &col)
 {
     if ((int)ptr.size() != nrows + 1 || ptr[0] != 0) return RS_ERR_BAD_PATTERN;
     for (int i = 0; i < nrows; ++i) {
@@ -773,18 +772,57 @@ static int validate_pattern(int nrows, int ncols, const std::vector<int> &ptr,
         bool diag = false;
         for (int p = ptr[i]; p < ptr[i + 1]; ++p) {
             const int c = col[p];
-            if (c < 0 || c >= ncols) return RS_ERR_BAD_PATTERN;
+            if (c < 0 || c >= nrows) return RS_ERR_BAD_PATTERN;
             if (p > ptr[i] && col[p - 1] >= c) return RS_ERR_BAD_PATTERN;
             if (c == i) diag = true;
         }
-        if (!diag && need_diag) return RS_ERR_BAD_PATTERN;
+        if (!diag) return RS_ERR_BAD_PATTERN;
     }
     if ((size_t)ptr[nrows] != col.size()) return RS_ERR_BAD_PATTERN;
     return RS_OK;
 }
 
+// The device copies of A's arrays (A's sizes are set) and the SpMV kernel for
+// its rows.  RS_MAT_PAD zeroed elements follow each array: the SpMV's bulk
+// copies widen their ranges to 16-byte boundaries.
+static int mat_fill(rs_mat *A, const int32_t *ptr, const int32_t *col, const double *val, cudaMemcpyKind kind)
+{
+    rs_ctx *ctx = A->ctx;
+    const int nrows = A->nrows, b2 = A->bs * A->bs;
+    const int64_t nnzb = A->nnzb;
+    int st = rs_alloc(ctx, (void **)&A->ptr, sizeof(int) * (nrows + 1 + RS_MAT_PAD));
+    st = st ? st : rs_alloc(ctx, (void **)&A->col, sizeof(int) * (nnzb + RS_MAT_PAD));
+    st = st ? st : rs_alloc(ctx, (void **)&A->val, sizeof(double) * (nnzb * b2 + RS_MAT_PAD));
+    if (st) return st;
+    RS_CUDA_TRY(cudaMemsetAsync(A->ptr + nrows + 1, 0, sizeof(int) * RS_MAT_PAD, ctx->stream));
+    RS_CUDA_TRY(cudaMemsetAsync(A->col + nnzb, 0, sizeof(int) * RS_MAT_PAD, ctx->stream));
+    RS_CUDA_TRY(cudaMemsetAsync(A->val + nnzb * b2, 0, sizeof(double) * RS_MAT_PAD, ctx->stream));
+    RS_CUDA_TRY(cudaMemcpyAsync(A->ptr, ptr, sizeof(int) * (nrows + 1), kind, ctx->stream));
+    if (nnzb) {
+        RS_CUDA_TRY(cudaMemcpyAsync(A->col, col, sizeof(int) * nnzb, kind, ctx->stream));
+        RS_CUDA_TRY(cudaMemcpyAsync(A->val, val, sizeof(double) * nnzb * b2, kind, ctx->stream));
+    }
+    // rows of at most 12 entries on average go to the pipelined row-per-thread
+    // kernel (lanes = 1); longer ones to the lane kernel with the smallest
+    // power of two L for which 4 L entries cover the mean row
+    const double mean = nrows ? (double)nnzb / nrows : 1.0;
+    int L = 1;
+    if (mean > 12.0)
+        while (L < 32 && 4.0 * L < mean) L <<= 1;
+    A->lanes = L;
+    return RS_OK;
+}
+
+static void mat_free(rs_mat *A)
+{
+    rs_free(A->ctx, A->ptr);
+    rs_free(A->ctx, A->col);
+    rs_free(A->ctx, A->val);
+    delete A;
+}
+
 static int mat_create(rs_ctx *ctx, int nrows, int bs, const int32_t *ptr, const int32_t *col,
-                      const double *val, int mem, rs_mat **out, int ncols = -1)
+                      const double *val, int mem, rs_mat **out)
 {
     if (!ctx || !out || nrows < 0 || bs < 1 || bs > 8 || !ptr) return RS_ERR_INVALID_ARG;
     if ((int64_t)nrows * bs > 0x7fffffffLL) return RS_ERR_INVALID_ARG;
@@ -811,33 +849,11 @@ static int mat_create(rs_ctx *ctx, int nrows, int bs, const int32_t *ptr, const 
         RS_CUDA_TRY(cudaMemcpyAsync(A->h_col.data(), col, sizeof(int) * nnzb, d2h, ctx->stream));
         RS_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
     }
-    // square matrices need every diagonal entry; rectangular operators
-    // (interpolation, restriction) only sorted, in-range columns
-    int st = validate_pattern(nrows, ncols < 0 ? nrows : ncols, A->h_ptr, A->h_col, ncols < 0);
+    int st = validate_pattern(nrows, A->h_ptr, A->h_col);
     if (st) { delete A; return st; }
-    // RS_MAT_PAD zeroed elements after each array: the SpMV's bulk copies
-    // widen their ranges to 16-byte boundaries
-    st = rs_alloc(ctx, (void **)&A->ptr, sizeof(int) * (nrows + 1 + RS_MAT_PAD));
-    st = st ? st : rs_alloc(ctx, (void **)&A->col, sizeof(int) * (nnzb + RS_MAT_PAD));
-    st = st ? st : rs_alloc(ctx, (void **)&A->val, sizeof(double) * (nnzb * bs * bs + RS_MAT_PAD));
-    if (st) { rs_free(ctx, A->ptr); rs_free(ctx, A->col); delete A; return st; }
-    RS_CUDA_TRY(cudaMemsetAsync(A->ptr + nrows + 1, 0, sizeof(int) * RS_MAT_PAD, ctx->stream));
-    RS_CUDA_TRY(cudaMemsetAsync(A->col + nnzb, 0, sizeof(int) * RS_MAT_PAD, ctx->stream));
-    RS_CUDA_TRY(cudaMemsetAsync(A->val + nnzb * bs * bs, 0, sizeof(double) * RS_MAT_PAD, ctx->stream));
-    RS_CUDA_TRY(cudaMemcpyAsync(A->ptr, ptr, sizeof(int) * (nrows + 1), h2d, ctx->stream));
-    if (nnzb) {
-        RS_CUDA_TRY(cudaMemcpyAsync(A->col, col, sizeof(int) * nnzb, h2d, ctx->stream));
-        RS_CUDA_TRY(cudaMemcpyAsync(A->val, val, sizeof(double) * nnzb * bs * bs, h2d, ctx->stream));
-    }
-    if (mem == RS_MEM_HOST) RS_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
-    // rows of at most 12 entries on average go to the pipelined row-per-thread
-    // kernel (lanes = 1); longer ones to the lane kernel with the smallest
-    // power of two L for which 4 L entries cover the mean row
-    const double mean = nrows ? (double)nnzb / nrows : 1.0;
-    int L = 1;
-    if (mean > 12.0)
-        while (L < 32 && 4.0 * L < mean) L <<= 1;
-    A->lanes = L;
+    st = mat_fill(A, ptr, col, val, h2d);
+    if (!st && mem == RS_MEM_HOST && cudaStreamSynchronize(ctx->stream) != cudaSuccess) st = RS_ERR_CUDA;
+    if (st) { mat_free(A); return st; }
     rs_ctx_retain(ctx);
     *out = A;
     return RS_OK;
@@ -849,18 +865,22 @@ extern "C" int rs_mat_create_csr(rs_ctx *ctx, int32_t n, const int32_t *rowptr,
     return mat_create(ctx, n, 1, rowptr, col, val, mem, A);
 }
 
-int rs_mat_create_rect(rs_ctx *ctx, int nrows, int ncols, const int32_t *ptr, const int32_t *col,
-                       const double *val, rs_mat **A)
+// an operator of the library's own setup kernels: sorted, in range, its size
+// known.  Neither validated nor copied to the host (nothing analyses its
+// pattern there), so nothing waits for the device.
+int rs_mat_create_dev(rs_ctx *ctx, int nrows, int64_t nnz, const int *ptr, const int *col, const double *val,
+                      rs_mat **out)
 {
-    if (ncols < 0) return RS_ERR_INVALID_ARG;
-    return mat_create(ctx, nrows, 1, ptr, col, val, RS_MEM_HOST, A, ncols);
-}
-
-// from device arrays (copied); ncols < 0: square, every diagonal entry present
-int rs_mat_create_rect_dev(rs_ctx *ctx, int nrows, int ncols, const int32_t *ptr, const int32_t *col,
-                           const double *val, rs_mat **A)
-{
-    return mat_create(ctx, nrows, 1, ptr, col, val, RS_MEM_DEVICE, A, ncols);
+    rs_mat *A = new rs_mat();
+    A->ctx = ctx;
+    A->bs = 1;
+    A->nrows = A->n = nrows;
+    A->nnzb = nnz;
+    const int st = mat_fill(A, ptr, col, val, cudaMemcpyDeviceToDevice);
+    if (st) { mat_free(A); return st; }
+    rs_ctx_retain(ctx);
+    *out = A;
+    return RS_OK;
 }
 
 extern "C" int rs_mat_create_bsr(rs_ctx *ctx, int32_t nb, int32_t bs, const int32_t *browptr,
@@ -874,10 +894,7 @@ extern "C" int rs_mat_destroy(rs_mat **pA)
     if (!pA || !*pA) return RS_OK;
     rs_mat *A = *pA;
     rs_ctx *ctx = A->ctx;
-    rs_free(ctx, A->ptr);
-    rs_free(ctx, A->col);
-    rs_free(ctx, A->val);
-    delete A;
+    mat_free(A);
     *pA = nullptr;
     rs_ctx_release(ctx);
     return RS_OK;

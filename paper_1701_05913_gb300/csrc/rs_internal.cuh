@@ -110,7 +110,7 @@ struct rs_mat {
     int64_t nnzb;            // stored blocks (scalars for CSR)
     int *ptr, *col;
     double *val;
-    std::vector<int> h_ptr, h_col;   // host copy of the pattern (analysis)
+    std::vector<int> h_ptr, h_col;   // host copy of a caller's pattern (analysis)
     int lanes;               // SpMV lanes per row (CSR; 1 = the pipelined row-per-thread kernel)
 };
 
@@ -301,11 +301,10 @@ int rs_check_launch(rs_ctx *ctx);
 int rs_alloc(rs_ctx *ctx, void **p, size_t bytes);
 void rs_free(rs_ctx *ctx, void *p);
 
-// an nrows x ncols CSR operator from host arrays (no diagonal required)
-int rs_mat_create_rect_dev(rs_ctx *ctx, int nrows, int ncols, const int32_t *ptr, const int32_t *col,
-                           const double *val, rs_mat **A);
-int rs_mat_create_rect(rs_ctx *ctx, int nrows, int ncols, const int32_t *ptr, const int32_t *col,
-                       const double *val, rs_mat **A);
+// a CSR operator of nnz entries from the library's own device arrays (copied;
+// not validated, no host copy of the pattern, no synchronisation)
+int rs_mat_create_dev(rs_ctx *ctx, int nrows, int64_t nnz, const int *ptr, const int *col, const double *val,
+                      rs_mat **A);
 
 // y = alpha * A x + beta * y (beta == 0: y not read).  Kernels given a
 // non-null `skip` return at once when *skip != 0 (a device flag).
@@ -350,7 +349,7 @@ int rs_ras_apply(RasData *R, const double *r, double *z, const int *skip);
 void rs_ras_destroy(RasData *R);
 // A0: the level-0 matrix when the caller has one as an rs_mat (else built
 // from the host pattern and the device values d_val)
-int rs_amg_create(rs_ctx *ctx, int n, const int *d_ptr, const int *d_col, const double *d_val, const rs_mat *A0,
+int rs_amg_create(rs_ctx *ctx, int n, int64_t nnz, const int *d_ptr, const int *d_col, const double *d_val, const rs_mat *A0,
                   double theta, int max_levels, int max_coarse, int nu, int smoother, AmgData **out);
 // the hierarchy of Alg. 3 on the device (rs_amg_setup.cu): from M->A[0]
 int rs_amg_setup_device(AmgData *M, double theta, int max_levels, int max_coarse);
