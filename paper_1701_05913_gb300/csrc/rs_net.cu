@@ -98,7 +98,6 @@ struct rs_net {
     unsigned *ticket;
     int *flag;                              // non-finite output flag
     unsigned gen;                           // workspace generation: bumped on every (re)allocation
-    double *gout;                           // dL/d(output) (per voxel)
     double *outb;                           // network output during training
     float *headpart;                        // head gradient partials
 };
@@ -123,6 +122,20 @@ __device__ __forceinline__ void ldsm_x4_t(unsigned &r0, unsigned &r1, unsigned &
                  : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3) : "r"(smem_u32(p)));
 }
 
+__device__ __forceinline__ void ldsm_x2_t(unsigned &r0, unsigned &r1, const void *p)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0,%1}, [%2];"
+                 : "=r"(r0), "=r"(r1) : "r"(smem_u32(p)));
+}
+
+// 16 bytes global -> shared, or 16 zero bytes (src is not read then)
+__device__ __forceinline__ void cp_async16(void *dst, const void *src, bool in)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(in ? 16 : 0)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 __device__ __forceinline__ void mma_bf16(float (&c)[4], unsigned a0, unsigned a1, unsigned a2, unsigned a3,
                                          unsigned b0, unsigned b1)
 {
@@ -138,38 +151,41 @@ __device__ __forceinline__ bool skipped(const int *skip) { return skip && *(vola
 // halo loader shared by the convolution kernels
 // ---------------------------------------------------------------------------
 // Loads the 18x6x6 input halo of the brick at (tx0, ty0, tz0) into sx
-// (stride SIN bf16 per voxel), zero outside the grid.
+// (stride SIN bf16 per voxel), zero outside the grid.  Activations come by
+// cp.async, so that a thread's loads are all in flight at once: the caller
+// waits (cp_async_wait_all, then a barrier).
 template <int CIN, int MODE>
 __device__ __forceinline__ void load_halo(bf16 *sx, int SIN, int D, int H, int W, int tx0, int ty0, int tz0,
                                           const bf16 *X, const bf16 *U, const double *r, const double *logk,
                                           const double *rscale)
 {
     constexpr int CH8 = CIN / 8;
-    for (int i = threadIdx.x; i < HVOX * CH8; i += blockDim.x) {
+#pragma unroll(MODE == IN_FIRST ? 3 : 1)
+    for (int i = threadIdx.x; i < HVOX * CH8; i += CONV_THREADS) {
         const int hv = i / CH8, ch = i % CH8;
         const int hx = hv % HX, hy = (hv / HX) % HY, hz = hv / (HX * HY);
         const int gx = tx0 + hx - 1, gy = ty0 + hy - 1, gz = tz0 + hz - 1;
-        uint4 val = make_uint4(0, 0, 0, 0);
-        if (gx >= 0 && gx < W && gy >= 0 && gy < H && gz >= 0 && gz < D) {
-            const int64_t vi = ((int64_t)gz * H + gy) * W + gx;
-            if (MODE == IN_PLAIN) {
-                val = *(const uint4 *)(X + vi * CIN + ch * 8);
-            } else if (MODE == IN_CATUP) {
-                if (ch < 2) {
-                    const int W2 = W >> 1, H2 = H >> 1;
-                    const int64_t ci = ((int64_t)(gz >> 1) * H2 + (gy >> 1)) * W2 + (gx >> 1);
-                    val = *(const uint4 *)(U + ci * 16 + ch * 8);
-                } else {
-                    val = *(const uint4 *)(X + vi * 16 + (ch - 2) * 8);
-                }
-            } else {   // IN_FIRST: channels (r * rscale, logk, 0, ...)
-                if (ch == 0) {
-                    __nv_bfloat162 p0 = __floats2bfloat162_rn((float)(r[vi] * *rscale), (float)logk[vi]);
-                    val.x = *(unsigned *)&p0;
-                }
+        const bool in = gx >= 0 && gx < W && gy >= 0 && gy < H && gz >= 0 && gz < D;
+        const int64_t vi = in ? ((int64_t)gz * H + gy) * W + gx : 0;
+        bf16 *dst = sx + hv * SIN + ch * 8;
+        if (MODE == IN_PLAIN) {
+            cp_async16(dst, X + vi * CIN + ch * 8, in);
+        } else if (MODE == IN_CATUP) {
+            if (ch < 2) {
+                const int W2 = W >> 1, H2 = H >> 1;
+                const int64_t ci = in ? ((int64_t)(gz >> 1) * H2 + (gy >> 1)) * W2 + (gx >> 1) : 0;
+                cp_async16(dst, U + ci * 16 + ch * 8, in);
+            } else {
+                cp_async16(dst, X + vi * 16 + (ch - 2) * 8, in);
             }
+        } else {   // IN_FIRST: channels (r * rscale, logk, 0, ...)
+            uint4 val = make_uint4(0, 0, 0, 0);
+            if (in && ch == 0) {
+                __nv_bfloat162 p0 = __floats2bfloat162_rn((float)(r[vi] * *rscale), (float)logk[vi]);
+                val.x = *(unsigned *)&p0;
+            }
+            *(uint4 *)dst = val;
         }
-        *(uint4 *)(sx + hv * SIN + ch * 8) = val;
     }
 }
 
@@ -178,9 +194,7 @@ __device__ __forceinline__ void load_halo(bf16 *sx, int SIN, int D, int H, int W
 // ---------------------------------------------------------------------------
 template <int CIN, int COUT, int MODE>
 __global__ void __launch_bounds__(CONV_THREADS)
-k_conv3(int D, int H, int W, const bf16 *__restrict__ X, const bf16 *__restrict__ U,
-        const double *__restrict__ r, const double *__restrict__ logk, const double *__restrict__ rscale,
-        const bf16 *__restrict__ Wp, const float *__restrict__ bias, int relu, bf16 *__restrict__ Y,
+k_conv3(int D, int H, int W, const bf16 *__restrict__ X, const bf16 *__restrict__ U, const bf16 *__restrict__ Wp, const float *__restrict__ bias, int relu, bf16 *__restrict__ Y,
         const int *skip)
 {
     if (skipped(skip)) return;
@@ -196,9 +210,10 @@ k_conv3(int D, int H, int W, const bf16 *__restrict__ X, const bf16 *__restrict_
     constexpr int WCH = CIN / 8;
     for (int i = threadIdx.x; i < 27 * COUT * WCH; i += blockDim.x) {
         const int row = i / WCH, ch = i % WCH;
-        *(uint4 *)(sw + row * SW + ch * 8) = *(const uint4 *)(Wp + (size_t)row * CIN + ch * 8);
+        cp_async16(sw + row * SW + ch * 8, Wp + (size_t)row * CIN + ch * 8, true);
     }
-    load_halo<CIN, MODE>(sx, SIN, D, H, W, tx0, ty0, tz0, X, U, r, logk, rscale);
+    load_halo<CIN, MODE>(sx, SIN, D, H, W, tx0, ty0, tz0, X, U, nullptr, nullptr, nullptr);
+    cp_async_wait_all();
     __syncthreads();
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -542,7 +557,7 @@ k_conv3_tc(int D, int H, int W, const __grid_constant__ CUtensorMap xmap, const 
     __shared__ float sbias[16], swh[17];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     // with wh (16 input channels only) the output head is applied in the
-    // epilogue and out written instead of Y: out[v] = (sum_c wh[c] y[v][c] +
+    // epilogue and out written, and Y only if it is given: out[v] = (sum_c wh[c] y[v][c] +
     // wh[16]) rms s, summed in channel order, non-finite values flagged
     const bool head = CIN == 16 && wh != nullptr;
     const int nbx = (W + C::BX - 1) / C::BX, nby = (H + C::BY - 1) / C::BY, nbz = (D + C::BZ - 1) / C::BZ;
@@ -693,8 +708,8 @@ k_conv3_tc(int D, int H, int W, const __grid_constant__ CUtensorMap xmap, const 
                         }
                         const double o = (double)hs * (scal[0] * (double)out_scale);
                         out[vi] = o;
-                        if (!isfinite(o)) atomicOr(flag, 1);
-                        continue;
+                        if (flag && !isfinite(o)) atomicOr(flag, 1);
+                        if (!Y) continue;
                     }
                 }
                 uint4 *dst = (uint4 *)(Y + vi * 16 + c0);
@@ -728,34 +743,35 @@ __global__ void k_upsample2(int D, int H, int W, const bf16 *__restrict__ Uc, bf
 }
 
 // ---------------------------------------------------------------------------
-// weight gradient: partial[blk][t][co][ci] = sum over the brick of
-// G[v][co] * X[v + off_t][ci];  partial[blk][27*16*CIN + co] = sum_v G[v][co]
+// weight gradient of one convolution + ReLU: the gradient of the layer's
+// output (Gp) times its ReLU mask (Yact > 0) is G, written to Gm (if given)
+// for the data gradient; over a block's bricks,
+//   partial[blk][t][co][ci] = sum_v G[v][co] X[v + off_t][ci],
+//   partial[blk][27*16*CIN + co] = sum_v G[v][co].
+// The first layer (CIN = 8) has 2 real input channels.
+//
+// What bounds it: the latency of a brick's loads, then shared-memory reads
+// (one ldmatrix per two MMAs).  Persistent blocks, two to four per SM, keep
+// the sums of all their bricks in the MMA accumulators: a 64^3 layer leaves
+// 304 to 608 partial sums instead of 1024, and the halo comes by cp.async,
+// all of it in flight at once.
 // ---------------------------------------------------------------------------
+__host__ __device__ constexpr int dw_sin(int cin) { return cin == 32 ? 40 : 24; }   // conflict-free ldmatrix rows
+constexpr int dw_blocks_per_sm(int cin) { return cin == 32 ? 2 : cin == 16 ? 3 : 4; }
+
 template <int CIN, int MODE>
-__global__ void __launch_bounds__(CONV_THREADS)
+__global__ void __launch_bounds__(CONV_THREADS, dw_blocks_per_sm(CIN))
 k_conv3_dw(int D, int H, int W, const bf16 *__restrict__ X, const bf16 *__restrict__ U,
            const double *__restrict__ r, const double *__restrict__ logk, const double *__restrict__ rscale,
-           const bf16 *__restrict__ G, float *__restrict__ partial)
+           const bf16 *__restrict__ Gp, const bf16 *__restrict__ Yact, bf16 *__restrict__ Gm,
+           float *__restrict__ partial)
 {
-    constexpr int SIN = CIN + 8, SG = 24;
+    constexpr int SIN = dw_sin(CIN), SG = 24;
     extern __shared__ __align__(16) unsigned char smraw[];
     bf16 *sx = (bf16 *)smraw;
     bf16 *sg = sx + HVOX * SIN;
     const int ntx = (W + TX - 1) / TX, nty = (H + TY - 1) / TY;
-    int b = blockIdx.x;
-    const int tx0 = (b % ntx) * TX;
-    b /= ntx;
-    const int ty0 = (b % nty) * TY, tz0 = (b / nty) * TZ;
-    load_halo<CIN, MODE>(sx, SIN, D, H, W, tx0, ty0, tz0, X, U, r, logk, rscale);
-    for (int i = threadIdx.x; i < TVOX * 2; i += blockDim.x) {
-        const int tv = i >> 1, ch = i & 1;
-        const int lx = tv % TX, ly = (tv / TX) % TY, lz = tv / (TX * TY);
-        const int gx = tx0 + lx, gy = ty0 + ly, gz = tz0 + lz;
-        uint4 val = make_uint4(0, 0, 0, 0);
-        if (gx < W && gy < H && gz < D) val = *(const uint4 *)(G + (((int64_t)gz * H + gy) * W + gx) * 16 + ch * 8);
-        *(uint4 *)(sg + tv * SG + ch * 8) = val;
-    }
-    __syncthreads();
+    const int nbricks = ntx * nty * ((D + TZ - 1) / TZ);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int q = lane >> 3, rr = lane & 7;
     constexpr int NT = CIN / 8;
@@ -766,26 +782,68 @@ k_conv3_dw(int D, int H, int W, const bf16 *__restrict__ X, const bf16 *__restri
         for (int n = 0; n < NT; ++n)
 #pragma unroll
             for (int j = 0; j < 4; ++j) acc[a][n][j] = 0.f;
-    for (int row = 0; row < TY * TZ; ++row) {
-        const int ly = row % TY, lz = row / TY;
-        unsigned a0, a1, a2, a3;
-        // A = G^T: rows co, columns = the 16 voxels of this x-row
-        ldsm_x4_t(a0, a1, a2, a3, sg + (row * TX + (q >> 1) * 8 + rr) * SG + (q & 1) * 8);
+    float bsum = 0.f;                        // bias gradient: channel threadIdx.x % 16, voxels = threadIdx.x / 16 mod 16
+    for (int b = blockIdx.x; b < nbricks; b += gridDim.x) {
+        const int tx0 = (b % ntx) * TX, ty0 = ((b / ntx) % nty) * TY, tz0 = (b / (ntx * nty)) * TZ;
+        load_halo<CIN, MODE>(sx, SIN, D, H, W, tx0, ty0, tz0, X, U, r, logk, rscale);
+        uint4 gv[2], yv[2];
+        int64_t vi[2];
 #pragma unroll
-        for (int s = 0; s < 4; ++s) {
-            const int t = warp + 8 * s;
-            if (t >= 27) continue;
-            const int dz = t / 9, dy = (t / 3) % 3, dx = t % 3;
-            const int lx = (q & 1) * 8 + rr;
-            const int hv = ((lz + dz) * HY + (ly + dy)) * HX + lx + dx;
-#pragma unroll
-            for (int np = 0; np < NT / 2; ++np) {
-                unsigned b0, b1, b2, b3;
-                ldsm_x4_t(b0, b1, b2, b3, sx + hv * SIN + np * 16 + (q >> 1) * 8);
-                mma_bf16(acc[s][np * 2], a0, a1, a2, a3, b0, b1);
-                mma_bf16(acc[s][np * 2 + 1], a0, a1, a2, a3, b2, b3);
+        for (int u = 0; u < 2; ++u) {
+            const int i = threadIdx.x + u * CONV_THREADS, tv = i >> 1, ch = i & 1;
+            const int gx = tx0 + tv % TX, gy = ty0 + (tv / TX) % TY, gz = tz0 + tv / (TX * TY);
+            vi[u] = gx < W && gy < H && gz < D ? (((int64_t)gz * H + gy) * W + gx) * 16 + ch * 8 : -1;
+            gv[u] = yv[u] = make_uint4(0, 0, 0, 0);
+            if (vi[u] >= 0) {
+                gv[u] = *(const uint4 *)(Gp + vi[u]);
+                yv[u] = *(const uint4 *)(Yact + vi[u]);
             }
         }
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int i = threadIdx.x + u * CONV_THREADS;
+            const bf16 *ye = (const bf16 *)&yv[u];
+            bf16 *ge = (bf16 *)&gv[u];
+#pragma unroll
+            for (int c = 0; c < 8; ++c)
+                if (!(__bfloat162float(ye[c]) > 0.f)) ge[c] = __float2bfloat16_rn(0.f);
+            *(uint4 *)(sg + (i >> 1) * SG + (i & 1) * 8) = gv[u];
+            if (Gm && vi[u] >= 0) *(uint4 *)(Gm + vi[u]) = gv[u];
+        }
+        cp_async_wait_all();
+        __syncthreads();
+#pragma unroll 2
+        for (int row = 0; row < TY * TZ; ++row) {
+            const int ly = row % TY, lz = row / TY;
+            unsigned a0, a1, a2, a3;
+            // A = G^T: rows co, columns = the 16 voxels of this x-row
+            ldsm_x4_t(a0, a1, a2, a3, sg + (row * TX + (q >> 1) * 8 + rr) * SG + (q & 1) * 8);
+#pragma unroll
+            for (int s = 0; s < 4; ++s) {
+                const int t = warp + 8 * s;
+                if (t >= 27) continue;
+                const int dz = t / 9, dy = (t / 3) % 3, dx = t % 3;
+                const int lx = (q & 1) * 8 + rr;
+                const int hv = ((lz + dz) * HY + (ly + dy)) * HX + lx + dx;
+                if constexpr (NT == 1) {
+                    unsigned b0, b1;
+                    ldsm_x2_t(b0, b1, sx + hv * SIN);
+                    mma_bf16(acc[s][0], a0, a1, a2, a3, b0, b1);
+                } else {
+#pragma unroll
+                    for (int np = 0; np < NT / 2; ++np) {
+                        unsigned b0, b1, b2, b3;
+                        ldsm_x4_t(b0, b1, b2, b3, sx + hv * SIN + np * 16 + (q >> 1) * 8);
+                        mma_bf16(acc[s][np * 2], a0, a1, a2, a3, b0, b1);
+                        mma_bf16(acc[s][np * 2 + 1], a0, a1, a2, a3, b2, b3);
+                    }
+                }
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < TVOX / 16; ++k)
+            bsum += __bfloat162float(sg[((threadIdx.x >> 4) + 16 * k) * SG + (threadIdx.x & 15)]);
+        __syncthreads();                     // before the next brick's loads
     }
     float *out = partial + (size_t)blockIdx.x * (27 * 16 * CIN + 16);
 #pragma unroll
@@ -795,41 +853,55 @@ k_conv3_dw(int D, int H, int W, const bf16 *__restrict__ X, const bf16 *__restri
 #pragma unroll
         for (int n = 0; n < NT; ++n) {
             const int co = lane >> 2, ci = n * 8 + (lane & 3) * 2;
-            out[(t * 16 + co) * CIN + ci] = acc[s][n][0];
-            out[(t * 16 + co) * CIN + ci + 1] = acc[s][n][1];
-            out[(t * 16 + co + 8) * CIN + ci] = acc[s][n][2];
-            out[(t * 16 + co + 8) * CIN + ci + 1] = acc[s][n][3];
+            *(float2 *)(out + (t * 16 + co) * CIN + ci) = make_float2(acc[s][n][0], acc[s][n][1]);
+            *(float2 *)(out + (t * 16 + co + 8) * CIN + ci) = make_float2(acc[s][n][2], acc[s][n][3]);
         }
     }
-    // bias gradient: sum of G over the brick
+    float *sb = (float *)smraw;              // bias sums of the 16 voxel groups, added in group order
+    sb[threadIdx.x] = bsum;
+    __syncthreads();
     if (threadIdx.x < 16) {
         float sum = 0.f;
-        for (int tv = 0; tv < TVOX; ++tv) sum += __bfloat162float(sg[tv * SG + threadIdx.x]);
+#pragma unroll
+        for (int k = 0; k < 16; ++k) sum += sb[k * 16 + threadIdx.x];
         out[27 * 16 * CIN + threadIdx.x] = sum;
     }
 }
 
-// grad[woff + (t*16+co)*cin + ci] += w * sum_b partial[b][(t*16+co)*cinp + ci]; bias likewise
-__global__ void k_dw_reduce(int nblocks, int cin, int cinp, const float *__restrict__ partial, float *grad,
-                            int64_t woff, int64_t boff, float wscale)
+// grad[woff + (t*16+co)*cin + ci] += w * sum_b partial[b][(t*16+co)*cinp + ci];
+// bias likewise.  A block sums 32 outputs, 16 threads each over every 16th
+// partial (coalesced 128-byte reads, four in flight); with one thread per
+// output over all 1024 partials of a 64^3 layer the 14 layers' sums took 730
+// of the training pass's 1290 us.
+#define DWR_GROUPS 16
+__global__ void __launch_bounds__(32 * DWR_GROUPS)
+k_dw_reduce(int nblocks, int cin, int cinp, const float *__restrict__ partial, float *grad, int64_t woff, int64_t boff,
+            float wscale)
 {
+    __shared__ float sm[DWR_GROUPS][32];
     const int stride = 27 * 16 * cinp + 16;
-    const int nw = 27 * 16 * cin;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nw + 16; i += gridDim.x * blockDim.x) {
-        int src;
-        int64_t dst;
-        if (i < nw) {
-            const int tc = i / cin, ci = i % cin;
-            src = tc * cinp + ci;
-            dst = woff + i;
-        } else {
-            src = 27 * 16 * cinp + (i - nw);
-            dst = boff + (i - nw);
+    const int c = threadIdx.x & 31, g = threadIdx.x >> 5;
+    const int src = blockIdx.x * 32 + c;
+    float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
+    if (src < stride) {
+        const float *p = partial + src;
+        int b = g;
+        for (; b + 3 * DWR_GROUPS < nblocks; b += 4 * DWR_GROUPS) {
+            s0 += p[(size_t)b * stride];
+            s1 += p[(size_t)(b + DWR_GROUPS) * stride];
+            s2 += p[(size_t)(b + 2 * DWR_GROUPS) * stride];
+            s3 += p[(size_t)(b + 3 * DWR_GROUPS) * stride];
         }
-        float s = 0.f;
-        for (int bk = 0; bk < nblocks; ++bk) s += partial[(size_t)bk * stride + src];
-        grad[dst] += wscale * s;
+        for (; b < nblocks; b += DWR_GROUPS) s0 += p[(size_t)b * stride];
     }
+    sm[g][c] = (s0 + s1) + (s2 + s3);
+    __syncthreads();
+    if (g || src >= stride) return;
+    float t = 0.f;
+#pragma unroll
+    for (int k = 0; k < DWR_GROUPS; ++k) t += sm[k][c];
+    if (src >= 27 * 16 * cinp) grad[boff + src - 27 * 16 * cinp] += wscale * t;
+    else if (src % cinp < cin) grad[woff + (src / cinp) * cin + src % cinp] += wscale * t;
 }
 
 // ---------------------------------------------------------------------------
@@ -870,46 +942,57 @@ __global__ void k_avgpool(int Dc, int Hc, int Wc, const bf16 *__restrict__ X, bf
     }
 }
 
-// g_pre = g * (y > 0)
-__global__ void k_relu_mask(int64_t n, const bf16 *__restrict__ g, const bf16 *__restrict__ y, bf16 *__restrict__ out)
-{
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        out[i] = __bfloat162float(y[i]) > 0.f ? g[i] : __float2bfloat16_rn(0.f);
-}
-
 // coarse gradient of a nearest-upsampled input: sum over the 8 children of
-// channels 0..15 of a 32-channel fine gradient
+// channels 0..15 of a 32-channel fine gradient; a thread per coarse voxel and
+// 8-channel half, 16-byte loads
 __global__ void k_up_backward(int Dc, int Hc, int Wc, const bf16 *__restrict__ gcat, bf16 *__restrict__ gc)
 {
-    const int64_t n = (int64_t)Dc * Hc * Wc * 16;
+    const int64_t n = (int64_t)Dc * Hc * Wc * 2;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const int c = (int)(i % 16);
-        const int64_t vc = i / 16;
+        const int h = (int)(i & 1);
+        const int64_t vc = i >> 1;
         const int x = (int)(vc % Wc), y = (int)((vc / Wc) % Hc), z = (int)(vc / ((int64_t)Wc * Hc));
         const int W = Wc * 2, H = Hc * 2;
-        float s = 0.f;
+        uint4 in[8];
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
             const int64_t vf = ((int64_t)(2 * z + (k >> 2)) * H + (2 * y + ((k >> 1) & 1))) * W + 2 * x + (k & 1);
-            s += __bfloat162float(gcat[vf * 32 + c]);
+            in[k] = *(const uint4 *)(gcat + vf * 32 + h * 8);
         }
-        gc[i] = __float2bfloat16_rn(s);
+        uint4 o;
+        bf16 *oe = (bf16 *)&o;
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+            float s = 0.f;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) s += __bfloat162float(((const bf16 *)&in[k])[c]);
+            oe[c] = __float2bfloat16_rn(s);
+        }
+        *(uint4 *)(gc + vc * 16 + h * 8) = o;
     }
 }
 
 // gradient of a skip tensor: skip part of the decoder's gradient (channels
-// 16..31 of gcat) plus the average-pooling adjoint of the coarse gradient
+// 16..31 of gcat) plus the average-pooling adjoint of the coarse gradient;
+// a thread per voxel and 8-channel half
 __global__ void k_pool_backward_add(int D, int H, int W, const bf16 *__restrict__ gcoarse,
                                     const bf16 *__restrict__ gcat, bf16 *__restrict__ out)
 {
-    const int64_t n = (int64_t)D * H * W * 16;
+    const int64_t n = (int64_t)D * H * W * 2;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const int c = (int)(i % 16);
-        const int64_t v = i / 16;
+        const int h = (int)(i & 1);
+        const int64_t v = i >> 1;
         const int x = (int)(v % W), y = (int)((v / W) % H), z = (int)(v / ((int64_t)W * H));
         const int64_t vc = ((int64_t)(z >> 1) * (H >> 1) + (y >> 1)) * (W >> 1) + (x >> 1);
-        const float s = __bfloat162float(gcat[v * 32 + 16 + c]) + 0.125f * __bfloat162float(gcoarse[vc * 16 + c]);
-        out[i] = __float2bfloat16_rn(s);
+        const uint4 a = *(const uint4 *)(gcat + v * 32 + 16 + h * 8);
+        const uint4 b = *(const uint4 *)(gcoarse + vc * 16 + h * 8);
+        const bf16 *ae = (const bf16 *)&a, *be = (const bf16 *)&b;
+        uint4 o;
+        bf16 *oe = (bf16 *)&o;
+#pragma unroll
+        for (int c = 0; c < 8; ++c)
+            oe[c] = __float2bfloat16_rn(__bfloat162float(ae[c]) + 0.125f * __bfloat162float(be[c]));
+        *(uint4 *)(out + v * 16 + h * 8) = o;
     }
 }
 
@@ -969,29 +1052,7 @@ k_rms(int64_t n, const double *__restrict__ r, double *red, unsigned *ticket, do
     }
 }
 
-// head: out[v] = (sum_c wh[c] x[v][c] + bh) * rms * s; flags non-finite output
-__global__ void k_head(int64_t n, const bf16 *__restrict__ x, const float *__restrict__ wh, const double *__restrict__ scal,
-                       float out_scale, double *__restrict__ out, int *flag, const int *skip)
-{
-    if (skipped(skip)) return;
-    const double sc = scal[0] * (double)out_scale;
-    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
-        const uint4 *p = (const uint4 *)(x + v * 16);
-        const uint4 a = p[0], b = p[1];
-        const bf16 *e0 = (const bf16 *)&a, *e1 = (const bf16 *)&b;
-        float s = wh[16];
-#pragma unroll
-        for (int c = 0; c < 8; ++c) s = fmaf(wh[c], __bfloat162float(e0[c]), s);
-#pragma unroll
-        for (int c = 0; c < 8; ++c) s = fmaf(wh[8 + c], __bfloat162float(e1[c]), s);
-        const double o = (double)s * sc;
-        out[v] = o;
-        if (flag && !isfinite(o)) atomicOr(flag, 1);
-    }
-}
-
-// loss = sum (o - e)^2 / sum e^2 (two sums with a last-block finish), and
-// gout = w * 2 (o - e) / sum e^2 computed after the sums by k_loss_grad
+// loss = sum (o - e)^2 / sum e^2: two sums with a last-block finish
 __global__ void __launch_bounds__(256)
 k_loss_sums(int64_t n, const double *__restrict__ o, const double *__restrict__ e, double *red, unsigned *ticket,
             double *scal)
@@ -1017,69 +1078,81 @@ k_loss_sums(int64_t n, const double *__restrict__ o, const double *__restrict__ 
         last = atomicAdd(ticket, 1u) == gridDim.x - 1;
     }
     __syncthreads();
-    if (!last || threadIdx.x >= 32) return;
+    if (!last) return;
     __threadfence();
     double a = 0.0, b = 0.0;
-    for (int bk = threadIdx.x; bk < (int)gridDim.x; bk += 32) { a += __ldcg(red + 2 * bk); b += __ldcg(red + 2 * bk + 1); }
+    for (int bk = threadIdx.x; bk < (int)gridDim.x; bk += blockDim.x) { a += __ldcg(red + 2 * bk); b += __ldcg(red + 2 * bk + 1); }
     a = warp_sum(a);
     b = warp_sum(b);
+    if ((threadIdx.x & 31) == 0) { sm[0][threadIdx.x >> 5] = a; sm[1][threadIdx.x >> 5] = b; }
+    __syncthreads();
     if (threadIdx.x == 0) {
+        a = b = 0.0;
+        for (int k = 0; k < 8; ++k) { a += sm[0][k]; b += sm[1][k]; }
         scal[2] = b > 0.0 ? a / b : 0.0;
         scal[3] = b;
         *ticket = 0;
     }
 }
 
-__global__ void k_loss_grad(int64_t n, const double *__restrict__ o, const double *__restrict__ e,
-                            const double *__restrict__ scal, double w, double *__restrict__ g)
-{
-    const double den = scal[3] > 0.0 ? scal[3] : 1.0;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        g[i] = w * 2.0 * (o[i] - e[i]) / den;
-}
-
-// head backward: ge = g * rms * s; dx[v][c] = ge * wh[c]; per-block partial
-// sums of ge * x[v][c] (16) and ge (1) into hp[block][17]
+// loss and head backward: dL/d(out) = w 2 (o - e) / sum e^2; ge = that *
+// rms * s; dx[v][c] = ge * wh[c]; per-block partial sums of ge * x[v][c] (16)
+// and ge (1) into hp[block][17].  A thread per voxel, 16-byte accesses.
 __global__ void __launch_bounds__(256)
 k_head_backward(int64_t n, const bf16 *__restrict__ x, const float *__restrict__ wh, const double *__restrict__ scal,
-                float out_scale, const double *__restrict__ g, bf16 *__restrict__ dx, float *__restrict__ hp)
+                float out_scale, const double *__restrict__ o, const double *__restrict__ e, double w,
+                bf16 *__restrict__ dx, float *__restrict__ hp)
 {
     __shared__ float sm[8][17];
     const double sc = scal[0] * (double)out_scale;
-    float acc[17];
+    const double den = scal[3] > 0.0 ? scal[3] : 1.0;
+    float acc[17], whr[16];
 #pragma unroll
     for (int c = 0; c < 17; ++c) acc[c] = 0.f;
+#pragma unroll
+    for (int c = 0; c < 16; ++c) whr[c] = wh[c];
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
-        const float ge = (float)(g[v] * sc);
+        uint4 in[2], od[2];
+        in[0] = *(const uint4 *)(x + v * 16);
+        in[1] = *(const uint4 *)(x + v * 16 + 8);
+        const double g = w * 2.0 * (o[v] - e[v]) / den;
+        const float ge = (float)(g * sc);
+        const bf16 *ie = (const bf16 *)in;
+        bf16 *oe = (bf16 *)od;
 #pragma unroll
         for (int c = 0; c < 16; ++c) {
-            acc[c] = fmaf(ge, __bfloat162float(x[v * 16 + c]), acc[c]);
-            dx[v * 16 + c] = __float2bfloat16_rn(ge * wh[c]);
+            acc[c] = fmaf(ge, __bfloat162float(ie[c]), acc[c]);
+            oe[c] = __float2bfloat16_rn(ge * whr[c]);
         }
         acc[16] += ge;
+        *(uint4 *)(dx + v * 16) = od[0];
+        *(uint4 *)(dx + v * 16 + 8) = od[1];
     }
 #pragma unroll
     for (int c = 0; c < 17; ++c) {
         float s = acc[c];
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        for (int k = 16; k > 0; k >>= 1) s += __shfl_xor_sync(0xffffffffu, s, k);
         if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5][c] = s;
     }
     __syncthreads();
     if (threadIdx.x < 17) {
         float s = 0.f;
-        for (int w = 0; w < 8; ++w) s += sm[w][threadIdx.x];
+        for (int k = 0; k < 8; ++k) s += sm[k][threadIdx.x];
         hp[blockIdx.x * 17 + threadIdx.x] = s;
     }
 }
 
-__global__ void k_head_reduce(int nblocks, const float *__restrict__ hp, float *grad, int64_t hoff)
+// a warp per head parameter
+__global__ void __launch_bounds__(17 * 32)
+k_head_reduce(int nblocks, const float *__restrict__ hp, float *grad, int64_t hoff)
 {
-    const int c = threadIdx.x;
-    if (c >= 17) return;
+    const int c = threadIdx.x >> 5, lane = threadIdx.x & 31;
     float s = 0.f;
-    for (int b = 0; b < nblocks; ++b) s += hp[b * 17 + c];
-    grad[hoff + c] += s;
+    for (int b = lane; b < nblocks; b += 32) s += hp[b * 17 + c];
+#pragma unroll
+    for (int k = 16; k > 0; k >>= 1) s += __shfl_xor_sync(0xffffffffu, s, k);
+    if (lane == 0) grad[hoff + c] += s;
 }
 
 // FP32 master -> bf16 forward [27][16][cinp] and data-gradient [27][cin][16] weights
@@ -1112,7 +1185,7 @@ __global__ void k_adam(int64_t n, float *p, float *g, float *m, float *v, float 
 // host side
 // ---------------------------------------------------------------------------
 static int conv_smem(int cin, int cout) { return (HVOX * (cin + 8) + 27 * cout * (cin + 8)) * 2; }
-static int dw_smem(int cin) { return (HVOX * (cin + 8) + TVOX * 24) * 2; }
+static int dw_smem(int cin) { return (HVOX * dw_sin(cin) + TVOX * 24) * 2; }
 
 static int64_t nbricks(const Level &L)
 {
@@ -1142,11 +1215,10 @@ static void ensure_attrs()
 {
     if (g_attrs_set) return;
     set_attr<16, 16, IN_PLAIN>();
-    set_attr<16, 16, IN_FIRST>();
     set_attr<32, 16, IN_CATUP>();
     set_attr<16, 32, IN_PLAIN>();
     set_attr_dw<16, IN_PLAIN>();
-    set_attr_dw<16, IN_FIRST>();
+    set_attr_dw<8, IN_FIRST>();
     set_attr_dw<32, IN_CATUP>();
     cudaFuncSetAttribute(k_conv3_tc<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, TcCfg<16>::SMEM);
     cudaFuncSetAttribute(k_conv3_tc<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, TcCfg<32>::SMEM);
@@ -1224,11 +1296,9 @@ static void free_workspace(rs_net *net)
         net->pool[l] = net->g16a[l] = net->g16b[l] = net->g32[l] = nullptr;
     }
     rs_free(c, net->partials);
-    rs_free(c, net->gout);
     rs_free(c, net->outb);
     rs_free(c, net->headpart);
     net->partials = nullptr;
-    net->gout = nullptr;
     net->outb = nullptr;
     net->headpart = nullptr;
     net->nx = net->ny = net->nz = 0;
@@ -1257,12 +1327,12 @@ static int ensure_workspace(rs_net *net, int nx, int ny, int nz)
         if (!st) st = rs_alloc(c, (void **)&net->g16a[l], sizeof(bf16) * 16 * nv);
         if (!st) st = rs_alloc(c, (void **)&net->g16b[l], sizeof(bf16) * 16 * nv);
         if (!st) st = rs_alloc(c, (void **)&net->g32[l], sizeof(bf16) * 32 * nv);
-        maxp = std::max(maxp, nbricks(net->lv[l]) * (27 * 16 * 32 + 16));
+        // at most the blocks of k_conv3_dw: 2 per SM with 32 input channels (3 with 16 are less)
+        maxp = std::max(maxp, std::min<int64_t>(nbricks(net->lv[l]), 2 * c->num_sms) * (27 * 16 * 32 + 16));
     }
     if (!st) st = rs_alloc(c, (void **)&net->partials, sizeof(float) * maxp);
-    if (!st) st = rs_alloc(c, (void **)&net->gout, sizeof(double) * net->lv[0].nvox);
     if (!st) st = rs_alloc(c, (void **)&net->outb, sizeof(double) * net->lv[0].nvox);
-    if (!st) st = rs_alloc(c, (void **)&net->headpart, sizeof(float) * 17 * c->num_sms * 8);
+    if (!st) st = rs_alloc(c, (void **)&net->headpart, sizeof(float) * 17 * c->num_sms * 4);
     if (st) { free_workspace(net); return st; }
     net->partials_len = maxp;
     net->nx = nx;
@@ -1297,7 +1367,8 @@ static bool use_tc(const rs_net *net, int level)
 }
 
 // hout: the last layer applies the output head in its epilogue and writes
-// the network output there instead of Y (finest level, tcgen05 kernel only)
+// the network output there, and Y if it is not null (finest level, tcgen05
+// kernel only)
 static int conv_forward(rs_net *net, int l, const bf16 *X, const bf16 *U, const double *r, const double *logk,
                         bf16 *Y, const int *skip, double *hout = nullptr)
 {
@@ -1336,11 +1407,11 @@ static int conv_forward(rs_net *net, int l, const bf16 *X, const bf16 *U, const 
         break;
     case IN_CATUP:
         k_conv3<32, 16, IN_CATUP><<<grid, CONV_THREADS, conv_smem(32, 16), c->stream>>>(
-            L.nz, L.ny, L.nx, X, U, nullptr, nullptr, nullptr, net->wf[l], bias, 1, Y, skip);
+            L.nz, L.ny, L.nx, X, U, net->wf[l], bias, 1, Y, skip);
         break;
     default:
         k_conv3<16, 16, IN_PLAIN><<<grid, CONV_THREADS, conv_smem(16, 16), c->stream>>>(
-            L.nz, L.ny, L.nx, X, nullptr, nullptr, nullptr, nullptr, net->wf[l], bias, 1, Y, skip);
+            L.nz, L.ny, L.nx, X, nullptr, net->wf[l], bias, 1, Y, skip);
     }
     return rs_check_launch(c);
 }
@@ -1354,7 +1425,7 @@ static int pool_forward(rs_net *net, int lvl, const bf16 *X, bf16 *Y, const int 
 }
 
 // forward pass; out (FP64, nvox) = network(r, logk) * rms * out_scale.
-// keep: the last layer's activations are kept for a backward pass; else the
+// keep: the last layer's activations are kept for a backward pass.  The
 // output head runs in the last convolution's epilogue
 static int net_forward(rs_net *net, const double *r, const double *logk, double *out, const int *skip,
                        bool keep = false)
@@ -1383,39 +1454,35 @@ static int net_forward(rs_net *net, const double *r, const double *logk, double 
     RS_TRY(conv_forward(net, D1A, A[E1B], A[D2B], nullptr, nullptr, A[D1A], skip));
     RS_TRY(conv_forward(net, D1B, A[D1A], nullptr, nullptr, nullptr, A[D1B], skip));
     RS_TRY(conv_forward(net, D0A, A[E0B], A[D1B], nullptr, nullptr, A[D0A], skip));
-    if (!keep) return conv_forward(net, D0B, A[D0A], nullptr, nullptr, nullptr, A[D0B], skip, out);
-    RS_TRY(conv_forward(net, D0B, A[D0A], nullptr, nullptr, nullptr, A[D0B], skip));
-    k_head<<<ew_grid(c, n0), 256, 0, c->stream>>>(n0, A[D0B], net->p + net->hoff, net->scal, net->out_scale, out,
-                                                 net->flag, skip);
-    return rs_check_launch(c);
+    return conv_forward(net, D0B, A[D0A], nullptr, nullptr, nullptr, keep ? A[D0B] : nullptr, skip, out);
 }
 
-// weight gradient of layer l for output gradient G (pre-activation), input as in the forward pass
-static int conv_dw(rs_net *net, int l, const bf16 *X, const bf16 *U, const double *r, const double *logk,
-                   const bf16 *G, float wscale)
+// weight gradient of layer l from the gradient Gp of its output, input as in
+// the forward pass; the pre-activation gradient goes to Gm (if not null)
+template <int CIN, int MODE>
+static int launch_dw(rs_net *net, int l, const bf16 *X, const bf16 *U, const double *r, const double *logk,
+                     const bf16 *Gp, bf16 *Gm, float wscale)
 {
     rs_ctx *c = net->ctx;
     const Level &L = net->lv[kLayers[l].level];
-    const int grid = (int)nbricks(L);
-    RsProfScope prof(c, RS_PROF_NET);
-    switch (kLayers[l].mode) {
-    case IN_FIRST:
-        k_conv3_dw<16, IN_FIRST><<<grid, CONV_THREADS, dw_smem(16), c->stream>>>(L.nz, L.ny, L.nx, nullptr, nullptr, r,
-                                                                                logk, net->scal + 1, G, net->partials);
-        break;
-    case IN_CATUP:
-        k_conv3_dw<32, IN_CATUP><<<grid, CONV_THREADS, dw_smem(32), c->stream>>>(L.nz, L.ny, L.nx, X, U, nullptr,
-                                                                                nullptr, nullptr, G, net->partials);
-        break;
-    default:
-        k_conv3_dw<16, IN_PLAIN><<<grid, CONV_THREADS, dw_smem(16), c->stream>>>(L.nz, L.ny, L.nx, X, nullptr, nullptr,
-                                                                                nullptr, nullptr, G, net->partials);
-    }
+    const int grid = (int)std::min<int64_t>(nbricks(L), (int64_t)dw_blocks_per_sm(CIN) * c->num_sms);
+    k_conv3_dw<CIN, MODE><<<grid, CONV_THREADS, dw_smem(CIN), c->stream>>>(
+        L.nz, L.ny, L.nx, X, U, r, logk, net->scal + 1, Gp, net->act[l], Gm, net->partials);
     RS_TRY(rs_check_launch(c));
-    const int cin = kLayers[l].cin, cinp = cin_pad(l);
-    k_dw_reduce<<<ew_grid(c, 27 * 16 * cin + 16), 256, 0, c->stream>>>(grid, cin, cinp, net->partials, net->g,
-                                                                        net->woff[l], net->boff[l], wscale);
+    k_dw_reduce<<<(27 * 16 * CIN + 16 + 31) / 32, 32 * DWR_GROUPS, 0, c->stream>>>(
+        grid, kLayers[l].cin, CIN, net->partials, net->g, net->woff[l], net->boff[l], wscale);
     return rs_check_launch(c);
+}
+
+static int conv_dw(rs_net *net, int l, const bf16 *X, const bf16 *U, const double *r, const double *logk,
+                   const bf16 *Gp, bf16 *Gm, float wscale)
+{
+    RsProfScope prof(net->ctx, RS_PROF_NET);
+    switch (kLayers[l].mode) {
+    case IN_FIRST: return launch_dw<8, IN_FIRST>(net, l, X, U, r, logk, Gp, Gm, wscale);
+    case IN_CATUP: return launch_dw<32, IN_CATUP>(net, l, X, U, r, logk, Gp, Gm, wscale);
+    default: return launch_dw<16, IN_PLAIN>(net, l, X, U, r, logk, Gp, Gm, wscale);
+    }
 }
 
 // data gradient: dX = conv(G, flipped transposed weights)
@@ -1427,18 +1494,10 @@ static int conv_dx(rs_net *net, int l, const bf16 *G, bf16 *dX)
     RsProfScope prof(c, RS_PROF_NET);
     if (kLayers[l].cin == 32)
         k_conv3<16, 32, IN_PLAIN><<<grid, CONV_THREADS, conv_smem(16, 32), c->stream>>>(
-            L.nz, L.ny, L.nx, G, nullptr, nullptr, nullptr, nullptr, net->wb[l], nullptr, 0, dX, nullptr);
+            L.nz, L.ny, L.nx, G, nullptr, net->wb[l], nullptr, 0, dX, nullptr);
     else
         k_conv3<16, 16, IN_PLAIN><<<grid, CONV_THREADS, conv_smem(16, 16), c->stream>>>(
-            L.nz, L.ny, L.nx, G, nullptr, nullptr, nullptr, nullptr, net->wb[l], nullptr, 0, dX, nullptr);
-    return rs_check_launch(c);
-}
-
-static int relu_mask(rs_net *net, int lvl, const bf16 *g, const bf16 *y, bf16 *out)
-{
-    rs_ctx *c = net->ctx;
-    const int64_t n = net->lv[lvl].nvox * 16;
-    k_relu_mask<<<ew_grid(c, n), 256, 0, c->stream>>>(n, g, y, out);
+            L.nz, L.ny, L.nx, G, nullptr, net->wb[l], nullptr, 0, dX, nullptr);
     return rs_check_launch(c);
 }
 
@@ -1447,24 +1506,23 @@ static int relu_mask(rs_net *net, int lvl, const bf16 *g, const bf16 *y, bf16 *o
 static int layer_backward(rs_net *net, int l, const bf16 *g_post, bf16 *gpre, const bf16 *X, const bf16 *U,
                           const double *r, const double *logk, bf16 *dX, float wscale)
 {
-    const int lvl = kLayers[l].level;
-    RS_TRY(relu_mask(net, lvl, g_post, net->act[l], gpre));
-    RS_TRY(conv_dw(net, l, X, U, r, logk, gpre, wscale));
+    RS_TRY(conv_dw(net, l, X, U, r, logk, g_post, dX ? gpre : nullptr, wscale));
     if (dX) RS_TRY(conv_dx(net, l, gpre, dX));
     return RS_OK;
 }
 
-static int net_backward(rs_net *net, const double *r, const double *logk, float wscale)
+static int net_backward(rs_net *net, const double *r, const double *logk, const double *e, double weight,
+                        float wscale)
 {
     rs_ctx *c = net->ctx;
     bf16 **A = net->act;
     const int64_t n0 = net->lv[0].nvox;
     {
         RsProfScope prof(c, RS_PROF_NET);
-        const int hb = std::min<int64_t>((n0 + 255) / 256, (int64_t)c->num_sms * 8);
+        const int hb = std::min<int64_t>((n0 + 255) / 256, (int64_t)c->num_sms * 4);
         k_head_backward<<<hb, 256, 0, c->stream>>>(n0, A[D0B], net->p + net->hoff, net->scal, net->out_scale,
-                                                   net->gout, net->g16a[0], net->headpart);
-        k_head_reduce<<<1, 32, 0, c->stream>>>(hb, net->headpart, net->g, net->hoff);
+                                                   net->outb, e, weight, net->g16a[0], net->headpart);
+        k_head_reduce<<<1, 17 * 32, 0, c->stream>>>(hb, net->headpart, net->g, net->hoff);
         c->launches++;
         RS_TRY(rs_check_launch(c));
     }
@@ -1478,7 +1536,7 @@ static int net_backward(rs_net *net, const double *r, const double *logk, float 
         RS_TRY(layer_backward(net, la, net->g16a[lvl], net->g16b[lvl], A[skip_src[lvl]], A[up_src[lvl]], nullptr,
                               nullptr, net->g32[lvl], wscale));
         const Level &C = net->lv[lvl + 1];
-        k_up_backward<<<ew_grid(c, C.nvox * 16), 256, 0, c->stream>>>(C.nz, C.ny, C.nx, net->g32[lvl], net->g16a[lvl + 1]);
+        k_up_backward<<<ew_grid(c, C.nvox * 2), 256, 0, c->stream>>>(C.nz, C.ny, C.nx, net->g32[lvl], net->g16a[lvl + 1]);
         RS_TRY(rs_check_launch(c));
     }
     // encoder, coarse to fine
@@ -1493,7 +1551,7 @@ static int net_backward(rs_net *net, const double *r, const double *logk, float 
             RS_TRY(layer_backward(net, la, net->g16a[lvl], net->g16b[lvl], net->pool[lvl], nullptr, nullptr, nullptr,
                                   net->g16a[lvl], wscale));
             const Level &F = net->lv[lvl - 1];
-            k_pool_backward_add<<<ew_grid(c, F.nvox * 16), 256, 0, c->stream>>>(F.nz, F.ny, F.nx, net->g16a[lvl],
+            k_pool_backward_add<<<ew_grid(c, F.nvox * 2), 256, 0, c->stream>>>(F.nz, F.ny, F.nx, net->g16a[lvl],
                                                                                  net->g32[lvl - 1], net->g16a[lvl - 1]);
             RS_TRY(rs_check_launch(c));
         }
@@ -1635,10 +1693,8 @@ extern "C" int rs_net_accumulate(rs_net *net, int32_t nx, int32_t ny, int32_t nz
     const int64_t n0 = net->lv[0].nvox;
     RS_TRY(net_forward(net, r, logk, net->outb, nullptr, true));
     k_loss_sums<<<c->red_blocks, 256, 0, c->stream>>>(n0, net->outb, e, net->red, net->ticket, net->scal);
-    k_loss_grad<<<ew_grid(c, n0), 256, 0, c->stream>>>(n0, net->outb, e, net->scal, weight, net->gout);
-    c->launches++;
     RS_TRY(rs_check_launch(c));
-    RS_TRY(net_backward(net, r, logk, 1.0f));
+    RS_TRY(net_backward(net, r, logk, e, weight, 1.0f));
     if (loss_host) {
         RS_CUDA_TRY(cudaMemcpyAsync(c->h_pinned + 8, net->scal + 2, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
         RS_CUDA_TRY(cudaStreamSynchronize(c->stream));
