@@ -344,6 +344,12 @@ k_dot(int n, const double *__restrict__ x, const double *__restrict__ y, double 
     }
 }
 
+// no block without elements: the last block adds one partial per block
+static int dot_grid(rs_ctx *ctx, int n)
+{
+    return std::max(1, std::min(ctx->red_blocks, (n + RS_RED_THREADS - 1) / RS_RED_THREADS));
+}
+
 int rs_axpby_launch(rs_ctx *ctx, int n, double a, const double *x, double b, double *y)
 {
     if (n <= 0) return RS_OK;
@@ -359,7 +365,7 @@ int rs_dot_launch(rs_ctx *ctx, int n, const double *x, const double *y, double *
         return RS_OK;
     }
     RsProfScope prof(ctx, RS_PROF_BLAS1);
-    k_dot<<<ctx->red_blocks, RS_RED_THREADS, 0, ctx->stream>>>(n, x, y, ctx->red_partials,
+    k_dot<<<dot_grid(ctx, n), RS_RED_THREADS, 0, ctx->stream>>>(n, x, y, ctx->red_partials,
                                                                ctx->red_ticket, out_dev, 0);
     return rs_check_launch(ctx);
 }
@@ -458,7 +464,7 @@ extern "C" int rs_vec_axpbyz(double a, const rs_vec *x, double b, const rs_vec *
 static int dot_to_host(rs_ctx *ctx, int n, const double *x, const double *y, int sq, double *out)
 {
     if (n == 0) { *out = 0.0; return RS_OK; }
-    k_dot<<<ctx->red_blocks, RS_RED_THREADS, 0, ctx->stream>>>(n, x, y, ctx->red_partials,
+    k_dot<<<dot_grid(ctx, n), RS_RED_THREADS, 0, ctx->stream>>>(n, x, y, ctx->red_partials,
                                                                ctx->red_ticket, ctx->d_scalars, sq);
     RS_TRY(rs_check_launch(ctx));
     RS_CUDA_TRY(cudaMemcpyAsync(ctx->h_pinned, ctx->d_scalars, sizeof(double),

@@ -33,6 +33,7 @@ struct GmresDev {
     int iters, k, cycle_done, converged, maxit, m, noupd, status;
     double augn2;           // ||Z y||^2 of the last cycle (LGMRES)
     double *hist;           // residual history (device), hist_len entries
+    int *host_done;         // pinned host copy of cycle_done
     int hist_len, pad_;
 };
 
@@ -329,31 +330,50 @@ k_cgs_pass(int n, int ld, int nc, const double *__restrict__ V, double *w, doubl
     } else {
         double a1[1] = {extra};
         if (reduce_partials<1, C::NW>(a1, 1, partials, ticket, &d->r2)) {
+            // the new Hessenberg column and the rotations through shared
+            // memory: one thread's chain of rotations then waits for no load
+            // (the ring is free: every tile has been consumed)
+            const int i = nc - 1, m1 = d->m + 1;
+            double *h = ring, *cs = ring + NC + 1, *sn = ring + 2 * NC + 2;
+            double *hcol = d->H + (size_t)i * m1;
+            for (int k = threadIdx.x; k < nc; k += blockDim.x) {
+                h[k] = hcol[k];
+                cs[k] = d->cs[k];
+                sn[k] = d->sn[k];
+            }
+            __syncthreads();
             if (threadIdx.x == 0) {
-                const int i = nc - 1, m1 = d->m + 1;
-                double *h = d->H + (size_t)i * m1;
                 const double hnext = sqrt(d->r2);
+                double a = h[0];
                 for (int k = 0; k < i; ++k) {
-                    const double a = h[k], b = h[k + 1];
-                    h[k] = __dadd_rn(__dmul_rn(d->cs[k], a), __dmul_rn(d->sn[k], b));
-                    h[k + 1] = __dadd_rn(__dmul_rn(-d->sn[k], a), __dmul_rn(d->cs[k], b));
+                    const double b = h[k + 1];
+                    h[k] = __dadd_rn(__dmul_rn(cs[k], a), __dmul_rn(sn[k], b));
+                    a = __dadd_rn(__dmul_rn(-sn[k], a), __dmul_rn(cs[k], b));
                 }
-                const double rho = hypot(h[i], hnext);
-                d->cs[i] = __ddiv_rn(h[i], rho);
-                d->sn[i] = __ddiv_rn(hnext, rho);
+                const double rho = hypot(a, hnext);
+                const double c = __ddiv_rn(a, rho), s = __ddiv_rn(hnext, rho), g = d->g[i];
+                d->cs[i] = c;
+                d->sn[i] = s;
                 h[i] = rho;
-                h[i + 1] = 0.0;
-                d->g[i + 1] = __dmul_rn(-d->sn[i], d->g[i]);
-                d->g[i] = __dmul_rn(d->cs[i], d->g[i]);
-                d->iters += 1;
+                h[nc] = 0.0;
+                const double g1 = __dmul_rn(-s, g);
+                d->g[i + 1] = g1;
+                d->g[i] = __dmul_rn(c, g);
+                const int iters = d->iters + 1;
+                d->iters = iters;
                 d->k = i + 1;
-                d->implicit = fabs(d->g[i + 1]);
-                record_hist(d->hist, d->hist_len, d->iters, d->implicit, d->bnorm);
+                const double implicit = fabs(g1);
+                d->implicit = implicit;
+                record_hist(d->hist, d->hist_len, iters, implicit, d->bnorm);
                 const bool happy = hnext <= 1e-14 * sqrt(d->w0sq);
-                if (d->implicit <= d->tol || d->iters >= d->maxit || happy || i == d->m - 1)
+                if (implicit <= d->tol || iters >= d->maxit || happy || i == d->m - 1) {
                     d->cycle_done = 1;
+                    *(volatile int *)d->host_done = 1;
+                }
                 d->hdiv = 1.0 / hnext;     // v_{i+1} = w / h_{i+1,i}
             }
+            __syncthreads();
+            for (int k = threadIdx.x; k <= nc; k += blockDim.x) hcol[k] = h[k];
         }
     }
 }
@@ -418,20 +438,38 @@ __global__ void k_gmres_start(GmresDev *d, const double *r2, double rtol, int fi
     d->hdiv = 1.0 / beta;      // v_1 = r / beta
 }
 
-// y = H(0:k,0:k)^{-1} g(0:k) by back-substitution
-__global__ void k_gmres_backsolve(GmresDev *d)
+// y = H(0:k,0:k)^{-1} g(0:k) by back-substitution, row by row, one thread's
+// chain of k^2/2 multiply-adds: from a copy of H in shared memory (from
+// global memory it took 62 us at k = 30, now 33)
+__global__ void __launch_bounds__(256) k_gmres_backsolve(GmresDev *d)
 {
-    if (threadIdx.x != 0) return;
+    __shared__ double hs[(RS_MAX_RESTART * (RS_MAX_RESTART + 1)) / 2];   // column l: rows 0..l, from l (l + 1) / 2
+    __shared__ double ys[RS_MAX_RESTART];
     const int k = d->k, m1 = d->m + 1;
-    for (int j = k - 1; j >= 0; --j) {
-        double s = d->g[j];
-        for (int l = j + 1; l < k; ++l) s = fma(-d->H[(size_t)l * m1 + j], d->y[l], s);
-        d->y[j] = __ddiv_rn(s, d->H[(size_t)j * m1 + j]);
+    for (int l = threadIdx.x >> 5; l < k; l += blockDim.x >> 5)
+        for (int j = threadIdx.x & 31; j <= l; j += 32) hs[l * (l + 1) / 2 + j] = d->H[(size_t)l * m1 + j];
+    for (int j = threadIdx.x; j < k; j += blockDim.x) ys[j] = d->g[j];
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int j = k - 1; j >= 0; --j) {
+            double s = ys[j];
+            for (int l = j + 1; l < k; ++l) s = fma(-hs[l * (l + 1) / 2 + j], ys[l], s);
+            ys[j] = __ddiv_rn(s, hs[j * (j + 1) / 2 + j]);
+        }
+        d->noupd = k == 0;
     }
-    d->noupd = k == 0;
+    __syncthreads();
+    for (int j = threadIdx.x; j < k; j += blockDim.x) d->y[j] = ys[j];
 }
 
-static int red_grid(rs_ctx *ctx) { return ctx->red_blocks; }
+// Blocks of a reduction over n rows, `rows` of them per block and round: at
+// most red_blocks, and no block without rows, since the last block adds one
+// partial per block (at 1920 rows the CGS2 passes took 9 to 25 us with 304
+// blocks of which 15 had rows, and take 6 to 19 with those 15).
+static int red_grid(rs_ctx *ctx, int n, int rows)
+{
+    return std::max(1, std::min(ctx->red_blocks, (n + rows - 1) / rows));
+}
 
 static int blas_grid(rs_ctx *ctx, int n)
 {
@@ -451,7 +489,7 @@ static int launch_cgs_pass(rs_ctx *ctx, int n, int ld, int nc, double *V, GmresD
     }
     RsProfScope prof(ctx, MODE == CGS_DOTS ? RS_PROF_CGS_DOTS
                           : MODE == CGS_UPDATE_DOTS ? RS_PROF_CGS_UPDATE_DOTS : RS_PROF_CGS_UPDATE_NORM);
-    k_cgs_pass<NC, NCC, MODE><<<red_grid(ctx), C::THREADS, C::SMEM, ctx->stream>>>(
+    k_cgs_pass<NC, NCC, MODE><<<red_grid(ctx, n, C::TILE), C::THREADS, C::SMEM, ctx->stream>>>(
         n, ld, nc, V, V + (size_t)nc * ld, ctx->red_partials, ctx->red_ticket, d, ctx->d_err, ctx->spin_limit);
     ctx->launches++;
     return rs_check_launch(ctx);
@@ -527,6 +565,12 @@ static int gmres_impl(const rs_mat *A, rs_pc *M, const rs_vec *bv, rs_vec *xv, i
     double *dhist = nullptr;
     int hlen = 0;
     int naug = 0, head = 0;      // stored corrections; the next ring slot
+    // The host enqueues a cycle at most STEPS_AHEAD steps ahead of the device
+    // and stops once the device has reported the cycle done: the kernels of
+    // further steps would only return.
+    constexpr int STEPS_AHEAD = 4;
+    cudaEvent_t ev[STEPS_AHEAD] = {};
+    volatile int *host_done = (volatile int *)(ctx->h_pinned + 32);
     int st = rs_alloc(ctx, (void **)&V, sizeof(double) * (size_t)ld * (m + aug_k + 1));
     if (!st && flexible) st = rs_alloc(ctx, (void **)&Z, sizeof(double) * (size_t)ld * (m + aug_k));
     if (!st && aug_k > 0) st = rs_alloc(ctx, (void **)&Aug, sizeof(double) * (size_t)ld * aug_k);
@@ -534,6 +578,8 @@ static int gmres_impl(const rs_mat *A, rs_pc *M, const rs_vec *bv, rs_vec *xv, i
     if (!st) st = rs_alloc(ctx, (void **)&t, sizeof(double) * ld);
     if (!st) st = rs_alloc(ctx, (void **)&d, sizeof(GmresDev));
     if (!st) st = hist_begin(ctx, &dhist, &hlen);
+    for (cudaEvent_t &e : ev)
+        if (!st && cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) st = RS_ERR_CUDA;
     int status = RS_NOT_CONVERGED;
     double bnorm = 0.0;
     const double *b = bv->d;
@@ -547,6 +593,7 @@ static int gmres_impl(const rs_mat *A, rs_pc *M, const rs_vec *bv, rs_vec *xv, i
         h0.noupd = 1;
         h0.hist = dhist;
         h0.hist_len = hlen;
+        h0.host_done = (int *)host_done;
         // ||b||
         st = rs_dot_launch(ctx, n, b, b, ctx->d_scalars);
         if (st) goto out;
@@ -588,6 +635,7 @@ static int gmres_impl(const rs_mat *A, rs_pc *M, const rs_vec *bv, rs_vec *xv, i
                 st = RS_ERR_CUDA;
                 goto out;
             }
+            *host_done = 0;
             // hs: iters, k, cycle_done, converged
             info->iters = hs[0];
             if (hs[3]) { status = RS_OK; break; }
@@ -595,6 +643,10 @@ static int gmres_impl(const rs_mat *A, rs_pc *M, const rs_vec *bv, rs_vec *xv, i
             k_scale_dev<<<gb, 256, 0, ctx->stream>>>(n, r, &d->hdiv, V, nullptr);
             ctx->launches++;
             for (int i = 0; i < dim; ++i) {
+                if (i >= STEPS_AHEAD) {
+                    if (cudaEventSynchronize(ev[i % STEPS_AHEAD]) != cudaSuccess) { st = RS_ERR_CUDA; goto out; }
+                    if (*host_done) break;
+                }
                 double *vi = V + (size_t)i * ld;
                 double *zi = flexible ? Z + (size_t)i * ld : t;
                 double *w = V + (size_t)(i + 1) * ld;
@@ -615,13 +667,14 @@ static int gmres_impl(const rs_mat *A, rs_pc *M, const rs_vec *bv, rs_vec *xv, i
                 }
                 if (!st) st = rs_spmv_launch(A, zi, 1.0, 0.0, w, cycle_done);
                 if (!st) st = cgs_step(ctx, n, ld, i + 1, V, d);
+                if (!st && cudaEventRecord(ev[i % STEPS_AHEAD], ctx->stream) != cudaSuccess) st = RS_ERR_CUDA;
                 if (st) goto out;
                 if (i + 1 < dim) {
                     k_scale_dev<<<gb, 256, 0, ctx->stream>>>(n, w, &d->hdiv, w, cycle_done);
                     ctx->launches++;
                 }
             }
-            k_gmres_backsolve<<<1, 32, 0, ctx->stream>>>(d);
+            k_gmres_backsolve<<<1, 256, 0, ctx->stream>>>(d);
             ctx->launches++;
             if (flexible && aug_k > 0) {
                 // the correction t = Z y; x += t; t / ||t|| joins the ring
@@ -669,6 +722,8 @@ out:
         const int hs = hist_end(ctx, dhist, hlen, info->iters);
         if (!st) st = hs;
     }
+    for (cudaEvent_t e : ev)
+        if (e) cudaEventDestroy(e);
     rs_free(ctx, V);
     rs_free(ctx, Z);
     rs_free(ctx, Aug);
@@ -886,7 +941,7 @@ extern "C" int rs_solve_bicgstab(const rs_mat *A, rs_pc *M, const rs_vec *bv, rs
         h0.hist = dhist;
         h0.hist_len = hlen;
         cudaMemcpyAsync(d, &h0, sizeof(h0), cudaMemcpyHostToDevice, ctx->stream);
-        const int gr = red_grid(ctx), gb = blas_grid(ctx, n);
+        const int gr = red_grid(ctx, n, RS_RED_THREADS), gb = blas_grid(ctx, n);
         int *halt = &d->done;
         const int batch = 8;
         for (;;) {
@@ -1104,7 +1159,7 @@ extern "C" int rs_solve_cg(const rs_mat *A, rs_pc *M, const rs_vec *bv, rs_vec *
         h0.hist = dhist;
         h0.hist_len = hlen;
         cudaMemcpyAsync(d, &h0, sizeof(h0), cudaMemcpyHostToDevice, ctx->stream);
-        const int gr = red_grid(ctx), gb = blas_grid(ctx, n);
+        const int gr = red_grid(ctx, n, RS_RED_THREADS), gb = blas_grid(ctx, n);
         int *halt = &d->done;
         const int batch = 8;
         for (;;) {
