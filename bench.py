@@ -313,7 +313,7 @@ def cgs_fmas(n, iters_list, m=30):
 
 
 def source_sha(kernel):
-    files = {"spmv": ["rs_core.cu"], "net": ["rs_net.cu"], "cpr_resid": ["rs_precond.cu"]}.get(
+    files = {"spmv": ["rs_core.cu", "rs_spmv.cu"], "net": ["rs_net.cu"], "cpr_resid": ["rs_precond.cu", "rs_spmv.cu"]}.get(
         kernel, ["rs_ilu.cu", "rs_wave.cu"] if "sweep" in kernel else ["rs_krylov.cu"])
     h = hashlib.sha256()
     for f in files:

@@ -177,7 +177,7 @@ void rs_amg_destroy(AmgData *M)
 }
 
 int rs_amg_create(rs_ctx *ctx, int n, int64_t nnz, const int *d_ptr, const int *d_col, const double *d_val, const rs_mat *A0,
-                  double theta, int max_levels, int max_coarse, int nu, int smoother, AmgData **out)
+                  const rs_mat *like,                  double theta, int max_levels, int max_coarse, int nu, int smoother, AmgData **out)
 {
     *out = nullptr;
     if (n < 1 || max_levels < 1 || max_levels > RS_AMG_MAXLEV || max_coarse < 1 || nu < 1 || !(theta >= 0.0) ||
@@ -192,7 +192,7 @@ int rs_amg_create(rs_ctx *ctx, int n, int64_t nnz, const int *d_ptr, const int *
         M->A[0] = const_cast<rs_mat *>(A0);
     } else {
         M->own0 = true;
-        st = rs_mat_create_dev(ctx, n, nnz, d_ptr, d_col, d_val, &M->A[0]);
+        st = rs_mat_create_dev(ctx, n, nnz, d_ptr, d_col, d_val, like, &M->A[0]);
     }
     // the hierarchy (Alg. 3), smoother diagonals and the coarsest inverse
     if (!st) st = rs_amg_setup_device(M, theta, max_levels, max_coarse);

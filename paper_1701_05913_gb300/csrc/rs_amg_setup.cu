@@ -875,9 +875,9 @@ int rs_amg_setup_device(AmgData *M, double theta, int max_levels, int max_coarse
         int64_t nx = 0, ncn = 0;
         RS_TRY(spgemm(ctx, D, n, A->ptr, A->col, A->val, pptr, pcol, pval, &xptr, &xcol, &xval, &nx));
         RS_TRY(spgemm(ctx, D, nc, rptr, rcol, rval, xptr, xcol, xval, &cptr, &ccol, &cval, &ncn));
-        RS_TRY(rs_mat_create_dev(ctx, n, np, pptr, pcol, pval, &M->P[l]));
-        RS_TRY(rs_mat_create_dev(ctx, nc, np, rptr, rcol, rval, &M->R[l]));
-        RS_TRY(rs_mat_create_dev(ctx, nc, ncn, cptr, ccol, cval, &M->A[l + 1]));
+        RS_TRY(rs_mat_create_dev(ctx, n, np, pptr, pcol, pval, nullptr, &M->P[l]));
+        RS_TRY(rs_mat_create_dev(ctx, nc, np, rptr, rcol, rval, nullptr, &M->R[l]));
+        RS_TRY(rs_mat_create_dev(ctx, nc, ncn, cptr, ccol, cval, nullptr, &M->A[l + 1]));
     }
     M->nlev = l + 1;
     const int ncoarse = M->A[l]->n;

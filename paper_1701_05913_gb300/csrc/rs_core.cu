@@ -699,6 +699,7 @@ static int spmv_dispatch(const rs_mat *A, const double *x, double alpha, double 
     rs_ctx *ctx = A->ctx;
     if (A->n == 0) return RS_OK;
     RsProfScope prof(ctx, RS_PROF_SPMV);
+    if (rs_spmv_layout(A)) return rs_spmv_layout_launch(A, x, alpha, beta, bvec, y, skip, dinv);
     if (A->bs == 1 && A->lanes == 1) {
         static unsigned long long raised = 0;   // devices whose shared-memory limit was raised
         const unsigned long long bit = 1ull << (ctx->device & 63);
@@ -791,7 +792,8 @@ static int validate_pattern(int nrows, const std::vector<int> &ptr, const std::v
 // The device copies of A's arrays (A's sizes are set) and the SpMV kernel for
 // its rows.  RS_MAT_PAD zeroed elements follow each array: the SpMV's bulk
 // copies widen their ranges to 16-byte boundaries.
-static int mat_fill(rs_mat *A, const int32_t *ptr, const int32_t *col, const double *val, cudaMemcpyKind kind)
+static int mat_fill(rs_mat *A, const int32_t *ptr, const int32_t *col, const double *val, cudaMemcpyKind kind,
+                    const rs_mat *like)
 {
     rs_ctx *ctx = A->ctx;
     const int nrows = A->nrows, b2 = A->bs * A->bs;
@@ -816,11 +818,18 @@ static int mat_fill(rs_mat *A, const int32_t *ptr, const int32_t *col, const dou
     if (mean > 12.0)
         while (L < 32 && 4.0 * L < mean) L <<= 1;
     A->lanes = L;
-    return RS_OK;
+    st = rs_spmv_layout_build(A, like);
+    if (st == RS_ERR_OOM) {           // no room for a second copy: CSR / BSR as it is
+        cudaGetLastError();
+        rs_spmv_layout_free(A);
+        st = RS_OK;
+    }
+    return st;
 }
 
 static void mat_free(rs_mat *A)
 {
+    rs_spmv_layout_free(A);
     rs_free(A->ctx, A->ptr);
     rs_free(A->ctx, A->col);
     rs_free(A->ctx, A->val);
@@ -857,7 +866,7 @@ static int mat_create(rs_ctx *ctx, int nrows, int bs, const int32_t *ptr, const 
     }
     int st = validate_pattern(nrows, A->h_ptr, A->h_col);
     if (st) { delete A; return st; }
-    st = mat_fill(A, ptr, col, val, h2d);
+    st = mat_fill(A, ptr, col, val, h2d, nullptr);
     if (!st && mem == RS_MEM_HOST && cudaStreamSynchronize(ctx->stream) != cudaSuccess) st = RS_ERR_CUDA;
     if (st) { mat_free(A); return st; }
     rs_ctx_retain(ctx);
@@ -873,16 +882,16 @@ extern "C" int rs_mat_create_csr(rs_ctx *ctx, int32_t n, const int32_t *rowptr,
 
 // an operator of the library's own setup kernels: sorted, in range, its size
 // known.  Neither validated nor copied to the host (nothing analyses its
-// pattern there), so nothing waits for the device.
+// pattern there).
 int rs_mat_create_dev(rs_ctx *ctx, int nrows, int64_t nnz, const int *ptr, const int *col, const double *val,
-                      rs_mat **out)
+                      const rs_mat *like, rs_mat **out)
 {
     rs_mat *A = new rs_mat();
     A->ctx = ctx;
     A->bs = 1;
     A->nrows = A->n = nrows;
     A->nnzb = nnz;
-    const int st = mat_fill(A, ptr, col, val, cudaMemcpyDeviceToDevice);
+    const int st = mat_fill(A, ptr, col, val, cudaMemcpyDeviceToDevice, like);
     if (st) { mat_free(A); return st; }
     rs_ctx_retain(ctx);
     *out = A;

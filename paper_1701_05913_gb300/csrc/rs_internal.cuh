@@ -112,6 +112,22 @@ struct rs_mat {
     double *val;
     std::vector<int> h_ptr, h_col;   // host copy of a caller's pattern (analysis)
     int lanes;               // SpMV lanes per row (CSR; 1 = the pipelined row-per-thread kernel)
+    // SpMV layouts (rs_spmv.cu), built with the matrix; at most one is present
+    // (else CSR / BSR)
+    struct {
+        int nd = 0;              // distinct offsets col - row, ascending; 0: no such layout
+        int off[8];
+        int64_t ld = 0;          // (scalar) rows, rounded up to 32
+        double *val = nullptr;   // [nd][bs][ld]: entry (offset k, block column c) of each scalar row
+        unsigned char *mask = nullptr;   // [nrows] bit k: the row has an entry at offset k
+    } dia;
+    struct {
+        int nslice = 0;          // 0: no such layout
+        int2 *rows = nullptr;    // [nslice * 32] row (-1: none) and its number of entries
+        int *sptr = nullptr;     // [nslice + 1] first entry of each slice
+        int *col = nullptr;      // [sptr[nslice]] entry k of lane l at sptr[s] + 32 k + l
+        double *val = nullptr;
+    } sell;
 };
 
 struct rs_vec {
@@ -265,7 +281,8 @@ struct rs_pc {
     int *diagA;              // diagonal block positions of A (CPR with a RAS F stage)
     double *rp, *zp;         // pressure-stage vectors [nb]
     double *t1, *t2;         // full-size work vectors [n]
-    double *pcol;            // PF form on blocks: column 0 of every block of A [nnzb*bs]
+    bool pf_blocks;          // PF form on a block matrix: the residual takes A's pressure columns only
+    double *pcol;            // those columns [nnzb*bs], when A has no stencil layout to take them from
     // learned pressure stage
     const rs_net *net;
     const double *log_perm;
@@ -302,9 +319,23 @@ int rs_alloc(rs_ctx *ctx, void **p, size_t bytes);
 void rs_free(rs_ctx *ctx, void *p);
 
 // a CSR operator of nnz entries from the library's own device arrays (copied;
-// not validated, no host copy of the pattern, no synchronisation)
+// not validated, no host copy of the pattern); like: a matrix of the same
+// (block) pattern, if there is one
 int rs_mat_create_dev(rs_ctx *ctx, int nrows, int64_t nnz, const int *ptr, const int *col, const double *val,
-                      rs_mat **A);
+                      const rs_mat *like, rs_mat **A);
+
+// SpMV layouts (rs_spmv.cu).  build: the stencil layout of A's pattern, else
+// the sliced one, else none (A is left as it was).  Rows from which the
+// sliced layout's thread per row fills the GPU: below, the lane kernel's
+// several lanes per row are faster.
+#define RS_SELL_MIN_ROWS 32768
+int rs_spmv_layout_build(rs_mat *A, const rs_mat *like);
+void rs_spmv_layout_free(rs_mat *A);
+bool rs_spmv_layout(const rs_mat *A);
+int rs_spmv_layout_launch(const rs_mat *A, const double *x, double alpha, double beta, const double *bvec, double *y,
+                          const int *skip, const double *dinv);
+// t = f - A (Pi_p p) of a block matrix with a stencil layout
+int rs_presid_dia_launch(const rs_mat *A, const double *p, const double *f, double *t, const int *skip);
 
 // y = alpha * A x + beta * y (beta == 0: y not read).  Kernels given a
 // non-null `skip` return at once when *skip != 0 (a device flag).
@@ -348,8 +379,9 @@ int rs_ras_create(rs_ctx *ctx, const rs_mat *A, int nparts, const int32_t *part,
 int rs_ras_apply(RasData *R, const double *r, double *z, const int *skip);
 void rs_ras_destroy(RasData *R);
 // A0: the level-0 matrix when the caller has one as an rs_mat (else built
-// from the host pattern and the device values d_val)
+// from the arrays; like: a block matrix of that pattern)
 int rs_amg_create(rs_ctx *ctx, int n, int64_t nnz, const int *d_ptr, const int *d_col, const double *d_val, const rs_mat *A0,
+                  const rs_mat *like,
                   double theta, int max_levels, int max_coarse, int nu, int smoother, AmgData **out);
 // the hierarchy of Alg. 3 on the device (rs_amg_setup.cu): from M->A[0]
 int rs_amg_setup_device(AmgData *M, double theta, int max_levels, int max_coarse);

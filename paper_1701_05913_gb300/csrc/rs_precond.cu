@@ -159,11 +159,15 @@ static int cpr_apply_pf_blocks(rs_pc *M, const double *r, double *z, const int *
         RsProfScope prof(ctx, RS_PROF_CPR_RESID);
         const int64_t threads = (int64_t)A->n;
         const int grid = (int)((threads + 255) / 256);
-        if (bs == 3)
-            k_cpr_presid<3><<<grid, 256, 0, ctx->stream>>>(nb, 3, A->ptr, A->col, M->pcol, M->zp, r, M->t1, skip);
-        else
-            k_cpr_presid<0><<<grid, 256, 0, ctx->stream>>>(nb, bs, A->ptr, A->col, M->pcol, M->zp, r, M->t1, skip);
-        RS_TRY(rs_check_launch(ctx));
+        if (!M->pcol) {
+            RS_TRY(rs_presid_dia_launch(A, M->zp, r, M->t1, skip));
+        } else {
+            if (bs == 3)
+                k_cpr_presid<3><<<grid, 256, 0, ctx->stream>>>(nb, 3, A->ptr, A->col, M->pcol, M->zp, r, M->t1, skip);
+            else
+                k_cpr_presid<0><<<grid, 256, 0, ctx->stream>>>(nb, bs, A->ptr, A->col, M->pcol, M->zp, r, M->t1, skip);
+            RS_TRY(rs_check_launch(ctx));
+        }
     }
     RS_TRY(cpr_stage(M, 'F', M->t1, M->t2, skip));
     k_prolong_add<<<grid_for(ctx, A->n), 256, 0, ctx->stream>>>(nb, bs, M->zp, M->t2, z, skip);
@@ -178,7 +182,7 @@ static int cpr_apply(rs_pc *M, const double *r, double *z, const int *skip)
     const rs_mat *A = M->A;
     static const char *forms[4] = {"PF", "FP", "FPF", "FFPF"};
     const char *seq = forms[M->form];
-    if (M->pcol) return cpr_apply_pf_blocks(M, r, z, skip);
+    if (M->pf_blocks) return cpr_apply_pf_blocks(M, r, z, skip);
     RS_TRY(cpr_stage(M, seq[0], r, z, skip));
     for (int k = 1; seq[k]; ++k) {
         RS_TRY(rs_residual_launch(A, r, z, M->t1, nullptr, skip));
@@ -357,7 +361,7 @@ extern "C" int rs_precond_setup(rs_ctx *ctx, const rs_mat *A, int type, const rs
             st = RS_ERR_INVALID_ARG;
             break;
         }
-        st = rs_amg_create(ctx, A->nrows, A->nnzb, A->ptr, A->col, A->val, A, th, lev, nc, nu, sm, &M->amg);
+        st = rs_amg_create(ctx, A->nrows, A->nnzb, A->ptr, A->col, A->val, A, nullptr, th, lev, nc, nu, sm, &M->amg);
         break;
     }
     case RS_PC_RAS: {
@@ -406,7 +410,7 @@ extern "C" int rs_precond_setup(rs_ctx *ctx, const rs_mat *A, int type, const rs
         if (bs == 1) {
             // pressure stage on A itself: its ILU(0), or an AMG V-cycle
             if (pstage == 1 && type == RS_PC_CPR) {
-                st = rs_amg_create(ctx, nb, A->nnzb, A->ptr, A->col, A->val, A, th, lev, ncoarse, nu, sm, &M->amg);
+                st = rs_amg_create(ctx, nb, A->nnzb, A->ptr, A->col, A->val, A, nullptr, th, lev, ncoarse, nu, sm, &M->amg);
             } else if (fras) {
                 st = rs_ilu_create(ctx, 1, nb, A->nnzb, A->ptr, A->col, A->h_ptr, A->h_col, fp32, sweep, run_cap, &M->ilu, &bad);
                 if (!st) st = rs_ilu_factor(M->ilu, A->val, &bad);
@@ -419,7 +423,8 @@ extern "C" int rs_precond_setup(rs_ctx *ctx, const rs_mat *A, int type, const rs
         if (!st) st = rs_alloc(ctx, (void **)&M->app_val, sizeof(double) * (A->nnzb > 0 ? A->nnzb : 1));
         if (!st) st = rs_alloc(ctx, (void **)&M->rp, sizeof(double) * (nb > 0 ? nb : 1));
         if (!st) st = rs_alloc(ctx, (void **)&M->zp, sizeof(double) * (nb > 0 ? nb : 1));
-        if (!st && M->form == RS_CPR_PF) {
+        M->pf_blocks = M->form == RS_CPR_PF;
+        if (!st && M->pf_blocks && !A->dia.nd) {
             st = rs_alloc(ctx, (void **)&M->pcol, sizeof(double) * bs * (A->nnzb > 0 ? A->nnzb : 1));
             if (!st && A->nnzb > 0) {
                 k_pcol_gather<<<grid_for(ctx, A->nnzb * bs), 256, 0, ctx->stream>>>(A->nnzb, bs, A->val, M->pcol);
@@ -451,7 +456,7 @@ extern "C" int rs_precond_setup(rs_ctx *ctx, const rs_mat *A, int type, const rs
         if (st) break;
         if (pstage == 1 && type == RS_PC_CPR) {
             // AMG V-cycle on the decoupled pressure matrix (the paper's CPR pressure stage)
-            st = rs_amg_create(ctx, nb, A->nnzb, A->ptr, A->col, M->app_val, nullptr, th, lev, ncoarse, nu, sm, &M->amg);
+            st = rs_amg_create(ctx, nb, A->nnzb, A->ptr, A->col, M->app_val, nullptr, A, th, lev, ncoarse, nu, sm, &M->amg);
             break;
         }
         st = rs_ilu_create(ctx, 1, nb, A->nnzb, A->ptr, A->col, A->h_ptr, A->h_col, fp32, sweep, run_cap, &M->ilu, &bad);

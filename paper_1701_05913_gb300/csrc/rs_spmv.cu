@@ -1,0 +1,466 @@
+// SpMV layouts and kernels for the patterns whose CSR / BSR product is bound
+// by something other than its bytes (y = A x, Figs. 20-21; the residual; the
+// Jacobi-type sweep x + (b - A x) d^-1).
+//
+// FP64 multiply-adds are scarce on this GPU (about two per clock and SM, 600 G
+// per second in all): a 7-point matrix takes as long for them as for its
+// bytes, and every idle or padded lane costs as much as a working one.  Both
+// layouts therefore give each thread one row, whose sum runs in column order
+// (the order of the row-per-thread CSR kernel and of the BSR kernel, so the
+// results are the same bit for bit), and issue a row's loads together.
+//
+// Stencil layout (DIA): the distinct offsets col - row are few (at most 8, a
+// structured grid), so a value's column follows from its place: [offset][row],
+// no column indices and no row pointers, and the loads of values and of x are
+// coalesced without staging.  A byte per row says which entries exist; absent
+// ones are neither multiplied nor added, so a NaN or infinity in x reaches
+// only the rows that refer to it.
+//
+// Sliced layout (SELL): 32 rows a slice, a row per lane, entry k of the 32
+// rows side by side.  The rows of a window are sorted by length first, so
+// the lanes of a slice finish together.
+#include <algorithm>
+#include <vector>
+
+#include "rs_internal.cuh"
+
+namespace {
+
+constexpr int DIA_MAX = 8;
+// Share of the layout's places that hold an entry from which it pays: a place
+// costs 8 bytes, an entry in CSR 12 and its row 4.
+constexpr double DIA_FILL = 0.7;
+
+struct DiaArgs {
+    int n;                   // block rows
+    int off[DIA_MAX];
+    int64_t ld;
+    const double *val;
+    const unsigned char *mask;
+};
+
+DiaArgs dia_args(const rs_mat *A)
+{
+    DiaArgs a;
+    a.n = A->nrows;
+    for (int k = 0; k < DIA_MAX; ++k) a.off[k] = k < A->dia.nd ? A->dia.off[k] : 0;
+    a.ld = A->dia.ld;
+    a.val = A->dia.val;
+    a.mask = A->dia.mask;
+    return a;
+}
+
+// the epilogue of row i: y = alpha acc (+ beta y), y = b - acc, or with dinv
+// y = x + (b - acc) dinv
+__device__ __forceinline__ void spmv_store(int64_t i, double acc, const double *__restrict__ x, double alpha,
+                                           double beta, const double *__restrict__ bvec, double *__restrict__ y,
+                                           const double *__restrict__ dinv)
+{
+    if (dinv) y[i] = fma(__dsub_rn(bvec[i], acc), dinv[i], x[i]);
+    else if (bvec) y[i] = __dsub_rn(bvec[i], acc);
+    else if (beta == 0.0) y[i] = alpha == 1.0 ? acc : __dmul_rn(alpha, acc);
+    else y[i] = fma(alpha, acc, beta * y[i]);
+}
+
+// A thread per scalar row.  All loads are independent of one another and of
+// the mask (x's index is clamped, not predicated), so a warp has its whole
+// row in flight.
+template <int ND, int BS>
+__global__ void __launch_bounds__(256)
+k_spmv_dia(DiaArgs a, const double *__restrict__ x, double alpha, double beta, const double *__restrict__ bvec,
+           double *__restrict__ y, const int *skip, const double *__restrict__ dinv)
+{
+    if (skip && *(volatile const int *)skip) return;
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= (int64_t)a.n * BS) return;
+    const int I = BS == 1 ? (int)i : (int)(i / BS);
+    const unsigned m = a.mask[I];
+    double v[ND][BS], xv[ND][BS];
+#pragma unroll
+    for (int k = 0; k < ND; ++k) {
+        const int J = min(max(I + a.off[k], 0), a.n - 1);
+#pragma unroll
+        for (int c = 0; c < BS; ++c) {
+            v[k][c] = __ldg(a.val + (int64_t)(k * BS + c) * a.ld + i);
+            xv[k][c] = __ldg(x + (int64_t)J * BS + c);
+        }
+    }
+    double acc = 0.0;
+#pragma unroll
+    for (int k = 0; k < ND; ++k)
+        if (m >> k & 1) {
+#pragma unroll
+            for (int c = 0; c < BS; ++c) acc = fma(v[k][c], xv[k][c], acc);
+        }
+    spmv_store(i, acc, x, alpha, beta, bvec, y, dinv);
+}
+
+// t = f - A (Pi_p p): only block column 0 meets the prolonged pressure vector
+template <int ND, int BS>
+__global__ void __launch_bounds__(256)
+k_presid_dia(DiaArgs a, const double *__restrict__ p, const double *__restrict__ f, double *__restrict__ t,
+             const int *skip)
+{
+    if (skip && *(volatile const int *)skip) return;
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= (int64_t)a.n * BS) return;
+    const int I = (int)(i / BS);
+    const unsigned m = a.mask[I];
+    double v[ND], pv[ND];
+#pragma unroll
+    for (int k = 0; k < ND; ++k) {
+        v[k] = __ldg(a.val + (int64_t)k * BS * a.ld + i);
+        pv[k] = __ldg(p + min(max(I + a.off[k], 0), a.n - 1));
+    }
+    double acc = 0.0;
+#pragma unroll
+    for (int k = 0; k < ND; ++k)
+        if (m >> k & 1) acc = fma(v[k], pv[k], acc);
+    t[i] = __dsub_rn(f[i], acc);
+}
+
+// a warp per slice, a row per lane; U entries' loads at a time
+template <int U>
+__global__ void __launch_bounds__(256)
+k_spmv_sell(int nslice, const int2 *__restrict__ rows, const int *__restrict__ sptr, const int *__restrict__ col,
+            const double *__restrict__ val, const double *__restrict__ x, double alpha, double beta,
+            const double *__restrict__ bvec, double *__restrict__ y, const int *skip, const double *__restrict__ dinv)
+{
+    if (skip && *(volatile const int *)skip) return;
+    const int s = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+    if (s >= nslice) return;
+    const int2 rl = rows[(int64_t)s * 32 + lane];
+    const int base = sptr[s] + lane, len = rl.y;
+    double acc = 0.0;
+    for (int k0 = 0; k0 < len; k0 += U) {
+        int c[U];
+        double v[U], xv[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            c[u] = k0 + u < len ? col[base + 32 * (k0 + u)] : -1;
+            v[u] = k0 + u < len ? val[base + 32 * (k0 + u)] : 0.0;
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) xv[u] = c[u] >= 0 ? __ldg(x + c[u]) : 0.0;
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (c[u] >= 0) acc = fma(v[u], xv[u], acc);
+    }
+    if (rl.x >= 0) spmv_store(rl.x, acc, x, alpha, beta, bvec, y, dinv);
+}
+
+// ---------------------------------------------------------------------------
+// building the layouts
+// ---------------------------------------------------------------------------
+// values and masks; *bad |= 1 when an entry's offset is not among off[0..nd)
+template <int BS>
+__global__ void k_dia_fill(DiaArgs a, int nd, const int *__restrict__ ptr, const int *__restrict__ col,
+                           const double *__restrict__ src, double *__restrict__ val, unsigned char *__restrict__ mask,
+                           int *bad)
+{
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= (int64_t)a.n * BS) return;
+    const int I = (int)(i / BS), r = (int)(i - (int64_t)I * BS);
+    unsigned m = 0;
+    bool ok = true;
+    for (int p = ptr[I]; p < ptr[I + 1]; ++p) {
+        const int d = col[p] - I;
+        int k = 0;
+        while (k < nd && a.off[k] != d) ++k;
+        if (k == nd) {
+            ok = false;
+            continue;
+        }
+        m |= 1u << k;
+#pragma unroll
+        for (int c = 0; c < BS; ++c) val[(int64_t)(k * BS + c) * a.ld + i] = src[(int64_t)p * BS * BS + r * BS + c];
+    }
+    if (!ok) atomicOr(bad, 1);
+    if (r == 0) mask[I] = (unsigned char)m;
+}
+
+constexpr int SELL_WIN = 512;       // rows sorted by length together
+
+// one window a block: rows in descending order of length (ties: by row), and
+// the entries of each of its slices
+__global__ void __launch_bounds__(SELL_WIN)
+k_sell_sort(int n, const int *__restrict__ ptr, int2 *__restrict__ rows, int *__restrict__ cnt)
+{
+    __shared__ unsigned key[SELL_WIN];
+    const int t = threadIdx.x, r0 = blockIdx.x * SELL_WIN, r = r0 + t;
+    const int len = r < n ? ptr[r + 1] - ptr[r] : -1;
+    key[t] = (unsigned)(65535 - min(len, 65534)) * SELL_WIN + t;      // no row: after the empty rows
+    __syncthreads();
+    for (int k = 2; k <= SELL_WIN; k <<= 1)
+        for (int j = k >> 1; j > 0; j >>= 1) {
+            const int u = t ^ j;
+            if (u > t) {
+                const unsigned a = key[t], b = key[u];
+                if ((a > b) == ((t & k) == 0)) {
+                    key[t] = b;
+                    key[u] = a;
+                }
+            }
+            __syncthreads();
+        }
+    const int row = r0 + (int)(key[t] % SELL_WIN);
+    const int l = row < n ? ptr[row + 1] - ptr[row] : 0;
+    rows[(int64_t)r0 + t] = make_int2(row < n ? row : -1, l);
+    const int w = __reduce_max_sync(0xffffffffu, min(l, 1 << 25));     // longer rows: the layout is refused
+    if ((t & 31) == 0) cnt[(r0 + t) >> 5] = 32 * w;
+}
+
+// exclusive scan of cnt[0..n) in place, cnt[n] = the total; one block
+__global__ void __launch_bounds__(1024) k_sell_scan(int n, int *__restrict__ cnt, long long *total)
+{
+    __shared__ long long ws[32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    long long carry = 0;
+    for (int b = 0; b < n; b += 1024) {
+        const int i = b + threadIdx.x;
+        const long long v = i < n ? cnt[i] : 0;
+        long long s = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const long long u = __shfl_up_sync(0xffffffffu, s, o);
+            if (lane >= o) s += u;
+        }
+        if (lane == 31) ws[w] = s;
+        __syncthreads();
+        if (w == 0) {
+            long long u = ws[lane];
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const long long q = __shfl_up_sync(0xffffffffu, u, o);
+                if (lane >= o) u += q;
+            }
+            ws[lane] = u;
+        }
+        __syncthreads();
+        const long long excl = carry + (w ? ws[w - 1] : 0) + s - v;
+        if (i < n) cnt[i] = (int)excl;
+        carry += ws[31];
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) {
+        cnt[n] = (int)carry;
+        *total = carry;
+    }
+}
+
+__global__ void __launch_bounds__(256)
+k_sell_fill(int nslice, const int2 *__restrict__ rows, const int *__restrict__ sptr, const int *__restrict__ ptr,
+            const int *__restrict__ col, const double *__restrict__ val, int *__restrict__ scol,
+            double *__restrict__ sval)
+{
+    const int s = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+    if (s >= nslice) return;
+    const int2 rl = rows[(int64_t)s * 32 + lane];
+    const int base = sptr[s] + lane, w = (sptr[s + 1] - sptr[s]) >> 5;
+    const int p0 = rl.x >= 0 ? ptr[rl.x] : 0;
+    for (int k = 0; k < w; ++k) {
+        scol[base + 32 * k] = k < rl.y ? col[p0 + k] : -1;
+        sval[base + 32 * k] = k < rl.y ? val[p0 + k] : 0.0;
+    }
+}
+
+// The offsets of a few sample rows (on the host: a caller's pattern), the
+// candidates of a stencil layout, or those of a matrix of the same pattern;
+// 0 when there are too many or the layout would be too empty.
+int dia_candidates(const rs_mat *A, const rs_mat *like, int (&off)[DIA_MAX])
+{
+    if (like) {
+        std::copy(like->dia.off, like->dia.off + DIA_MAX, off);
+        return like->dia.nd;
+    }
+    const std::vector<int> &ptr = A->h_ptr, &col = A->h_col;
+    if (A->nrows < 1 || (int)ptr.size() != A->nrows + 1) return 0;
+    int nd = 0;
+    const int samples = 64;
+    for (int k = 0; k < samples; ++k) {
+        const int i = (int)((int64_t)(A->nrows - 1) * k / (samples - 1));
+        for (int p = ptr[i]; p < ptr[i + 1]; ++p) {
+            const int d = col[p] - i;
+            if (std::find(off, off + nd, d) != off + nd) continue;
+            if (nd == DIA_MAX) return 0;
+            off[nd++] = d;
+        }
+    }
+    std::sort(off, off + nd);
+    return (double)A->nnzb >= DIA_FILL * nd * (double)A->nrows ? nd : 0;
+}
+
+template <int BS>
+int dia_build(rs_mat *A, int nd, const int (&off)[DIA_MAX])
+{
+    rs_ctx *ctx = A->ctx;
+    const int64_t ld = ((int64_t)A->n + 31) / 32 * 32;
+    const size_t bytes = sizeof(double) * nd * BS * (size_t)ld;
+    int *bad = nullptr;
+    int st = rs_alloc(ctx, (void **)&A->dia.val, bytes);
+    st = st ? st : rs_alloc(ctx, (void **)&A->dia.mask, A->nrows);
+    st = st ? st : rs_alloc(ctx, (void **)&bad, sizeof(int));
+    int hbad = 1;
+    if (!st && (cudaMemsetAsync(A->dia.val, 0, bytes, ctx->stream) != cudaSuccess ||
+                cudaMemsetAsync(bad, 0, sizeof(int), ctx->stream) != cudaSuccess))
+        st = RS_ERR_CUDA;
+    if (!st) {
+        A->dia.ld = ld;
+        std::copy(off, off + nd, A->dia.off);
+        A->dia.nd = nd;
+        k_dia_fill<BS><<<(int)((A->n + 255) / 256), 256, 0, ctx->stream>>>(dia_args(A), nd, A->ptr, A->col, A->val,
+                                                                          A->dia.val, A->dia.mask, bad);
+        st = rs_check_launch(ctx);
+    }
+    if (!st && (cudaMemcpyAsync(&hbad, bad, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream) != cudaSuccess ||
+                cudaStreamSynchronize(ctx->stream) != cudaSuccess))
+        st = RS_ERR_CUDA;
+    rs_free(ctx, bad);
+    if (st || hbad) rs_spmv_layout_free(A);
+    return st;
+}
+
+int sell_build(rs_mat *A)
+{
+    rs_ctx *ctx = A->ctx;
+    const int win = (A->nrows + SELL_WIN - 1) / SELL_WIN, ns = win * (SELL_WIN / 32);
+    long long *tot = nullptr, htot = 0;
+    int st = rs_alloc(ctx, (void **)&A->sell.rows, sizeof(int2) * 32 * (size_t)ns);
+    st = st ? st : rs_alloc(ctx, (void **)&A->sell.sptr, sizeof(int) * ((size_t)ns + 1));
+    st = st ? st : rs_alloc(ctx, (void **)&tot, sizeof(long long));
+    if (!st) {
+        k_sell_sort<<<win, SELL_WIN, 0, ctx->stream>>>(A->nrows, A->ptr, A->sell.rows, A->sell.sptr);
+        k_sell_scan<<<1, 1024, 0, ctx->stream>>>(ns, A->sell.sptr, tot);
+        ctx->launches += 1;
+        st = rs_check_launch(ctx);
+    }
+    if (!st && (cudaMemcpyAsync(&htot, tot, sizeof(htot), cudaMemcpyDeviceToHost, ctx->stream) != cudaSuccess ||
+                cudaStreamSynchronize(ctx->stream) != cudaSuccess))
+        st = RS_ERR_CUDA;
+    rs_free(ctx, tot);
+    // a few very long rows would leave a slice to one lane: keep CSR
+    const bool fits = htot < 0x7fffffffLL && (double)htot <= 1.25 * (double)A->nnzb + 32.0 * 32;
+    if (!st && fits) {
+        st = rs_alloc(ctx, (void **)&A->sell.col, sizeof(int) * (size_t)htot);
+        st = st ? st : rs_alloc(ctx, (void **)&A->sell.val, sizeof(double) * (size_t)htot);
+        if (!st) {
+            k_sell_fill<<<(ns + 7) / 8, 256, 0, ctx->stream>>>(ns, A->sell.rows, A->sell.sptr, A->ptr, A->col, A->val,
+                                                              A->sell.col, A->sell.val);
+            st = rs_check_launch(ctx);
+            A->sell.nslice = ns;
+        }
+    }
+    if (st || !fits) rs_spmv_layout_free(A);
+    return st;
+}
+
+template <int BS>
+int dia_launch(const rs_mat *A, const double *x, double alpha, double beta, const double *bvec, double *y,
+               const int *skip, const double *dinv)
+{
+    const int grid = (int)((A->n + 255) / 256);
+    const DiaArgs a = dia_args(A);
+    switch (A->dia.nd) {
+#define RS_DIA_CASE(ND)                                                                                          \
+    case ND:                                                                                                     \
+        k_spmv_dia<ND, BS><<<grid, 256, 0, A->ctx->stream>>>(a, x, alpha, beta, bvec, y, skip, dinv);             \
+        break;
+        RS_DIA_CASE(1)
+        RS_DIA_CASE(2)
+        RS_DIA_CASE(3)
+        RS_DIA_CASE(4)
+        RS_DIA_CASE(5)
+        RS_DIA_CASE(6)
+        RS_DIA_CASE(7)
+        RS_DIA_CASE(8)
+#undef RS_DIA_CASE
+    default: return RS_ERR_INVALID_ARG;
+    }
+    return rs_check_launch(A->ctx);
+}
+
+template <int BS>
+int presid_launch(const rs_mat *A, const double *p, const double *f, double *t, const int *skip)
+{
+    const int grid = (int)((A->n + 255) / 256);
+    const DiaArgs a = dia_args(A);
+    switch (A->dia.nd) {
+#define RS_DIA_CASE(ND)                                                               \
+    case ND:                                                                          \
+        k_presid_dia<ND, BS><<<grid, 256, 0, A->ctx->stream>>>(a, p, f, t, skip);      \
+        break;
+        RS_DIA_CASE(1)
+        RS_DIA_CASE(2)
+        RS_DIA_CASE(3)
+        RS_DIA_CASE(4)
+        RS_DIA_CASE(5)
+        RS_DIA_CASE(6)
+        RS_DIA_CASE(7)
+        RS_DIA_CASE(8)
+#undef RS_DIA_CASE
+    default: return RS_ERR_INVALID_ARG;
+    }
+    return rs_check_launch(A->ctx);
+}
+
+}  // namespace
+
+void rs_spmv_layout_free(rs_mat *A)
+{
+    rs_ctx *ctx = A->ctx;
+    rs_free(ctx, A->dia.val);
+    rs_free(ctx, A->dia.mask);
+    rs_free(ctx, A->sell.rows);
+    rs_free(ctx, A->sell.sptr);
+    rs_free(ctx, A->sell.col);
+    rs_free(ctx, A->sell.val);
+    A->dia = {};
+    A->sell = {};
+}
+
+int rs_spmv_layout_build(rs_mat *A, const rs_mat *like)
+{
+    if (A->bs <= 3) {
+        int off[DIA_MAX];
+        const int nd = dia_candidates(A, like, off);
+        if (nd) {
+            RS_TRY(A->bs == 1 ? dia_build<1>(A, nd, off) : A->bs == 2 ? dia_build<2>(A, nd, off) : dia_build<3>(A, nd, off));
+            if (A->dia.nd) return RS_OK;
+        }
+    }
+    if (A->bs == 1 && A->nrows >= RS_SELL_MIN_ROWS) return sell_build(A);
+    return RS_OK;
+}
+
+bool rs_spmv_layout(const rs_mat *A) { return A->dia.nd > 0 || A->sell.nslice > 0; }
+
+int rs_spmv_layout_launch(const rs_mat *A, const double *x, double alpha, double beta, const double *bvec, double *y,
+                          const int *skip, const double *dinv)
+{
+    if (A->dia.nd > 0) {
+        switch (A->bs) {
+        case 1: return dia_launch<1>(A, x, alpha, beta, bvec, y, skip, dinv);
+        case 2: return dia_launch<2>(A, x, alpha, beta, bvec, y, skip, dinv);
+        case 3: return dia_launch<3>(A, x, alpha, beta, bvec, y, skip, dinv);
+        default: return RS_ERR_INVALID_ARG;
+        }
+    }
+    const int grid = (A->sell.nslice + 7) / 8;
+    // short rows (interpolation) need no more loads in flight than they have entries
+    if (A->nnzb <= 6 * (int64_t)A->nrows)
+        k_spmv_sell<4><<<grid, 256, 0, A->ctx->stream>>>(A->sell.nslice, A->sell.rows, A->sell.sptr, A->sell.col,
+                                                         A->sell.val, x, alpha, beta, bvec, y, skip, dinv);
+    else
+        k_spmv_sell<8><<<grid, 256, 0, A->ctx->stream>>>(A->sell.nslice, A->sell.rows, A->sell.sptr, A->sell.col,
+                                                         A->sell.val, x, alpha, beta, bvec, y, skip, dinv);
+    return rs_check_launch(A->ctx);
+}
+
+int rs_presid_dia_launch(const rs_mat *A, const double *p, const double *f, double *t, const int *skip)
+{
+    switch (A->bs) {
+    case 2: return presid_launch<2>(A, p, f, t, skip);
+    case 3: return presid_launch<3>(A, p, f, t, skip);
+    default: return RS_ERR_INVALID_ARG;
+    }
+}
