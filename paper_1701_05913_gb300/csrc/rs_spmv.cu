@@ -4,15 +4,17 @@
 //
 // FP64 multiply-adds are scarce on this GPU (about two per clock and SM, 600 G
 // per second in all): a 7-point matrix takes as long for them as for its
-// bytes, and every idle or padded lane costs as much as a working one.  Both
-// layouts therefore give each thread one row, whose sum runs in column order
-// (the order of the row-per-thread CSR kernel and of the BSR kernel, so the
-// results are the same bit for bit), and issue a row's loads together.
+// bytes, one of 3 x 3 blocks longer, and every idle or padded lane costs as
+// much as a working one.  Both layouts therefore give each thread one (block)
+// row, whose sum runs in column order (the order of the row-per-thread CSR
+// kernel and of the BSR kernel, so the results are the same bit for bit), and
+// issue a row's loads together.
 //
 // Stencil layout (DIA): the distinct offsets col - row are few (at most 8, a
-// structured grid), so a value's column follows from its place: [offset][row],
-// no column indices and no row pointers, and the loads of values and of x are
-// coalesced without staging.  A byte per row says which entries exist; absent
+// structured grid), so a value's column follows from its place (a plane per
+// offset and place in the block, a value per row): no column indices and no
+// row pointers, and the loads of values and of x are coalesced without
+// staging.  A byte per row says which entries exist; absent
 // ones are neither multiplied nor added, so a NaN or infinity in x reaches
 // only the rows that refer to it.
 //
@@ -51,7 +53,7 @@ DiaArgs dia_args(const rs_mat *A)
 }
 
 // the epilogue of row i: y = alpha acc (+ beta y), y = b - acc, or with dinv
-// y = x + (b - acc) dinv
+// y = x + (b - acc) dinv; factors of 1 cost no FP64 instruction
 __device__ __forceinline__ void spmv_store(int64_t i, double acc, const double *__restrict__ x, double alpha,
                                            double beta, const double *__restrict__ bvec, double *__restrict__ y,
                                            const double *__restrict__ dinv)
@@ -59,40 +61,58 @@ __device__ __forceinline__ void spmv_store(int64_t i, double acc, const double *
     if (dinv) y[i] = fma(__dsub_rn(bvec[i], acc), dinv[i], x[i]);
     else if (bvec) y[i] = __dsub_rn(bvec[i], acc);
     else if (beta == 0.0) y[i] = alpha == 1.0 ? acc : __dmul_rn(alpha, acc);
-    else y[i] = fma(alpha, acc, beta * y[i]);
+    else y[i] = fma(alpha, acc, beta == 1.0 ? y[i] : __dmul_rn(beta, y[i]));
 }
 
-// A thread per scalar row.  All loads are independent of one another and of
-// the mask (x's index is clamped, not predicated), so a warp has its whole
-// row in flight.
+// A thread per (block) row.  All loads are independent of one another and of
+// the mask (x's index is clamped, not predicated), so a warp keeps many of
+// its row's loads in flight.  Per product at the start and now: 7-point,
+// 1,048,576 rows 33.9 -> 19 us (76 MB moved; bytes and multiply-adds take
+// 11 and 12 us); 3 x 3 blocks, 500,000 rows 69 -> 60 us (52 us of
+// multiply-adds).
 template <int ND, int BS>
 __global__ void __launch_bounds__(256)
 k_spmv_dia(DiaArgs a, const double *__restrict__ x, double alpha, double beta, const double *__restrict__ bvec,
            double *__restrict__ y, const int *skip, const double *__restrict__ dinv)
 {
     if (skip && *(volatile const int *)skip) return;
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (int64_t)a.n * BS) return;
-    const int I = BS == 1 ? (int)i : (int)(i / BS);
+    const int64_t I = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (I >= a.n) return;
     const unsigned m = a.mask[I];
-    double v[ND][BS], xv[ND][BS];
+    double acc[BS];
 #pragma unroll
-    for (int k = 0; k < ND; ++k) {
-        const int J = min(max(I + a.off[k], 0), a.n - 1);
+    for (int r = 0; r < BS; ++r) acc[r] = 0.0;
+    auto at = [&](int k) { return min(max(I + a.off[k], (int64_t)0), (int64_t)a.n - 1); };
+    if constexpr (BS == 1) {
+        // the whole row's loads, then its multiply-adds (24.5 -> 22.8 us a call)
+        double v[ND], xv[ND];
 #pragma unroll
-        for (int c = 0; c < BS; ++c) {
-            v[k][c] = __ldg(a.val + (int64_t)(k * BS + c) * a.ld + i);
-            xv[k][c] = __ldg(x + (int64_t)J * BS + c);
+        for (int k = 0; k < ND; ++k) {
+            v[k] = __ldg(a.val + (int64_t)k * a.ld + I);
+            xv[k] = __ldg(x + at(k));
+        }
+#pragma unroll
+        for (int k = 0; k < ND; ++k)
+            if (m >> k & 1) acc[0] = fma(v[k], xv[k], acc[0]);
+    } else {
+#pragma unroll
+        for (int k = 0; k < ND; ++k) {
+            const int64_t J = at(k);
+            double v[BS * BS], xv[BS];
+#pragma unroll
+            for (int c = 0; c < BS; ++c) xv[c] = __ldg(x + J * BS + c);
+#pragma unroll
+            for (int e = 0; e < BS * BS; ++e) v[e] = __ldg(a.val + (int64_t)(k * BS * BS + e) * a.ld + I);
+            if (m >> k & 1) {
+#pragma unroll
+                for (int r = 0; r < BS; ++r)
+#pragma unroll
+                    for (int c = 0; c < BS; ++c) acc[r] = fma(v[r * BS + c], xv[c], acc[r]);
+            }
         }
     }
-    double acc = 0.0;
 #pragma unroll
-    for (int k = 0; k < ND; ++k)
-        if (m >> k & 1) {
-#pragma unroll
-            for (int c = 0; c < BS; ++c) acc = fma(v[k][c], xv[k][c], acc);
-        }
-    spmv_store(i, acc, x, alpha, beta, bvec, y, dinv);
+    for (int r = 0; r < BS; ++r) spmv_store(I * BS + r, acc[r], x, alpha, beta, bvec, y, dinv);
 }
 
 // t = f - A (Pi_p p): only block column 0 meets the prolonged pressure vector
@@ -102,21 +122,25 @@ k_presid_dia(DiaArgs a, const double *__restrict__ p, const double *__restrict__
              const int *skip)
 {
     if (skip && *(volatile const int *)skip) return;
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (int64_t)a.n * BS) return;
-    const int I = (int)(i / BS);
+    const int64_t I = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (I >= a.n) return;
     const unsigned m = a.mask[I];
-    double v[ND], pv[ND];
+    double acc[BS];
+#pragma unroll
+    for (int r = 0; r < BS; ++r) acc[r] = 0.0;
 #pragma unroll
     for (int k = 0; k < ND; ++k) {
-        v[k] = __ldg(a.val + (int64_t)k * BS * a.ld + i);
-        pv[k] = __ldg(p + min(max(I + a.off[k], 0), a.n - 1));
-    }
-    double acc = 0.0;
+        const double pv = __ldg(p + min(max(I + a.off[k], (int64_t)0), (int64_t)a.n - 1));
+        double v[BS];
 #pragma unroll
-    for (int k = 0; k < ND; ++k)
-        if (m >> k & 1) acc = fma(v[k], pv[k], acc);
-    t[i] = __dsub_rn(f[i], acc);
+        for (int r = 0; r < BS; ++r) v[r] = __ldg(a.val + (int64_t)(k * BS * BS + r * BS) * a.ld + I);
+        if (m >> k & 1) {
+#pragma unroll
+            for (int r = 0; r < BS; ++r) acc[r] = fma(v[r], pv, acc[r]);
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < BS; ++r) t[I * BS + r] = __dsub_rn(f[I * BS + r], acc[r]);
 }
 
 // a warp per slice, a row per lane; U entries' loads at a time
@@ -173,7 +197,8 @@ __global__ void k_dia_fill(DiaArgs a, int nd, const int *__restrict__ ptr, const
         }
         m |= 1u << k;
 #pragma unroll
-        for (int c = 0; c < BS; ++c) val[(int64_t)(k * BS + c) * a.ld + i] = src[(int64_t)p * BS * BS + r * BS + c];
+        for (int c = 0; c < BS; ++c)
+            val[(int64_t)(k * BS * BS + r * BS + c) * a.ld + I] = src[(int64_t)p * BS * BS + r * BS + c];
     }
     if (!ok) atomicOr(bad, 1);
     if (r == 0) mask[I] = (unsigned char)m;
@@ -294,8 +319,8 @@ template <int BS>
 int dia_build(rs_mat *A, int nd, const int (&off)[DIA_MAX])
 {
     rs_ctx *ctx = A->ctx;
-    const int64_t ld = ((int64_t)A->n + 31) / 32 * 32;
-    const size_t bytes = sizeof(double) * nd * BS * (size_t)ld;
+    const int64_t ld = ((int64_t)A->nrows + 31) / 32 * 32;
+    const size_t bytes = sizeof(double) * nd * BS * BS * (size_t)ld;
     int *bad = nullptr;
     int st = rs_alloc(ctx, (void **)&A->dia.val, bytes);
     st = st ? st : rs_alloc(ctx, (void **)&A->dia.mask, A->nrows);
@@ -308,7 +333,7 @@ int dia_build(rs_mat *A, int nd, const int (&off)[DIA_MAX])
         A->dia.ld = ld;
         std::copy(off, off + nd, A->dia.off);
         A->dia.nd = nd;
-        k_dia_fill<BS><<<(int)((A->n + 255) / 256), 256, 0, ctx->stream>>>(dia_args(A), nd, A->ptr, A->col, A->val,
+        k_dia_fill<BS><<<(int)(((int64_t)A->n + 255) / 256), 256, 0, ctx->stream>>>(dia_args(A), nd, A->ptr, A->col, A->val,
                                                                           A->dia.val, A->dia.mask, bad);
         st = rs_check_launch(ctx);
     }
@@ -358,7 +383,7 @@ template <int BS>
 int dia_launch(const rs_mat *A, const double *x, double alpha, double beta, const double *bvec, double *y,
                const int *skip, const double *dinv)
 {
-    const int grid = (int)((A->n + 255) / 256);
+    const int grid = (int)(((int64_t)A->nrows + 255) / 256);
     const DiaArgs a = dia_args(A);
     switch (A->dia.nd) {
 #define RS_DIA_CASE(ND)                                                                                          \
@@ -382,7 +407,7 @@ int dia_launch(const rs_mat *A, const double *x, double alpha, double beta, cons
 template <int BS>
 int presid_launch(const rs_mat *A, const double *p, const double *f, double *t, const int *skip)
 {
-    const int grid = (int)((A->n + 255) / 256);
+    const int grid = (int)(((int64_t)A->nrows + 255) / 256);
     const DiaArgs a = dia_args(A);
     switch (A->dia.nd) {
 #define RS_DIA_CASE(ND)                                                               \
