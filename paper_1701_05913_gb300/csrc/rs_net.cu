@@ -437,57 +437,91 @@ k_conv3_first(int D, int H, int W, const double *__restrict__ r, const double *_
 
 // ---------------------------------------------------------------------------
 // 3x3x3 convolution on the tcgen05 tensor cores (16 output channels), used
-// for the finest level.
+// for the finest level (and coarser ones, see use_tc).
 //
 // Implicit GEMM: D[voxel][co] = sum over taps t and input channels ci of
-// X[voxel + off_t][ci] W[t][co][ci].  A brick is 8 x 16 y BZ z output voxels;
-// per (tap, 16-channel chunk, z-plane) one tcgen05.mma with M = 128 (the
-// 8 x 16 voxels of a plane), N = 16, K = 16 accumulates in tensor memory.
+// X[voxel + off_t][ci] W[t][co][ci].  A block marches along z through columns
+// of 8 x 16 (x, y) voxels.  Per input plane h (10 x 18 with its halo), tap
+// (dy, dx) and 16-channel chunk, one tcgen05.mma with M = 128 (the voxels of
+// the column), K = 16 and N = 48 forms the plane's contribution to the three
+// output planes it touches: B = [W(dz = 0) | W(dz = 1) | W(dz = 2)] for the
+// planes h + 1, h and h - 1.  Each input plane has its own accumulator (48
+// columns of tensor memory); the epilogue of output plane z adds the three
+// partial sums of z's neighbours.
+//
+// Why N = 48 and a march: the tensor pipe takes an M = 128, K = 16 MMA about
+// every 42 cycles per SM for N up to 32 and 52 at N = 64, since each reads
+// 4 KB of A from shared memory.  Bricks of two output planes (N = 32, 36 MMAs
+// per 256 voxels, a quarter of them on zero weights, and each plane loaded
+// twice) took 1140 cycles per 128 voxels where the march has 9 MMAs.
 //
 // Operands sit in shared memory in the canonical no-swizzle K-major layout
-// (core matrix: 8 rows of 16 bytes).  The brick's input halo (10 x, 18 y,
-// BZ + 2 z) is one TMA box per 8-channel plane, stored [z][y][x][8 channels]:
-// a core matrix is 8 consecutive x of one y row (128 contiguous bytes), the
-// next core matrix along M is the next y row (160 bytes on) and the next 8
-// channels are the next plane.  A tap only moves the start address (by
-// 16 dx + 160 dy + one z slab dz), so one copy of the halo serves all 27.
+// (core matrix: 8 rows of 16 bytes).  A plane's halo is one TMA box per 8
+// channels, stored [y][x][8 channels]: a core matrix is 8 consecutive x of one
+// y row (128 contiguous bytes), the next one along M is the next y row (160
+// bytes on) and the next 8 channels are the next box.  A tap (dy, dx) only
+// moves the start address by 16 dx + 160 dy, so one copy serves all nine.
 //
-// The tensor pipe takes an M = 128, K = 16 MMA about every 42 cycles per SM
-// for N up to 32, so N = 16 caps the rate at a quarter of the dense peak.
-// The N dimension therefore stacks the brick's two z-planes: a halo plane hz
-// at tap (dy, dx) meets the weights of tap dz = hz - z for output plane z, so
-// one MMA with B = [W(hz) | W(hz - 1)] (zero blocks where dz is out of
-// range) serves both planes: 36 MMAs with N = 32 per brick and 16-channel
-// chunk instead of 54 with N = 16.  A single thread issues one MMA every
-// ~150 cycles, so four warps issue.  Warp roles, coupled only by mbarriers:
-//   warps 0-3   MMA issue (lane 0).  Warp w owns accumulator w of each TMEM
-//               set: halo plane w, both output planes; the four partial sums
-//               meet in the epilogue.
-//   warps 4-11  epilogue: tcgen05.ld of the partials, bias, ReLU, bf16 stores;
+// The planes of all columns are dealt to the blocks as one sequence, so every
+// block has the same number of output planes (plus two halo planes for each
+// piece of a column).  A single thread issues one MMA every ~150 cycles, so
+// four warps issue.  Warp roles, coupled only by mbarriers, t counting the
+// block's input planes:
+//   warps 0-3   MMA issue (lane 0): plane t on warp t mod 4, into accumulator
+//               set t mod NSET.
+//   warps 4-11  epilogue, two groups of four warps taking output planes in
+//               turn: tcgen05.ld of the partial sums, bias, ReLU, bf16 stores;
 //               a warp reads TMEM lanes 32 (warp mod 4) + 0..31.
 //   warp 12     producer (lane 0): TMA box loads into an NBUF-slot ring.
-// Barriers: full[slot] (TMA bytes), empty[slot] (the four issuers' MMAs
-// that read the slot completed), tfull[set] (accumulators ready), tempty[set]
-// (the epilogue has read them).  Every wait is bounded.
+// Barriers: full[slot] (TMA bytes), empty[slot] (the MMAs that read the slot
+// completed), tfull[set] (accumulator ready), tempty[set] (the three output
+// planes that use it have read it; the first and last plane of a piece, which
+// belong to one, are released by the epilogue steps beside them).  Every wait
+// is bounded.
 // ---------------------------------------------------------------------------
 template <int CIN>
 struct TcCfg {
-    static constexpr int BX = 8, BY = 16, BZ = 2;
-    static constexpr int HXb = BX + 2, HYb = BY + 2, HZb = BZ + 2;
+    static constexpr int BX = 8, BY = 16;
+    static constexpr int HXb = BX + 2, HYb = BY + 2;
     static constexpr int RS = HXb * 16;                      // bytes of one halo row (10 x, 8 channels)
-    static constexpr int BOX = HZb * HYb * RS;               // bytes of one plane's TMA box
-    static constexpr int PB = (BOX + 127) / 128 * 128;      // plane stride in shared memory
+    static constexpr int BOX = HYb * RS;                     // bytes of one TMA box: a plane's 8 channels
+    static constexpr int PB = (BOX + 127) / 128 * 128;       // box stride in shared memory
     static constexpr int NP = CIN / 8, KC = CIN / 16;
     static constexpr int SLOT = NP * PB;
-    static constexpr int NBUF = CIN == 16 ? 6 : 3;
-    // weights: [hz][dy dx][kc][k half][n = 16 z + co][8 channels], 1 KB a block
-    static constexpr int WB = 4 * 9 * KC * 1024;
+    static constexpr int NBUF = CIN == 16 ? 12 : 8;
+    // weights: [dy dx][kc][k half][n = 16 dz + co][8 channels]
+    static constexpr int N = 48, WBLK = N * 32, WHALF = N * 16;
+    static constexpr int WB = 9 * KC * WBLK;
     static constexpr int SMEM = NBUF * SLOT + WB;
-    static constexpr int ACC_COLS = 32;                     // one issuer's accumulator (N = 32)
-    static constexpr int NSET = 4, SET_COLS = 4 * ACC_COLS, TMEM_COLS = NSET * SET_COLS;
+    static constexpr int NSET = 8, SET_COLS = 64, TMEM_COLS = NSET * SET_COLS;
     static_assert(TMEM_COLS <= 512, "one CTA per SM holds all of TMEM at most");
     static_assert(SMEM <= 227 * 1024, "shared memory of one CTA");
     static constexpr int THREADS = 13 * 32;
+};
+
+// a block's share of the output planes, column after column, as pieces of
+// consecutive planes of one column
+struct TcPieces {
+    int nbx, D, p, end;
+    int bx, by, z0, lz;
+    __device__ __forceinline__ TcPieces(int D_, int H, int W) : D(D_)
+    {
+        nbx = (W + 7) / 8;
+        const int64_t total = (int64_t)nbx * ((H + 15) / 16) * D;
+        p = (int)(total * blockIdx.x / gridDim.x);
+        end = (int)(total * (blockIdx.x + 1) / gridDim.x);
+    }
+    __device__ __forceinline__ bool next()
+    {
+        if (p >= end) return false;
+        const int col = p / D;
+        bx = col % nbx;
+        by = col / nbx;
+        z0 = p - col * D;
+        lz = min(D - z0, end - p);
+        p += lz;
+        return true;
+    }
 };
 
 __device__ __forceinline__ uint64_t tc_desc(unsigned addr, unsigned lbo, unsigned sbo)
@@ -520,11 +554,10 @@ __device__ __forceinline__ void tc_mma(uint32_t tacc, uint64_t da, uint64_t db, 
                  : "memory");
 }
 
-// the MMAs of issuer WI for one brick: halo plane WI at the nine (dy, dx) and
-// each 16-channel chunk, N = 32 (both output planes).  With one chunk the
-// loop is unrolled (each descriptor is the slot's base plus a constant);
-// with two it is not, which keeps the descriptors out of registers.
-template <int CIN, int WI>
+// the MMAs of one input plane: the nine (dy, dx), each 16-channel chunk.  With
+// one chunk the loop is unrolled (each descriptor is the slot's base plus a
+// constant); with two it is not, which keeps the descriptors out of registers.
+template <int CIN>
 __device__ __forceinline__ void tc_issue(uint32_t tacc, uint64_t dA0, uint64_t dB0)
 {
     typedef TcCfg<CIN> C;
@@ -533,9 +566,9 @@ __device__ __forceinline__ void tc_issue(uint32_t tacc, uint64_t dA0, uint64_t d
         const int dy = j / 3, dx = j % 3;
 #pragma unroll
         for (int kc = 0; kc < C::KC; ++kc) {
-            const uint64_t da = dA0 + (uint64_t)((2 * kc * C::PB + (WI * C::HYb + dy) * C::RS + dx * 16) >> 4);
-            const uint64_t db = dB0 + (uint64_t)((((WI * 9 + j) * C::KC + kc) * 1024) >> 4);
-            tc_mma<32>(tacc, da, db, (j | kc) ? 1u : 0u);
+            const uint64_t da = dA0 + (uint64_t)((2 * kc * C::PB + dy * C::RS + dx * 16) >> 4);
+            const uint64_t db = dB0 + (uint64_t)(((j * C::KC + kc) * C::WBLK) >> 4);
+            tc_mma<C::N>(tacc, da, db, (j | kc) ? 1u : 0u);
         }
     }
 }
@@ -557,33 +590,28 @@ k_conv3_tc(int D, int H, int W, const __grid_constant__ CUtensorMap xmap, const 
     __shared__ float sbias[16], swh[17];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     // with wh (16 input channels only) the output head is applied in the
-    // epilogue and out written, and Y only if it is given: out[v] = (sum_c wh[c] y[v][c] +
-    // wh[16]) rms s, summed in channel order, non-finite values flagged
+    // epilogue and out written, and Y only if it is given: out[v] =
+    // (sum_c wh[c] y[v][c] + wh[16]) rms s, summed in channel order,
+    // non-finite values flagged
     const bool head = CIN == 16 && wh != nullptr;
-    const int nbx = (W + C::BX - 1) / C::BX, nby = (H + C::BY - 1) / C::BY, nbz = (D + C::BZ - 1) / C::BZ;
-    const int nbricks = nbx * nby * nbz;
-    const int nmine = blockIdx.x < nbricks ? (nbricks - 1 - blockIdx.x) / gridDim.x + 1 : 0;
 
-    // block (hz, dy dx, kc), column n = 16 z + co: W[dz = hz - z][dy][dx][co], zero for dz outside 0..2
-    for (int i = tid; i < 36 * C::KC * 32 * 2; i += blockDim.x) {
-        const int blk = i / 64, n = (i / 2) % 32, kh = i % 2;
-        const int kc = blk % C::KC, hz = blk / (9 * C::KC), j = (blk / C::KC) % 9, z = n >> 4, co = n & 15,
-                  dz = hz - z;
-        uint4 v = make_uint4(0, 0, 0, 0);
-        if (dz >= 0 && dz <= 2)
-            v = *(const uint4 *)(Wp + ((size_t)(dz * 9 + j) * 16 + co) * CIN + kc * 16 + kh * 8);
-        *(uint4 *)(wts + blk * 1024 + kh * 512 + (n >> 3) * 128 + (n & 7) * 16) = v;
+    // block (dy dx, kc), column n = 16 dz + co: W[dz][dy][dx][co]
+    for (int i = tid; i < 9 * C::KC * C::N * 2; i += blockDim.x) {
+        const int blk = i / (2 * C::N), n = (i / 2) % C::N, kh = i % 2;
+        const int kc = blk % C::KC, j = blk / C::KC, dz = n >> 4, co = n & 15;
+        *(uint4 *)(wts + blk * C::WBLK + kh * C::WHALF + (n >> 3) * 128 + (n & 7) * 16) =
+            *(const uint4 *)(Wp + ((size_t)(dz * 9 + j) * 16 + co) * CIN + kc * 16 + kh * 8);
     }
     if (tid < 16) sbias[tid] = bias[tid];
     if (head && tid < 17) swh[tid] = wh[tid];
     if (tid == 0) {
         for (int k = 0; k < C::NBUF; ++k) {
             mbar_init(&full[k], 1);
-            mbar_init(&empty[k], 4);
+            mbar_init(&empty[k], 1);
         }
         for (int k = 0; k < C::NSET; ++k) {
-            mbar_init(&tfull[k], 4);
-            mbar_init(&tempty[k], 256);
+            mbar_init(&tfull[k], 1);
+            mbar_init(&tempty[k], 12);          // three output planes, four warps each
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -597,125 +625,128 @@ k_conv3_tc(int D, int H, int W, const __grid_constant__ CUtensorMap xmap, const 
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 
+    TcPieces pc(D, H, W);
+    int t0 = 0;                                            // the piece's first input plane
     if (warp == 12) {
         // producer
         if (lane == 0) {
-            for (int k = 0; k < nmine; ++k) {
-                const int slot = k % C::NBUF, b = blockIdx.x + k * gridDim.x;
-                if (k >= C::NBUF) mbar_wait(&empty[slot], (unsigned)((k / C::NBUF - 1) & 1), limit, err);
-                const int bx = b % nbx, by = (b / nbx) % nby, bz = b / (nbx * nby);
-                mbar_arrive_expect_tx(&full[slot], (unsigned)(C::NP * C::BOX));
+            while (pc.next()) {
+                for (int i = 0; i < pc.lz + 2; ++i) {
+                    const int t = t0 + i, slot = t % C::NBUF;
+                    if (t >= C::NBUF) mbar_wait(&empty[slot], (unsigned)((t / C::NBUF - 1) & 1), limit, err);
+                    mbar_arrive_expect_tx(&full[slot], (unsigned)(C::NP * C::BOX));
 #pragma unroll
-                for (int pl = 0; pl < C::NP; ++pl) {
-                    // 16 input channels: both planes from X; 32: planes 0, 1 from the
-                    // upsampled coarse tensor, 2, 3 from X (the skip connection)
-                    const CUtensorMap *map = (CIN == 32 && pl < 2) ? &umap : &xmap;
-                    tma_load4(bufs + slot * C::SLOT + pl * C::PB, map, (pl & 1) * 8, bx * C::BX - 1, by * C::BY - 1,
-                              bz * C::BZ - 1, &full[slot]);
+                    for (int pl = 0; pl < C::NP; ++pl) {
+                        // 16 input channels: both boxes from X; 32: boxes 0, 1 from the
+                        // upsampled coarse tensor, 2, 3 from X (the skip connection)
+                        const CUtensorMap *map = (CIN == 32 && pl < 2) ? &umap : &xmap;
+                        tma_load4(bufs + slot * C::SLOT + pl * C::PB, map, (pl & 1) * 8, pc.bx * C::BX - 1,
+                                  pc.by * C::BY - 1, pc.z0 + i - 1, &full[slot]);
+                    }
                 }
+                t0 += pc.lz + 2;
             }
-            // the copies of the last bricks have landed before this block can end
-            for (int k = nmine > C::NBUF ? nmine - C::NBUF : 0; k < nmine; ++k)
-                mbar_wait(&full[k % C::NBUF], (unsigned)((k / C::NBUF) & 1), limit, err);
+            // the last copies have landed before this block can end
+            for (int t = t0 > C::NBUF ? t0 - C::NBUF : 0; t < t0; ++t)
+                mbar_wait(&full[t % C::NBUF], (unsigned)((t / C::NBUF) & 1), limit, err);
         }
     } else if (warp < 4) {
         // MMA issue
         if (lane == 0) {
-            // B: the k halves of a block are 512 bytes apart, 8-column groups 128
-            const uint64_t dB0 = tc_desc(smem_u32(wts), 512, 128);
-            for (int k = 0; k < nmine; ++k) {
-                const int slot = k % C::NBUF, set = k % C::NSET;
-                mbar_wait(&full[slot], (unsigned)((k / C::NBUF) & 1), limit, err);
-                if (k >= C::NSET) mbar_wait(&tempty[set], (unsigned)((k / C::NSET - 1) & 1), limit, err);
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t tacc = tmem_base + set * C::SET_COLS + warp * C::ACC_COLS;
-                const uint64_t dA0 = tc_desc(smem_u32(bufs + slot * C::SLOT), C::PB, C::RS);
-                switch (warp) {
-                case 0: tc_issue<CIN, 0>(tacc, dA0, dB0); break;
-                case 1: tc_issue<CIN, 1>(tacc, dA0, dB0); break;
-                case 2: tc_issue<CIN, 2>(tacc, dA0, dB0); break;
-                default: tc_issue<CIN, 3>(tacc, dA0, dB0); break;
+            // B: the k halves of a block are WHALF bytes apart, 8-column groups 128
+            const uint64_t dB0 = tc_desc(smem_u32(wts), C::WHALF, 128);
+            int last = -1;
+            while (pc.next()) {
+                for (int t = t0 + ((warp - t0) & 3); t < t0 + pc.lz + 2; t += 4) {
+                    const int slot = t % C::NBUF, set = t % C::NSET;
+                    mbar_wait(&full[slot], (unsigned)((t / C::NBUF) & 1), limit, err);
+                    if (t >= C::NSET) mbar_wait(&tempty[set], (unsigned)((t / C::NSET - 1) & 1), limit, err);
+                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    tc_issue<CIN>(tmem_base + set * C::SET_COLS, tc_desc(smem_u32(bufs + slot * C::SLOT), C::PB, C::RS),
+                                  dB0);
+                    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                                     smem_u32(&empty[slot]))
+                                 : "memory");
+                    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                                     smem_u32(&tfull[set]))
+                                 : "memory");
+                    last = t;
                 }
-                asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                                 smem_u32(&empty[slot]))
-                             : "memory");
-                asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                                 smem_u32(&tfull[set]))
-                             : "memory");
+                t0 += pc.lz + 2;
             }
             // this issuer's last MMAs have completed before TMEM is released
-            if (nmine > 0)
-                mbar_wait(&tfull[(nmine - 1) % C::NSET], (unsigned)(((nmine - 1) / C::NSET) & 1), limit, err);
+            if (last >= 0) mbar_wait(&tfull[last % C::NSET], (unsigned)((last / C::NSET) & 1), limit, err);
         }
     } else {
-        // epilogue: warps 4..11
-        const int e = warp - 4, q = warp & 3;
+        // epilogue: warps 4..11; step t reads the accumulators of planes
+        // t - 1, t, t + 1 and writes the output plane at t's z
+        const int grp = (warp - 4) >> 2, q = warp & 3;
         const int row = q * 32 + lane;                      // M row = TMEM lane
         const int x = row & 7, y = row >> 3;
-        const int z = C::BZ == 2 ? (e >> 2) : 0;
-        const int c0 = C::BZ == 2 ? 0 : (e >> 2) * 8;      // 32 input channels: two warps per quadrant
-        constexpr int NCOL = C::BZ == 2 ? 16 : 8;
-        for (int k = 0; k < nmine; ++k) {
-            const int set = k % C::NSET, b = blockIdx.x + k * gridDim.x;
-            mbar_wait(&tfull[set], (unsigned)((k / C::NSET) & 1), limit, err);
-            __syncwarp();   // the TMEM loads below are warp-collective
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            float f[NCOL];
+        const uint32_t tq = tmem_base + ((uint32_t)(q * 32) << 16);
+        auto ready = [&](int t) { mbar_wait(&tfull[t % C::NSET], (unsigned)((t / C::NSET) & 1), limit, err); };
+        auto release = [&](int t) { mbar_arrive(&tempty[t % C::NSET]); };
+        while (pc.next()) {
+            for (int i = (grp - t0) & 1; i < pc.lz + 2; i += 2) {
+                const int t = t0 + i;
+                const bool lo = i == 0, hi = i == pc.lz + 1;     // halo planes: nothing to write
+                if (!lo) ready(t - 1);
+                ready(t);
+                if (!hi) ready(t + 1);
+                __syncwarp();   // the TMEM loads below are warp-collective
+                float f[16];
+                if (!lo && !hi) {
+                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    uint32_t v[3][16];
 #pragma unroll
-            for (int j = 0; j < NCOL; ++j) f[j] = sbias[c0 + j];
+                    for (int dz = 0; dz < 3; ++dz) {
+                        const uint32_t ta = tq + ((t - 1 + dz) % C::NSET) * C::SET_COLS + 16 * dz;
+                        asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+                                     : "=r"(v[dz][0]), "=r"(v[dz][1]), "=r"(v[dz][2]), "=r"(v[dz][3]), "=r"(v[dz][4]),
+                                       "=r"(v[dz][5]), "=r"(v[dz][6]), "=r"(v[dz][7]), "=r"(v[dz][8]), "=r"(v[dz][9]),
+                                       "=r"(v[dz][10]), "=r"(v[dz][11]), "=r"(v[dz][12]), "=r"(v[dz][13]),
+                                       "=r"(v[dz][14]), "=r"(v[dz][15])
+                                     : "r"(ta));
+                    }
+                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-            for (int g = 0; g < 4; ++g) {
-                // issuer g's partial: plane z of its N = 32 accumulator, or its 16 columns
-                const uint32_t ta = tmem_base + ((uint32_t)(q * 32) << 16) + set * C::SET_COLS +
-                                    g * C::ACC_COLS + z * 16;
-                uint32_t v[16];
-                if constexpr (NCOL == 16) {
-                    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-                                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]),
-                                   "=r"(v[6]), "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]),
-                                   "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-                                 : "r"(ta));
-                } else {
-                    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]),
-                                   "=r"(v[6]), "=r"(v[7])
-                                 : "r"(ta));
+                    for (int j = 0; j < 16; ++j)
+                        f[j] = sbias[j] + __uint_as_float(v[0][j]) + __uint_as_float(v[1][j]) + __uint_as_float(v[2][j]);
                 }
-                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-                for (int j = 0; j < NCOL; ++j) f[j] += __uint_as_float(v[j]);
-            }
-            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-            mbar_arrive(&tempty[set]);
-            const int bx = b % nbx, by = (b / nbx) % nby, bz = b / (nbx * nby);
-            const int gx = bx * C::BX + x, gy = by * C::BY + y, gz = bz * C::BZ + z;
-            if (gx < W && gy < H && gz < D) {
+                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                __syncwarp();
+                if (lane == 0) {
+                    release(t);
+                    release(lo ? t : t - 1);
+                    release(hi ? t : t + 1);
+                }
+                const int gx = pc.bx * C::BX + x, gy = pc.by * C::BY + y, gz = pc.z0 + i - 1;
+                if (lo || hi || gx >= W || gy >= H) continue;
                 const int64_t vi = ((int64_t)gz * H + gy) * W + gx;
-                unsigned packed[NCOL / 2];
+                unsigned packed[8];
 #pragma unroll
-                for (int j = 0; j < NCOL / 2; ++j) {
+                for (int j = 0; j < 8; ++j) {
                     __nv_bfloat162 h = __floats2bfloat162_rn(fmaxf(f[2 * j], 0.f), fmaxf(f[2 * j + 1], 0.f));
                     packed[j] = *(unsigned *)&h;
                 }
-                if constexpr (NCOL == 16) {
-                    if (head) {
-                        float hs = swh[16];
+                if (head) {
+                    float hs = swh[16];
 #pragma unroll
-                        for (int j = 0; j < 8; ++j) {
-                            const __nv_bfloat162 h = *(const __nv_bfloat162 *)&packed[j];
-                            hs = fmaf(swh[2 * j], __low2float(h), hs);
-                            hs = fmaf(swh[2 * j + 1], __high2float(h), hs);
-                        }
-                        const double o = (double)hs * (scal[0] * (double)out_scale);
-                        out[vi] = o;
-                        if (flag && !isfinite(o)) atomicOr(flag, 1);
-                        if (!Y) continue;
+                    for (int j = 0; j < 8; ++j) {
+                        const __nv_bfloat162 h = *(const __nv_bfloat162 *)&packed[j];
+                        hs = fmaf(swh[2 * j], __low2float(h), hs);
+                        hs = fmaf(swh[2 * j + 1], __high2float(h), hs);
                     }
+                    const double o = (double)hs * (scal[0] * (double)out_scale);
+                    out[vi] = o;
+                    if (flag && !isfinite(o)) atomicOr(flag, 1);
+                    if (!Y) continue;
                 }
-                uint4 *dst = (uint4 *)(Y + vi * 16 + c0);
+                uint4 *dst = (uint4 *)(Y + vi * 16);
                 dst[0] = make_uint4(packed[0], packed[1], packed[2], packed[3]);
-                if constexpr (NCOL == 16) dst[1] = make_uint4(packed[4], packed[5], packed[6], packed[7]);
+                dst[1] = make_uint4(packed[4], packed[5], packed[6], packed[7]);
             }
+            t0 += pc.lz + 2;
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -1356,9 +1387,9 @@ static int pack_all(rs_net *net)
 
 // launches one forward convolution of layer l
 // The finest level's forward convolutions run on tcgen05, and so do a
-// coarser level's when it has at least two of the kernel's bricks (8 x 16 x 2
-// voxels) per SM: with fewer, the persistent pipeline's prologue (weights,
-// TMEM allocation, first copies) is not amortised and mma.sync is as fast.
+// coarser level's when it has at least two bricks of 8 x 16 x 2 voxels per
+// SM: with fewer, the persistent pipeline's prologue (weights, TMEM
+// allocation, first copies) is not amortised and mma.sync is as fast.
 static bool use_tc(const rs_net *net, int level)
 {
     const Level &L = net->lv[level];
@@ -1378,22 +1409,21 @@ static int conv_forward(rs_net *net, int l, const bf16 *X, const bf16 *U, const 
     const float *bias = net->p + net->boff[l];
     if (use_tc(net, kLayers[l].level) && kLayers[l].mode != IN_FIRST) {
         const CUtensorMap *xmap, *umap;
+        typedef TcCfg<16> TC;
+        RS_TRY(cached_tmap(net, &xmap, X, L.nx, L.ny, L.nz, TC::HXb, TC::HYb, 1));
+        // a block per SM; fewer when there are fewer output planes of 8 x 16 voxels
+        const int64_t planes = (int64_t)((L.nx + TC::BX - 1) / TC::BX) * ((L.ny + TC::BY - 1) / TC::BY) * L.nz;
+        const int tgrid = (int)std::min<int64_t>(planes, c->num_sms);
         if (kLayers[l].mode == IN_CATUP) {
             // the coarse input, upsampled to this level, is the first half of the concatenation
-            typedef TcCfg<32> TC;
-            RS_TRY(cached_tmap(net, &umap, net->up0, L.nx, L.ny, L.nz, TC::HXb, TC::HYb, TC::HZb));
-            RS_TRY(cached_tmap(net, &xmap, X, L.nx, L.ny, L.nz, TC::HXb, TC::HYb, TC::HZb));
+            RS_TRY(cached_tmap(net, &umap, net->up0, L.nx, L.ny, L.nz, TC::HXb, TC::HYb, 1));
             k_upsample2<<<ew_grid(c, L.nvox), 256, 0, c->stream>>>(L.nz, L.ny, L.nx, U, net->up0, skip);
             RS_TRY(rs_check_launch(c));
-            const int nb = ((L.nx + TC::BX - 1) / TC::BX) * ((L.ny + TC::BY - 1) / TC::BY) * ((L.nz + TC::BZ - 1) / TC::BZ);
-            k_conv3_tc<32><<<std::min(nb, c->num_sms), TC::THREADS, TC::SMEM, c->stream>>>(
+            k_conv3_tc<32><<<tgrid, TcCfg<32>::THREADS, TcCfg<32>::SMEM, c->stream>>>(
                 L.nz, L.ny, L.nx, *xmap, *umap, net->wf[l], bias, Y, c->d_err, c->spin_limit, skip, nullptr,
                 nullptr, 0.f, nullptr, nullptr);
         } else {
-            typedef TcCfg<16> TC;
-            RS_TRY(cached_tmap(net, &xmap, X, L.nx, L.ny, L.nz, TC::HXb, TC::HYb, TC::HZb));
-            const int nb = ((L.nx + TC::BX - 1) / TC::BX) * ((L.ny + TC::BY - 1) / TC::BY) * ((L.nz + TC::BZ - 1) / TC::BZ);
-            k_conv3_tc<16><<<std::min(nb, c->num_sms), TC::THREADS, TC::SMEM, c->stream>>>(
+            k_conv3_tc<16><<<tgrid, TC::THREADS, TC::SMEM, c->stream>>>(
                 L.nz, L.ny, L.nx, *xmap, *xmap, net->wf[l], bias, Y, c->d_err, c->spin_limit, skip,
                 hout ? net->p + net->hoff : nullptr, net->scal, net->out_scale, hout, net->flag);
         }
