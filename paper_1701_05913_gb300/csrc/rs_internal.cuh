@@ -117,8 +117,8 @@ struct rs_mat {
     struct {
         int nd = 0;              // distinct offsets col - row, ascending; 0: no such layout
         int off[8];
-        int64_t ld = 0;          // (scalar) rows, rounded up to 32
-        double *val = nullptr;   // [nd][bs][ld]: entry (offset k, block column c) of each scalar row
+        int64_t ld = 0;          // (block) rows, rounded up to 32
+        double *val = nullptr;   // [nd][bs][bs][ld]: entry (r, c) of each row's block at offset k
         unsigned char *mask = nullptr;   // [nrows] bit k: the row has an entry at offset k
     } dia;
     struct {
@@ -195,6 +195,11 @@ struct WaveLayout {
     void *lrec = nullptr, *urec = nullptr;  // L and U records in wave order (apply precision)
     void *rw = nullptr;                   // right-hand side in wave order
     void *yw = nullptr, *zw = nullptr;    // values of the L and U sweeps (sentinel protocol)
+    // small grids: both sweeps in one block (rs_level.cu); lrec and urec then
+    // hold its chunks, one per wavefront, and rw, yw, zw are not used
+    int one = 0, one_wc = 0, one_group = 2, one_nslots = 0, one_threads = 0;
+    int *one_place = nullptr;             // [n] padded cell of each natural row
+    int2 *one_cells = nullptr;            // [n] natural row, index in its wavefront
 };
 
 struct IluFactor {
@@ -373,6 +378,12 @@ int rs_wave_create(IluFactor *f, int nx, int ny, int nz);
 int rs_wave_gather(IluFactor *f);
 int rs_wave_apply(IluFactor *f, const double *r, double *z, const double *scale, const int *skip);
 void rs_wave_free(IluFactor *f);
+// one-block sweeps of small grids (rs_level.cu); fits: the rule, given the
+// hops between units on the wavefront sweeps' critical path
+bool rs_level_fits(int bs, int fp32, int nx, int ny, int nz, int hops);
+int rs_level_create(IluFactor *f);
+int rs_level_gather(IluFactor *f);
+int rs_level_apply(IluFactor *f, const double *r, double *z, const double *scale, const int *skip);
 // local: 0 = ILU(level), 1 = ILUT(ilut_p, ilut_tol) (scalar matrices)
 int rs_ras_create(rs_ctx *ctx, const rs_mat *A, int nparts, const int32_t *part, int overlap, int level, int local,
                   int ilut_p, double ilut_tol, int fp32, RasData **out, int *bad_row);

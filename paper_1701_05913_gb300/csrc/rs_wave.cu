@@ -963,6 +963,7 @@ int rs_wave_create(IluFactor *f, int nx, int ny, int nz)
     W.nyt = (ny + a - 1) / a;
     W.nzt = (nz + b - 1) / b;
     W.nunits = W.nyt * W.nzt;
+    if (rs_level_fits(bs, f->fp32, nx, ny, nz, W.nyt + W.nzt - 2)) return rs_level_create(f);
     const int nsteps = nx + a + b - 2;
     W.npad = (nsteps + G - 1) / G * G;       // whole chunks
     W.ncell = (int64_t)W.nunits * W.npad * 32;
@@ -1000,11 +1001,14 @@ void rs_wave_free(IluFactor *f)
     rs_free(ctx, W.rw);
     rs_free(ctx, W.yw);
     rs_free(ctx, W.zw);
+    rs_free(ctx, W.one_place);
+    rs_free(ctx, W.one_cells);
     W = WaveLayout();
 }
 
 int rs_wave_gather(IluFactor *f)
 {
+    if (f->W.one) return rs_level_gather(f);
     switch (f->bs) {
     case 1: return f->fp32 ? wave_gather_t<1, float>(f) : wave_gather_t<1, double>(f);
     case 2: return f->fp32 ? wave_gather_t<2, float>(f) : wave_gather_t<2, double>(f);
@@ -1016,6 +1020,7 @@ int rs_wave_gather(IluFactor *f)
 
 int rs_wave_apply(IluFactor *f, const double *r, double *z, const double *scale, const int *skip)
 {
+    if (f->W.one) return rs_level_apply(f, r, z, scale, skip);
     switch (f->bs) {
     case 1: return f->fp32 ? wave_apply_t<1, float>(f, r, z, scale, skip) : wave_apply_t<1, double>(f, r, z, scale, skip);
     case 2: return f->fp32 ? wave_apply_t<2, float>(f, r, z, scale, skip) : wave_apply_t<2, double>(f, r, z, scale, skip);

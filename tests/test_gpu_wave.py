@@ -55,6 +55,82 @@ def test_wave_ilu0_apply_matches_oracle_and_segments(rs, ctx, orc, shape):
         assert rel(zw.numpy(), zs.numpy()) <= 2 * tol
 
 
+# grids too large for the sweeps in one block (rs_level.cu), which the small
+# shapes here take: ragged tiles of the wavefront units
+@pytest.mark.parametrize("shape", [(33, 70, 40), (130, 37, 20), (5, 121, 67), (160, 10, 8)])
+@pytest.mark.parametrize("prec", ["fp64", "mixed"])
+def test_wave_units_ragged(rs, ctx, orc, shape, prec):
+    g = synth.Grid(*shape)
+    d = synth.pressure_7pt(g, 33, kz_scale=0.1)
+    A, Ao = rs.Mat.csr(ctx, d), orc.Mat.csr(d)
+    M = rs.Precond(ctx, A, "ilu0", prec=prec, sweep="wavefront")
+    _, _, lu = orc.ilu0(Ao)
+    r = np.random.default_rng(34).standard_normal(g.n)
+    z = rs.Vec.zeros(ctx, g.n)
+    for _ in range(2):
+        M.apply(rs.Vec(ctx, r), z)
+        assert rel(z.numpy(), orc.ilu0_solve(Ao, lu, r, fp32=(prec == "mixed"))) <= (1e-12 if prec == "fp64" else 1e-5)
+
+
+# the sweeps in one block: wavefronts of one cell, of an odd number, of more
+# than 128 rows; lines, planes and boxes; an odd number of wavefronts; blocks
+@pytest.mark.parametrize("shape,bs", [((2, 1, 2), 1), ((2, 2, 1), 1), ((64, 2, 1), 1), ((1, 9, 31), 1), ((17, 13, 11), 1),
+                                      ((20, 20, 20), 1), ((100, 9, 10), 1), ((6, 5, 7), 2), ((9, 8, 7), 3), ((16, 12, 9), 3),
+                                      ((5, 6, 4), 4)])
+@pytest.mark.parametrize("drop", [0.0, 0.3])
+def test_sweeps_in_one_block(rs, ctx, orc, shape, bs, drop):
+    g = synth.Grid(*shape)
+    if bs == 1:
+        m = synth.pressure_7pt(g, 35, kz_scale=0.1)
+        ptr, col, val = m["rowptr"], m["col"], m["val"].reshape(-1, 1)
+    else:
+        m = synth.black_oil_bsr3(g, 35)
+        if bs != 3:
+            m = _blocks_of_size(m, bs)
+        ptr, col, val = m["browptr"], m["bcol"], m["bval"].reshape(-1, bs * bs)
+    rows = np.repeat(np.arange(g.n), np.diff(ptr))
+    rng = np.random.default_rng(36)
+    keep = (rows == col) | (rng.random(col.size) >= drop)      # entries missing, diagonals never
+    ptr = np.concatenate([[0], np.cumsum(np.bincount(rows[keep], minlength=g.n))]).astype(np.int32)
+    col, val = col[keep], np.ascontiguousarray(val[keep]).reshape(-1)
+    r = rng.standard_normal(g.n * bs)
+    for prec in ("fp64", "mixed"):
+        fp32 = prec == "mixed"
+        if bs == 1:
+            d = dict(n=g.n, rowptr=ptr, col=col, val=val)
+            A, Ao = rs.Mat.csr(ctx, d), orc.Mat.csr(d)
+            ref = orc.ilu0_solve(Ao, orc.ilu0(Ao)[2], r, fp32=fp32)
+        else:
+            d = dict(nb=g.n, bs=bs, browptr=ptr, bcol=col, bval=val)
+            A, Ao = rs.Mat.bsr(ctx, d), orc.Mat.bsr(d)
+            _, _, lu, dinv = orc.bilu0(Ao)
+            ref = orc.bilu0_solve(Ao, lu, dinv, r, fp32=fp32)
+        M = rs.Precond(ctx, A, "ilu0" if bs == 1 else "bilu0", prec=prec)
+        z = rs.Vec.zeros(ctx, A.n)
+        for _ in range(2):
+            M.apply(rs.Vec(ctx, r), z)
+            assert rel(z.numpy(), ref) <= (1e-5 if fp32 else 1e-12)
+
+
+def test_sweeps_in_one_block_report_a_timeout(rs, ctx, orc):
+    """With a one-cycle limit a wait for the records records the timeout and
+    still sees them arrive: the result stays right and the context usable."""
+    g = synth.Grid(16, 12, 10)
+    d = synth.pressure_7pt(g, 37)
+    A, Ao = rs.Mat.csr(ctx, d), orc.Mat.csr(d)
+    M = rs.Precond(ctx, A, "ilu0")
+    r = np.random.default_rng(38).standard_normal(g.n)
+    z = rs.Vec.zeros(ctx, g.n)
+    ctx.set_spin_limit(1)
+    try:
+        M.apply(rs.Vec(ctx, r), z)
+        assert ctx.check() in (rs.OK, rs.ERR_DEVICE_TIMEOUT)
+    finally:
+        ctx.set_spin_limit(0)
+    assert rel(z.numpy(), orc.ilu0_solve(Ao, orc.ilu0(Ao)[2], r)) <= 1e-12
+    assert ctx.check() == rs.OK
+
+
 def test_wave_is_bit_stable_across_applies_and_scales(rs, ctx, orc):
     """The schedule is dynamic (tickets), the arithmetic is not: repeated
     applies give identical bits; a device scale multiplies r on entry."""
