@@ -26,12 +26,14 @@
 __global__ void k_amg_first(int n, const double *__restrict__ b, const double *__restrict__ dinv,
                             double *__restrict__ x, const int *skip)
 {
+    if (rs_pdl_wait()) return;
     if (skip && *(volatile const int *)skip) return;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) x[i] = b[i] * dinv[i];
 }
 
 __global__ void k_amg_copy(int n, const double *__restrict__ a, double *__restrict__ x, const int *skip)
 {
+    if (rs_pdl_wait()) return;
     if (skip && *(volatile const int *)skip) return;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) x[i] = a[i];
 }
@@ -52,6 +54,7 @@ __global__ void __launch_bounds__(32 * RS_HGS_WARPS)
 k_amg_hgs(int n, const int *__restrict__ ptr, const int *__restrict__ col, const double *__restrict__ val,
           const double *__restrict__ b, const double *__restrict__ xold, double *__restrict__ xnew, const int *skip)
 {
+    if (rs_pdl_wait()) return;
     __shared__ double xs[RS_HGS_WARPS][32];
     if (skip && *(volatile const int *)skip) return;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -140,6 +143,7 @@ k_amg_hgs(int n, const int *__restrict__ ptr, const int *__restrict__ col, const
 __global__ void k_amg_dense(int n, const double *__restrict__ inv, const double *__restrict__ b,
                             double *__restrict__ x, const int *skip)
 {
+    if (rs_pdl_wait()) return;
     if (skip && *(volatile const int *)skip) return;
     const int lane = threadIdx.x & 31;
     for (int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < n; i += (gridDim.x * blockDim.x) >> 5) {
@@ -221,7 +225,7 @@ static int vcycle(AmgData *M, int l, const double *b, double *x, const int *skip
     const int n = A->n;
     if (l == M->nlev - 1) {
         RsProfScope prof(ctx, RS_PROF_PRECOND_OTHER);
-        k_amg_dense<<<std::max(1, std::min((n + 7) / 8, ctx->num_sms * 4)), 256, 0, ctx->stream>>>(n, M->cinv, b, x,
+        rs_pdl(k_amg_dense, std::max(1, std::min((n + 7) / 8, ctx->num_sms * 4)), 256, 0, ctx)(n, M->cinv, b, x,
                                                                                                   skip);
         return rs_check_launch(ctx);
     }
@@ -236,13 +240,13 @@ static int vcycle(AmgData *M, int l, const double *b, double *x, const int *skip
     if (M->smoother == 1) {
         {
             RsProfScope prof(ctx, RS_PROF_PRECOND_OTHER);
-            k_amg_hgs<false><<<gh, 32 * RS_HGS_WARPS, 0, ctx->stream>>>(n, A->ptr, A->col, A->val, b, nullptr, cur, skip);
+            rs_pdl(k_amg_hgs<false>, gh, 32 * RS_HGS_WARPS, 0, ctx)(n, A->ptr, A->col, A->val, b, nullptr, cur, skip);
         }
         RS_TRY(rs_check_launch(ctx));
         for (int s = 1; s < nu; ++s) {
             {
                 RsProfScope prof(ctx, RS_PROF_PRECOND_OTHER);
-                k_amg_hgs<false><<<gh, 32 * RS_HGS_WARPS, 0, ctx->stream>>>(n, A->ptr, A->col, A->val, b, cur, oth, skip);
+                rs_pdl(k_amg_hgs<false>, gh, 32 * RS_HGS_WARPS, 0, ctx)(n, A->ptr, A->col, A->val, b, cur, oth, skip);
             }
             RS_TRY(rs_check_launch(ctx));
             std::swap(cur, oth);
@@ -250,7 +254,7 @@ static int vcycle(AmgData *M, int l, const double *b, double *x, const int *skip
     } else {
         {
             RsProfScope prof(ctx, RS_PROF_PRECOND_OTHER);
-            k_amg_first<<<g, 256, 0, ctx->stream>>>(n, b, M->d[l], cur, skip);
+            rs_pdl(k_amg_first, g, 256, 0, ctx)(n, b, M->d[l], cur, skip);
         }
         RS_TRY(rs_check_launch(ctx));
         for (int s = 1; s < nu; ++s) {
@@ -268,7 +272,7 @@ static int vcycle(AmgData *M, int l, const double *b, double *x, const int *skip
         if (M->smoother == 1) {   // backward sweeps: the adjoint of the forward ones
             {
                 RsProfScope prof(ctx, RS_PROF_PRECOND_OTHER);
-                k_amg_hgs<true><<<gh, 32 * RS_HGS_WARPS, 0, ctx->stream>>>(n, A->ptr, A->col, A->val, b, cur, oth, skip);
+                rs_pdl(k_amg_hgs<true>, gh, 32 * RS_HGS_WARPS, 0, ctx)(n, A->ptr, A->col, A->val, b, cur, oth, skip);
             }
             RS_TRY(rs_check_launch(ctx));
         } else {
@@ -279,7 +283,7 @@ static int vcycle(AmgData *M, int l, const double *b, double *x, const int *skip
     if (cur != X) {       // an odd number of post-smoothing sweeps
         {
             RsProfScope prof(ctx, RS_PROF_PRECOND_OTHER);
-            k_amg_copy<<<g, 256, 0, ctx->stream>>>(n, cur, X, skip);
+            rs_pdl(k_amg_copy, g, 256, 0, ctx)(n, cur, X, skip);
         }
         RS_TRY(rs_check_launch(ctx));
     }
@@ -325,8 +329,10 @@ int rs_amg_apply(AmgData *M, const double *r, double *z, const int *skip)
     int st = RS_ERR_CUDA;
     if (cudaStreamBeginCapture(M->capture, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
         ctx->stream = M->capture;
+        ctx->capturing = true;
         st = vcycle(M, 0, r, z, skip);
         ctx->stream = user;
+        ctx->capturing = false;
         const cudaError_t e = cudaStreamEndCapture(M->capture, &graph);
         if (e != cudaSuccess) st = RS_ERR_CUDA;
     }

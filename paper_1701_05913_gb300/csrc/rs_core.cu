@@ -286,11 +286,13 @@ static int blas_grid(rs_ctx *ctx, int n)
 
 __global__ void k_set(int n, double a, double *x)
 {
+    if (rs_pdl_wait()) return;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) x[i] = a;
 }
 
 __global__ void k_axpby(int n, double a, const double *__restrict__ x, double b, double *y)
 {
+    if (rs_pdl_wait()) return;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
         y[i] = b == 0.0 ? a * x[i] : fma(a, x[i], b * y[i]);
 }
@@ -298,6 +300,7 @@ __global__ void k_axpby(int n, double a, const double *__restrict__ x, double b,
 __global__ void k_axpbyz(int n, double a, const double *__restrict__ x, double b,
                          const double *__restrict__ y, double *__restrict__ z)
 {
+    if (rs_pdl_wait()) return;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
         z[i] = fma(a, x[i], b * y[i]);
 }
@@ -308,6 +311,7 @@ __global__ void __launch_bounds__(RS_RED_THREADS)
 k_dot(int n, const double *__restrict__ x, const double *__restrict__ y, double *partials,
       unsigned *ticket, double *out, int sqrt_out)
 {
+    if (rs_pdl_wait()) return;
     __shared__ double sm[RS_RED_THREADS / 32];
     __shared__ bool last;
     double a0 = 0, a1 = 0, a2 = 0, a3 = 0;
@@ -354,7 +358,7 @@ int rs_axpby_launch(rs_ctx *ctx, int n, double a, const double *x, double b, dou
 {
     if (n <= 0) return RS_OK;
     RsProfScope prof(ctx, RS_PROF_BLAS1);
-    k_axpby<<<blas_grid(ctx, n), 256, 0, ctx->stream>>>(n, a, x, b, y);
+    rs_pdl(k_axpby, blas_grid(ctx, n), 256, 0, ctx)(n, a, x, b, y);
     return rs_check_launch(ctx);
 }
 
@@ -365,7 +369,7 @@ int rs_dot_launch(rs_ctx *ctx, int n, const double *x, const double *y, double *
         return RS_OK;
     }
     RsProfScope prof(ctx, RS_PROF_BLAS1);
-    k_dot<<<dot_grid(ctx, n), RS_RED_THREADS, 0, ctx->stream>>>(n, x, y, ctx->red_partials,
+    rs_pdl(k_dot, dot_grid(ctx, n), RS_RED_THREADS, 0, ctx)(n, x, y, ctx->red_partials,
                                                                ctx->red_ticket, out_dev, 0);
     return rs_check_launch(ctx);
 }
@@ -441,7 +445,7 @@ extern "C" int rs_vec_set_value(rs_vec *x, double a)
 {
     if (!x) return RS_ERR_INVALID_ARG;
     if (x->n == 0) return RS_OK;
-    k_set<<<blas_grid(x->ctx, x->n), 256, 0, x->ctx->stream>>>(x->n, a, x->d);
+    rs_pdl(k_set, blas_grid(x->ctx, x->n), 256, 0, x->ctx)(x->n, a, x->d);
     return rs_check_launch(x->ctx);
 }
 
@@ -457,14 +461,14 @@ extern "C" int rs_vec_axpbyz(double a, const rs_vec *x, double b, const rs_vec *
     if (!x || !y || !z) return RS_ERR_INVALID_ARG;
     if (x->n != y->n || x->n != z->n) return RS_ERR_SIZE_MISMATCH;
     if (z->n == 0) return RS_OK;
-    k_axpbyz<<<blas_grid(z->ctx, z->n), 256, 0, z->ctx->stream>>>(z->n, a, x->d, b, y->d, z->d);
+    rs_pdl(k_axpbyz, blas_grid(z->ctx, z->n), 256, 0, z->ctx)(z->n, a, x->d, b, y->d, z->d);
     return rs_check_launch(z->ctx);
 }
 
 static int dot_to_host(rs_ctx *ctx, int n, const double *x, const double *y, int sq, double *out)
 {
     if (n == 0) { *out = 0.0; return RS_OK; }
-    k_dot<<<dot_grid(ctx, n), RS_RED_THREADS, 0, ctx->stream>>>(n, x, y, ctx->red_partials,
+    rs_pdl(k_dot, dot_grid(ctx, n), RS_RED_THREADS, 0, ctx)(n, x, y, ctx->red_partials,
                                                                ctx->red_ticket, ctx->d_scalars, sq);
     RS_TRY(rs_check_launch(ctx));
     RS_CUDA_TRY(cudaMemcpyAsync(ctx->h_pinned, ctx->d_scalars, sizeof(double),
@@ -503,6 +507,7 @@ k_spmv_csr(int n, const int *__restrict__ ptr, const int *__restrict__ col,
            const double *__restrict__ bvec, double *__restrict__ y, const int *skip,
            const double *__restrict__ dinv)
 {
+    if (rs_pdl_wait()) return;
     if (skip && *(volatile const int *)skip) return;
     const int gid = blockIdx.x * blockDim.x + threadIdx.x;
     const int row = gid / L;
@@ -565,6 +570,7 @@ k_spmv_csr_pipe(int n, const int *__restrict__ ptr, const int *__restrict__ col,
                 double *__restrict__ y, const int *skip, int *err, long long limit,
                 const double *__restrict__ dinv)
 {
+    if (rs_pdl_wait()) return;
     if (skip && *(volatile const int *)skip) return;
     extern __shared__ __align__(128) unsigned char spmv_smem[];
     SpmvStage *stg = (SpmvStage *)spmv_smem;
@@ -670,6 +676,7 @@ k_spmv_bsr(int nb, int bsr, const int *__restrict__ ptr, const int *__restrict__
            const double *__restrict__ val, const double *__restrict__ x, double alpha, double beta,
            const double *__restrict__ bvec, double *__restrict__ y, const int *skip)
 {
+    if (rs_pdl_wait()) return;
     if (skip && *(volatile const int *)skip) return;
     const int bs = BS > 0 ? BS : bsr;
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -710,7 +717,7 @@ static int spmv_dispatch(const rs_mat *A, const double *x, double alpha, double 
         }
         const int tiles = (A->n + RS_SPMV_TILE - 1) / RS_SPMV_TILE;
         const int grid = std::max(1, std::min(tiles, 3 * ctx->num_sms));
-        k_spmv_csr_pipe<<<grid, RS_SPMV_THREADS, RS_SPMV_SMEM, ctx->stream>>>(
+        rs_pdl(k_spmv_csr_pipe, grid, RS_SPMV_THREADS, RS_SPMV_SMEM, ctx)(
             A->n, A->ptr, A->col, A->val, x, alpha, beta, bvec, y, skip, ctx->d_err, ctx->spin_limit, dinv);
     } else if (A->bs == 1) {
         const int L = A->lanes;
@@ -719,7 +726,7 @@ static int spmv_dispatch(const rs_mat *A, const double *x, double alpha, double 
         switch (L) {
 #define RS_SPMV_CASE(LL)                                                                    \
     case LL:                                                                                \
-        k_spmv_csr<LL><<<grid, 256, 0, ctx->stream>>>(A->n, A->ptr, A->col, A->val, x, alpha, \
+        rs_pdl(k_spmv_csr<LL>, grid, 256, 0, ctx)(A->n, A->ptr, A->col, A->val, x, alpha, \
                                                       beta, bvec, y, skip, dinv);           \
         break;
             RS_SPMV_CASE(1)
@@ -735,13 +742,13 @@ static int spmv_dispatch(const rs_mat *A, const double *x, double alpha, double 
         const int64_t threads = (int64_t)A->nrows * A->bs;
         const int grid = (int)((threads + 255) / 256);
         if (A->bs == 3)
-            k_spmv_bsr<3><<<grid, 256, 0, ctx->stream>>>(A->nrows, 3, A->ptr, A->col, A->val, x,
+            rs_pdl(k_spmv_bsr<3>, grid, 256, 0, ctx)(A->nrows, 3, A->ptr, A->col, A->val, x,
                                                          alpha, beta, bvec, y, skip);
         else if (A->bs == 2)
-            k_spmv_bsr<2><<<grid, 256, 0, ctx->stream>>>(A->nrows, 2, A->ptr, A->col, A->val, x,
+            rs_pdl(k_spmv_bsr<2>, grid, 256, 0, ctx)(A->nrows, 2, A->ptr, A->col, A->val, x,
                                                          alpha, beta, bvec, y, skip);
         else
-            k_spmv_bsr<0><<<grid, 256, 0, ctx->stream>>>(A->nrows, A->bs, A->ptr, A->col, A->val,
+            rs_pdl(k_spmv_bsr<0>, grid, 256, 0, ctx)(A->nrows, A->bs, A->ptr, A->col, A->val,
                                                          x, alpha, beta, bvec, y, skip);
     }
     return rs_check_launch(ctx);

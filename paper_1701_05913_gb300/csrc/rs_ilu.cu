@@ -1097,6 +1097,7 @@ __global__ void __launch_bounds__(RS_SWEEP_THREADS)
 k_lsolve_seg(SegArgs g, const T *__restrict__ val, const T *__restrict__ mul, const double *__restrict__ r,
              const double *__restrict__ scale, T *y, T *zreset)
 {
+    if (rs_pdl_wait()) return;
     extern __shared__ __align__(16) unsigned char sweep_smem[];
     if (g.skip && *(volatile const int *)g.skip) return;
     const int lane = threadIdx.x & 31;
@@ -1195,6 +1196,7 @@ __global__ void __launch_bounds__(RS_SWEEP_THREADS)
 k_usolve_seg(SegArgs g, const T *__restrict__ val, const T *__restrict__ mul, const T *__restrict__ dinv, T *y,
              T *z, double *__restrict__ out)
 {
+    if (rs_pdl_wait()) return;
     extern __shared__ __align__(16) unsigned char sweep_smem[];
     if (g.skip && *(volatile const int *)g.skip) return;
     const int lane = threadIdx.x & 31;
@@ -1579,20 +1581,20 @@ static int apply_seg(IluFactor *f, const double *r, double *z, const double *sca
         RsProfScope prof(ctx, BS == 1 ? RS_PROF_LSWEEP : RS_PROF_BLSWEEP);
         const SegArgs a = seg_args(ctx, f->SL, f->nrows, f->state, skip);
         if (rl)
-            k_lsolve_seg<BS, T, BS == 1><<<gl, 32 * wl, sl, ctx->stream>>>(
+            rs_pdl(k_lsolve_seg<BS, T, BS == 1>, gl, 32 * wl, sl, ctx)(
                 a, (const T *)f->SL.val, (const T *)f->SL.mul, r, scale, y, zt);
         else
-            k_lsolve_seg<BS, T, false><<<gl, 32 * wl, sl, ctx->stream>>>(
+            rs_pdl(k_lsolve_seg<BS, T, false>, gl, 32 * wl, sl, ctx)(
                 a, (const T *)f->SL.val, (const T *)f->SL.mul, r, scale, y, zt);
     }
     RS_TRY(rs_check_launch(ctx));
     RsProfScope prof(ctx, BS == 1 ? RS_PROF_USWEEP : RS_PROF_BUSWEEP);
     const SegArgs a = seg_args(ctx, f->SU, f->nrows, f->state, skip);
     if (ru)
-        k_usolve_seg<BS, T, BS == 1><<<gu, 32 * wu, su, ctx->stream>>>(
+        rs_pdl(k_usolve_seg<BS, T, BS == 1>, gu, 32 * wu, su, ctx)(
             a, (const T *)f->SU.val, (const T *)f->SU.mul, (const T *)f->SU.rdiag, y, zt, z);
     else
-        k_usolve_seg<BS, T, false><<<gu, 32 * wu, su, ctx->stream>>>(
+        rs_pdl(k_usolve_seg<BS, T, false>, gu, 32 * wu, su, ctx)(
             a, (const T *)f->SU.val, (const T *)f->SU.mul, (const T *)f->SU.rdiag, y, zt, z);
     return rs_check_launch(ctx);
 }

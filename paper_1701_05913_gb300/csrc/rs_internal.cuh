@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <utility>
 #include <vector>
 
 #include "rs.h"
@@ -91,6 +92,7 @@ struct rs_ctx {
     // handles and context may be destroyed in any order
     int live = 0;
     bool closing = false;
+    bool capturing = false;  // the stream is being captured into a graph of the library's
 };
 
 // Records an event pair around the launches in its scope when profiling is on.
@@ -417,6 +419,53 @@ int rs_collect_device_error(rs_ctx *ctx, int *bad_row);
 // device helpers
 // ---------------------------------------------------------------------------
 #ifdef __CUDACC__
+// Programmatic dependent launch: rs_pdl(kernel, grid, block, smem, ctx)(args)
+// lets the kernel's blocks start while the kernel before it on the stream
+// drains, which hides launch latency (about 0.7 us a kernel of a chain) and
+// whatever the kernel does before rs_pdl_wait().  Every kernel launched this
+// way calls rs_pdl_wait() on every path before it reads or writes anything
+// that other kernels touch: it returns when the kernel before has completed
+// and its writes are visible.  The dependents are released after the wait, so
+// a kernel that runs early knows that all kernels but the last one are done.
+template <class... P>
+struct RsPdl {
+    void (*kernel)(P...);
+    dim3 grid, block;
+    size_t smem;
+    const rs_ctx *ctx;
+    template <class... A>
+    void operator()(A &&...a) const
+    {
+        cudaLaunchAttribute at;
+        at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at.val.programmaticStreamSerializationAllowed = 1;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = grid;
+        cfg.blockDim = block;
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = ctx->stream;
+        cfg.attrs = &at;
+        cfg.numAttrs = ctx->capturing ? 0 : 1;
+        cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(a)...);   // an error is read by rs_check_launch
+    }
+};
+template <class... P>
+RsPdl<P...> rs_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, const rs_ctx *ctx)
+{
+    return {kernel, grid, block, smem, ctx};
+}
+// Never true: `if (rs_pdl_wait()) return;` makes everything after it depend on
+// a value the compiler does not know, so that no load through a const
+// __restrict__ pointer (which it may take for one that never changes) is
+// moved up past the wait.
+__device__ __forceinline__ bool rs_pdl_wait()
+{
+    unsigned z;
+    asm volatile("griddepcontrol.wait;\n\tmov.u32 %0, 0;" : "=r"(z)::"memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    return z != 0;
+}
+
 __device__ __forceinline__ int ld_acquire(const int *p)
 {
     int v;

@@ -231,15 +231,12 @@ k_cgs_pass(int n, int ld, int nc, const double *__restrict__ V, double *w, doubl
            GmresDev *d, int *err, long long limit)
 {
     typedef CgsCfg<NC> C;
-    if (*(volatile int *)&d->cycle_done) return;
     extern __shared__ __align__(128) unsigned char cgs_smem[];
     double *ring = (double *)cgs_smem;
     unsigned long long *full = (unsigned long long *)(ring + C::S * C::STAGE);
     unsigned long long *empty = full + C::S;
     __shared__ double hs[NC];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (MODE != CGS_DOTS)
-        for (int k = threadIdx.x; k < nc; k += blockDim.x) hs[k] = MODE == CGS_UPDATE_DOTS ? d->h1[k] : d->h2[k];
     if (threadIdx.x == 0) {
         for (int s = 0; s < C::S; ++s) {
             mbar_init(&full[s], 1);
@@ -247,6 +244,10 @@ k_cgs_pass(int n, int ld, int nc, const double *__restrict__ V, double *w, doubl
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    if (rs_pdl_wait()) return;
+    if (*(volatile int *)&d->cycle_done) return;
+    if (MODE != CGS_DOTS)
+        for (int k = threadIdx.x; k < nc; k += blockDim.x) hs[k] = MODE == CGS_UPDATE_DOTS ? d->h1[k] : d->h2[k];
     __syncthreads();
     const int ntiles = (n + C::TILE - 1) / C::TILE;
     double acc[NC];
@@ -382,6 +383,7 @@ k_cgs_pass(int n, int ld, int nc, const double *__restrict__ V, double *w, doubl
 __global__ void k_basis_combine(int n, int ld, const double *__restrict__ B, const GmresDev *d,
                                 double *__restrict__ x, int add)
 {
+    if (rs_pdl_wait()) return;
     if (*(volatile const int *)&d->noupd) return;
     __shared__ double ys[RS_MAX_RESTART];
     const int k = d->k;
@@ -398,6 +400,7 @@ __global__ void k_basis_combine(int n, int ld, const double *__restrict__ B, con
 __global__ void k_scale_dev(int n, const double *__restrict__ r, const double *__restrict__ s,
                             double *__restrict__ v, const int *skip)
 {
+    if (rs_pdl_wait()) return;
     if (skip && *(volatile const int *)skip) return;
     const double a = *s;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) v[i] = r[i] * a;
@@ -407,6 +410,7 @@ __global__ void k_scale_dev(int n, const double *__restrict__ r, const double *_
 __global__ void k_scale_rsqrt(int n, const double *__restrict__ x, const double *__restrict__ n2,
                               double *__restrict__ y, const int *skip)
 {
+    if (rs_pdl_wait()) return;
     if (skip && *(volatile const int *)skip) return;
     const double s = *n2;
     const double a = s > 0.0 ? 1.0 / sqrt(s) : 0.0;
@@ -415,6 +419,7 @@ __global__ void k_scale_rsqrt(int n, const double *__restrict__ x, const double 
 
 __global__ void k_axpy_skip(int n, const double *__restrict__ x, double *__restrict__ y, const int *skip)
 {
+    if (rs_pdl_wait()) return;
     if (skip && *(volatile const int *)skip) return;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) y[i] += x[i];
 }
@@ -422,6 +427,7 @@ __global__ void k_axpy_skip(int n, const double *__restrict__ x, double *__restr
 // cycle start: beta = ||r||, convergence test on the true residual
 __global__ void k_gmres_start(GmresDev *d, const double *r2, double rtol, int first)
 {
+    if (rs_pdl_wait()) return;
     if (threadIdx.x != 0) return;
     const double beta = sqrt(*r2);
     if (first) {
@@ -443,6 +449,7 @@ __global__ void k_gmres_start(GmresDev *d, const double *r2, double rtol, int fi
 // global memory it took 62 us at k = 30, now 33)
 __global__ void __launch_bounds__(256) k_gmres_backsolve(GmresDev *d)
 {
+    if (rs_pdl_wait()) return;
     __shared__ double hs[(RS_MAX_RESTART * (RS_MAX_RESTART + 1)) / 2];   // column l: rows 0..l, from l (l + 1) / 2
     __shared__ double ys[RS_MAX_RESTART];
     const int k = d->k, m1 = d->m + 1;
@@ -489,7 +496,7 @@ static int launch_cgs_pass(rs_ctx *ctx, int n, int ld, int nc, double *V, GmresD
     }
     RsProfScope prof(ctx, MODE == CGS_DOTS ? RS_PROF_CGS_DOTS
                           : MODE == CGS_UPDATE_DOTS ? RS_PROF_CGS_UPDATE_DOTS : RS_PROF_CGS_UPDATE_NORM);
-    k_cgs_pass<NC, NCC, MODE><<<red_grid(ctx, n, C::TILE), C::THREADS, C::SMEM, ctx->stream>>>(
+    rs_pdl(k_cgs_pass<NC, NCC, MODE>, red_grid(ctx, n, C::TILE), C::THREADS, C::SMEM, ctx)(
         n, ld, nc, V, V + (size_t)nc * ld, ctx->red_partials, ctx->red_ticket, d, ctx->d_err, ctx->spin_limit);
     ctx->launches++;
     return rs_check_launch(ctx);
@@ -626,7 +633,7 @@ static int gmres_impl(const rs_mat *A, rs_pc *M, const rs_vec *bv, rs_vec *xv, i
             // true residual and cycle start
             st = rs_residual_launch(A, b, x, r, &d->r2, nullptr);
             if (st) goto out;
-            k_gmres_start<<<1, 32, 0, ctx->stream>>>(d, &d->r2, rtol, first);
+            rs_pdl(k_gmres_start, 1, 32, 0, ctx)(d, &d->r2, rtol, first);
             first = 0;
             ctx->launches++;
             int hs[4];
@@ -640,7 +647,7 @@ static int gmres_impl(const rs_mat *A, rs_pc *M, const rs_vec *bv, rs_vec *xv, i
             info->iters = hs[0];
             if (hs[3]) { status = RS_OK; break; }
             if (hs[2]) { status = RS_NOT_CONVERGED; break; }
-            k_scale_dev<<<gb, 256, 0, ctx->stream>>>(n, r, &d->hdiv, V, nullptr);
+            rs_pdl(k_scale_dev, gb, 256, 0, ctx)(n, r, &d->hdiv, V, nullptr);
             ctx->launches++;
             for (int i = 0; i < dim; ++i) {
                 if (i >= STEPS_AHEAD) {
@@ -670,35 +677,35 @@ static int gmres_impl(const rs_mat *A, rs_pc *M, const rs_vec *bv, rs_vec *xv, i
                 if (!st && cudaEventRecord(ev[i % STEPS_AHEAD], ctx->stream) != cudaSuccess) st = RS_ERR_CUDA;
                 if (st) goto out;
                 if (i + 1 < dim) {
-                    k_scale_dev<<<gb, 256, 0, ctx->stream>>>(n, w, &d->hdiv, w, cycle_done);
+                    rs_pdl(k_scale_dev, gb, 256, 0, ctx)(n, w, &d->hdiv, w, cycle_done);
                     ctx->launches++;
                 }
             }
-            k_gmres_backsolve<<<1, 256, 0, ctx->stream>>>(d);
+            rs_pdl(k_gmres_backsolve, 1, 256, 0, ctx)(d);
             ctx->launches++;
             if (flexible && aug_k > 0) {
                 // the correction t = Z y; x += t; t / ||t|| joins the ring
-                k_basis_combine<<<gb, 256, 0, ctx->stream>>>(n, ld, Z, d, t, 0);
-                k_axpy_skip<<<gb, 256, 0, ctx->stream>>>(n, t, x, noupd);
+                rs_pdl(k_basis_combine, gb, 256, 0, ctx)(n, ld, Z, d, t, 0);
+                rs_pdl(k_axpy_skip, gb, 256, 0, ctx)(n, t, x, noupd);
                 ctx->launches += 2;
                 st = rs_dot_launch(ctx, n, t, t, &d->augn2);
                 if (st) goto out;
-                k_scale_rsqrt<<<gb, 256, 0, ctx->stream>>>(n, t, &d->augn2, Aug + (size_t)head * ld, noupd);
+                rs_pdl(k_scale_rsqrt, gb, 256, 0, ctx)(n, t, &d->augn2, Aug + (size_t)head * ld, noupd);
                 ctx->launches++;
                 head = (head + 1) % aug_k;
                 naug = std::min(naug + 1, aug_k);
             } else if (flexible) {
-                k_basis_combine<<<gb, 256, 0, ctx->stream>>>(n, ld, Z, d, x, 1);
+                rs_pdl(k_basis_combine, gb, 256, 0, ctx)(n, ld, Z, d, x, 1);
                 ctx->launches++;
             } else {
-                k_basis_combine<<<gb, 256, 0, ctx->stream>>>(n, ld, V, d, r, 0);
+                rs_pdl(k_basis_combine, gb, 256, 0, ctx)(n, ld, V, d, r, 0);
                 ctx->launches++;
                 if (M) {
                     st = rs_pc_apply_dev(M, r, t, noupd);
                     if (st) goto out;
-                    k_axpy_skip<<<gb, 256, 0, ctx->stream>>>(n, t, x, noupd);
+                    rs_pdl(k_axpy_skip, gb, 256, 0, ctx)(n, t, x, noupd);
                 } else {
-                    k_axpy_skip<<<gb, 256, 0, ctx->stream>>>(n, r, x, noupd);
+                    rs_pdl(k_axpy_skip, gb, 256, 0, ctx)(n, r, x, noupd);
                 }
                 ctx->launches++;
             }
@@ -777,6 +784,7 @@ k_bicg(int op, int n, double *p, double *r, const double *__restrict__ v, double
        const double *__restrict__ sh, const double *__restrict__ rh, double *partials,
        unsigned *ticket, BicgDev *d)
 {
+    if (rs_pdl_wait()) return;
     if (op != 5 && (*(volatile int *)&d->done || *(volatile int *)&d->half)) return;
     if (op == 5 && !*(volatile int *)&d->half) return;
     const double alpha = d->alpha, omega = d->omega, beta = d->beta;
@@ -865,6 +873,7 @@ k_bicg(int op, int n, double *p, double *r, const double *__restrict__ v, double
 __global__ void k_bicg_restart(int n, const double *__restrict__ r, double *rh, double *p, double *v,
                                BicgDev *d)
 {
+    if (rs_pdl_wait()) return;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         rh[i] = r[i];
         p[i] = 0.0;
@@ -874,6 +883,7 @@ __global__ void k_bicg_restart(int n, const double *__restrict__ r, double *rh, 
 
 __global__ void k_bicg_restart_scalars(BicgDev *d, const double *r2)
 {
+    if (rs_pdl_wait()) return;
     if (threadIdx.x) return;
     const double rn = sqrt(*r2);
     d->implicit = rn;
@@ -948,15 +958,15 @@ extern "C" int rs_solve_bicgstab(const rs_mat *A, rs_pc *M, const rs_vec *bv, rs
             // (re)start from the true residual
             st = rs_residual_launch(A, b, x, r, &d->red[1], nullptr);
             if (st) goto out;
-            k_bicg_restart<<<gb, 256, 0, ctx->stream>>>(n, r, rh, p, v, d);
-            k_bicg_restart_scalars<<<1, 32, 0, ctx->stream>>>(d, &d->red[1]);
+            rs_pdl(k_bicg_restart, gb, 256, 0, ctx)(n, r, rh, p, v, d);
+            rs_pdl(k_bicg_restart_scalars, 1, 32, 0, ctx)(d, &d->red[1]);
             ctx->launches += 2;
             bool restart = false;
             while (!restart) {
                 for (int it = 0; it < batch; ++it) {
                     {
                         RsProfScope prof(ctx, RS_PROF_BLAS1);
-                        k_bicg<<<gr, RS_RED_THREADS, 0, ctx->stream>>>(0, n, p, r, v, s, t, x, ph, sh, rh,
+                        rs_pdl(k_bicg, gr, RS_RED_THREADS, 0, ctx)(0, n, p, r, v, s, t, x, ph, sh, rh,
                                                                        ctx->red_partials, ctx->red_ticket, d);
                     }
                     ctx->launches++;
@@ -966,17 +976,17 @@ extern "C" int rs_solve_bicgstab(const rs_mat *A, rs_pc *M, const rs_vec *bv, rs
                     if (st) goto out;
                     {
                         RsProfScope prof(ctx, RS_PROF_BLAS1);
-                        k_bicg<<<gr, RS_RED_THREADS, 0, ctx->stream>>>(3, n, p, r, v, s, t, x, ph, sh, rh,
+                        rs_pdl(k_bicg, gr, RS_RED_THREADS, 0, ctx)(3, n, p, r, v, s, t, x, ph, sh, rh,
                                                                        ctx->red_partials, ctx->red_ticket, d);
                     }
                     {
                         RsProfScope prof(ctx, RS_PROF_BLAS1);
-                        k_bicg<<<gr, RS_RED_THREADS, 0, ctx->stream>>>(1, n, p, r, v, s, t, x, ph, sh, rh,
+                        rs_pdl(k_bicg, gr, RS_RED_THREADS, 0, ctx)(1, n, p, r, v, s, t, x, ph, sh, rh,
                                                                        ctx->red_partials, ctx->red_ticket, d);
                     }
                     {
                         RsProfScope prof(ctx, RS_PROF_BLAS1);
-                        k_bicg<<<gr, RS_RED_THREADS, 0, ctx->stream>>>(5, n, p, r, v, s, t, x, ph, sh, rh,
+                        rs_pdl(k_bicg, gr, RS_RED_THREADS, 0, ctx)(5, n, p, r, v, s, t, x, ph, sh, rh,
                                                                        ctx->red_partials, ctx->red_ticket, d);
                     }
                     ctx->launches += 3;
@@ -986,12 +996,12 @@ extern "C" int rs_solve_bicgstab(const rs_mat *A, rs_pc *M, const rs_vec *bv, rs
                     if (st) goto out;
                     {
                         RsProfScope prof(ctx, RS_PROF_BLAS1);
-                        k_bicg<<<gr, RS_RED_THREADS, 0, ctx->stream>>>(4, n, p, r, v, s, t, x, ph, sh, rh,
+                        rs_pdl(k_bicg, gr, RS_RED_THREADS, 0, ctx)(4, n, p, r, v, s, t, x, ph, sh, rh,
                                                                        ctx->red_partials, ctx->red_ticket, d);
                     }
                     {
                         RsProfScope prof(ctx, RS_PROF_BLAS1);
-                        k_bicg<<<gr, RS_RED_THREADS, 0, ctx->stream>>>(2, n, p, r, v, s, t, x, ph, sh, rh,
+                        rs_pdl(k_bicg, gr, RS_RED_THREADS, 0, ctx)(2, n, p, r, v, s, t, x, ph, sh, rh,
                                                                        ctx->red_partials, ctx->red_ticket, d);
                     }
                     ctx->launches += 2;
@@ -1051,6 +1061,7 @@ __global__ void __launch_bounds__(RS_RED_THREADS)
 k_cg(int op, int n, double *x, double *r, const double *__restrict__ z, double *p,
      const double *__restrict__ q, double *partials, unsigned *ticket, CgDev *d)
 {
+    if (rs_pdl_wait()) return;
     if (*(volatile int *)&d->done) return;
     const double alpha = d->alpha, beta = d->beta;
     double acc[1] = {0.0};
@@ -1102,6 +1113,7 @@ k_cg(int op, int n, double *x, double *r, const double *__restrict__ z, double *
 // restart from the true residual (in r, ||r||^2 in *r2): p = 0, first pass
 __global__ void k_cg_restart(int n, double *p, CgDev *d, const double *r2)
 {
+    if (rs_pdl_wait()) return;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) p[i] = 0.0;
     if (blockIdx.x || threadIdx.x) return;
     const double rn = sqrt(*r2);
@@ -1165,7 +1177,7 @@ extern "C" int rs_solve_cg(const rs_mat *A, rs_pc *M, const rs_vec *bv, rs_vec *
         for (;;) {
             st = rs_residual_launch(A, b, x, r, &d->red[1], nullptr);
             if (st) goto out;
-            k_cg_restart<<<gb, 256, 0, ctx->stream>>>(n, p, d, &d->red[1]);
+            rs_pdl(k_cg_restart, gb, 256, 0, ctx)(n, p, d, &d->red[1]);
             ctx->launches++;
             bool restart = false;
             while (!restart) {
@@ -1174,12 +1186,12 @@ extern "C" int rs_solve_cg(const rs_mat *A, rs_pc *M, const rs_vec *bv, rs_vec *
                     if (st) goto out;
                     {
                         RsProfScope prof(ctx, RS_PROF_BLAS1);
-                        k_cg<<<gr, RS_RED_THREADS, 0, ctx->stream>>>(0, n, x, r, z, p, q, ctx->red_partials,
+                        rs_pdl(k_cg, gr, RS_RED_THREADS, 0, ctx)(0, n, x, r, z, p, q, ctx->red_partials,
                                                                      ctx->red_ticket, d);
                     }
                     {
                         RsProfScope prof(ctx, RS_PROF_BLAS1);
-                        k_cg<<<gb, RS_RED_THREADS, 0, ctx->stream>>>(1, n, x, r, z, p, q, ctx->red_partials,
+                        rs_pdl(k_cg, gb, RS_RED_THREADS, 0, ctx)(1, n, x, r, z, p, q, ctx->red_partials,
                                                                      ctx->red_ticket, d);
                     }
                     ctx->launches += 2;
@@ -1187,12 +1199,12 @@ extern "C" int rs_solve_cg(const rs_mat *A, rs_pc *M, const rs_vec *bv, rs_vec *
                     if (st) goto out;
                     {
                         RsProfScope prof(ctx, RS_PROF_BLAS1);
-                        k_cg<<<gr, RS_RED_THREADS, 0, ctx->stream>>>(2, n, x, r, z, p, q, ctx->red_partials,
+                        rs_pdl(k_cg, gr, RS_RED_THREADS, 0, ctx)(2, n, x, r, z, p, q, ctx->red_partials,
                                                                      ctx->red_ticket, d);
                     }
                     {
                         RsProfScope prof(ctx, RS_PROF_BLAS1);
-                        k_cg<<<gr, RS_RED_THREADS, 0, ctx->stream>>>(3, n, x, r, z, p, q, ctx->red_partials,
+                        rs_pdl(k_cg, gr, RS_RED_THREADS, 0, ctx)(3, n, x, r, z, p, q, ctx->red_partials,
                                                                      ctx->red_ticket, d);
                     }
                     ctx->launches += 2;

@@ -109,7 +109,6 @@ __global__ void __launch_bounds__(LV_MAX_ROWS + 32)
 k_level_solve(LevelArgs g, const unsigned char *__restrict__ lbuf, const unsigned char *__restrict__ ubuf,
               const double *__restrict__ r, const double *__restrict__ scale, double *__restrict__ z)
 {
-    if (g.skip && *(volatile const int *)g.skip) return;
     extern __shared__ __align__(128) unsigned char lv_smem[];
     unsigned long long *full = (unsigned long long *)lv_smem;
     const int vbytes = lv_values<BS, T>(g.ncell);
@@ -134,6 +133,8 @@ k_level_solve(LevelArgs g, const unsigned char *__restrict__ lbuf, const unsigne
                 ((int *)(ring + sl * sb + w * ub))[tid] = -1;
             }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    if (rs_pdl_wait()) return;
+    if (g.skip && *(volatile const int *)g.skip) return;
     __syncthreads();
     const int groups = 2 * g.ngroup;
     if (tid >= nio) {
@@ -463,7 +464,7 @@ int level_apply(IluFactor *f, const double *r, double *z, const double *scale, c
                         (size_t)g.nslots * g.group * lv_chunk<BS, T, 4>(g.wc);
     // L and U are one kernel: the profiler counts it as the L sweep
     RsProfScope prof(ctx, BS == 1 ? RS_PROF_LSWEEP : RS_PROF_BLSWEEP);
-    k_level_solve<BS, T><<<1, std::max(W.one_threads, LV_IO_THREADS) + 32, smem, ctx->stream>>>(
+    rs_pdl(k_level_solve<BS, T>, 1, std::max(W.one_threads, LV_IO_THREADS) + 32, smem, ctx)(
         g, (const unsigned char *)W.lrec, (const unsigned char *)W.urec, r, scale, z);
     return rs_check_launch(ctx);
 }

@@ -197,7 +197,6 @@ __global__ void __launch_bounds__(CONV_THREADS)
 k_conv3(int D, int H, int W, const bf16 *__restrict__ X, const bf16 *__restrict__ U, const bf16 *__restrict__ Wp, const float *__restrict__ bias, int relu, bf16 *__restrict__ Y,
         const int *skip)
 {
-    if (skipped(skip)) return;
     constexpr int SIN = CIN + 8, SW = CIN + 8;
     extern __shared__ __align__(16) unsigned char smraw[];
     bf16 *sx = (bf16 *)smraw;
@@ -212,8 +211,12 @@ k_conv3(int D, int H, int W, const bf16 *__restrict__ X, const bf16 *__restrict_
         const int row = i / WCH, ch = i % WCH;
         cp_async16(sw + row * SW + ch * 8, Wp + (size_t)row * CIN + ch * 8, true);
     }
-    load_halo<CIN, MODE>(sx, SIN, D, H, W, tx0, ty0, tz0, X, U, nullptr, nullptr, nullptr);
+    // the weights were written at least two kernels ago: under way before the wait
+    if (rs_pdl_wait()) return;
+    const bool off = skipped(skip);
+    if (!off) load_halo<CIN, MODE>(sx, SIN, D, H, W, tx0, ty0, tz0, X, U, nullptr, nullptr, nullptr);
     cp_async_wait_all();
+    if (off) return;
     __syncthreads();
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -322,6 +325,7 @@ k_conv3_first(int D, int H, int W, const double *__restrict__ r, const double *_
               const double *__restrict__ rscale, const bf16 *__restrict__ Wp, const float *__restrict__ bias,
               bf16 *__restrict__ Y, const int *skip)
 {
+    if (rs_pdl_wait()) return;
     if (skipped(skip)) return;
     __shared__ __align__(16) bf16 sb[16 * FKS];
     __shared__ unsigned sh[FSH];            // the halo, then zeros for the padding taps
@@ -581,7 +585,6 @@ k_conv3_tc(int D, int H, int W, const __grid_constant__ CUtensorMap xmap, const 
            float out_scale, double *__restrict__ out, int *flag)
 {
     typedef TcCfg<CIN> C;
-    if (skipped(skip)) return;
     extern __shared__ __align__(1024) unsigned char tc_smem[];
     unsigned char *bufs = tc_smem;                         // NBUF x SLOT
     unsigned char *wts = tc_smem + C::NBUF * C::SLOT;      // WB
@@ -625,7 +628,11 @@ k_conv3_tc(int D, int H, int W, const __grid_constant__ CUtensorMap xmap, const 
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 
+    // up to here nothing of the kernel before is read: the weights and biases
+    // were written at least two kernels ago
+    if (rs_pdl_wait()) return;
     TcPieces pc(D, H, W);
+    if (skipped(skip)) pc.end = pc.p;
     int t0 = 0;                                            // the piece's first input plane
     if (warp == 12) {
         // producer
@@ -760,6 +767,7 @@ k_conv3_tc(int D, int H, int W, const __grid_constant__ CUtensorMap xmap, const 
 // nearest-neighbour x2 upsampling of a 16-channel tensor: Uf[z][y][x] = Uc[z/2][y/2][x/2]
 __global__ void k_upsample2(int D, int H, int W, const bf16 *__restrict__ Uc, bf16 *__restrict__ Uf, const int *skip)
 {
+    if (rs_pdl_wait()) return;
     if (skipped(skip)) return;
     const int64_t n = (int64_t)D * H * W;
     const int W2 = W >> 1, H2 = H >> 1;
@@ -797,6 +805,7 @@ k_conv3_dw(int D, int H, int W, const bf16 *__restrict__ X, const bf16 *__restri
            const bf16 *__restrict__ Gp, const bf16 *__restrict__ Yact, bf16 *__restrict__ Gm,
            float *__restrict__ partial)
 {
+    if (rs_pdl_wait()) return;
     constexpr int SIN = dw_sin(CIN), SG = 24;
     extern __shared__ __align__(16) unsigned char smraw[];
     bf16 *sx = (bf16 *)smraw;
@@ -909,6 +918,7 @@ __global__ void __launch_bounds__(32 * DWR_GROUPS)
 k_dw_reduce(int nblocks, int cin, int cinp, const float *__restrict__ partial, float *grad, int64_t woff, int64_t boff,
             float wscale)
 {
+    if (rs_pdl_wait()) return;
     __shared__ float sm[DWR_GROUPS][32];
     const int stride = 27 * 16 * cinp + 16;
     const int c = threadIdx.x & 31, g = threadIdx.x >> 5;
@@ -943,6 +953,7 @@ k_dw_reduce(int nblocks, int cin, int cinp, const float *__restrict__ partial, f
 // FP32 in (dz, dy, dx) order
 __global__ void k_avgpool(int Dc, int Hc, int Wc, const bf16 *__restrict__ X, bf16 *__restrict__ Y, const int *skip)
 {
+    if (rs_pdl_wait()) return;
     if (skipped(skip)) return;
     const int64_t n = (int64_t)Dc * Hc * Wc * 2;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
@@ -978,6 +989,7 @@ __global__ void k_avgpool(int Dc, int Hc, int Wc, const bf16 *__restrict__ X, bf
 // 8-channel half, 16-byte loads
 __global__ void k_up_backward(int Dc, int Hc, int Wc, const bf16 *__restrict__ gcat, bf16 *__restrict__ gc)
 {
+    if (rs_pdl_wait()) return;
     const int64_t n = (int64_t)Dc * Hc * Wc * 2;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const int h = (int)(i & 1);
@@ -1009,6 +1021,7 @@ __global__ void k_up_backward(int Dc, int Hc, int Wc, const bf16 *__restrict__ g
 __global__ void k_pool_backward_add(int D, int H, int W, const bf16 *__restrict__ gcoarse,
                                     const bf16 *__restrict__ gcat, bf16 *__restrict__ out)
 {
+    if (rs_pdl_wait()) return;
     const int64_t n = (int64_t)D * H * W * 2;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const int h = (int)(i & 1);
@@ -1031,6 +1044,7 @@ __global__ void k_pool_backward_add(int D, int H, int W, const bf16 *__restrict_
 __global__ void __launch_bounds__(256)
 k_rms(int64_t n, const double *__restrict__ r, double *red, unsigned *ticket, double *scal, const int *skip)
 {
+    if (rs_pdl_wait()) return;
     if (skipped(skip)) return;
     __shared__ double sm[8];
     __shared__ bool last;
@@ -1088,6 +1102,7 @@ __global__ void __launch_bounds__(256)
 k_loss_sums(int64_t n, const double *__restrict__ o, const double *__restrict__ e, double *red, unsigned *ticket,
             double *scal)
 {
+    if (rs_pdl_wait()) return;
     __shared__ double sm[2][8];
     __shared__ bool last;
     double s0 = 0.0, s1 = 0.0;
@@ -1134,6 +1149,7 @@ k_head_backward(int64_t n, const bf16 *__restrict__ x, const float *__restrict__
                 float out_scale, const double *__restrict__ o, const double *__restrict__ e, double w,
                 bf16 *__restrict__ dx, float *__restrict__ hp)
 {
+    if (rs_pdl_wait()) return;
     __shared__ float sm[8][17];
     const double sc = scal[0] * (double)out_scale;
     const double den = scal[3] > 0.0 ? scal[3] : 1.0;
@@ -1178,6 +1194,7 @@ k_head_backward(int64_t n, const bf16 *__restrict__ x, const float *__restrict__
 __global__ void __launch_bounds__(17 * 32)
 k_head_reduce(int nblocks, const float *__restrict__ hp, float *grad, int64_t hoff)
 {
+    if (rs_pdl_wait()) return;
     const int c = threadIdx.x >> 5, lane = threadIdx.x & 31;
     float s = 0.f;
     for (int b = lane; b < nblocks; b += 32) s += hp[b * 17 + c];
@@ -1417,13 +1434,13 @@ static int conv_forward(rs_net *net, int l, const bf16 *X, const bf16 *U, const 
         if (kLayers[l].mode == IN_CATUP) {
             // the coarse input, upsampled to this level, is the first half of the concatenation
             RS_TRY(cached_tmap(net, &umap, net->up0, L.nx, L.ny, L.nz, TC::HXb, TC::HYb, 1));
-            k_upsample2<<<ew_grid(c, L.nvox), 256, 0, c->stream>>>(L.nz, L.ny, L.nx, U, net->up0, skip);
+            rs_pdl(k_upsample2, ew_grid(c, L.nvox), 256, 0, c)(L.nz, L.ny, L.nx, U, net->up0, skip);
             RS_TRY(rs_check_launch(c));
-            k_conv3_tc<32><<<tgrid, TcCfg<32>::THREADS, TcCfg<32>::SMEM, c->stream>>>(
+            rs_pdl(k_conv3_tc<32>, tgrid, TcCfg<32>::THREADS, TcCfg<32>::SMEM, c)(
                 L.nz, L.ny, L.nx, *xmap, *umap, net->wf[l], bias, Y, c->d_err, c->spin_limit, skip, nullptr,
                 nullptr, 0.f, nullptr, nullptr);
         } else {
-            k_conv3_tc<16><<<tgrid, TC::THREADS, TC::SMEM, c->stream>>>(
+            rs_pdl(k_conv3_tc<16>, tgrid, TC::THREADS, TC::SMEM, c)(
                 L.nz, L.ny, L.nx, *xmap, *xmap, net->wf[l], bias, Y, c->d_err, c->spin_limit, skip,
                 hout ? net->p + net->hoff : nullptr, net->scal, net->out_scale, hout, net->flag);
         }
@@ -1432,15 +1449,15 @@ static int conv_forward(rs_net *net, int l, const bf16 *X, const bf16 *U, const 
     if (hout) return RS_ERR_INVALID_ARG;        // the head is fused on the tcgen05 path only
     switch (kLayers[l].mode) {
     case IN_FIRST:
-        k_conv3_first<<<std::min(grid, c->num_sms * 4), CONV_THREADS, 0, c->stream>>>(
+        rs_pdl(k_conv3_first, std::min(grid, c->num_sms * 4), CONV_THREADS, 0, c)(
             L.nz, L.ny, L.nx, r, logk, net->scal + 1, net->wf[l], bias, Y, skip);
         break;
     case IN_CATUP:
-        k_conv3<32, 16, IN_CATUP><<<grid, CONV_THREADS, conv_smem(32, 16), c->stream>>>(
+        rs_pdl(k_conv3<32, 16, IN_CATUP>, grid, CONV_THREADS, conv_smem(32, 16), c)(
             L.nz, L.ny, L.nx, X, U, net->wf[l], bias, 1, Y, skip);
         break;
     default:
-        k_conv3<16, 16, IN_PLAIN><<<grid, CONV_THREADS, conv_smem(16, 16), c->stream>>>(
+        rs_pdl(k_conv3<16, 16, IN_PLAIN>, grid, CONV_THREADS, conv_smem(16, 16), c)(
             L.nz, L.ny, L.nx, X, nullptr, net->wf[l], bias, 1, Y, skip);
     }
     return rs_check_launch(c);
@@ -1450,7 +1467,7 @@ static int pool_forward(rs_net *net, int lvl, const bf16 *X, bf16 *Y, const int 
 {
     rs_ctx *c = net->ctx;
     const Level &L = net->lv[lvl];
-    k_avgpool<<<ew_grid(c, L.nvox * 2), 256, 0, c->stream>>>(L.nz, L.ny, L.nx, X, Y, skip);
+    rs_pdl(k_avgpool, ew_grid(c, L.nvox * 2), 256, 0, c)(L.nz, L.ny, L.nx, X, Y, skip);
     return rs_check_launch(c);
 }
 
@@ -1465,7 +1482,7 @@ static int net_forward(rs_net *net, const double *r, const double *logk, double 
     // one profiler interval over the whole pass: the kernels, without the
     // host work between their launches
     RsProfScope prof(c, RS_PROF_NET);
-    k_rms<<<c->red_blocks, 256, 0, c->stream>>>(n0, r, net->red, net->ticket, net->scal, skip);
+    rs_pdl(k_rms, c->red_blocks, 256, 0, c)(n0, r, net->red, net->ticket, net->scal, skip);
     RS_TRY(rs_check_launch(c));
     bf16 **A = net->act;
     RS_TRY(conv_forward(net, E0A, nullptr, nullptr, r, logk, A[E0A], skip));
@@ -1496,10 +1513,10 @@ static int launch_dw(rs_net *net, int l, const bf16 *X, const bf16 *U, const dou
     rs_ctx *c = net->ctx;
     const Level &L = net->lv[kLayers[l].level];
     const int grid = (int)std::min<int64_t>(nbricks(L), (int64_t)dw_blocks_per_sm(CIN) * c->num_sms);
-    k_conv3_dw<CIN, MODE><<<grid, CONV_THREADS, dw_smem(CIN), c->stream>>>(
+    rs_pdl(k_conv3_dw<CIN, MODE>, grid, CONV_THREADS, dw_smem(CIN), c)(
         L.nz, L.ny, L.nx, X, U, r, logk, net->scal + 1, Gp, net->act[l], Gm, net->partials);
     RS_TRY(rs_check_launch(c));
-    k_dw_reduce<<<(27 * 16 * CIN + 16 + 31) / 32, 32 * DWR_GROUPS, 0, c->stream>>>(
+    rs_pdl(k_dw_reduce, (27 * 16 * CIN + 16 + 31) / 32, 32 * DWR_GROUPS, 0, c)(
         grid, kLayers[l].cin, CIN, net->partials, net->g, net->woff[l], net->boff[l], wscale);
     return rs_check_launch(c);
 }
@@ -1523,10 +1540,10 @@ static int conv_dx(rs_net *net, int l, const bf16 *G, bf16 *dX)
     const int grid = (int)nbricks(L);
     RsProfScope prof(c, RS_PROF_NET);
     if (kLayers[l].cin == 32)
-        k_conv3<16, 32, IN_PLAIN><<<grid, CONV_THREADS, conv_smem(16, 32), c->stream>>>(
+        rs_pdl(k_conv3<16, 32, IN_PLAIN>, grid, CONV_THREADS, conv_smem(16, 32), c)(
             L.nz, L.ny, L.nx, G, nullptr, net->wb[l], nullptr, 0, dX, nullptr);
     else
-        k_conv3<16, 16, IN_PLAIN><<<grid, CONV_THREADS, conv_smem(16, 16), c->stream>>>(
+        rs_pdl(k_conv3<16, 16, IN_PLAIN>, grid, CONV_THREADS, conv_smem(16, 16), c)(
             L.nz, L.ny, L.nx, G, nullptr, net->wb[l], nullptr, 0, dX, nullptr);
     return rs_check_launch(c);
 }
@@ -1550,9 +1567,9 @@ static int net_backward(rs_net *net, const double *r, const double *logk, const 
     {
         RsProfScope prof(c, RS_PROF_NET);
         const int hb = std::min<int64_t>((n0 + 255) / 256, (int64_t)c->num_sms * 4);
-        k_head_backward<<<hb, 256, 0, c->stream>>>(n0, A[D0B], net->p + net->hoff, net->scal, net->out_scale,
+        rs_pdl(k_head_backward, hb, 256, 0, c)(n0, A[D0B], net->p + net->hoff, net->scal, net->out_scale,
                                                    net->outb, e, weight, net->g16a[0], net->headpart);
-        k_head_reduce<<<1, 17 * 32, 0, c->stream>>>(hb, net->headpart, net->g, net->hoff);
+        rs_pdl(k_head_reduce, 1, 17 * 32, 0, c)(hb, net->headpart, net->g, net->hoff);
         c->launches++;
         RS_TRY(rs_check_launch(c));
     }
@@ -1566,7 +1583,7 @@ static int net_backward(rs_net *net, const double *r, const double *logk, const 
         RS_TRY(layer_backward(net, la, net->g16a[lvl], net->g16b[lvl], A[skip_src[lvl]], A[up_src[lvl]], nullptr,
                               nullptr, net->g32[lvl], wscale));
         const Level &C = net->lv[lvl + 1];
-        k_up_backward<<<ew_grid(c, C.nvox * 2), 256, 0, c->stream>>>(C.nz, C.ny, C.nx, net->g32[lvl], net->g16a[lvl + 1]);
+        rs_pdl(k_up_backward, ew_grid(c, C.nvox * 2), 256, 0, c)(C.nz, C.ny, C.nx, net->g32[lvl], net->g16a[lvl + 1]);
         RS_TRY(rs_check_launch(c));
     }
     // encoder, coarse to fine
@@ -1581,7 +1598,7 @@ static int net_backward(rs_net *net, const double *r, const double *logk, const 
             RS_TRY(layer_backward(net, la, net->g16a[lvl], net->g16b[lvl], net->pool[lvl], nullptr, nullptr, nullptr,
                                   net->g16a[lvl], wscale));
             const Level &F = net->lv[lvl - 1];
-            k_pool_backward_add<<<ew_grid(c, F.nvox * 2), 256, 0, c->stream>>>(F.nz, F.ny, F.nx, net->g16a[lvl],
+            rs_pdl(k_pool_backward_add, ew_grid(c, F.nvox * 2), 256, 0, c)(F.nz, F.ny, F.nx, net->g16a[lvl],
                                                                                  net->g32[lvl - 1], net->g16a[lvl - 1]);
             RS_TRY(rs_check_launch(c));
         }
@@ -1722,7 +1739,7 @@ extern "C" int rs_net_accumulate(rs_net *net, int32_t nx, int32_t ny, int32_t nz
     rs_ctx *c = net->ctx;
     const int64_t n0 = net->lv[0].nvox;
     RS_TRY(net_forward(net, r, logk, net->outb, nullptr, true));
-    k_loss_sums<<<c->red_blocks, 256, 0, c->stream>>>(n0, net->outb, e, net->red, net->ticket, net->scal);
+    rs_pdl(k_loss_sums, c->red_blocks, 256, 0, c)(n0, net->outb, e, net->red, net->ticket, net->scal);
     RS_TRY(rs_check_launch(c));
     RS_TRY(net_backward(net, r, logk, e, weight, 1.0f));
     if (loss_host) {
@@ -1797,13 +1814,14 @@ extern "C" int rs_net_load(rs_ctx *ctx, const char *path, rs_net **out)
 // network output had a non-finite value (flag[0])
 __global__ void k_fallback_flag(int *flag, const int *skip)
 {
+    if (rs_pdl_wait()) return;
     flag[1] = (skip && *(volatile const int *)skip) || flag[0] == 0;
 }
 
 static int rs_ilu_fallback(rs_pc *M, const double *rp, double *zp, int *flag, const int *skip)
 {
     rs_ctx *c = M->ctx;
-    k_fallback_flag<<<1, 1, 0, c->stream>>>(flag, skip);
+    rs_pdl(k_fallback_flag, 1, 1, 0, c)(flag, skip);
     RS_TRY(rs_check_launch(c));
     return rs_ilu_apply(M->ilu, rp, zp, nullptr, flag + 1);
 }

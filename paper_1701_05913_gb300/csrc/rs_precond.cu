@@ -41,6 +41,7 @@ __global__ void k_qimpes_restrict(int nb, int bs, const double *__restrict__ w,
                                   const double *__restrict__ f, double *__restrict__ rp,
                                   const int *skip)
 {
+    if (rs_pdl_wait()) return;
     if (skip && *(volatile const int *)skip) return;
     for (int I = blockIdx.x * blockDim.x + threadIdx.x; I < nb; I += gridDim.x * blockDim.x) {
         double s = f[(size_t)I * bs];
@@ -53,6 +54,7 @@ __global__ void k_qimpes_restrict(int nb, int bs, const double *__restrict__ w,
 __global__ void k_prolong(int nb, int bs, const double *__restrict__ p, double *__restrict__ z,
                           const int *skip)
 {
+    if (rs_pdl_wait()) return;
     if (skip && *(volatile const int *)skip) return;
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < (int64_t)nb * bs;
          t += (int64_t)gridDim.x * blockDim.x) {
@@ -64,6 +66,7 @@ __global__ void k_prolong(int nb, int bs, const double *__restrict__ p, double *
 __global__ void k_copy_add(int64_t n, const double *__restrict__ a, double *__restrict__ z,
                            int add, const int *skip)
 {
+    if (rs_pdl_wait()) return;
     if (skip && *(volatile const int *)skip) return;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x)
@@ -90,6 +93,7 @@ k_cpr_presid(int nb, int bsr, const int *__restrict__ ptr, const int *__restrict
              const double *__restrict__ pcol, const double *__restrict__ p, const double *__restrict__ f,
              double *__restrict__ t, const int *skip)
 {
+    if (rs_pdl_wait()) return;
     if (skip && *(volatile const int *)skip) return;
     const int bs = BS > 0 ? BS : bsr;
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -104,6 +108,7 @@ k_cpr_presid(int nb, int bsr, const int *__restrict__ ptr, const int *__restrict
 __global__ void k_prolong_add(int nb, int bs, const double *__restrict__ p, const double *__restrict__ t,
                               double *__restrict__ z, const int *skip)
 {
+    if (rs_pdl_wait()) return;
     if (skip && *(volatile const int *)skip) return;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < (int64_t)nb * bs;
          i += (int64_t)gridDim.x * blockDim.x) {
@@ -130,7 +135,7 @@ static int cpr_stage(rs_pc *M, char kind, const double *v, double *out, const in
     const int nb = A->nrows, bs = A->bs;
     const double *rp = v;
     if (bs > 1) {
-        k_qimpes_restrict<<<grid_for(ctx, nb), 256, 0, ctx->stream>>>(nb, bs, M->w, v, M->rp, skip);
+        rs_pdl(k_qimpes_restrict, grid_for(ctx, nb), 256, 0, ctx)(nb, bs, M->w, v, M->rp, skip);
         RS_TRY(rs_check_launch(ctx));
         rp = M->rp;
     }
@@ -139,7 +144,7 @@ static int cpr_stage(rs_pc *M, char kind, const double *v, double *out, const in
     else if (M->amg) RS_TRY(rs_amg_apply(M->amg, rp, zp, skip));
     else RS_TRY(rs_ilu_apply(M->ilu, rp, zp, nullptr, skip));
     if (bs > 1 && prolong) {
-        k_prolong<<<grid_for(ctx, A->n), 256, 0, ctx->stream>>>(nb, bs, M->zp, out, skip);
+        rs_pdl(k_prolong, grid_for(ctx, A->n), 256, 0, ctx)(nb, bs, M->zp, out, skip);
         RS_TRY(rs_check_launch(ctx));
     }
     return RS_OK;
@@ -163,14 +168,14 @@ static int cpr_apply_pf_blocks(rs_pc *M, const double *r, double *z, const int *
             RS_TRY(rs_presid_dia_launch(A, M->zp, r, M->t1, skip));
         } else {
             if (bs == 3)
-                k_cpr_presid<3><<<grid, 256, 0, ctx->stream>>>(nb, 3, A->ptr, A->col, M->pcol, M->zp, r, M->t1, skip);
+                rs_pdl(k_cpr_presid<3>, grid, 256, 0, ctx)(nb, 3, A->ptr, A->col, M->pcol, M->zp, r, M->t1, skip);
             else
-                k_cpr_presid<0><<<grid, 256, 0, ctx->stream>>>(nb, bs, A->ptr, A->col, M->pcol, M->zp, r, M->t1, skip);
+                rs_pdl(k_cpr_presid<0>, grid, 256, 0, ctx)(nb, bs, A->ptr, A->col, M->pcol, M->zp, r, M->t1, skip);
             RS_TRY(rs_check_launch(ctx));
         }
     }
     RS_TRY(cpr_stage(M, 'F', M->t1, M->t2, skip));
-    k_prolong_add<<<grid_for(ctx, A->n), 256, 0, ctx->stream>>>(nb, bs, M->zp, M->t2, z, skip);
+    rs_pdl(k_prolong_add, grid_for(ctx, A->n), 256, 0, ctx)(nb, bs, M->zp, M->t2, z, skip);
     return rs_check_launch(ctx);
 }
 
@@ -187,7 +192,7 @@ static int cpr_apply(rs_pc *M, const double *r, double *z, const int *skip)
     for (int k = 1; seq[k]; ++k) {
         RS_TRY(rs_residual_launch(A, r, z, M->t1, nullptr, skip));
         RS_TRY(cpr_stage(M, seq[k], M->t1, M->t2, skip));
-        k_copy_add<<<grid_for(ctx, A->n), 256, 0, ctx->stream>>>(A->n, M->t2, z, 1, skip);
+        rs_pdl(k_copy_add, grid_for(ctx, A->n), 256, 0, ctx)(A->n, M->t2, z, 1, skip);
         RS_TRY(rs_check_launch(ctx));
     }
     return RS_OK;
@@ -239,8 +244,10 @@ static int cpr_apply_graph(rs_pc *M, const double *r, double *z, const int *skip
     int st = RS_ERR_CUDA;
     if (cudaStreamBeginCapture(M->capture, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
         ctx->stream = M->capture;
+        ctx->capturing = true;
         st = cpr_apply(M, r, z, skip);
         ctx->stream = user;
+        ctx->capturing = false;
         if (cudaStreamEndCapture(M->capture, &graph) != cudaSuccess) st = RS_ERR_CUDA;
     }
     if (!st && (!graph || cudaGraphInstantiate(&exec, graph, 0) != cudaSuccess)) st = RS_ERR_CUDA;
@@ -262,7 +269,7 @@ int rs_pc_apply_dev(rs_pc *M, const double *r, double *z, const int *skip)
     const rs_mat *A = M->A;
     switch (M->type) {
     case RS_PC_NONE:
-        k_copy_add<<<grid_for(ctx, A->n), 256, 0, ctx->stream>>>(A->n, r, z, 0, skip);
+        rs_pdl(k_copy_add, grid_for(ctx, A->n), 256, 0, ctx)(A->n, r, z, 0, skip);
         return rs_check_launch(ctx);
     case RS_PC_ILU0:
         return rs_ilu_apply(M->ilu, r, z, nullptr, skip);

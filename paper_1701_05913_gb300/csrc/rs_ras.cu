@@ -38,6 +38,7 @@ __global__ void k_ras_values(int64_t nnz, int b2, const int *__restrict__ src, c
 __global__ void k_ras_gather(int next, int bs, const int *__restrict__ gidx, const double *__restrict__ r,
                              double *__restrict__ rh, const int *skip)
 {
+    if (rs_pdl_wait()) return;
     if (skip && *(volatile const int *)skip) return;
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < (int64_t)next * bs;
          e += (int64_t)gridDim.x * blockDim.x) {
@@ -50,6 +51,7 @@ __global__ void k_ras_gather(int next, int bs, const int *__restrict__ gidx, con
 __global__ void k_ras_scatter(int nrows, int bs, const int *__restrict__ own, const double *__restrict__ zh,
                               double *__restrict__ z, const int *skip)
 {
+    if (rs_pdl_wait()) return;
     if (skip && *(volatile const int *)skip) return;
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < (int64_t)nrows * bs;
          e += (int64_t)gridDim.x * blockDim.x) {
@@ -600,13 +602,13 @@ int rs_ras_apply(RasData *R, const double *r, double *z, const int *skip)
     if (R->nrows == 0) return RS_OK;
     {
         RsProfScope prof(ctx, RS_PROF_PRECOND_OTHER);
-        k_ras_gather<<<ras_grid(ctx, (int64_t)R->next * R->bs), 256, 0, ctx->stream>>>(R->next, R->bs, R->gidx, r,
+        rs_pdl(k_ras_gather, ras_grid(ctx, (int64_t)R->next * R->bs), 256, 0, ctx)(R->next, R->bs, R->gidx, r,
                                                                                       R->rhat, skip);
     }
     RS_TRY(rs_check_launch(ctx));
     RS_TRY(rs_ilu_apply(R->f, R->rhat, R->zhat, nullptr, skip));
     RsProfScope prof(ctx, RS_PROF_PRECOND_OTHER);
-    k_ras_scatter<<<ras_grid(ctx, (int64_t)R->nrows * R->bs), 256, 0, ctx->stream>>>(R->nrows, R->bs, R->own,
+    rs_pdl(k_ras_scatter, ras_grid(ctx, (int64_t)R->nrows * R->bs), 256, 0, ctx)(R->nrows, R->bs, R->own,
                                                                                     R->zhat, z, skip);
     return rs_check_launch(ctx);
 }

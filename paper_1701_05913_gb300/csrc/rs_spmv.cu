@@ -75,6 +75,7 @@ __global__ void __launch_bounds__(256)
 k_spmv_dia(DiaArgs a, const double *__restrict__ x, double alpha, double beta, const double *__restrict__ bvec,
            double *__restrict__ y, const int *skip, const double *__restrict__ dinv)
 {
+    if (rs_pdl_wait()) return;
     if (skip && *(volatile const int *)skip) return;
     const int64_t I = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (I >= a.n) return;
@@ -121,6 +122,7 @@ __global__ void __launch_bounds__(256)
 k_presid_dia(DiaArgs a, const double *__restrict__ p, const double *__restrict__ f, double *__restrict__ t,
              const int *skip)
 {
+    if (rs_pdl_wait()) return;
     if (skip && *(volatile const int *)skip) return;
     const int64_t I = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (I >= a.n) return;
@@ -150,6 +152,7 @@ k_spmv_sell(int nslice, const int2 *__restrict__ rows, const int *__restrict__ s
             const double *__restrict__ val, const double *__restrict__ x, double alpha, double beta,
             const double *__restrict__ bvec, double *__restrict__ y, const int *skip, const double *__restrict__ dinv)
 {
+    if (rs_pdl_wait()) return;
     if (skip && *(volatile const int *)skip) return;
     const int s = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
     if (s >= nslice) return;
@@ -388,7 +391,7 @@ int dia_launch(const rs_mat *A, const double *x, double alpha, double beta, cons
     switch (A->dia.nd) {
 #define RS_DIA_CASE(ND)                                                                                          \
     case ND:                                                                                                     \
-        k_spmv_dia<ND, BS><<<grid, 256, 0, A->ctx->stream>>>(a, x, alpha, beta, bvec, y, skip, dinv);             \
+        rs_pdl(k_spmv_dia<ND, BS>, grid, 256, 0, A->ctx)(a, x, alpha, beta, bvec, y, skip, dinv);             \
         break;
         RS_DIA_CASE(1)
         RS_DIA_CASE(2)
@@ -412,7 +415,7 @@ int presid_launch(const rs_mat *A, const double *p, const double *f, double *t, 
     switch (A->dia.nd) {
 #define RS_DIA_CASE(ND)                                                               \
     case ND:                                                                          \
-        k_presid_dia<ND, BS><<<grid, 256, 0, A->ctx->stream>>>(a, p, f, t, skip);      \
+        rs_pdl(k_presid_dia<ND, BS>, grid, 256, 0, A->ctx)(a, p, f, t, skip);      \
         break;
         RS_DIA_CASE(1)
         RS_DIA_CASE(2)
@@ -473,10 +476,10 @@ int rs_spmv_layout_launch(const rs_mat *A, const double *x, double alpha, double
     const int grid = (A->sell.nslice + 7) / 8;
     // short rows (interpolation) need no more loads in flight than they have entries
     if (A->nnzb <= 6 * (int64_t)A->nrows)
-        k_spmv_sell<4><<<grid, 256, 0, A->ctx->stream>>>(A->sell.nslice, A->sell.rows, A->sell.sptr, A->sell.col,
+        rs_pdl(k_spmv_sell<4>, grid, 256, 0, A->ctx)(A->sell.nslice, A->sell.rows, A->sell.sptr, A->sell.col,
                                                          A->sell.val, x, alpha, beta, bvec, y, skip, dinv);
     else
-        k_spmv_sell<8><<<grid, 256, 0, A->ctx->stream>>>(A->sell.nslice, A->sell.rows, A->sell.sptr, A->sell.col,
+        rs_pdl(k_spmv_sell<8>, grid, 256, 0, A->ctx)(A->sell.nslice, A->sell.rows, A->sell.sptr, A->sell.col,
                                                          A->sell.val, x, alpha, beta, bvec, y, skip, dinv);
     return rs_check_launch(A->ctx);
 }

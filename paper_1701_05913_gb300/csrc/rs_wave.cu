@@ -250,6 +250,7 @@ template <int BS, typename T, bool LOWER>
 __global__ void __launch_bounds__(WaveCfg<BS, T>::THREADS)
 k_wave_sweep(WaveArgs g, const T *__restrict__ rec, const T *__restrict__ rhs, T *xv)
 {
+    if (rs_pdl_wait()) return;
     using C = WaveCfg<BS, T>;
     constexpr int B2 = C::B2;
     constexpr int RB = LOWER ? C::RL : C::RU;
@@ -672,6 +673,7 @@ __global__ void __launch_bounds__(WAVE_PERM_THREADS)
 k_wave_in(WaveArgs g, const double *__restrict__ r, const double *__restrict__ scale, T *__restrict__ rw,
           T *__restrict__ zreset)
 {
+    if (rs_pdl_wait()) return;
     constexpr int W = 32 * BS + 1;                 // tile row: one lane's 32 cells, padded
     __shared__ double tile[32 * W];
     if (g.skip && *(volatile const int *)g.skip) return;
@@ -712,6 +714,7 @@ template <int BS, typename T>
 __global__ void __launch_bounds__(WAVE_PERM_THREADS)
 k_wave_out(WaveArgs g, const T *__restrict__ zw, T *__restrict__ yreset, double *__restrict__ out)
 {
+    if (rs_pdl_wait()) return;
     constexpr int W = 32 * BS + 1;
     __shared__ double tile[32 * W];
     if (g.skip && *(volatile const int *)g.skip) return;
@@ -833,16 +836,16 @@ int wave_apply_t(IluFactor *f, const double *r, double *z, const double *scale, 
     RS_TRY((raise_sweep_smem<BS, T, false>(ctx)));
     {
         RsProfScope prof(ctx, BS == 1 ? RS_PROF_LSWEEP : RS_PROF_BLSWEEP);
-        k_wave_in<BS, T><<<gp, WAVE_PERM_THREADS, 0, ctx->stream>>>(g, r, scale, (T *)W.rw, (T *)W.zw);
-        k_wave_sweep<BS, T, true><<<gw, C::THREADS, sl, ctx->stream>>>(g, (const T *)W.lrec, (const T *)W.rw,
+        rs_pdl(k_wave_in<BS, T>, gp, WAVE_PERM_THREADS, 0, ctx)(g, r, scale, (T *)W.rw, (T *)W.zw);
+        rs_pdl(k_wave_sweep<BS, T, true>, gw, C::THREADS, sl, ctx)(g, (const T *)W.lrec, (const T *)W.rw,
                                                                        (T *)W.yw);
     }
     RS_TRY(rs_check_launch(ctx));
     {
         RsProfScope prof(ctx, BS == 1 ? RS_PROF_USWEEP : RS_PROF_BUSWEEP);
-        k_wave_sweep<BS, T, false><<<gw, C::THREADS, su, ctx->stream>>>(g, (const T *)W.urec, (const T *)W.yw,
+        rs_pdl(k_wave_sweep<BS, T, false>, gw, C::THREADS, su, ctx)(g, (const T *)W.urec, (const T *)W.yw,
                                                                         (T *)W.zw);
-        k_wave_out<BS, T><<<gp, WAVE_PERM_THREADS, 0, ctx->stream>>>(g, (const T *)W.zw, (T *)W.yw, z);
+        rs_pdl(k_wave_out<BS, T>, gp, WAVE_PERM_THREADS, 0, ctx)(g, (const T *)W.zw, (T *)W.yw, z);
     }
     ctx->launches += 2;   // rs_check_launch counts one per call
     RS_TRY(rs_check_launch(ctx));
