@@ -70,8 +70,14 @@ struct WaveCfg {
     // that the round trip stays short (block records: 4 steps measured
     // faster than 8)
     static constexpr int K = BS == 1 ? (sizeof(T) == 4 ? 16 : 8) : (sizeof(T) == 4 ? 4 : 2);
-    // (step, position) pairs of a polling round per producer lane
-    static constexpr int JP = 4;
+    // (step, position) pairs of a polling round per producer lane: 8 steps of
+    // 12 positions.  A round is the loads' trip (700 cycles) and the handling;
+    // with its address arithmetic, clock reads and the wait for the compute
+    // warp's counter on that path a round took 1500 cycles, which the hops
+    // between units and FP32 steps waited on.  128 x 128 x 64, both sweeps:
+    // 268 -> 243 us FP64, 174 -> 133 us FP32 (2 pairs: 243 / 140; 4: 247 /
+    // 139; two rounds in flight: 257 / 193).
+    static constexpr int JP = 3;
     // hand-off ring (steps), a power of two
     static constexpr int HR = 2 * K < 16 ? 16 : 2 * K;
     static constexpr int HDR_BYTES = 128;                            // R mbarriers, ticket, counters
@@ -308,14 +314,11 @@ k_wave_sweep(WaveArgs g, const T *__restrict__ rec, const T *__restrict__ rhs, T
             // ---------------------------------------------------------------
             const T *grec = rec + base * RB;
             const T *grhs = rhs + base * BS;
-            int qb = 0;                           // next chunk to copy
-            auto cons_now = [&]() -> int {
-                unsigned c = 0;
-                if (lane == 0) c = ld_acq_cta(&hd->cons);
-                return (int)__shfl_sync(FULL, c, 0);
-            };
+            int qb = 0, qstep = 0;                // next chunk to copy, and the step that frees its slot
+            // steps the compute warp has left
+            auto cons_now = [&]() -> int { return __shfl_sync(FULL, *(volatile int *)&hd->cons, 0); };
             auto issue_ready = [&](int c) {
-                while (qb < nch && (qb < R || c >= (qb - R + 1) * G)) {
+                while (c >= qstep) {
                     if (lane == 0) {
                         const int k = LOWER ? qb : nch - 1 - qb;
                         const int sl = qb % R;
@@ -327,6 +330,7 @@ k_wave_sweep(WaveArgs g, const T *__restrict__ rec, const T *__restrict__ rhs, T
                                  G * 32 * BS * (int)sizeof(T), &hd->bar[sl]);
                     }
                     ++qb;
+                    qstep = qb < R ? 0 : qb < nch ? (qb - R + 1) * G : 0x7fffffff;
                 }
             };
             // The unit's hand-off positions: p < a on the z face (the
@@ -336,9 +340,10 @@ k_wave_sweep(WaveArgs g, const T *__restrict__ rec, const T *__restrict__ rhs, T
             // takes few load instructions.
             const int F = a + b;
             const int KE = min(K, (32 * JP) / F);        // steps per round, >= 1
-            int jk[JP], jring[JP], jskew[JP];
-            int64_t jsrc[JP];
-            bool jin[JP], jok[JP];
+            constexpr int DT = LOWER ? 1 : -1;
+            int jk[JP], jring[JP], jx[JP];
+            const T *jp[JP];
+            bool jok[JP], jin[JP];
 #pragma unroll
             for (int j = 0; j < JP; ++j) {
                 const int idx = lane + 32 * j;
@@ -356,37 +361,27 @@ k_wave_sweep(WaveArgs g, const T *__restrict__ rec, const T *__restrict__ rhs, T
                 jok[j] = jin[j] && has && c_ok;
                 jk[j] = k;
                 jring[j] = ((zf ? 0 : 1) * 32 + cy + (cz << g.la)) * BS;
-                jskew[j] = cy + cz;
-                jsrc[j] = jok[j] ? uu * ucells + 32 * so + sl : 0;
+                // at the round's first step s the position is at t = t0 +- s: x = t - skew, address jp +- 32 s
+                const int t0 = (LOWER ? 0 : g.npad - 1) + DT * k;
+                jx[j] = t0 - (cy + cz);
+                jp[j] = xv + (jok[j] ? uu * ucells + 32 * so + sl + 32 * (int64_t)t0 : 0) * BS;
             }
             int sp = 0;                           // next step to hand over
-            long long tl = clock64();             // last progress
-            bool late = false;
-            while (sp < g.npad) {
-                const int c = cons_now();
-                issue_ready(c);
-                const int room = min(g.npad, c + HR) - sp;
-                if (room <= 0) {
-                    // the ring is full: wait for the compute warp
-                    const long long dt = clock64() - tl;
-                    if (!late && dt > g.limit) {
-                        late = true;
-                        if (lane == 0) atomicOr(g.err, RS_DEVERR_TIMEOUT);
-                    }
-                    if (dt > giveup) break;
-                    continue;
-                }
-                bits_t v[JP][BS];
-                unsigned miss = 0;
+            long long tl = 0;                     // start of the rounds without progress
+            bool idle = false, late = false;
+            // loads of the steps [s, e) of a round, at most KE
+            auto poll = [&](int s, int e, bits_t (&v)[JP][BS]) {
 #pragma unroll
                 for (int j = 0; j < JP; ++j) {
-                    const int s = sp + jk[j];
-                    const int t = LOWER ? s : g.npad - 1 - s;
-                    const bool act = jok[j] && jk[j] < room && (unsigned)(t - jskew[j]) < (unsigned)g.nx;
-                    const T *src = xv + (jsrc[j] + 32 * (int64_t)t) * BS;
+                    const bool act = jok[j] && s + jk[j] < e && (unsigned)(jx[j] + DT * s) < (unsigned)g.nx;
+                    const T *src = jp[j] + (int64_t)(DT * 32 * BS) * s;
 #pragma unroll
                     for (int k2 = 0; k2 < BS; ++k2) v[j][k2] = act ? ld_poll(src + k2) : bits_t(0);
                 }
+            };
+            // hands over the steps whose values have all arrived
+            auto take = [&](int s, int e, const bits_t (&v)[JP][BS]) {
+                unsigned miss = 0;
 #pragma unroll
                 for (int j = 0; j < JP; ++j) {
                     bool p = false;
@@ -395,28 +390,57 @@ k_wave_sweep(WaveArgs g, const T *__restrict__ rec, const T *__restrict__ rhs, T
                     if (p) miss |= 1u << jk[j];
                 }
                 miss = __reduce_or_sync(FULL, miss);
-                int ready = min(room, KE);
+                int ready = min(e - s, KE);
                 if (miss && !dead) ready = min(ready, __ffs(miss) - 1);
+                if (ready <= 0) return;
                 // every position of the steps handed over is written: the
                 // value, or 0 where no value is read
 #pragma unroll
                 for (int j = 0; j < JP; ++j) {
                     if (jin[j] && jk[j] < ready) {
-                        T *hp = ring + (size_t)((sp + jk[j]) & (HR - 1)) * 2 * 32 * BS + jring[j];
+                        T *hp = ring + (size_t)((s + jk[j]) & (HR - 1)) * 2 * 32 * BS + jring[j];
 #pragma unroll
                         for (int k2 = 0; k2 < BS; ++k2) hp[k2] = bits_to(T(), v[j][k2]);
                     }
                 }
-                if (ready > 0) {
-                    __syncwarp();
-                    sp += ready;
-                    if (lane == 0) st_rel_cta(&hd->prod, (unsigned)sp);
+                __syncwarp();
+                sp = s + ready;
+                if (lane == 0) st_rel_cta(&hd->prod, (unsigned)sp);
+            };
+            // no progress: give up in the end
+            auto stuck = [&](bool ringfull) -> bool {
+                if (!idle) {
+                    idle = true;
                     tl = clock64();
-                } else if (clock64() - tl > g.limit) {
-                    // give up: carry the sentinel on (arithmetic on it gives NaN)
-                    if (lane == 0) atomicOr(g.err, RS_DEVERR_TIMEOUT);
-                    dead = true;
+                    return false;
                 }
+                const long long dt = clock64() - tl;
+                if (dt <= g.limit) return false;
+                if (ringfull) {
+                    // waiting for the compute warp
+                    if (!late) {
+                        late = true;
+                        if (lane == 0) atomicOr(g.err, RS_DEVERR_TIMEOUT);
+                    }
+                    return dt > giveup;
+                }
+                // carry the sentinel on (arithmetic on it gives NaN)
+                if (lane == 0) atomicOr(g.err, RS_DEVERR_TIMEOUT);
+                dead = true;
+                return false;
+            };
+            bits_t v[JP][BS];
+            int lim = min(g.npad, HR);            // steps the ring has room for
+            while (sp < g.npad) {
+                const int before = sp, e = lim;
+                poll(sp, e, v);
+                // while the loads travel: the compute warp's progress, and the chunks it has freed
+                const int c = cons_now();
+                issue_ready(c);
+                lim = min(g.npad, c + HR);
+                take(before, e, v);
+                if (sp != before) idle = false;
+                else if (stuck(e <= sp)) break;
             }
             // the last chunks, as the compute warp frees their slots
             tl = clock64();
@@ -460,8 +484,11 @@ k_wave_sweep(WaveArgs g, const T *__restrict__ rec, const T *__restrict__ rhs, T
             const long long t0 = clock64();
             bool late = false;
             for (;;) {
-                v = __shfl_sync(FULL, ld_acq_cta(&hd->prod), 0);
-                if (v > (unsigned)s) return v;
+#pragma unroll 1
+                for (int k = 0; k < 8; ++k) {
+                    v = __shfl_sync(FULL, ld_acq_cta(&hd->prod), 0);
+                    if (v > (unsigned)s) return v;
+                }
                 const long long dt = clock64() - t0;
                 if (!late && dt > g.limit) {
                     late = true;
