@@ -240,6 +240,7 @@ struct RasData {
     double *rhat = nullptr, *zhat = nullptr;   // [next*bs] work vectors
     std::vector<int> h_gidx;
     IluFactor *f = nullptr;
+    struct PartSweep *ps = nullptr;   // one-block-per-subdomain sweeps (rs_part.cu), when its rule takes them
 };
 
 // Algebraic multigrid (rs_amg.cu): operators of every level as rs_mat,
@@ -386,6 +387,16 @@ bool rs_level_fits(int bs, int fp32, int nx, int ny, int nz, int hops);
 int rs_level_create(IluFactor *f);
 int rs_level_gather(IluFactor *f);
 int rs_level_apply(IluFactor *f, const double *r, double *z, const double *scale, const int *skip);
+// sweeps of independent parts, a block per part (rs_part.cu).  create: from the
+// parts' first rows, the stacked pattern and its factor f, *out null when the
+// rule leaves them to the segment sweeps (of seg_levels levels, L and U
+// together); apply: rows gidx of r in, owned rows of z out (r and z must not
+// overlap)
+struct PartSweep;
+int rs_part_create(rs_ctx *ctx, const std::vector<int> &sbase, const std::vector<int> &ptr, const std::vector<int> &col,
+                   const IluFactor *f, int seg_levels, PartSweep **out);
+int rs_part_apply(const PartSweep *S, const int *gidx, const int *own, const double *r, double *z, const int *skip);
+void rs_part_destroy(PartSweep *S);
 // local: 0 = ILU(level), 1 = ILUT(ilut_p, ilut_tol) (scalar matrices)
 int rs_ras_create(rs_ctx *ctx, const rs_mat *A, int nparts, const int32_t *part, int overlap, int level, int local,
                   int ilut_p, double ilut_tol, int fp32, RasData **out, int *bad_row);

@@ -464,6 +464,7 @@ int rs_ras_create(rs_ctx *ctx, const rs_mat *A, int nparts, const int32_t *part,
     std::vector<int> mark(n, -1), loc(n, 0), set, frontier, next;
     std::vector<int> lptr, lcol, lsrc;
     int64_t total_nnz = 0;
+    std::vector<int> pbase(1, 0);             // first stacked row of every subdomain
     for (int s = 0; s < nparts; ++s) {
         set.assign(prow.begin() + pstart[s], prow.begin() + pstart[s + 1]);
         for (int g : set) mark[g] = s;
@@ -521,6 +522,7 @@ int rs_ras_create(rs_ctx *ctx, const rs_mat *A, int nparts, const int32_t *part,
         total_nnz = (int64_t)hcol.size();
         if (total_nnz > INT_MAX) return RS_ERR_INVALID_ARG;
         gidx.insert(gidx.end(), set.begin(), set.end());
+        pbase.push_back(base + ns);
         for (int r = pstart[s]; r < pstart[s + 1]; ++r) own[prow[r]] = base + loc[prow[r]];
     }
     const int nx = (int)gidx.size();
@@ -584,6 +586,7 @@ int rs_ras_create(rs_ctx *ctx, const rs_mat *A, int nparts, const int32_t *part,
     if (local == 1) st = st ? st : rs_ilu_set_factors(R->f, R->val, &bad);
     else st = st ? st : rs_ilu_factor(R->f, R->val, &bad);
     if (bad >= 0 && bad < nx && bad_row) *bad_row = gidx[bad];
+    if (!st && bs == 1) st = rs_part_create(ctx, pbase, hptr, hcol, R->f, R->f->SL.nlevels + R->f->SU.nlevels, &R->ps);
     if (st == RS_ERR_ZERO_PIVOT) {
         *out = R;            // the caller keeps the object to report the row
         return st;
@@ -600,6 +603,8 @@ int rs_ras_apply(RasData *R, const double *r, double *z, const int *skip)
 {
     rs_ctx *ctx = R->ctx;
     if (R->nrows == 0) return RS_OK;
+    // a block per subdomain reads r and writes z as it goes: not when they overlap
+    if (R->ps && (r + R->nrows <= z || z + R->nrows <= r)) return rs_part_apply(R->ps, R->gidx, R->own, r, z, skip);
     {
         RsProfScope prof(ctx, RS_PROF_PRECOND_OTHER);
         rs_pdl(k_ras_gather, ras_grid(ctx, (int64_t)R->next * R->bs), 256, 0, ctx)(R->next, R->bs, R->gidx, r,
@@ -617,6 +622,7 @@ void rs_ras_destroy(RasData *R)
 {
     if (!R) return;
     rs_ctx *ctx = R->ctx;
+    rs_part_destroy(R->ps);
     if (R->f) rs_ilu_destroy(R->f);     // borrows ptr / col: released first
     rs_free(ctx, R->ptr);
     rs_free(ctx, R->col);

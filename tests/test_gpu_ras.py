@@ -154,6 +154,30 @@ def test_ras_block_matrix(rs, ctx, orc):
         assert rel(z.numpy(), want) <= 1e-12, overlap
 
 
+# subdomains swept by one block each (rs_part.cu): levels of more than 128
+# rows (two chunks), rows of more than 8 entries per triangle, an odd number of
+# levels, more subdomains than SMs, and a subdomain too large for it
+@pytest.mark.parametrize("shape,parts,overlap,level", [
+    ((24, 24, 24), (1, 1, 1), 0, 0), ((14, 12, 10), (2, 1, 1), 1, 3), ((17, 11, 9), (1, 1, 1), 0, 1),
+    ((40, 36, 30), (6, 6, 6), 1, 1), ((64, 40, 30), (2, 1, 1), 1, 0)])
+@pytest.mark.parametrize("prec", ["fp64", "mixed"])
+def test_ras_subdomains_in_one_block(rs, ctx, orc, shape, parts, overlap, level, prec):
+    g = synth.Grid(*shape)
+    d = synth.pressure_7pt(g, 58, kz_scale=0.1)
+    part, nparts = rs.box_partition(shape, parts), int(np.prod(parts))
+    M = rs.Precond(ctx, rs.Mat.csr(ctx, d), "ras", prec=prec, nparts=nparts, part=part, overlap=overlap, level=level)
+    r = np.random.default_rng(59).standard_normal(g.n)
+    want = orc.Ras(orc.Mat.csr(d), nparts, part=part, overlap=overlap, level=level).apply(r)
+    tol = 1e-12 if prec == "fp64" else 1e-5
+    z = rs.Vec.zeros(ctx, g.n)
+    for _ in range(2):
+        M.apply(rs.Vec(ctx, r), z)
+        assert rel(z.numpy(), want) <= tol
+    same = rs.Vec(ctx, r.copy())                  # in place: r and z are one vector
+    M.apply(same, same)
+    assert rel(same.numpy(), want) <= tol
+
+
 def test_ras_sweep_levels_shrink_with_subdomains(rs, ctx):
     g = synth.Grid(64, 64, 32)
     d = synth.pressure_7pt(g, 55)
