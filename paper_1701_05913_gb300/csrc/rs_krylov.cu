@@ -225,6 +225,43 @@ struct CgsCfg {
 // nc - NCC (0 to 3) columns take a warp-uniform branch, so that no FP64
 // multiply-add is issued for a column that does not exist (predicated-off
 // FP64 instructions still occupy the FP64 pipe on this GPU).
+// One thread: the Givens rotations on the new Hessenberg column h[0..nc) with
+// h_{nc,nc-1} = hnext (h[nc] is set to 0), the rotated residual, the
+// convergence and happy-breakdown tests and the next vector's scale.  cs, sn:
+// the earlier rotations (nc - 1 of them are read).
+__device__ __forceinline__ void givens_update(GmresDev *d, int nc, double *h, const double *cs, const double *sn,
+                                              double hnext, double w0sq)
+{
+    const int i = nc - 1;
+    double a = h[0];
+    for (int k = 0; k < i; ++k) {
+        const double b = h[k + 1];
+        h[k] = __dadd_rn(__dmul_rn(cs[k], a), __dmul_rn(sn[k], b));
+        a = __dadd_rn(__dmul_rn(-sn[k], a), __dmul_rn(cs[k], b));
+    }
+    const double rho = hypot(a, hnext);
+    const double c = __ddiv_rn(a, rho), s = __ddiv_rn(hnext, rho), g = d->g[i];
+    d->cs[i] = c;
+    d->sn[i] = s;
+    h[i] = rho;
+    h[nc] = 0.0;
+    const double g1 = __dmul_rn(-s, g);
+    d->g[i + 1] = g1;
+    d->g[i] = __dmul_rn(c, g);
+    const int iters = d->iters + 1;
+    d->iters = iters;
+    d->k = i + 1;
+    const double implicit = fabs(g1);
+    d->implicit = implicit;
+    record_hist(d->hist, d->hist_len, iters, implicit, d->bnorm);
+    const bool happy = hnext <= 1e-14 * sqrt(w0sq);
+    if (implicit <= d->tol || iters >= d->maxit || happy || i == d->m - 1) {
+        d->cycle_done = 1;
+        *(volatile int *)d->host_done = 1;
+    }
+    d->hdiv = 1.0 / hnext;     // v_{i+1} = w / h_{i+1,i}
+}
+
 template <int NC, int NCC, int MODE>
 __global__ void __launch_bounds__(CgsCfg<NC>::THREADS)
 k_cgs_pass(int n, int ld, int nc, const double *__restrict__ V, double *w, double *partials, unsigned *ticket,
@@ -334,49 +371,143 @@ k_cgs_pass(int n, int ld, int nc, const double *__restrict__ V, double *w, doubl
             // the new Hessenberg column and the rotations through shared
             // memory: one thread's chain of rotations then waits for no load
             // (the ring is free: every tile has been consumed)
-            const int i = nc - 1, m1 = d->m + 1;
             double *h = ring, *cs = ring + NC + 1, *sn = ring + 2 * NC + 2;
-            double *hcol = d->H + (size_t)i * m1;
+            double *hcol = d->H + (size_t)(nc - 1) * (d->m + 1);
             for (int k = threadIdx.x; k < nc; k += blockDim.x) {
                 h[k] = hcol[k];
                 cs[k] = d->cs[k];
                 sn[k] = d->sn[k];
             }
             __syncthreads();
-            if (threadIdx.x == 0) {
-                const double hnext = sqrt(d->r2);
-                double a = h[0];
-                for (int k = 0; k < i; ++k) {
-                    const double b = h[k + 1];
-                    h[k] = __dadd_rn(__dmul_rn(cs[k], a), __dmul_rn(sn[k], b));
-                    a = __dadd_rn(__dmul_rn(-sn[k], a), __dmul_rn(cs[k], b));
-                }
-                const double rho = hypot(a, hnext);
-                const double c = __ddiv_rn(a, rho), s = __ddiv_rn(hnext, rho), g = d->g[i];
-                d->cs[i] = c;
-                d->sn[i] = s;
-                h[i] = rho;
-                h[nc] = 0.0;
-                const double g1 = __dmul_rn(-s, g);
-                d->g[i + 1] = g1;
-                d->g[i] = __dmul_rn(c, g);
-                const int iters = d->iters + 1;
-                d->iters = iters;
-                d->k = i + 1;
-                const double implicit = fabs(g1);
-                d->implicit = implicit;
-                record_hist(d->hist, d->hist_len, iters, implicit, d->bnorm);
-                const bool happy = hnext <= 1e-14 * sqrt(d->w0sq);
-                if (implicit <= d->tol || iters >= d->maxit || happy || i == d->m - 1) {
-                    d->cycle_done = 1;
-                    *(volatile int *)d->host_done = 1;
-                }
-                d->hdiv = 1.0 / hnext;     // v_{i+1} = w / h_{i+1,i}
-            }
+            if (threadIdx.x == 0) givens_update(d, nc, h, cs, sn, sqrt(d->r2), d->w0sq);
             __syncthreads();
             for (int k = threadIdx.x; k <= nc; k += blockDim.x) hcol[k] = h[k];
         }
     }
+}
+
+// ---------------------------------------------------------------------------
+// The same step of a small system in one launch: a cluster of CS_CTAS blocks,
+// each with its rows of the nc basis vectors and of w in shared memory from
+// the first product to the last.  Column sums go block to block through
+// distributed shared memory and are added in block order, and the new basis
+// vector is written already scaled by 1 / h_{i+1,i}.  What bounds it: three
+// cluster barriers and the FP64 multiply-adds of CS_CTAS SMs (4 n nc in all:
+// about 5 us at 1920 rows and 15 columns); three passes and the scaling took
+// 30 us there, of which 12 were launches.
+// ---------------------------------------------------------------------------
+#define CS_CTAS 8
+#define CS_THREADS 256
+#define CS_MAX_ROWS 6144                            // beyond, the passes' more SMs win
+#define CS_SMEM (190 * 1024)
+
+static size_t cgs_small_smem(int n, int nc)
+{
+    return sizeof(double) * (size_t)((n + CS_CTAS - 1) / CS_CTAS) * (nc + 1);
+}
+
+__global__ void __cluster_dims__(CS_CTAS, 1, 1) __launch_bounds__(CS_THREADS)
+k_cgs_small(int n, int ld, int nc, double *__restrict__ V, GmresDev *d)
+{
+    extern __shared__ __align__(16) double cs_tile[];           // [nc + 1][R]: basis vectors, then w
+    __shared__ double ex[3][CS_CTAS][RS_MAX_RESTART + 2];       // the blocks' sums, one buffer an exchange
+    __shared__ double part[RS_MAX_RESTART + 2], h[RS_MAX_RESTART + 2], h2[RS_MAX_RESTART + 2];
+    __shared__ double cs[RS_MAX_RESTART], sn[RS_MAX_RESTART];
+    if (rs_pdl_wait()) return;
+    if (*(volatile int *)&d->cycle_done) return;                // set by this step at the earliest after its barriers
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int rank = blockIdx.x;                                // one cluster: the grid
+    const int R = (n + CS_CTAS - 1) / CS_CTAS, r0 = rank * R, rows = max(0, min(R, n - r0));
+    double *w = cs_tile + (size_t)nc * R;
+    for (int k = warp; k <= nc; k += CS_THREADS / 32) {
+        const double *src = V + (size_t)k * ld + r0;
+#pragma unroll 4
+        for (int r = lane; r < rows; r += 32) cs_tile[(size_t)k * R + r] = src[r];
+    }
+    __syncthreads();
+    // part[k] = this block's rows of <V_k, w>, k < cols (k = nc: <w, w>)
+    auto dots = [&](int cols) {
+        for (int k0 = 4 * warp; k0 < cols; k0 += 4 * (CS_THREADS / 32)) {
+            double acc[4] = {0.0, 0.0, 0.0, 0.0};
+            for (int r = lane; r < rows; r += 32) {
+                const double wr = w[r];
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    if (k0 + j < cols) acc[j] = fma(cs_tile[(size_t)(k0 + j) * R + r], wr, acc[j]);
+            }
+            warp_reduce_scatter<4>(acc, lane);
+            if (lane % 8 == 0 && k0 + lane / 8 < cols) part[k0 + lane / 8] = acc[0];
+        }
+        __syncthreads();
+    };
+    // out[k] = the sum of every block's part[k], added in block order
+    auto exchange = [&](int which, int cols, double *out) {
+        for (int t = tid; t < cols * CS_CTAS; t += CS_THREADS) {
+            const int q = t / cols, k = t - q * cols;
+            unsigned dst;
+            asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(dst) : "r"(smem_addr(&ex[which][rank][k])), "r"(q));
+            asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(dst), "d"(part[k]) : "memory");
+        }
+        asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+        asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+        for (int k = tid; k < cols; k += CS_THREADS) {
+            double s = 0.0;
+#pragma unroll
+            for (int q = 0; q < CS_CTAS; ++q) s += ex[which][q][k];
+            out[k] = s;
+        }
+        __syncthreads();
+    };
+    // w -= V c; the block's rows of <w, w> if asked for
+    auto update = [&](const double *c) -> double {
+        double sq = 0.0;
+        for (int r = tid; r < rows; r += CS_THREADS) {
+            double s0 = 0.0, s1 = 0.0;
+            int k = 0;
+            for (; k + 1 < nc; k += 2) {
+                s0 = fma(cs_tile[(size_t)k * R + r], c[k], s0);
+                s1 = fma(cs_tile[(size_t)(k + 1) * R + r], c[k + 1], s1);
+            }
+            if (k < nc) s0 = fma(cs_tile[(size_t)k * R + r], c[k], s0);
+            const double v = w[r] - (s0 + s1);
+            w[r] = v;
+            sq = fma(v, v, sq);
+        }
+        return sq;
+    };
+    // h1 = V^T w and ||w||^2; w -= V h1; h2 = V^T w; w -= V h2; ||w||
+    dots(nc + 1);
+    exchange(0, nc + 1, h);
+    const double w0sq = h[nc];
+    update(h);
+    __syncthreads();
+    dots(nc);
+    exchange(1, nc, h2);
+    double sq = warp_sum(update(h2));
+    __syncthreads();
+    if (lane == 0) part[1 + warp] = sq;
+    __syncthreads();
+    if (tid == 0) {
+        sq = 0.0;
+        for (int q = 0; q < CS_THREADS / 32; ++q) sq += part[1 + q];
+        part[0] = sq;
+    }
+    __syncthreads();
+    __shared__ double total[1];
+    exchange(2, 1, total);
+    const double hnext = sqrt(total[0]), inv = 1.0 / hnext;
+    for (int r = tid; r < rows; r += CS_THREADS) V[(size_t)nc * ld + r0 + r] = w[r] * inv;
+    if (rank != 0) return;
+    double *hcol = d->H + (size_t)(nc - 1) * (d->m + 1);
+    for (int k = tid; k < nc; k += CS_THREADS) {
+        h[k] += h2[k];
+        cs[k] = d->cs[k];
+        sn[k] = d->sn[k];
+    }
+    __syncthreads();
+    if (tid == 0) givens_update(d, nc, h, cs, sn, hnext, w0sq);
+    __syncthreads();
+    for (int k = tid; k <= nc; k += CS_THREADS) hcol[k] = h[k];
 }
 
 // x[r] (or u[r]) = sum_j B[j][r] y[j] for j < k; add = 1 accumulates into x
@@ -514,8 +645,22 @@ static int launch_cgs(rs_ctx *ctx, int n, int ld, int nc, double *V, GmresDev *d
     return st;
 }
 
+// small systems: one launch, and V[:, nc] comes out scaled
+static bool cgs_is_small(int n, int nc) { return n <= CS_MAX_ROWS && cgs_small_smem(n, nc) <= CS_SMEM; }
+
 static int cgs_step(rs_ctx *ctx, int n, int ld, int nc, double *V, GmresDev *d)
 {
+    if (cgs_is_small(n, nc)) {
+        static unsigned long long raised = 0;   // devices whose shared-memory limit was raised
+        const unsigned long long bit = 1ull << (ctx->device & 63);
+        if (!(raised & bit)) {
+            RS_CUDA_TRY(cudaFuncSetAttribute(k_cgs_small, cudaFuncAttributeMaxDynamicSharedMemorySize, CS_SMEM));
+            raised |= bit;
+        }
+        RsProfScope prof(ctx, RS_PROF_CGS_UPDATE_DOTS);
+        rs_pdl(k_cgs_small, CS_CTAS, CS_THREADS, cgs_small_smem(n, nc), ctx)(n, ld, nc, V, d);
+        return rs_check_launch(ctx);
+    }
     switch (nc / 4) {
     case 0: return launch_cgs<0>(ctx, n, ld, nc, V, d);
     case 1: return launch_cgs<4>(ctx, n, ld, nc, V, d);
@@ -676,7 +821,7 @@ static int gmres_impl(const rs_mat *A, rs_pc *M, const rs_vec *bv, rs_vec *xv, i
                 if (!st) st = cgs_step(ctx, n, ld, i + 1, V, d);
                 if (!st && cudaEventRecord(ev[i % STEPS_AHEAD], ctx->stream) != cudaSuccess) st = RS_ERR_CUDA;
                 if (st) goto out;
-                if (i + 1 < dim) {
+                if (i + 1 < dim && !cgs_is_small(n, i + 1)) {
                     rs_pdl(k_scale_dev, gb, 256, 0, ctx)(n, w, &d->hdiv, w, cycle_done);
                     ctx->launches++;
                 }

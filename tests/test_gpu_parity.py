@@ -409,6 +409,25 @@ def test_gmres_mixed_precision_error_vs_oracle(rs, ctx, orc):
     assert rel(x.numpy(), xo12) <= 1e-6, rel(x.numpy(), xo12)
 
 
+# the one-launch Arnoldi step of small systems (at most 6144 rows while the
+# basis fits in shared memory): fewer rows than blocks, ragged rows, the switch
+# to the three passes in mid-cycle (31 columns at 6144 rows), the largest
+# restart, and one size beyond the rule
+@pytest.mark.parametrize("shape,restart", [((3, 2, 1), 30), ((11, 7, 5), 64), ((24, 16, 16), 50), ((25, 16, 16), 30)])
+@pytest.mark.parametrize("solver", ["gmres", "fgmres"])
+def test_small_system_arnoldi(rs, ctx, orc, shape, restart, solver):
+    g = synth.Grid(*shape)
+    d = synth.pressure_7pt(g, 21, kz_scale=0.1)
+    A, Ao = rs.Mat.csr(ctx, d), orc.Mat.csr(d)
+    b = orc.spmv(Ao, synth.x_true(g.n, 21))
+    xo, io, _ = orc.gmres(Ao, orc.PC(Ao, "ilu0"), b, restart=restart, rtol=1e-10)
+    x = rs.Vec.zeros(ctx, g.n)
+    info = getattr(rs, "solve_" + solver)(A, rs.Precond(ctx, A, "ilu0"), vec(rs, ctx, b), x, restart=restart, rtol=1e-10)
+    assert info["status"] == 0 and abs(info["iters"] - io["iters"]) <= 2, (info, io)
+    assert orc.norm2(b - orc.spmv(Ao, x.numpy())) <= 1e-10 * orc.norm2(b)
+    assert rel(x.numpy(), xo) <= 1e-6
+
+
 def test_unpreconditioned_and_edge_cases(rs, ctx, orc):
     g = synth.Grid(8, 7, 6)
     d = synth.pressure_7pt(g, 3, accum=0.5)     # well conditioned: short, smooth convergence
