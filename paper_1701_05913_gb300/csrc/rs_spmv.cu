@@ -66,9 +66,9 @@ __device__ __forceinline__ void spmv_store(int64_t i, double acc, const double *
 
 // A thread per (block) row.  All loads are independent of one another and of
 // the mask (x's index is clamped, not predicated), so a warp keeps many of
-// its row's loads in flight.  Per product at the start and now: 7-point,
-// 1,048,576 rows 33.9 -> 19 us (76 MB moved; bytes and multiply-adds take
-// 11 and 12 us); 3 x 3 blocks, 500,000 rows 69 -> 60 us (52 us of
+// its row's loads in flight.  Per product, against the CSR and BSR kernels:
+// 7-point, 1,048,576 rows 33.9 -> 19 us (76 MB moved; bytes and multiply-adds
+// take 11 and 12 us); 3 x 3 blocks, 500,000 rows 69 -> 60 us (52 us of
 // multiply-adds).
 template <int ND, int BS>
 __global__ void __launch_bounds__(256)
@@ -159,19 +159,32 @@ k_spmv_sell(int nslice, const int2 *__restrict__ rows, const int *__restrict__ s
     const int2 rl = rows[(int64_t)s * 32 + lane];
     const int base = sptr[s] + lane, len = rl.y;
     double acc = 0.0;
-    for (int k0 = 0; k0 < len; k0 += U) {
-        int c[U];
-        double v[U], xv[U];
+    // the next U entries' loads are issued before the products of these wait
+    // for their gathers: one memory latency a round instead of two (a V-cycle
+    // at 128 x 128 x 64: 404 -> 398 us)
+    int c[U];
+    double v[U];
+    auto load = [&](int k0) {
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            c[u] = k0 + u < len ? col[base + 32 * (k0 + u)] : -1;
-            v[u] = k0 + u < len ? val[base + 32 * (k0 + u)] : 0.0;
+            c[u] = k0 + u < len ? __ldg(col + base + 32 * (k0 + u)) : -1;
+            v[u] = k0 + u < len ? __ldg(val + base + 32 * (k0 + u)) : 0.0;
         }
+    };
+    load(0);
+    for (int k0 = 0; k0 < len; k0 += U) {
+        double xv[U], vv[U];
+        bool in[U];
 #pragma unroll
-        for (int u = 0; u < U; ++u) xv[u] = c[u] >= 0 ? __ldg(x + c[u]) : 0.0;
+        for (int u = 0; u < U; ++u) {
+            in[u] = c[u] >= 0;
+            vv[u] = v[u];
+            xv[u] = in[u] ? __ldg(x + c[u]) : 0.0;
+        }
+        load(k0 + U);
 #pragma unroll
         for (int u = 0; u < U; ++u)
-            if (c[u] >= 0) acc = fma(v[u], xv[u], acc);
+            if (in[u]) acc = fma(vv[u], xv[u], acc);
     }
     if (rl.x >= 0) spmv_store(rl.x, acc, x, alpha, beta, bvec, y, dinv);
 }
