@@ -416,6 +416,7 @@ k_cgs_small(int n, int ld, int nc, double *__restrict__ V, GmresDev *d)
     __shared__ double cs[RS_MAX_RESTART], sn[RS_MAX_RESTART];
     if (rs_pdl_wait()) return;
     if (*(volatile int *)&d->cycle_done) return;                // set by this step at the earliest after its barriers
+    asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory");   // a block that has not started has no memory to write to
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int rank = blockIdx.x;                                // one cluster: the grid
     const int R = (n + CS_CTAS - 1) / CS_CTAS, r0 = rank * R, rows = max(0, min(R, n - r0));
@@ -478,6 +479,7 @@ k_cgs_small(int n, int ld, int nc, double *__restrict__ V, GmresDev *d)
     };
     // h1 = V^T w and ||w||^2; w -= V h1; h2 = V^T w; w -= V h2; ||w||
     dots(nc + 1);
+    asm volatile("barrier.cluster.wait;" ::: "memory");
     exchange(0, nc + 1, h);
     const double w0sq = h[nc];
     update(h);
