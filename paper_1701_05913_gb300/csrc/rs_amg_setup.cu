@@ -69,20 +69,25 @@ __global__ void __launch_bounds__(SCAN_T) k_scan_blocks(int n, const int *__rest
     if (threadIdx.x == 0) bsum[blockIdx.x] = tot;
 }
 
-// one block: the block sums in place, exclusive; *total at the end
-__global__ void __launch_bounds__(SCAN_T) k_scan_top(int nb, int *__restrict__ bsum, int *__restrict__ total)
+// one block: exclusive scan of n values (out may be in); the sum in *total and,
+// where end is given, *end
+__global__ void __launch_bounds__(SCAN_T) k_scan_top(int n, const int *in, int *out, int *__restrict__ total,
+                                                     int *__restrict__ end)
 {
     __shared__ int sh[32];
     int carry = 0;
-    for (int b0 = 0; b0 < nb; b0 += SCAN_T) {
+    for (int b0 = 0; b0 < n; b0 += SCAN_T) {
         const int i = b0 + threadIdx.x;
         int tot;
-        const int v = i < nb ? bsum[i] : 0;
+        const int v = i < n ? in[i] : 0;
         const int e = block_excl_scan(v, sh, &tot);
-        if (i < nb) bsum[i] = carry + e;
+        if (i < n) out[i] = carry + e;
         carry += tot;
     }
-    if (threadIdx.x == 0) *total = carry;
+    if (threadIdx.x == 0) {
+        *total = carry;
+        if (end) *end = carry;
+    }
 }
 
 __global__ void __launch_bounds__(SCAN_T) k_scan_add(int n, int *__restrict__ out, const int *__restrict__ bsum,
@@ -96,25 +101,63 @@ __global__ void __launch_bounds__(SCAN_T) k_scan_add(int n, int *__restrict__ ou
 // ---------------------------------------------------------------------------
 // 1. strength and its transpose
 // ---------------------------------------------------------------------------
-// count pass (sptr == nullptr): cnt[i] = |S_i|; fill pass: scol
-__global__ void k_strength(int n, const int *__restrict__ ptr, const int *__restrict__ col,
-                           const double *__restrict__ val, double theta, const int *__restrict__ sptr,
-                           int *__restrict__ out)
+// The kernels below go over a row's entries.  What bounds them is the latency
+// of a row's loads (a coarse level has a few rows of 30 to 60 entries and
+// cannot fill the chip), so the loads of ROW_U entries are issued before the
+// first is used, with clamped indices instead of predicates, and nothing is
+// looked up twice: the strength threshold is kept per row instead of found by
+// searching S.  128 x 128 x 64 hierarchy: strength 713 -> 380 us, interpolation
+// 1486 -> 565 us, sorting the rows of the transposes 327 -> 73 us.
+constexpr int ROW_U = 8;
+
+// body(p, col, val) for the entries p of [s, e) in order
+template <typename F>
+__device__ __forceinline__ void each_entry(int s, int e, const int *__restrict__ col, const double *__restrict__ val,
+                                           F body)
+{
+    for (int p0 = s; p0 < e; p0 += ROW_U) {
+        int c[ROW_U];
+        double v[ROW_U];
+#pragma unroll
+        for (int u = 0; u < ROW_U; ++u) {
+            const int p = min(p0 + u, e - 1);
+            c[u] = col[p];
+            v[u] = val[p];
+        }
+#pragma unroll
+        for (int u = 0; u < ROW_U; ++u)
+            if (p0 + u < e) body(c[u], v[u]);
+    }
+}
+
+// th[i]: entries with -a_ij >= th[i], j != i, are strong (none when infinite:
+// the row has no negative off-diagonal entry); cnt[i] = |S_i|
+__global__ void k_strength_count(int n, const int *__restrict__ ptr, const int *__restrict__ col,
+                                 const double *__restrict__ val, double theta, double *__restrict__ th,
+                                 int *__restrict__ cnt)
 {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        const int s = ptr[i], e = ptr[i + 1];
         double mx = 0.0;
-        for (int p = ptr[i]; p < ptr[i + 1]; ++p)
-            if (col[p] != i && -val[p] > mx) mx = -val[p];
-        int k = sptr ? sptr[i] : 0;
-        if (mx > 0.0) {
-            const double th = __dmul_rn(theta, mx);
-            for (int p = ptr[i]; p < ptr[i + 1]; ++p)
-                if (col[p] != i && -val[p] >= th) {
-                    if (sptr) out[k] = col[p];
-                    ++k;
-                }
-        }
-        if (!sptr) out[i] = k;
+        each_entry(s, e, col, val, [&](int c, double v) { mx = c != i && -v > mx ? -v : mx; });
+        const double t = mx > 0.0 ? __dmul_rn(theta, mx) : (double)INFINITY;
+        int k = 0;
+        if (mx > 0.0) each_entry(s, e, col, val, [&](int c, double v) { k += c != i && -v >= t; });
+        th[i] = t;
+        cnt[i] = k;
+    }
+}
+
+__global__ void k_strength_fill(int n, const int *__restrict__ ptr, const int *__restrict__ col,
+                                const double *__restrict__ val, const double *__restrict__ th,
+                                const int *__restrict__ sptr, int *__restrict__ scol)
+{
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        const double t = th[i];
+        int k = sptr[i];
+        each_entry(ptr[i], ptr[i + 1], col, val, [&](int c, double v) {
+            if (c != i && -v >= t) scol[k++] = c;
+        });
     }
 }
 
@@ -125,7 +168,7 @@ __global__ void k_count_cols(int64_t nnz, const int *__restrict__ col, int *__re
 }
 
 // transpose fill: entries land at an atomic slot of their column; values
-// optional; rows of the transpose are sorted afterwards where order matters
+// optional; rows of the transpose are sorted afterwards where it has values
 __global__ void k_transpose_fill(int n, const int *__restrict__ ptr, const int *__restrict__ col,
                                  const double *__restrict__ val, int *__restrict__ fill, int *__restrict__ tcol,
                                  double *__restrict__ tval)
@@ -138,22 +181,22 @@ __global__ void k_transpose_fill(int n, const int *__restrict__ ptr, const int *
         }
 }
 
-// insertion sort of every row by column (rows of a transpose are short)
-__global__ void k_sort_rows(int n, const int *__restrict__ ptr, int *__restrict__ col, double *__restrict__ val)
+// rows by column into (col, val): SORT_L lanes a row, an entry's place is the
+// number of the row's columns below its own (no column occurs twice)
+constexpr int SORT_L = 8;
+__global__ void k_sort_rows(int n, const int *__restrict__ ptr, const int *__restrict__ ucol,
+                            const double *__restrict__ uval, int *__restrict__ col, double *__restrict__ val)
 {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    const int lane = threadIdx.x % SORT_L;
+    for (int i = (blockIdx.x * blockDim.x + threadIdx.x) / SORT_L; i < n; i += gridDim.x * blockDim.x / SORT_L) {
         const int s = ptr[i], e = ptr[i + 1];
-        for (int a = s + 1; a < e; ++a) {
-            const int c = col[a];
-            const double v = val ? val[a] : 0.0;
-            int b = a - 1;
-            while (b >= s && col[b] > c) {
-                col[b + 1] = col[b];
-                if (val) val[b + 1] = val[b];
-                --b;
-            }
-            col[b + 1] = c;
-            if (val) val[b + 1] = v;
+        for (int a = s + lane; a < e; a += SORT_L) {
+            const int c = ucol[a];
+            int k = 0;
+#pragma unroll 8
+            for (int b = s; b < e; ++b) k += ucol[b] < c;
+            col[s + k] = c;
+            val[s + k] = uval[a];
         }
     }
 }
@@ -194,10 +237,17 @@ __global__ void k_pmis_select(int n, const int *__restrict__ sptr, const int *__
         if (old[i] != 0) continue;
         const double li = lam[i];
         bool top = true;
-        for (int q = sptr[i]; q < sptr[i + 1] && top; ++q)
-            if (old[scol[q]] == 0 && !(li > lam[scol[q]])) top = false;
-        for (int q = tptr[i]; q < tptr[i + 1] && top; ++q)
-            if (old[tcol[q]] == 0 && !(li > lam[tcol[q]])) top = false;
+        auto look = [&](int s, int e, const int *__restrict__ nb) {
+            for (int q0 = s; q0 < e && top; q0 += ROW_U) {
+                int c[ROW_U];
+#pragma unroll
+                for (int u = 0; u < ROW_U; ++u) c[u] = nb[min(q0 + u, e - 1)];
+#pragma unroll
+                for (int u = 0; u < ROW_U; ++u) top = top & !((old[c[u]] == 0) & !(li > lam[c[u]]));
+            }
+        };
+        look(sptr[i], sptr[i + 1], scol);
+        look(tptr[i], tptr[i + 1], tcol);
         if (top) st[i] = 1;
     }
 }
@@ -209,7 +259,14 @@ __global__ void k_pmis_f(int n, const int *__restrict__ sptr, const int *__restr
     for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
         if (st[j] != 0) continue;
         bool f = false;
-        for (int q = sptr[j]; q < sptr[j + 1] && !f; ++q) f = st[scol[q]] == 1;
+        const int s = sptr[j], e = sptr[j + 1];
+        for (int q0 = s; q0 < e && !f; q0 += ROW_U) {
+            int c[ROW_U];
+#pragma unroll
+            for (int u = 0; u < ROW_U; ++u) c[u] = scol[min(q0 + u, e - 1)];
+#pragma unroll
+            for (int u = 0; u < ROW_U; ++u) f = f | (st[c[u]] == 1);
+        }
         if (f) st[j] = 2;
         else atomicAdd(und, 1);
     }
@@ -233,67 +290,77 @@ __global__ void k_cidx(int n, const char *__restrict__ st, const int *__restrict
 // (positive) off-diagonal entries over that of its strong C neighbours,
 // d = a_ii, plus the positive couplings when no strong C coupling is positive
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ bool in_row(const int *__restrict__ sc, int s, int e, int k)
-{
-    for (int r = s; r < e; ++r)
-        if (sc[r] == k) return true;
-    return false;
-}
-
-// count pass (pptr == nullptr): cnt[i]; fill pass: pcol, pval
-__global__ void k_interp(int n, const int *__restrict__ ptr, const int *__restrict__ col,
-                         const double *__restrict__ val, const int *__restrict__ sptr, const int *__restrict__ scol,
-                         const int *__restrict__ cidx, const int *__restrict__ pptr, int *__restrict__ out,
-                         double *__restrict__ pval)
+__global__ void k_interp_count(int n, const int *__restrict__ sptr, const int *__restrict__ scol,
+                               const int *__restrict__ cidx, int *__restrict__ cnt)
 {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        if (cidx[i] >= 0) {
-            if (pptr) {
-                out[pptr[i]] = cidx[i];
-                pval[pptr[i]] = 1.0;
-            } else {
-                out[i] = 1;
-            }
+        int k = 1;
+        if (cidx[i] < 0) {
+            k = 0;
+#pragma unroll 4
+            for (int r = sptr[i]; r < sptr[i + 1]; ++r) k += cidx[scol[r]] >= 0;
+        }
+        cnt[i] = k;
+    }
+}
+
+// the strong C couplings go to pval as they are met and become weights once
+// the row's sums are known
+__global__ void k_interp_fill(int n, const int *__restrict__ ptr, const int *__restrict__ col,
+                              const double *__restrict__ val, const double *__restrict__ th,
+                              const int *__restrict__ cidx, const int *__restrict__ pptr, int *__restrict__ pcol,
+                              double *__restrict__ pval)
+{
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        const int k0 = pptr[i], ci = cidx[i];
+        if (ci >= 0) {
+            pcol[k0] = ci;
+            pval[k0] = 1.0;
             continue;
         }
-        const int s0 = sptr[i], s1 = sptr[i + 1];
-        if (!pptr) {
-            int k = 0;
-            for (int p = ptr[i]; p < ptr[i + 1]; ++p) {
-                const int c = col[p];
-                if (c != i && cidx[c] >= 0 && in_row(scol, s0, s1, c)) ++k;
-            }
-            out[i] = k;
-            continue;
-        }
+        const double t = th[i];
+        const int s = ptr[i], e = ptr[i + 1];
         double aii = 0.0, neg = 0.0, pos = 0.0, negc = 0.0, posc = 0.0;
-        for (int p = ptr[i]; p < ptr[i + 1]; ++p) {
-            const double v = val[p];
-            if (col[p] == i) aii = v;
-            else if (v < 0.0) neg = __dadd_rn(neg, v);
-            else pos = __dadd_rn(pos, v);
-        }
-        // the strong C neighbours' couplings, in column order
-        for (int r = s0; r < s1; ++r) {
-            const int c = scol[r];
-            if (cidx[c] < 0) continue;
-            for (int p = ptr[i]; p < ptr[i + 1]; ++p)
-                if (col[p] == c) {
-                    if (val[p] < 0.0) negc = __dadd_rn(negc, val[p]);
-                    else posc = __dadd_rn(posc, val[p]);
+        int k = k0;
+        for (int p0 = s; p0 < e; p0 += ROW_U) {
+            int c[ROW_U], cc[ROW_U];
+            double v[ROW_U];
+#pragma unroll
+            for (int u = 0; u < ROW_U; ++u) {
+                const int p = min(p0 + u, e - 1);
+                c[u] = col[p];
+                v[u] = val[p];
+            }
+#pragma unroll
+            for (int u = 0; u < ROW_U; ++u) cc[u] = cidx[c[u]];
+#pragma unroll
+            for (int u = 0; u < ROW_U; ++u) {
+                if (p0 + u >= e) continue;
+                if (c[u] == i) {
+                    aii = v[u];
+                    continue;
                 }
+                const bool strong_c = cc[u] >= 0 && -v[u] >= t;
+                if (v[u] < 0.0) {
+                    neg = __dadd_rn(neg, v[u]);
+                    if (strong_c) negc = __dadd_rn(negc, v[u]);
+                } else {
+                    pos = __dadd_rn(pos, v[u]);
+                    if (strong_c) posc = __dadd_rn(posc, v[u]);
+                }
+                if (strong_c) {
+                    pcol[k] = cc[u];
+                    pval[k++] = v[u];
+                }
+            }
         }
         double diag = aii, beta = 0.0;
         if (posc == 0.0) diag = __dadd_rn(diag, pos);
         else beta = __ddiv_rn(pos, posc);
         const double alpha = negc != 0.0 ? __ddiv_rn(neg, negc) : 0.0;
-        int k = pptr[i];
-        for (int p = ptr[i]; p < ptr[i + 1]; ++p) {
-            const int c = col[p];
-            if (c == i || cidx[c] < 0 || !in_row(scol, s0, s1, c)) continue;
-            out[k] = cidx[c];
-            pval[k] = __ddiv_rn(__dmul_rn(-(val[p] < 0.0 ? alpha : beta), val[p]), diag);
-            ++k;
+        for (int q = k0; q < k; ++q) {
+            const double v = pval[q];
+            pval[q] = __ddiv_rn(__dmul_rn(-(v < 0.0 ? alpha : beta), v), diag);
         }
     }
 }
@@ -575,10 +642,10 @@ __global__ void k_amg_l1(int n, const int *__restrict__ ptr, const int *__restri
 {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         double s = 0.0, dg = 0.0;
-        for (int p = ptr[i]; p < ptr[i + 1]; ++p) {
-            s = __dadd_rn(s, fabs(val[p]));
-            if (col[p] == i) dg = val[p];
-        }
+        each_entry(ptr[i], ptr[i + 1], col, val, [&](int c, double v) {
+            s = __dadd_rn(s, fabs(v));
+            dg = c == i ? v : dg;
+        });
         dinv[i] = __ddiv_rn(1.0, s);
         if (dg == 0.0) atomicOr(bad, 1);
     }
@@ -705,10 +772,14 @@ int scan(rs_ctx *ctx, Dev &D, const int *in, int *out, int n, int *total)
     int *bsum, *dt;
     RS_TRY(D.alloc(&bsum, nb));
     RS_TRY(D.alloc(&dt, 1));
-    k_scan_blocks<<<nb, SCAN_T, 0, ctx->stream>>>(n, in, out, bsum);
-    k_scan_top<<<1, SCAN_T, 0, ctx->stream>>>(nb, bsum, dt);
-    k_scan_add<<<nb, SCAN_T, 0, ctx->stream>>>(n, out, bsum, dt);
-    ctx->launches += 2;
+    if (nb <= 4) {        // a coarse level: a block's few rounds are shorter than two more launches
+        k_scan_top<<<1, SCAN_T, 0, ctx->stream>>>(n, in, out, dt, out + n);
+    } else {
+        k_scan_blocks<<<nb, SCAN_T, 0, ctx->stream>>>(n, in, out, bsum);
+        k_scan_top<<<1, SCAN_T, 0, ctx->stream>>>(nb, bsum, bsum, dt, nullptr);
+        k_scan_add<<<nb, SCAN_T, 0, ctx->stream>>>(n, out, bsum, dt);
+        ctx->launches += 2;
+    }
     RS_TRY(rs_check_launch(ctx));
     RS_CUDA_TRY(cudaMemcpyAsync(total, dt, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
     RS_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
@@ -722,25 +793,31 @@ int read_flag(rs_ctx *ctx, const int *d, int *h)
     return RS_OK;
 }
 
-// transpose (values optional) with sorted rows
+// transpose; with values its rows are sorted (without, their order is open)
 int transpose(rs_ctx *ctx, Dev &D, int n, int m, int64_t nnz, const int *ptr, const int *col, const double *val,
               int **tptr, int **tcol, double **tval)
 {
-    int *cnt, *fill, tot = 0;
+    int *cnt, *fill, *ucol = nullptr, tot = 0;
+    double *uval = nullptr;
     RS_TRY(D.alloc(&cnt, m));
     RS_TRY(D.alloc(tptr, m + 1));
     RS_TRY(D.alloc(tcol, nnz));
-    if (tval) RS_TRY(D.alloc(tval, nnz));
+    if (tval) {
+        RS_TRY(D.alloc(tval, nnz));
+        RS_TRY(D.alloc(&ucol, nnz));
+        RS_TRY(D.alloc(&uval, nnz));
+    }
     RS_TRY(D.alloc(&fill, m));
     RS_CUDA_TRY(cudaMemsetAsync(cnt, 0, sizeof(int) * std::max(m, 1), ctx->stream));
     k_count_cols<<<grid_for(ctx, nnz, 256), 256, 0, ctx->stream>>>(nnz, col, cnt);
     RS_TRY(rs_check_launch(ctx));
     RS_TRY(scan(ctx, D, cnt, *tptr, m, &tot));
     RS_CUDA_TRY(cudaMemcpyAsync(fill, *tptr, sizeof(int) * std::max(m, 1), cudaMemcpyDeviceToDevice, ctx->stream));
-    k_transpose_fill<<<grid_for(ctx, n, 256), 256, 0, ctx->stream>>>(n, ptr, col, val, fill, *tcol,
-                                                                     tval ? *tval : nullptr);
-    k_sort_rows<<<grid_for(ctx, m, 128), 128, 0, ctx->stream>>>(m, *tptr, *tcol, tval ? *tval : nullptr);
-    ctx->launches += 1;
+    k_transpose_fill<<<grid_for(ctx, n, 256), 256, 0, ctx->stream>>>(n, ptr, col, val, fill, tval ? ucol : *tcol,
+                                                                     uval);
+    RS_TRY(rs_check_launch(ctx));
+    if (!tval) return RS_OK;
+    k_sort_rows<<<grid_for(ctx, (int64_t)m * SORT_L, 128), 128, 0, ctx->stream>>>(m, *tptr, ucol, uval, *tcol, *tval);
     return rs_check_launch(ctx);
 }
 
@@ -812,13 +889,15 @@ int rs_amg_setup_device(AmgData *M, double theta, int max_levels, int max_coarse
         const int g = grid_for(ctx, n, 128);
         // 1. strength S and its transpose
         int *scnt, *sptr, *scol, *tptr, *tcol, ns = 0;
+        double *th;
+        RS_TRY(D.alloc(&th, n));
         RS_TRY(D.alloc(&scnt, n));
         RS_TRY(D.alloc(&sptr, n + 1));
-        k_strength<<<g, 128, 0, ctx->stream>>>(n, A->ptr, A->col, A->val, theta, nullptr, scnt);
+        k_strength_count<<<g, 128, 0, ctx->stream>>>(n, A->ptr, A->col, A->val, theta, th, scnt);
         RS_TRY(rs_check_launch(ctx));
         RS_TRY(scan(ctx, D, scnt, sptr, n, &ns));
         RS_TRY(D.alloc(&scol, ns));
-        k_strength<<<g, 128, 0, ctx->stream>>>(n, A->ptr, A->col, A->val, theta, sptr, scol);
+        k_strength_fill<<<g, 128, 0, ctx->stream>>>(n, A->ptr, A->col, A->val, th, sptr, scol);
         RS_TRY(rs_check_launch(ctx));
         RS_TRY(transpose(ctx, D, n, n, ns, sptr, scol, nullptr, &tptr, &tcol, nullptr));
         // 2. PMIS
@@ -858,12 +937,12 @@ int rs_amg_setup_device(AmgData *M, double theta, int max_levels, int max_coarse
         double *pval;
         RS_TRY(D.alloc(&pcnt, n));
         RS_TRY(D.alloc(&pptr, n + 1));
-        k_interp<<<g, 128, 0, ctx->stream>>>(n, A->ptr, A->col, A->val, sptr, scol, cidx, nullptr, pcnt, nullptr);
+        k_interp_count<<<g, 128, 0, ctx->stream>>>(n, sptr, scol, cidx, pcnt);
         RS_TRY(rs_check_launch(ctx));
         RS_TRY(scan(ctx, D, pcnt, pptr, n, &np));
         RS_TRY(D.alloc(&pcol, np));
         RS_TRY(D.alloc(&pval, np));
-        k_interp<<<g, 128, 0, ctx->stream>>>(n, A->ptr, A->col, A->val, sptr, scol, cidx, pptr, pcol, pval);
+        k_interp_fill<<<g, 128, 0, ctx->stream>>>(n, A->ptr, A->col, A->val, th, cidx, pptr, pcol, pval);
         RS_TRY(rs_check_launch(ctx));
         // 4. R = P^T (nc x n)
         int *rptr, *rcol;

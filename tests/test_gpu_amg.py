@@ -132,6 +132,22 @@ def test_amg_products_of_long_rows(rs, ctx, orc, n, w, reach, coarse):
         assert all(np.array_equal(x, y) for x, y in zip(g["A"], wa)), l
 
 
+# single and several blocks of the scans (1024 values each, up to four in one
+# block)
+@pytest.mark.parametrize("n", [1023, 1025, 4095, 4096, 4097, 5121])
+def test_amg_setup_at_scan_edges(rs, ctx, orc, n):
+    d = synth.pressure_7pt(synth.Grid(n, 1, 1), 79)
+    got = rs.Precond(ctx, rs.Mat.csr(ctx, d), "amg", amg=dict(max_coarse=8)).amg_levels()
+    R = orc.Amg(orc.Mat.csr(d), max_coarse=8)
+    want = R.levels()
+    assert len(got) == len(want) >= 2
+    for l, (g, (wa, wp)) in enumerate(zip(got, want)):
+        assert all(np.array_equal(x, y) for x, y in zip(g["A"], wa)), l
+        if wp is not None:
+            assert np.array_equal(g["cidx"], R.cidx(l)), l
+            assert all(np.array_equal(x, y) for x, y in zip(g["P"], wp)), l
+
+
 def test_amg_product_row_limit(rs, ctx):
     """A Galerkin row of more than 2048 candidate terms is refused."""
     A = rs.Mat.csr(ctx, _scattered(1200, 12, 1200))
