@@ -739,6 +739,154 @@ __global__ void k_dense_take(int n, const double *__restrict__ m, double *__rest
     }
 }
 
+// The same elimination of a small coarsest matrix in one launch: a cluster of
+// GJ_CTAS blocks holds the matrix in shared memory, row s in block s % GJ_CTAS.
+// Of [A | I] only n columns are ever live: at step c column c of the left half
+// is done, and of the right half only the columns of rows that have been
+// pivots differ from the identity, so the column of pivot row sp takes the
+// place of column c.
+// Rows stay where they are; slot_of and pos_of say which row stands where
+// after the swaps, and every block keeps them alike.  Per column: each block's
+// pivot candidate goes to all blocks, one cluster barrier, then every block
+// reads the pivot row from its owner, divides it by the pivot and eliminates
+// its own rows.  The owner puts the divided row in place after the next barrier, when
+// all blocks have read the old one.  Same pivots, operations and order per
+// element as the two kernels above.
+//
+// What bounds it: n steps of a cluster barrier, n divisions per block (about
+// 4 us a step together) and n / 8 rows of FP64 on one SM (4 us more at n =
+// 256), against two launches a step and all SMs.  Setup of one dense level,
+// us, at n = 24, 97, 160, 256, 300: 316, 1090, 1764, 3200, 3818 -> 137, 527,
+// 899, 2182, 3364; the lines meet a little above GJ_MAX_N.
+constexpr int GJ_CTAS = 8, GJ_THREADS = 256;
+constexpr int GJ_MAX_N = 304;
+constexpr size_t gj_smem(int n) { return sizeof(double) * ((size_t)(n + GJ_CTAS - 1) / GJ_CTAS + 2) * n; }
+static_assert(gj_smem(GJ_MAX_N) <= 200 * 1024, "the coarsest matrix fits in a cluster's shared memory");
+
+__device__ __forceinline__ unsigned cluster_addr(const void *p, int rank)
+{
+    unsigned a;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_addr(p)), "r"(rank));
+    return a;
+}
+__device__ __forceinline__ double ld_cluster(unsigned a)
+{
+    double v;
+    asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+}
+
+__global__ void __cluster_dims__(GJ_CTAS, 1, 1) __launch_bounds__(GJ_THREADS)
+k_gj_cluster(int n, const int *__restrict__ ptr, const int *__restrict__ col, const double *__restrict__ val,
+             double *__restrict__ inv, int *__restrict__ bad)
+{
+    extern __shared__ __align__(16) double gj[];
+    __shared__ double cv[2][GJ_CTAS];                   // candidates of the blocks, by the step's parity
+    __shared__ int cp[2][GJ_CTAS];
+    __shared__ int slot_of[GJ_MAX_N], pos_of[GJ_MAX_N];
+    const int R = (n + GJ_CTAS - 1) / GJ_CTAS;
+    double *tile = gj, *row = gj + (size_t)R * n;       // row: the divided pivot rows of two steps
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, rank = blockIdx.x;   // one cluster: the grid
+    for (int t = tid; t < R * n; t += GJ_THREADS) tile[t] = 0.0;
+    for (int t = tid; t < n; t += GJ_THREADS) slot_of[t] = pos_of[t] = t;
+    __syncthreads();
+    for (int i = warp; rank + GJ_CTAS * i < n; i += GJ_THREADS / 32) {
+        const int s = rank + GJ_CTAS * i;
+        for (int p = ptr[s] + lane; p < ptr[s + 1]; p += 32) tile[(size_t)i * n + col[p]] = val[p];
+    }
+    cluster_sync();                                     // every block has started
+    int last = -1;                                      // the row divided in the step before
+    bool singular = false;
+    for (int c = 0; c < n; ++c) {
+        const int b = c & 1;
+        double *rb = row + (size_t)b * n, *ro = row + (size_t)(b ^ 1) * n;
+        __syncthreads();
+        if (warp == 0) {                                // largest |a|, lowest position on ties
+            double best = -1.0;
+            int bp = n;
+            for (int i = lane; rank + GJ_CTAS * i < n; i += 32) {
+                const int ps = pos_of[rank + GJ_CTAS * i];
+                const double a = fabs(tile[(size_t)i * n + c]);
+                if (ps >= c && (a > best || (a == best && ps < bp))) {
+                    best = a;
+                    bp = ps;
+                }
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                const double a = __shfl_xor_sync(0xffffffffu, best, o);
+                const int ps = __shfl_xor_sync(0xffffffffu, bp, o);
+                if (a > best || (a == best && ps < bp)) {
+                    best = a;
+                    bp = ps;
+                }
+            }
+            if (lane < GJ_CTAS) {
+                asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(cluster_addr(&cv[b][rank], lane)), "d"(best)
+                             : "memory");
+                asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(cluster_addr(&cp[b][rank], lane)), "r"(bp)
+                             : "memory");
+            }
+        }
+        cluster_sync();
+        if (last >= 0 && last % GJ_CTAS == rank)
+            for (int j = tid; j < n; j += GJ_THREADS) tile[(size_t)(last / GJ_CTAS) * n + j] = ro[j];
+        double best = -1.0;
+        int p = n;
+#pragma unroll
+        for (int q = 0; q < GJ_CTAS; ++q)
+            if (cv[b][q] > best || (cv[b][q] == best && cp[b][q] < p)) {
+                best = cv[b][q];
+                p = cp[b][q];
+            }
+        if (p >= n) p = c;                              // a column of NaN: refused below
+        const int sp = slot_of[p], sc = slot_of[c];
+        const unsigned src = cluster_addr(tile + (size_t)(sp / GJ_CTAS) * n, sp % GJ_CTAS);
+        const double piv = ld_cluster(src + 8 * c);
+        if (!(piv != 0.0) || !isfinite(piv)) {          // the same value in every block
+            singular = true;
+            break;
+        }
+        for (int j = tid; j < n; j += GJ_THREADS) rb[j] = __ddiv_rn(j == c ? 1.0 : ld_cluster(src + 8 * j), piv);
+        __syncthreads();
+        if (tid == 0) {
+            slot_of[p] = sc;
+            slot_of[c] = sp;
+            pos_of[sc] = p;
+            pos_of[sp] = c;
+        }
+        for (int i = warp; rank + GJ_CTAS * i < n; i += GJ_THREADS / 32) {
+            if (rank + GJ_CTAS * i == sp) continue;
+            double *t = tile + (size_t)i * n;
+            const double f = t[c];
+            __syncwarp();                               // every lane has f
+            if (f != 0.0) {
+#pragma unroll 4
+                for (int j = lane; j < n; j += 32) t[j] = __dsub_rn(j == c ? 0.0 : t[j], __dmul_rn(f, rb[j]));
+            } else if (lane == 0) {
+                t[c] = 0.0;
+            }
+        }
+        last = sp;
+    }
+    __syncthreads();
+    if (singular) {
+        if (rank == 0 && tid == 0) atomicOr(bad, 1);
+    } else {
+        for (int i = warp; rank + GJ_CTAS * i < n; i += GJ_THREADS / 32) {
+            const int s = rank + GJ_CTAS * i;
+            const double *t = s == last ? row + (size_t)((n - 1) & 1) * n : tile + (size_t)i * n;
+            for (int j = lane; j < n; j += 32) inv[(size_t)pos_of[s] * n + slot_of[j]] = t[j];
+        }
+    }
+    cluster_sync();                                     // no block leaves while another reads its rows
+}
+
 // ---------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------
@@ -976,10 +1124,24 @@ int rs_amg_setup_device(AmgData *M, double theta, int max_levels, int max_coarse
     }
     // the coarsest matrix's dense inverse
     double *aug;
-    RS_TRY(D.alloc(&aug, (size_t)ncoarse * 2 * ncoarse));
     RS_TRY(rs_alloc(ctx, (void **)&M->cinv, sizeof(double) * (size_t)ncoarse * ncoarse));
     const rs_mat *Cm = M->A[l];
     RS_CUDA_TRY(cudaMemsetAsync(bad, 0, sizeof(int), ctx->stream));
+    if (ncoarse <= GJ_MAX_N) {
+        static unsigned long long raised = 0;  // one bit per device
+        const unsigned long long bit = 1ull << (ctx->device & 63);
+        if (!(raised & bit)) {
+            RS_CUDA_TRY(cudaFuncSetAttribute(k_gj_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)gj_smem(GJ_MAX_N)));
+            raised |= bit;
+        }
+        k_gj_cluster<<<GJ_CTAS, GJ_THREADS, gj_smem(ncoarse), ctx->stream>>>(ncoarse, Cm->ptr, Cm->col, Cm->val,
+                                                                             M->cinv, bad);
+        RS_TRY(rs_check_launch(ctx));
+        RS_TRY(read_flag(ctx, bad, &hbad));
+        return hbad ? RS_ERR_ZERO_PIVOT : RS_OK;
+    }
+    RS_TRY(D.alloc(&aug, (size_t)ncoarse * 2 * ncoarse));
     k_dense_aug<<<grid_for(ctx, (int64_t)ncoarse * 2 * ncoarse, 256), 256, 0, ctx->stream>>>(ncoarse, Cm->ptr,
                                                                                           Cm->col, Cm->val, aug);
     k_dense_scatter<<<grid_for(ctx, ncoarse, 128), 128, 0, ctx->stream>>>(ncoarse, Cm->ptr, Cm->col, Cm->val, aug);

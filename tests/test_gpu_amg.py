@@ -148,6 +148,27 @@ def test_amg_setup_at_scan_edges(rs, ctx, orc, n):
             assert all(np.array_equal(x, y) for x, y in zip(g["P"], wp)), l
 
 
+# one dense level with rows swapped at most columns, around the largest matrix
+# inverted in one launch and at ragged shares of its eight blocks.  The inverse
+# meets the system: |A (A^-1 r) - r| <= c n eps cond(A) |r|, with cond below
+# 1e4 for these matrices and growth below 10
+@pytest.mark.parametrize("n", [1, 2, 7, 8, 9, 97, 255, 303, 304, 305])
+def test_amg_coarsest_inverse(rs, ctx, n):
+    rng = np.random.default_rng(80 + n)
+    D = rng.standard_normal((n, n)) + 2.0 * np.sqrt(n) * np.eye(n)[rng.permutation(n)]
+    assert np.linalg.cond(D) < 1e4
+    d = dict(n=n, rowptr=(np.arange(n + 1) * n).astype(np.int32), col=np.tile(np.arange(n), n).astype(np.int32),
+             val=D.ravel().copy())
+    M = rs.Precond(ctx, rs.Mat.csr(ctx, d), "amg", amg=dict(max_coarse=n))
+    z = rs.Vec.zeros(ctx, n)
+    r = rng.standard_normal(n)
+    M.apply(rs.Vec(ctx, r), z)
+    assert rel(D @ z.numpy(), r) <= 10 * max(n, 8) * 2.2e-16 * 1e4
+    D[:, n // 2] = 0.0                                    # no pivot in this column
+    d["val"] = D.ravel().copy()
+    assert rs.Precond(ctx, rs.Mat.csr(ctx, d), "amg", amg=dict(max_coarse=n)).status == rs.ERR_ZERO_PIVOT
+
+
 def test_amg_product_row_limit(rs, ctx):
     """A Galerkin row of more than 2048 candidate terms is refused."""
     A = rs.Mat.csr(ctx, _scattered(1200, 12, 1200))
