@@ -12,8 +12,9 @@
 // the gather and scatter passes of the apply go too.
 //
 // The rows' records come in chunks of at most PT_ROWS rows of a level (places;
-// values by entry; columns by entry, 16-bit and local), streamed through a ring of shared-memory slots, two chunks a slot and copy,
-// by a producer warp that joins the barrier once per slot (as in rs_level.cu).
+// values by entry; columns by entry, 16-bit and local), streamed through a
+// ring of shared-memory slots, two chunks a slot and copy, by a producer warp
+// that joins the barrier once per slot (as in rs_level.cu).
 // A row with fewer entries than its chunk's widest reads a zero at the end of
 // the values.
 //
