@@ -314,7 +314,7 @@ def cgs_fmas(n, iters_list, m=30):
 
 def source_sha(kernel):
     files = {"spmv": ["rs_core.cu", "rs_spmv.cu"], "net": ["rs_net.cu"], "cpr_resid": ["rs_precond.cu", "rs_spmv.cu"]}.get(
-        kernel, ["rs_ilu.cu", "rs_wave.cu"] if "sweep" in kernel else ["rs_krylov.cu"])
+        kernel, ["rs_ilu.cu", "rs_wave.cu", "rs_level.cu", "rs_part.cu"] if "sweep" in kernel else ["rs_krylov.cu"])
     h = hashlib.sha256()
     for f in files:
         h.update(open(os.path.join(ROOT, "paper_1701_05913_gb300", "csrc", f), "rb").read())
