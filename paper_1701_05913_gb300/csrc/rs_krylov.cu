@@ -393,19 +393,21 @@ k_cgs_pass(int n, int ld, int nc, const double *__restrict__ V, double *w, doubl
 // distributed shared memory and are added in block order, and the new basis
 // vector is written already scaled by 1 / h_{i+1,i}.  What bounds it: three
 // cluster barriers and the FP64 multiply-adds of CS_CTAS SMs (4 n nc in all:
-// 13 of 34 us at 1920 rows and 15 columns).  Against three passes and the
-// scaling, GMRES(30) with ILU(0) at 16x12x10: 3521 -> 3136 us, 57 -> 51 us an
-// iteration.
+// about 4 of 23 us at 1920 rows and 15 columns).  The basis is loaded while the
+// product before still runs.  Against three passes and the scaling, GMRES(30)
+// with ILU(0) at 16x12x10: 3521 -> 2890 us, 57 -> 47 us an iteration (3136 with the
+// loads after the wait; a cluster of 16 blocks took 5 % longer than 8, with
+// more to exchange).
 // ---------------------------------------------------------------------------
 #define CS_CTAS 8
 #define CS_THREADS 256
 #define CS_MAX_ROWS 6144                            // beyond, the passes' more SMs win
 #define CS_SMEM (190 * 1024)
 
-static size_t cgs_small_smem(int n, int nc)
-{
-    return sizeof(double) * (size_t)((n + CS_CTAS - 1) / CS_CTAS) * (nc + 1);
-}
+// rows of a block: even, so that a column's rows are whole 16-byte copies
+__host__ __device__ __forceinline__ int cgs_small_rows(int n) { return ((n + CS_CTAS - 1) / CS_CTAS + 1) & ~1; }
+
+static size_t cgs_small_smem(int n, int nc) { return sizeof(double) * (size_t)cgs_small_rows(n) * (nc + 1); }
 
 __global__ void __cluster_dims__(CS_CTAS, 1, 1) __launch_bounds__(CS_THREADS)
 k_cgs_small(int n, int ld, int nc, double *__restrict__ V, GmresDev *d)
@@ -414,18 +416,28 @@ k_cgs_small(int n, int ld, int nc, double *__restrict__ V, GmresDev *d)
     __shared__ double ex[3][CS_CTAS][RS_MAX_RESTART + 2];       // the blocks' sums, one buffer an exchange
     __shared__ double part[RS_MAX_RESTART + 2], h[RS_MAX_RESTART + 2], h2[RS_MAX_RESTART + 2];
     __shared__ double cs[RS_MAX_RESTART], sn[RS_MAX_RESTART];
-    if (rs_pdl_wait()) return;
-    if (*(volatile int *)&d->cycle_done) return;                // set by this step at the earliest after its barriers
-    asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory");   // a block that has not started has no memory to write to
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int rank = blockIdx.x;                                // one cluster: the grid
-    const int R = (n + CS_CTAS - 1) / CS_CTAS, r0 = rank * R, rows = max(0, min(R, n - r0));
+    const int R = cgs_small_rows(n), r0 = rank * R, rows = max(0, min(R, n - r0));
     double *w = cs_tile + (size_t)nc * R;
-    for (int k = warp; k <= nc; k += CS_THREADS / 32) {
-        const double *src = V + (size_t)k * ld + r0;
-#pragma unroll 4
-        for (int r = lane; r < rows; r += 32) cs_tile[(size_t)k * R + r] = src[r];
-    }
+    // columns [k0, k1) through L2; ld has room for an odd last row's neighbour
+    auto load = [&](int k0, int k1) {
+        const int pairs = (rows + 1) / 2;
+        for (int t = tid; t < (k1 - k0) * pairs; t += CS_THREADS) {
+            const int k = t / pairs, q = 2 * (t - k * pairs);
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(cs_tile + (size_t)(k0 + k) * R + q)),
+                         "l"(V + (size_t)(k0 + k) * ld + r0 + q)
+                         : "memory");
+        }
+    };
+    // the kernel before is the product that writes w: the basis is older
+    load(0, nc);
+    const bool never = rs_pdl_wait(), done = never || *(volatile int *)&d->cycle_done;  // set by this step at the
+                                                                                        // earliest after its barriers
+    if (!done) load(nc, nc + 1);
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    if (done) return;
+    asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory");   // a block that has not started has no memory to write to
     __syncthreads();
     // part[k] = this block's rows of <V_k, w>, k < cols (k = nc: <w, w>)
     auto dots = [&](int cols) {
