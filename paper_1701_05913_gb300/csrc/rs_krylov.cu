@@ -225,22 +225,47 @@ struct CgsCfg {
 // nc - NCC (0 to 3) columns take a warp-uniform branch, so that no FP64
 // multiply-add is issued for a column that does not exist (predicated-off
 // FP64 instructions still occupy the FP64 pipe on this GPU).
-// One thread: the Givens rotations on the new Hessenberg column h[0..nc) with
+// The Givens rotations on the new Hessenberg column h[0..nc) with
 // h_{nc,nc-1} = hnext (h[nc] is set to 0), the rotated residual, the
 // convergence and happy-breakdown tests and the next vector's scale.  cs, sn:
 // the earlier rotations (nc - 1 of them are read).
+// A warp calls it.  An FP64 instruction takes a warp 64 cycles whether one lane
+// works or all, so only what depends on the rotation before stays in the chain
+// (two of the six operations a rotation); the products beside it, the new
+// column and the three quotients are taken lane by lane.  Same operations.
 __device__ __forceinline__ void givens_update(GmresDev *d, int nc, double *h, const double *cs, const double *sn,
-                                              double hnext, double w0sq)
+                                              double hnext, double w0sq, int lane)
 {
+    __shared__ double av[RS_MAX_RESTART], cb[RS_MAX_RESTART];
     const int i = nc - 1;
+    double sb[(RS_MAX_RESTART + 31) / 32];
+#pragma unroll
+    for (int q = 0; q < (RS_MAX_RESTART + 31) / 32; ++q) {
+        const int k = lane + 32 * q;
+        if (k >= i) continue;
+        cb[k] = __dmul_rn(cs[k], h[k + 1]);
+        sb[q] = __dmul_rn(sn[k], h[k + 1]);
+    }
+    __syncwarp();
     double a = h[0];
+#pragma unroll 4
     for (int k = 0; k < i; ++k) {
-        const double b = h[k + 1];
-        h[k] = __dadd_rn(__dmul_rn(cs[k], a), __dmul_rn(sn[k], b));
-        a = __dadd_rn(__dmul_rn(-sn[k], a), __dmul_rn(cs[k], b));
+        if (lane == 0) av[k] = a;
+        a = __dadd_rn(__dmul_rn(-sn[k], a), cb[k]);
+    }
+    __syncwarp();
+#pragma unroll
+    for (int q = 0; q < (RS_MAX_RESTART + 31) / 32; ++q) {
+        const int k = lane + 32 * q;
+        if (k < i) h[k] = __dadd_rn(__dmul_rn(cs[k], av[k]), sb[q]);
     }
     const double rho = hypot(a, hnext);
-    const double c = __ddiv_rn(a, rho), s = __ddiv_rn(hnext, rho), g = d->g[i];
+    const double quot = __ddiv_rn(lane == 0 ? a : lane == 1 ? hnext : 1.0, lane < 2 ? rho : hnext);
+    const double c = __shfl_sync(0xffffffffu, quot, 0), s = __shfl_sync(0xffffffffu, quot, 1);
+    const double hinv = __shfl_sync(0xffffffffu, quot, 2);
+    __syncwarp();
+    if (lane != 0) return;
+    const double g = d->g[i];
     d->cs[i] = c;
     d->sn[i] = s;
     h[i] = rho;
@@ -259,7 +284,7 @@ __device__ __forceinline__ void givens_update(GmresDev *d, int nc, double *h, co
         d->cycle_done = 1;
         *(volatile int *)d->host_done = 1;
     }
-    d->hdiv = 1.0 / hnext;     // v_{i+1} = w / h_{i+1,i}
+    d->hdiv = hinv;            // v_{i+1} = w / h_{i+1,i}
 }
 
 template <int NC, int NCC, int MODE>
@@ -379,7 +404,7 @@ k_cgs_pass(int n, int ld, int nc, const double *__restrict__ V, double *w, doubl
                 sn[k] = d->sn[k];
             }
             __syncthreads();
-            if (threadIdx.x == 0) givens_update(d, nc, h, cs, sn, sqrt(d->r2), d->w0sq);
+            if (warp == 0) givens_update(d, nc, h, cs, sn, sqrt(d->r2), d->w0sq, lane);
             __syncthreads();
             for (int k = threadIdx.x; k <= nc; k += blockDim.x) hcol[k] = h[k];
         }
@@ -393,9 +418,9 @@ k_cgs_pass(int n, int ld, int nc, const double *__restrict__ V, double *w, doubl
 // distributed shared memory and are added in block order, and the new basis
 // vector is written already scaled by 1 / h_{i+1,i}.  What bounds it: three
 // cluster barriers and the FP64 multiply-adds of CS_CTAS SMs (4 n nc in all:
-// about 4 of 23 us at 1920 rows and 15 columns).  The basis is loaded while the
+// about 4 of 21 us at 1920 rows and 15 columns).  The basis is loaded while the
 // product before still runs.  Against three passes and the scaling, GMRES(30)
-// with ILU(0) at 16x12x10: 3521 -> 2890 us, 57 -> 47 us an iteration (3136 with the
+// with ILU(0) at 16x12x10: 3521 -> 2830 us, 57 -> 46 us an iteration (3136 with the
 // loads after the wait; a cluster of 16 blocks took 5 % longer than 8, with
 // more to exchange).
 // ---------------------------------------------------------------------------
@@ -520,7 +545,7 @@ k_cgs_small(int n, int ld, int nc, double *__restrict__ V, GmresDev *d)
         sn[k] = d->sn[k];
     }
     __syncthreads();
-    if (tid == 0) givens_update(d, nc, h, cs, sn, hnext, w0sq);
+    if (warp == 0) givens_update(d, nc, h, cs, sn, hnext, w0sq, lane);
     __syncthreads();
     for (int k = tid; k <= nc; k += CS_THREADS) hcol[k] = h[k];
 }
