@@ -46,6 +46,7 @@
 #include <algorithm>
 #include <vector>
 
+#include "rs_bounds.cuh"
 #include "rs_internal.cuh"
 
 #define RS_WAVE_MAX_NX 4096
@@ -314,7 +315,7 @@ k_wave_sweep(WaveArgs g, const T *__restrict__ rec, const T *__restrict__ rhs, T
             // ---------------------------------------------------------------
             const T *grec = rec + base * RB;
             const T *grhs = rhs + base * BS;
-            int qb = 0, qstep = 0;                // next chunk to copy, and the step that frees its slot
+            int qb = 0, qstep = rs_wave_chunk_step(0, nch, R, G);    // next chunk to copy, and the step that frees its slot
             // steps the compute warp has left
             auto cons_now = [&]() -> int { return __shfl_sync(FULL, *(volatile int *)&hd->cons, 0); };
             auto issue_ready = [&](int c) {
@@ -330,7 +331,7 @@ k_wave_sweep(WaveArgs g, const T *__restrict__ rec, const T *__restrict__ rhs, T
                                  G * 32 * BS * (int)sizeof(T), &hd->bar[sl]);
                     }
                     ++qb;
-                    qstep = qb < R ? 0 : qb < nch ? (qb - R + 1) * G : 0x7fffffff;
+                    qstep = rs_wave_chunk_step(qb, nch, R, G);
                 }
             };
             // The unit's hand-off positions: p < a on the z face (the

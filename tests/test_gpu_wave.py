@@ -72,6 +72,40 @@ def test_wave_units_ragged(rs, ctx, orc, shape, prec):
         assert rel(z.numpy(), orc.ilu0_solve(Ao, lu, r, fp32=(prec == "mixed"))) <= (1e-12 if prec == "fp64" else 1e-5)
 
 
+def _launches(ctx, M, r, z):
+    n0 = ctx.launches()
+    M.apply(r, z)
+    return ctx.launches() - n0
+
+
+# units of 1 to 5 chunks of records (the ring has 4 slots): short lines on
+# grids too large for the sweeps in one block
+@pytest.mark.parametrize("shape,bs,prec", [
+    ((4, 70, 60), 1, "fp64"), ((12, 60, 50), 1, "fp64"), ((20, 90, 40), 1, "fp64"), ((30, 60, 50), 1, "fp64"),
+    ((5, 121, 67), 1, "mixed"), ((12, 60, 50), 1, "mixed"), ((30, 60, 50), 1, "mixed"), ((45, 60, 40), 1, "mixed"),
+    ((60, 50, 40), 1, "mixed"), ((2, 70, 60), 2, "fp64"), ((2, 70, 60), 2, "mixed"), ((4, 70, 60), 2, "mixed")])
+def test_wave_units_of_few_chunks(rs, ctx, orc, shape, bs, prec):
+    g, fp32 = synth.Grid(*shape), prec == "mixed"
+    if bs == 1:
+        d = synth.pressure_7pt(g, 33, kz_scale=0.1)
+        A, Ao = rs.Mat.csr(ctx, d), orc.Mat.csr(d)
+    else:
+        d = _blocks_of_size(synth.black_oil_bsr3(g, 33), bs)
+        A, Ao = rs.Mat.bsr(ctx, d), orc.Mat.bsr(d)
+    M = rs.Precond(ctx, A, "ilu0" if bs == 1 else "bilu0", prec=prec, sweep="wavefront")
+    r = np.random.default_rng(34).standard_normal(A.n)
+    if bs == 1:
+        ref = orc.ilu0_solve(Ao, orc.ilu0(Ao)[2], r, fp32=fp32)
+    else:
+        _, _, lu, dinv = orc.bilu0(Ao)
+        ref = orc.bilu0_solve(Ao, lu, dinv, r, fp32=fp32)
+    z = rs.Vec.zeros(ctx, A.n)
+    for _ in range(3):
+        assert _launches(ctx, M, rs.Vec(ctx, r), z) == 4       # in, L, U, out: not the sweeps in one block
+        assert rel(z.numpy(), ref) <= (1e-5 if fp32 else 1e-12)
+    assert ctx.check() == rs.OK
+
+
 # the sweeps in one block: wavefronts of one cell, of an odd number, of more
 # than 128 rows; lines, planes and boxes; an odd number of wavefronts; blocks
 @pytest.mark.parametrize("shape,bs", [((2, 1, 2), 1), ((2, 2, 1), 1), ((64, 2, 1), 1), ((1, 9, 31), 1), ((17, 13, 11), 1),
