@@ -18,3 +18,9 @@ RS_HD int rs_wave_chunk_step(int q, int nch, int nslots, int steps)
 {
     return q >= nch ? RS_NO_STEP : q < nslots ? 0 : (q - nslots + 1) * steps;
 }
+
+// Sweeps of a part of nrow rows: places are 16 bits, idle records hold 0xFFFF.
+// Once a copy has been given up on, RS_PART_LOST is in every place read, and the
+// record, which is then whatever its ring slot held before, is not used.
+#define RS_PART_LOST 0x10000
+RS_HD bool rs_part_place(int e, int nrow) { return e < nrow; }

@@ -30,6 +30,7 @@
 #include <algorithm>
 #include <vector>
 
+#include "rs_bounds.cuh"
 #include "rs_internal.cuh"
 
 namespace {
@@ -40,7 +41,8 @@ constexpr int PT_GROUP = 2;                         // chunks a slot
 constexpr int PT_IO = 512;                          // threads that move the vectors in and out
 constexpr int PT_MIN_SLOTS = 3, PT_MAX_SLOTS = 6;
 constexpr int PT_MAX_GROUPS = 2048;                 // of both sweeps of a part (their table is in shared memory)
-constexpr int PT_HDR = 128;                         // mbarriers
+constexpr int PT_HDR = 128;                         // mbarriers; at PT_LOST the mark of a copy given up on
+constexpr int PT_LOST = 64;
 constexpr size_t PT_SMEM = 220 * 1024;
 constexpr long long PT_DRAIN = 1LL << 30;           // cycles a late copy is still waited for
 constexpr unsigned short PT_IDLE = 0xFFFF;
@@ -84,13 +86,13 @@ struct PartRec {
     unsigned short c[PT_REG];
     const unsigned char *vals;                      // of this thread's row
     const unsigned char *cols;
-    __device__ __forceinline__ void load(const unsigned char *ch, int wm, int t, const T *y)
+    __device__ __forceinline__ void load(const unsigned char *ch, int wm, int t, const T *y, int nrow, const volatile int *lost)
     {
         w = wm & 0xFFFF;
         m = wm >> 16;
         e = PT_IDLE;
         if (t < w) {
-            e = ((const unsigned short *)ch)[t];
+            e = ((const unsigned short *)ch)[t] | *lost;
             vals = ch + 2 * w + t * sizeof(T);
             cols = ch + 2 * w + (m + (LOWER ? 0 : 1)) * w * sizeof(T) + 2 * t;
             const unsigned char *pv = vals, *pc = cols;
@@ -103,7 +105,7 @@ struct PartRec {
                     pc += 2 * w;
                 }
             // no other row writes y[e]: out of the step's chain
-            acc = y[e == PT_IDLE ? 0 : e];
+            acc = y[rs_part_place(e, nrow) ? e : nrow];
             if (!LOWER) acc = mad(*(const T *)(vals + m * w * sizeof(T)), acc, T(0));
         }
     }
@@ -117,7 +119,8 @@ struct PartRec {
         for (int k = 0; k < PT_REG; ++k)
             if (k < m) s = msub(s, v[k], x[k]);
         for (int k = PT_REG; k < m; ++k)
-            s = msub(s, *(const T *)(vals + k * w * sizeof(T)), y[*(const unsigned short *)(cols + 2 * k * w)]);
+            s = msub(s, *(const T *)(vals + k * w * sizeof(T)),
+                     y[*(const unsigned short *)(cols + 2 * k * w)]);
         y[e] = s;
     }
 };
@@ -132,14 +135,12 @@ k_part_solve(PartArgs g, const double *__restrict__ r, double *__restrict__ z)
     T *y = (T *)(pt_smem + PT_HDR + g.tbytes);
     unsigned char *ring = pt_smem + PT_HDR + g.tbytes + g.vbytes;
     const int tid = threadIdx.x;
+    volatile int *lost = (volatile int *)(pt_smem + PT_LOST);
     if (tid == 0) {
+        *lost = 0;
         for (int s = 0; s < g.nslots; ++s) mbar_init(&full[s], 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    // zeros everywhere: a copy that never arrives (a timeout) leads to no
-    // place outside the values
-    for (int k = tid; k < g.nslots * g.slot / 16; k += blockDim.x) ((uint4 *)ring)[k] = make_uint4(0, 0, 0, 0);
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     if (rs_pdl_wait()) return;
     if (g.skip && *(volatile const int *)g.skip) return;
     const PartInfo P = g.part[blockIdx.x];
@@ -177,6 +178,7 @@ k_part_solve(PartArgs g, const double *__restrict__ r, double *__restrict__ z)
                 }
                 if (dt > giveup) {
                     dead = true;
+                    *lost = RS_PART_LOST;
                     break;
                 }
             }
@@ -187,7 +189,8 @@ k_part_solve(PartArgs g, const double *__restrict__ r, double *__restrict__ z)
         }
         __syncthreads();
         // the barrier at the end of group j's first chunk: group j + 1 has
-        // arrived, and group j - 1 has been read
+        // arrived (or is marked lost, and no record of it is used), and group
+        // j - 1 has been read
         for (int j = 0; j < groups; ++j) {
             if (lane == 0 && j + 1 < groups) arrived();
             __syncwarp();
@@ -227,28 +230,28 @@ k_part_solve(PartArgs g, const double *__restrict__ r, double *__restrict__ z)
         PartRec<T, true> ql;
         PartRec<T, false> qu;
         PtGroup t = tab[0], tn;                      // this group and the next one
-        ql.load(slot, t.c0, tid, y);
+        ql.load(slot, t.c0, tid, y, P.nrow, lost);
         for (int j = 0; j < P.nl; ++j) {
             tn = tab[min(j + 1, groups - 1)];
-            if (ql.e != PT_IDLE) ql.solve(y);
-            ql.load(slot + pt_bytes<T, true>(t.c0), t.c1, tid, y);
+            if (rs_part_place(ql.e, P.nrow)) ql.solve(y);
+            ql.load(slot + pt_bytes<T, true>(t.c0), t.c1, tid, y, P.nrow, lost);
             barrier(true);
-            if (ql.e != PT_IDLE) ql.solve(y);
+            if (rs_part_place(ql.e, P.nrow)) ql.solve(y);
             advance();
             // U's first right-hand side may be a value of this step: after the barrier
-            if (j + 1 < P.nl) ql.load(slot, tn.c0, tid, y);
+            if (j + 1 < P.nl) ql.load(slot, tn.c0, tid, y, P.nrow, lost);
             t = tn;
             barrier(false);
         }
-        qu.load(slot, t.c0, tid, y);
+        qu.load(slot, t.c0, tid, y, P.nrow, lost);
         for (int j = 0; j < P.nu; ++j) {
             tn = tab[min(P.nl + j + 1, groups - 1)];
-            if (qu.e != PT_IDLE) qu.solve(y);
-            qu.load(slot + pt_bytes<T, false>(t.c0), t.c1, tid, y);
+            if (rs_part_place(qu.e, P.nrow)) qu.solve(y);
+            qu.load(slot + pt_bytes<T, false>(t.c0), t.c1, tid, y, P.nrow, lost);
             barrier(true);
-            if (qu.e != PT_IDLE) qu.solve(y);
+            if (rs_part_place(qu.e, P.nrow)) qu.solve(y);
             advance();
-            if (j + 1 < P.nu) qu.load(slot, tn.c0, tid, y);
+            if (j + 1 < P.nu) qu.load(slot, tn.c0, tid, y, P.nrow, lost);
             t = tn;
             barrier(false);
         }

@@ -12,6 +12,8 @@ CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
 SRC = """
 #include "rs_bounds.cuh"
 extern "C" int wave_chunk_step(int q, int nch, int nslots, int steps) { return rs_wave_chunk_step(q, nch, nslots, steps); }
+extern "C" int part_place(int e, int nrow) { return rs_part_place(e, nrow); }
+extern "C" int part_lost() { return RS_PART_LOST; }
 """
 
 
@@ -42,3 +44,10 @@ def test_wave_producer_copies_every_chunk_of_a_unit_once_and_no_other(rules, nsl
             # the consumer's own chunk is on its way when it gets there
             assert len(issued) > c // steps, (nch, c)
         assert len(issued) == nch
+
+
+@pytest.mark.parametrize("nrow", [1, 2, 31, 1000, 65534])
+def test_part_sweep_takes_its_rows_and_none_that_is_lost(rules, nrow):
+    for e in range(0x10000):
+        assert bool(rules.part_place(e, nrow)) == (e < nrow)
+        assert not rules.part_place(e | rules.part_lost(), nrow)
