@@ -14,7 +14,7 @@
 //     plane and two planes, so a row reads its three neighbours at fixed
 //     distances and none is tested for;
 //   - the records (a row's place, its L or U entries) come in chunks of one
-//     size, a wavefront each, idle threads marked by place -1; a thread reads
+//     size for both sweeps, a wavefront each, idle threads marked by place -1; a thread reads
 //     its next one into registers before the barrier;
 //   - they stream through a ring of shared-memory slots, two or four
 //     wavefronts a slot and copy.  A producer warp waits for the copies and
@@ -53,11 +53,16 @@ struct LevelArgs {
     const int *skip;
 };
 
-// bytes of a chunk: a place per cell, then NB block rows of BS values per row
+// Bytes of a chunk: a place per cell, then the block rows of BS values per row,
+// 4 of U, 3 of L (the fourth is left out).  One size for both, so that a ring slot
+// has its places at the same offsets whatever it holds: a copy that has been
+// given up on, or lands later than that, leaves there the -1 of the start or places of
+// the grid, never a value's bits.  (A test of every place before its use took
+// 0.4 to 1 us of an apply's 13 to 42, in the steps' chain; L's larger copies take none.)
 template <int BS, typename T>
 __host__ __device__ __forceinline__ int lv_plane(int wc) { return wc * BS * (int)sizeof(T); }
-template <int BS, typename T, int NB>
-__host__ __device__ __forceinline__ int lv_chunk(int wc) { return 4 * wc + NB * BS * lv_plane<BS, T>(wc); }
+template <int BS, typename T>
+__host__ __device__ __forceinline__ int lv_chunk(int wc) { return 4 * wc + 4 * BS * lv_plane<BS, T>(wc); }
 // bytes of a value array on the padded grid; blocks keep y and z apart, since
 // a cell's rows all read its y
 template <int BS, typename T>
@@ -114,8 +119,7 @@ k_level_solve(LevelArgs g, const unsigned char *__restrict__ lbuf, const unsigne
     const int vbytes = lv_values<BS, T>(g.ncell);
     T *yv = (T *)(lv_smem + LV_HDR), *zv = BS > 1 ? (T *)(lv_smem + LV_HDR + vbytes) : yv;
     unsigned char *ring = lv_smem + LV_HDR + (BS > 1 ? 2 : 1) * vbytes;
-    const int lb = lv_chunk<BS, T, 3>(g.wc), ub = lv_chunk<BS, T, 4>(g.wc);
-    const int sb = g.group * ub;                    // bytes of a slot
+    const int cb = lv_chunk<BS, T>(g.wc), sb = g.group * cb;      // bytes of a chunk and of a slot
     // threads: nt compute, then helpers that only move r and z (up to nio in
     // all), then the producer warp
     const int nt = g.nt, nio = blockDim.x - 32, tid = threadIdx.x;
@@ -123,15 +127,11 @@ k_level_solve(LevelArgs g, const unsigned char *__restrict__ lbuf, const unsigne
         for (int s = 0; s < g.nslots; ++s) mbar_init(&full[s], 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    // the padding to 0, and every slot's places to -1: a chunk that never
-    // arrives (a timeout) leads to no place outside the grid
+    // the padding to 0, and the places of every slot's chunks to -1
     for (int k = tid; k < (BS > 1 ? 2 : 1) * vbytes / 16; k += blockDim.x) ((uint4 *)yv)[k] = make_uint4(0, 0, 0, 0);
     if (tid < g.wc)
         for (int sl = 0; sl < g.nslots; ++sl)
-            for (int w = 0; w < g.group; ++w) {     // the places of an L chunk, and of a U chunk
-                ((int *)(ring + sl * sb + w * lb))[tid] = -1;
-                ((int *)(ring + sl * sb + w * ub))[tid] = -1;
-            }
+            for (int w = 0; w < g.group; ++w) ((int *)(ring + sl * sb + w * cb))[tid] = -1;
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     if (rs_pdl_wait()) return;
     if (g.skip && *(volatile const int *)g.skip) return;
@@ -144,10 +144,9 @@ k_level_solve(LevelArgs g, const unsigned char *__restrict__ lbuf, const unsigne
         unsigned wph = 0;
         const unsigned char *src = lbuf;
         auto issue = [&]() {
-            const unsigned bytes = g.group * (ij < g.ngroup ? lb : ub);
-            mbar_arrive_expect_tx(&full[isl], bytes);
-            bulk_g2s(ring + isl * sb, src, bytes, &full[isl]);
-            src += bytes;
+            mbar_arrive_expect_tx(&full[isl], sb);
+            bulk_g2s(ring + isl * sb, src, sb, &full[isl]);
+            src += sb;
             if (++ij == g.ngroup) src = ubuf;
             if (++isl == g.nslots) isl = 0;
         };
@@ -235,7 +234,7 @@ k_level_solve(LevelArgs g, const unsigned char *__restrict__ lbuf, const unsigne
             const unsigned char *c = slot;
             for (int k = 1; k < g.group; ++k) {
                 if (ql.e >= 0) ql.solve(yv, zv, i, g.px, g.pxy);
-                c += lb;
+                c += cb;
                 if (in) ql.load(c, cell, tid, g.wc, ps);
                 barrier(k == 1);
             }
@@ -251,7 +250,7 @@ k_level_solve(LevelArgs g, const unsigned char *__restrict__ lbuf, const unsigne
             const unsigned char *c = slot;
             for (int k = 1; k < g.group; ++k) {
                 if (qu.e >= 0) qu.solve(yv, zv, i, g.px, g.pxy);
-                c += ub;
+                c += cb;
                 if (in) qu.load(c, cell, tid, g.wc, ps);
                 barrier(k == 1);
             }
@@ -292,8 +291,8 @@ __global__ void k_level_gather(LevelArgs g, int ny, const int2 *__restrict__ cel
     if (t >= g.n) return;
     const int i = cells[t].x, p = cells[t].y;
     const int h = i % g.nx + (i / g.nx) % ny + i / g.nxy;
-    unsigned char *lc = lbuf + (size_t)h * lv_chunk<BS, T, 3>(g.wc);
-    unsigned char *uc = ubuf + (size_t)(g.nlev - 1 - h) * lv_chunk<BS, T, 4>(g.wc);
+    unsigned char *lc = lbuf + (size_t)h * lv_chunk<BS, T>(g.wc);
+    unsigned char *uc = ubuf + (size_t)(g.nlev - 1 - h) * lv_chunk<BS, T>(g.wc);
     ((int *)lc)[p] = ((int *)uc)[p] = g.place[i];
     const int ps = lv_plane<BS, T>(g.wc);
     auto put = [&](unsigned char *c, int blk, int a, int b, double v) {
@@ -395,7 +394,7 @@ int lv_slots(int64_t ncell, int wc, int *group)
     const size_t fixed = LV_HDR + (BS > 1 ? 2 : 1) * (size_t)lv_values<BS, T>((int)ncell);
     if (fixed >= LV_SMEM) return 0;
     for (*group = 4; *group >= 2; *group /= 2) {
-        const size_t ns = (LV_SMEM - fixed) / (*group * lv_chunk<BS, T, 4>(wc));
+        const size_t ns = (LV_SMEM - fixed) / (*group * lv_chunk<BS, T>(wc));
         if (ns >= LV_MIN_SLOTS) return (int)std::min<size_t>(ns, LV_MAX_SLOTS);
     }
     return 0;
@@ -420,16 +419,16 @@ int level_create(IluFactor *f, const std::vector<int> &w)
                 cells[i] = make_int2(i, at[x + y + z]++);
             }
     const int64_t chunks = (int64_t)g.ngroup * g.group;    // the last group filled up with empty ones
-    const int64_t lw = chunks * lv_chunk<BS, T, 3>(W.one_wc) / 4, uw = chunks * lv_chunk<BS, T, 4>(W.one_wc) / 4;
+    const int64_t words = chunks * lv_chunk<BS, T>(W.one_wc) / 4;
     int st = rs_alloc(ctx, (void **)&W.one_place, sizeof(int) * n);
     st = st ? st : rs_alloc(ctx, (void **)&W.one_cells, sizeof(int2) * n);
-    st = st ? st : rs_alloc(ctx, &W.lrec, 4 * (size_t)lw);
-    st = st ? st : rs_alloc(ctx, &W.urec, 4 * (size_t)uw);
+    st = st ? st : rs_alloc(ctx, &W.lrec, 4 * (size_t)words);
+    st = st ? st : rs_alloc(ctx, &W.urec, 4 * (size_t)words);
     if (st) return st;
     RS_CUDA_TRY(cudaMemcpyAsync(W.one_place, place.data(), sizeof(int) * n, cudaMemcpyHostToDevice, ctx->stream));
     RS_CUDA_TRY(cudaMemcpyAsync(W.one_cells, cells.data(), sizeof(int2) * n, cudaMemcpyHostToDevice, ctx->stream));
-    k_level_clear<<<256, 256, 0, ctx->stream>>>(lw, lv_chunk<BS, T, 3>(W.one_wc) / 4, W.one_wc, (int *)W.lrec);
-    k_level_clear<<<256, 256, 0, ctx->stream>>>(uw, lv_chunk<BS, T, 4>(W.one_wc) / 4, W.one_wc, (int *)W.urec);
+    k_level_clear<<<256, 256, 0, ctx->stream>>>(words, lv_chunk<BS, T>(W.one_wc) / 4, W.one_wc, (int *)W.lrec);
+    k_level_clear<<<256, 256, 0, ctx->stream>>>(words, lv_chunk<BS, T>(W.one_wc) / 4, W.one_wc, (int *)W.urec);
     ctx->launches += 1;
     RS_TRY(rs_check_launch(ctx));
     RS_CUDA_TRY(cudaStreamSynchronize(ctx->stream));        // the host arrays end here
@@ -461,7 +460,7 @@ int level_apply(IluFactor *f, const double *r, double *z, const double *scale, c
     }
     const LevelArgs g = level_args(f, skip);
     const size_t smem = LV_HDR + (BS > 1 ? 2 : 1) * (size_t)lv_values<BS, T>(g.ncell) +
-                        (size_t)g.nslots * g.group * lv_chunk<BS, T, 4>(g.wc);
+                        (size_t)g.nslots * g.group * lv_chunk<BS, T>(g.wc);
     // L and U are one kernel: the profiler counts it as the L sweep
     RsProfScope prof(ctx, BS == 1 ? RS_PROF_LSWEEP : RS_PROF_BLSWEEP);
     rs_pdl(k_level_solve<BS, T>, 1, std::max(W.one_threads, LV_IO_THREADS) + 32, smem, ctx)(
