@@ -150,7 +150,8 @@ k_level_solve(LevelArgs g, const unsigned char *__restrict__ lbuf, const unsigne
             if (++ij == g.ngroup) src = ubuf;
             if (++isl == g.nslots) isl = 0;
         };
-        // bounded: records a timeout after the limit, gives up only much later
+        // bounded: a wait longer than the limit, however short the limit, is
+        // recorded as a timeout; given up only much later
         bool dead = false;
         auto arrived = [&]() {
             unsigned long long *b = &full[wsl];
@@ -159,15 +160,17 @@ k_level_solve(LevelArgs g, const unsigned char *__restrict__ lbuf, const unsigne
                 wsl = 0;
                 wph ^= 1;
             }
-            if (dead || mbar_try_wait(b, par)) return;
+            if (dead) return;
             const long long t0 = clock64(), giveup = 4 * g.limit + LV_DRAIN;
             bool late = false;
-            while (!mbar_try_wait(b, par)) {
+            for (;;) {
+                const bool in = mbar_try_wait(b, par);
                 const long long dt = clock64() - t0;
                 if (!late && dt > g.limit) {
                     late = true;
                     atomicOr(g.err, RS_DEVERR_TIMEOUT);
                 }
+                if (in) break;
                 if (dt > giveup) {
                     dead = true;
                     break;

@@ -159,7 +159,8 @@ k_part_solve(PartArgs g, const double *__restrict__ r, double *__restrict__ z)
             bulk_g2s(ring + isl * g.slot, g.buf + 16 * (size_t)t.off, 16u * t.size, &full[isl]);
             if (++isl == g.nslots) isl = 0;
         };
-        // bounded: records a timeout after the limit, gives up only much later
+        // bounded: a wait longer than the limit, however short the limit, is
+        // recorded as a timeout; given up only much later
         auto arrived = [&]() {
             unsigned long long *b = &full[wsl];
             const unsigned par = wph;
@@ -167,15 +168,17 @@ k_part_solve(PartArgs g, const double *__restrict__ r, double *__restrict__ z)
                 wsl = 0;
                 wph ^= 1;
             }
-            if (dead || mbar_try_wait(b, par)) return;
+            if (dead) return;
             const long long t0 = clock64(), giveup = 4 * g.limit + PT_DRAIN;
             bool late = false;
-            while (!mbar_try_wait(b, par)) {
+            for (;;) {
+                const bool in = mbar_try_wait(b, par);
                 const long long dt = clock64() - t0;
                 if (!late && dt > g.limit) {
                     late = true;
                     atomicOr(g.err, RS_DEVERR_TIMEOUT);
                 }
+                if (in) break;
                 if (dt > giveup) {
                     dead = true;
                     *lost = RS_PART_LOST;

@@ -178,6 +178,30 @@ def test_ras_subdomains_in_one_block(rs, ctx, orc, shape, parts, overlap, level,
     assert rel(same.numpy(), want) <= tol
 
 
+@pytest.mark.parametrize("prec", ["fp64", "mixed"])
+def test_ras_subdomains_in_one_block_report_every_wait_over_the_limit(rs, ctx, prec):
+    """A limit of one cycle has run out when the first copy arrives, however
+    early that is: the apply in one launch reports it, and is right."""
+    g = synth.Grid(16, 14, 12)
+    A = rs.Mat.csr(ctx, synth.pressure_7pt(g, 58))
+    M = rs.Precond(ctx, A, "ras", prec=prec, nparts=8, part=rs.box_partition((16, 14, 12), (2, 2, 2)), overlap=1, level=1)
+    r = rs.Vec(ctx, np.random.default_rng(59).standard_normal(g.n))
+    z = rs.Vec.zeros(ctx, g.n)
+    n0 = ctx.launches()
+    M.apply(r, z)
+    assert ctx.launches() - n0 == 1 and ctx.check() == rs.OK
+    want = z.numpy()
+    ctx.set_spin_limit(1)
+    try:
+        M.apply(r, z)
+        assert ctx.check() == rs.ERR_DEVICE_TIMEOUT
+    finally:
+        ctx.set_spin_limit(0)
+    assert np.array_equal(z.numpy(), want)
+    M.apply(r, z)
+    assert ctx.check() == rs.OK and np.array_equal(z.numpy(), want)
+
+
 def test_ras_sweep_levels_shrink_with_subdomains(rs, ctx):
     g = synth.Grid(64, 64, 32)
     d = synth.pressure_7pt(g, 55)

@@ -165,6 +165,29 @@ def test_sweeps_in_one_block_report_a_timeout(rs, ctx, orc):
     assert ctx.check() == rs.OK
 
 
+@pytest.mark.parametrize("bs,prec", [(1, "fp64"), (1, "mixed"), (3, "mixed")])
+def test_sweeps_in_one_block_report_every_wait_over_the_limit(rs, ctx, orc, bs, prec):
+    """A limit of one cycle has run out when the first copy arrives, however
+    early that is: the apply in one launch reports it, and is right."""
+    g = synth.Grid(16, 12, 9)
+    d = synth.pressure_7pt(g, 37) if bs == 1 else synth.black_oil_bsr3(g, 37)
+    A, Ao = (rs.Mat.csr(ctx, d), orc.Mat.csr(d)) if bs == 1 else (rs.Mat.bsr(ctx, d), orc.Mat.bsr(d))
+    M = rs.Precond(ctx, A, "ilu0" if bs == 1 else "bilu0", prec=prec)
+    r = np.random.default_rng(38).standard_normal(A.n)
+    z = rs.Vec.zeros(ctx, A.n)
+    assert _launches(ctx, M, rs.Vec(ctx, r), z) == 1 and ctx.check() == rs.OK
+    want = z.numpy()
+    ctx.set_spin_limit(1)
+    try:
+        M.apply(rs.Vec(ctx, r), z)
+        assert ctx.check() == rs.ERR_DEVICE_TIMEOUT
+    finally:
+        ctx.set_spin_limit(0)
+    assert np.array_equal(z.numpy(), want)
+    M.apply(rs.Vec(ctx, r), z)
+    assert ctx.check() == rs.OK and np.array_equal(z.numpy(), want)
+
+
 def test_wave_is_bit_stable_across_applies_and_scales(rs, ctx, orc):
     """The schedule is dynamic (tickets), the arithmetic is not: repeated
     applies give identical bits; a device scale multiplies r on entry."""
