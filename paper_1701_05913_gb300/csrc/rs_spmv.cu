@@ -5,10 +5,10 @@
 // FP64 multiply-adds are scarce on this GPU (about two per clock and SM, 600 G
 // per second in all): a 7-point matrix takes as long for them as for its
 // bytes, one of 3 x 3 blocks longer, and every idle or padded lane costs as
-// much as a working one.  Both layouts therefore give each thread one (block)
-// row, whose sum runs in column order (the order of the row-per-thread CSR
-// kernel and of the BSR kernel, so the results are the same bit for bit), and
-// issue a row's loads together.
+// much as a working one.  Both layouts therefore give each thread a row (or a
+// whole block row), whose sum runs in column order (the order of the
+// row-per-thread CSR kernel and of the BSR kernel, so the results are the same
+// bit for bit), and issue a row's loads together.
 //
 // Stencil layout (DIA): the distinct offsets col - row are few (at most 8, a
 // structured grid), so a value's column follows from its place (a plane per
@@ -22,6 +22,7 @@
 // rows side by side.  The rows of a window are sorted by length first, so
 // the lanes of a slice finish together.
 #include <algorithm>
+#include <type_traits>
 #include <vector>
 
 #include "rs_internal.cuh"
@@ -64,13 +65,14 @@ __device__ __forceinline__ void spmv_store(int64_t i, double acc, const double *
     else y[i] = fma(alpha, acc, beta == 1.0 ? y[i] : __dmul_rn(beta, y[i]));
 }
 
-// A thread per (block) row.  All loads are independent of one another and of
-// the mask (x's index is clamped, not predicated), so a warp keeps many of
-// its row's loads in flight.  Per product, against the CSR and BSR kernels:
-// 7-point, 1,048,576 rows 33.9 -> 19 us (76 MB moved; bytes and multiply-adds
-// take 11 and 12 us); 3 x 3 blocks, 500,000 rows 69 -> 60 us (52 us of
-// multiply-adds).
-template <int ND, int BS>
+// A thread per RB scalar rows of a block row: all BS, or one (threadIdx.y says
+// which; the block row is blockIdx.x blockDim.x + threadIdx.x).  All loads are
+// independent of one another and of the mask (x's index is clamped, not
+// predicated), so a warp keeps many of its row's loads in flight.  Per product,
+// against the CSR and BSR kernels: 7-point, 1,048,576 rows 33.9 -> 19 us (76 MB
+// moved; bytes and multiply-adds take 11 and 12 us); 3 x 3 blocks, 500,000 block
+// rows 69.7 -> 62.1 us (52 us of multiply-adds), 27,000 8.3 -> 4.9, 8,000 6.2 -> 3.0.
+template <int ND, int BS, int RB>
 __global__ void __launch_bounds__(256)
 k_spmv_dia(DiaArgs a, const double *__restrict__ x, double alpha, double beta, const double *__restrict__ bvec,
            double *__restrict__ y, const int *skip, const double *__restrict__ dinv)
@@ -79,10 +81,11 @@ k_spmv_dia(DiaArgs a, const double *__restrict__ x, double alpha, double beta, c
     if (skip && *(volatile const int *)skip) return;
     const int64_t I = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (I >= a.n) return;
+    const int r0 = RB == BS ? 0 : threadIdx.y;
     const unsigned m = a.mask[I];
-    double acc[BS];
+    double acc[RB];
 #pragma unroll
-    for (int r = 0; r < BS; ++r) acc[r] = 0.0;
+    for (int r = 0; r < RB; ++r) acc[r] = 0.0;
     auto at = [&](int k) { return min(max(I + a.off[k], (int64_t)0), (int64_t)a.n - 1); };
     if constexpr (BS == 1) {
         // the whole row's loads, then its multiply-adds (24.5 -> 22.8 us a call)
@@ -99,24 +102,26 @@ k_spmv_dia(DiaArgs a, const double *__restrict__ x, double alpha, double beta, c
 #pragma unroll
         for (int k = 0; k < ND; ++k) {
             const int64_t J = at(k);
-            double v[BS * BS], xv[BS];
+            double v[RB * BS], xv[BS];
 #pragma unroll
             for (int c = 0; c < BS; ++c) xv[c] = __ldg(x + J * BS + c);
 #pragma unroll
-            for (int e = 0; e < BS * BS; ++e) v[e] = __ldg(a.val + (int64_t)(k * BS * BS + e) * a.ld + I);
+            for (int e = 0; e < RB * BS; ++e) v[e] = __ldg(a.val + (int64_t)(k * BS * BS + r0 * BS + e) * a.ld + I);
             if (m >> k & 1) {
 #pragma unroll
-                for (int r = 0; r < BS; ++r)
+                for (int r = 0; r < RB; ++r)
 #pragma unroll
                     for (int c = 0; c < BS; ++c) acc[r] = fma(v[r * BS + c], xv[c], acc[r]);
             }
         }
     }
 #pragma unroll
-    for (int r = 0; r < BS; ++r) spmv_store(I * BS + r, acc[r], x, alpha, beta, bvec, y, dinv);
+    for (int r = 0; r < RB; ++r) spmv_store(I * BS + r0 + r, acc[r], x, alpha, beta, bvec, y, dinv);
 }
 
-// t = f - A (Pi_p p): only block column 0 meets the prolonged pressure vector
+// t = f - A (Pi_p p): only block column 0 meets the prolonged pressure vector.
+// A thread per scalar row: against one per block row 8,000 3 x 3 block rows take
+// 2.9 instead of 4.4 us, 100,000 5.9 instead of 6.0, 210,000 12.4 instead of 13.3.
 template <int ND, int BS>
 __global__ void __launch_bounds__(256)
 k_presid_dia(DiaArgs a, const double *__restrict__ p, const double *__restrict__ f, double *__restrict__ t,
@@ -126,23 +131,16 @@ k_presid_dia(DiaArgs a, const double *__restrict__ p, const double *__restrict__
     if (skip && *(volatile const int *)skip) return;
     const int64_t I = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (I >= a.n) return;
+    const int r = threadIdx.y;
     const unsigned m = a.mask[I];
-    double acc[BS];
-#pragma unroll
-    for (int r = 0; r < BS; ++r) acc[r] = 0.0;
+    double acc = 0.0;
 #pragma unroll
     for (int k = 0; k < ND; ++k) {
         const double pv = __ldg(p + min(max(I + a.off[k], (int64_t)0), (int64_t)a.n - 1));
-        double v[BS];
-#pragma unroll
-        for (int r = 0; r < BS; ++r) v[r] = __ldg(a.val + (int64_t)(k * BS * BS + r * BS) * a.ld + I);
-        if (m >> k & 1) {
-#pragma unroll
-            for (int r = 0; r < BS; ++r) acc[r] = fma(v[r], pv, acc[r]);
-        }
+        const double v = __ldg(a.val + (int64_t)(k * BS * BS + r * BS) * a.ld + I);
+        if (m >> k & 1) acc = fma(v, pv, acc);
     }
-#pragma unroll
-    for (int r = 0; r < BS; ++r) t[I * BS + r] = __dsub_rn(f[I * BS + r], acc[r]);
+    t[I * BS + r] = __dsub_rn(f[I * BS + r], acc);
 }
 
 // a warp per slice, a row per lane; U entries' loads at a time
@@ -395,53 +393,57 @@ int sell_build(rs_mat *A)
     return st;
 }
 
-template <int BS>
-int dia_launch(const rs_mat *A, const double *x, double alpha, double beta, const double *bvec, double *y,
-               const int *skip, const double *dinv)
+// Block rows from which a thread takes a whole one: it loads x once, but its
+// chain of multiply-adds is BS times as long and its registers leave about
+// 156,000 rows resident at once.  Below, thread blocks of 32 block rows, a warp
+// per row of the block.  Thread per scalar row / per block row, us: 3 x 3 blocks
+// 8,000 rows 3.0 / 6.1, 100,000 14.0 / 14.7, 180,000 25.2 / 39.5, 245,000 33.9 /
+// 39.0, 294,000 39.6 / 39.3, 500,000 64.8 / 62.1; 2 x 2 blocks 27,000 3.4 / 4.4,
+// 210,000 14.1 / 18.2, 280,000 18.3 / 18.5, 500,000 32.2 / 30.5.
+constexpr int DIA_BLOCK_ROWS = 280000;
+
+// launch(ND) with A's number of offsets as a constant
+template <typename F>
+int dia_dispatch(const rs_mat *A, F launch)
 {
-    const int grid = (int)(((int64_t)A->nrows + 255) / 256);
-    const DiaArgs a = dia_args(A);
     switch (A->dia.nd) {
-#define RS_DIA_CASE(ND)                                                                                          \
-    case ND:                                                                                                     \
-        rs_pdl(k_spmv_dia<ND, BS>, grid, 256, 0, A->ctx)(a, x, alpha, beta, bvec, y, skip, dinv);             \
-        break;
-        RS_DIA_CASE(1)
-        RS_DIA_CASE(2)
-        RS_DIA_CASE(3)
-        RS_DIA_CASE(4)
-        RS_DIA_CASE(5)
-        RS_DIA_CASE(6)
-        RS_DIA_CASE(7)
-        RS_DIA_CASE(8)
-#undef RS_DIA_CASE
+    case 1: launch(std::integral_constant<int, 1>()); break;
+    case 2: launch(std::integral_constant<int, 2>()); break;
+    case 3: launch(std::integral_constant<int, 3>()); break;
+    case 4: launch(std::integral_constant<int, 4>()); break;
+    case 5: launch(std::integral_constant<int, 5>()); break;
+    case 6: launch(std::integral_constant<int, 6>()); break;
+    case 7: launch(std::integral_constant<int, 7>()); break;
+    case 8: launch(std::integral_constant<int, 8>()); break;
     default: return RS_ERR_INVALID_ARG;
     }
     return rs_check_launch(A->ctx);
 }
 
+int dia_grid(const rs_mat *A, int rows) { return (int)(((int64_t)A->nrows + rows - 1) / rows); }
+
+template <int BS>
+int dia_launch(const rs_mat *A, const double *x, double alpha, double beta, const double *bvec, double *y,
+               const int *skip, const double *dinv)
+{
+    return dia_dispatch(A, [&](auto nd) {
+        constexpr int ND = decltype(nd)::value;
+        if (BS == 1 || A->nrows >= DIA_BLOCK_ROWS)
+            rs_pdl(k_spmv_dia<ND, BS, BS>, dia_grid(A, 256), 256, 0, A->ctx)(dia_args(A), x, alpha, beta, bvec, y, skip,
+                                                                            dinv);
+        else
+            rs_pdl(k_spmv_dia<ND, BS, 1>, dia_grid(A, 32), dim3(32, BS), 0, A->ctx)(dia_args(A), x, alpha, beta, bvec,
+                                                                                   y, skip, dinv);
+    });
+}
+
 template <int BS>
 int presid_launch(const rs_mat *A, const double *p, const double *f, double *t, const int *skip)
 {
-    const int grid = (int)(((int64_t)A->nrows + 255) / 256);
-    const DiaArgs a = dia_args(A);
-    switch (A->dia.nd) {
-#define RS_DIA_CASE(ND)                                                               \
-    case ND:                                                                          \
-        rs_pdl(k_presid_dia<ND, BS>, grid, 256, 0, A->ctx)(a, p, f, t, skip);      \
-        break;
-        RS_DIA_CASE(1)
-        RS_DIA_CASE(2)
-        RS_DIA_CASE(3)
-        RS_DIA_CASE(4)
-        RS_DIA_CASE(5)
-        RS_DIA_CASE(6)
-        RS_DIA_CASE(7)
-        RS_DIA_CASE(8)
-#undef RS_DIA_CASE
-    default: return RS_ERR_INVALID_ARG;
-    }
-    return rs_check_launch(A->ctx);
+    return dia_dispatch(A, [&](auto nd) {
+        rs_pdl(k_presid_dia<decltype(nd)::value, BS>, dia_grid(A, 32), dim3(32, BS), 0, A->ctx)(dia_args(A), p, f, t,
+                                                                                              skip);
+    });
 }
 
 }  // namespace

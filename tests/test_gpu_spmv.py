@@ -70,6 +70,31 @@ def test_stencil_layout(rs, ctx, orc, bs, n, offs, keep):
     _check(rs, ctx, orc, _offsets_matrix(n, offs, keep, bs, rng), rng, shift=n % 2 == 1)
 
 
+# block rows on both sides of 280,000, from which a thread takes a whole block
+# row; sizes off the thread blocks of 32 and 256; odd offsets; 7 and 3 of them
+@pytest.mark.parametrize("bs", [2, 3])
+@pytest.mark.parametrize("n,offs", [(31, [-5, -1, 0, 1, 5]), (279999, [-700, -31, -1, 0, 1, 31, 700]),
+                                    (280001, [-700, -31, -1, 0, 1, 31, 700]), (300015, [-1, 0, 64])])
+def test_stencil_products_of_small_and_large_block_systems(rs, ctx, bs, n, offs):
+    rng = np.random.default_rng(n + bs)
+    i = np.arange(n)
+    on = np.stack([(i + o >= 0) & (i + o < n) for o in offs], axis=1) & (rng.random((n, len(offs))) < 0.9)
+    on[:, offs.index(0)] = True
+    ptr = np.concatenate([[0], np.cumsum(on.sum(1))]).astype(np.int32)
+    row, k = np.nonzero(on)
+    col = row + np.array(offs)[k]
+    val = rng.integers(-5, 6, size=(row.size, bs, bs)).astype(float)
+    A = rs.Mat.bsr(ctx, dict(nb=n, bs=bs, browptr=ptr, bcol=col.astype(np.int32), bval=val.reshape(-1)))
+    x, y0 = (rng.integers(-9, 10, size=n * bs).astype(float) for _ in range(2))
+    ref = np.zeros((n, bs))
+    np.add.at(ref, row, np.einsum("eij,ej->ei", val, x.reshape(n, bs)[col]))
+    xv, y = rs.Vec(ctx, x), rs.Vec(ctx, y0)
+    A.amxpby(-1.0, xv, 1.0, y)
+    assert np.array_equal(y.numpy(), y0 - ref.reshape(-1))
+    A.spmv(xv, y)
+    assert np.array_equal(y.numpy(), ref.reshape(-1))
+
+
 def test_stencil_layout_rejects_a_late_offset(rs, ctx, orc):
     """One entry off the sampled rows' offsets: the matrix keeps CSR."""
     rng = np.random.default_rng(7)
