@@ -438,12 +438,15 @@ int rs_collect_device_error(rs_ctx *ctx, int *bad_row);
 // that other kernels touch: it returns when the kernel before has completed
 // and its writes are visible.  The dependents are released after the wait, so
 // a kernel that runs early knows that all kernels but the last one are done.
+// Blocks that start early are placed beside the ones that are still there, so
+// they are spread unevenly; plain = true launches without, where that costs more.
 template <class... P>
 struct RsPdl {
     void (*kernel)(P...);
     dim3 grid, block;
     size_t smem;
     const rs_ctx *ctx;
+    bool plain;
     template <class... A>
     void operator()(A &&...a) const
     {
@@ -456,14 +459,14 @@ struct RsPdl {
         cfg.dynamicSmemBytes = smem;
         cfg.stream = ctx->stream;
         cfg.attrs = &at;
-        cfg.numAttrs = ctx->capturing ? 0 : 1;
+        cfg.numAttrs = plain || ctx->capturing ? 0 : 1;
         cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(a)...);   // an error is read by rs_check_launch
     }
 };
 template <class... P>
-RsPdl<P...> rs_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, const rs_ctx *ctx)
+RsPdl<P...> rs_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, const rs_ctx *ctx, bool plain = false)
 {
-    return {kernel, grid, block, smem, ctx};
+    return {kernel, grid, block, smem, ctx, plain};
 }
 // Never true: `if (rs_pdl_wait()) return;` makes everything after it depend on
 // a value the compiler does not know, so that no load through a const

@@ -331,6 +331,26 @@ def test_wave_block_ilu0_other_block_sizes(rs, ctx, orc, bs):
         assert rel(z.numpy(), ref) <= (1e-12 if prec == "fp64" else 1e-5)
 
 
+@pytest.mark.parametrize("bs", [2, 3, 4])
+@pytest.mark.parametrize("shape", [(40, 36, 30), (8, 64, 64), (5, 100, 100)])
+def test_wave_block_units(rs, ctx, orc, shape, bs):
+    """Block systems beyond the sweeps in one block, with 40, 128 and 325 units:
+    fewer than SMs, about as many, more than twice as many."""
+    m = synth.black_oil_bsr3(synth.Grid(*shape), 18)
+    m = m if bs == 3 else _blocks_of_size(m, bs)
+    A, Ao = rs.Mat.bsr(ctx, m), orc.Mat.bsr(m)
+    _, _, lu_ref, dinv_ref = orc.bilu0(Ao)
+    r = np.random.default_rng(19).standard_normal(A.n)
+    for prec in ("fp64", "mixed"):
+        M = rs.Precond(ctx, A, "bilu0", prec=prec, sweep="wavefront")
+        ref = orc.bilu0_solve(Ao, lu_ref, dinv_ref, r, fp32=(prec == "mixed"))
+        z = rs.Vec.zeros(ctx, A.n)
+        for _ in range(2):
+            assert _launches(ctx, M, rs.Vec(ctx, r), z) == 4
+            assert rel(z.numpy(), ref) <= (1e-12 if prec == "fp64" else 1e-5)
+    assert ctx.check() == rs.OK
+
+
 @pytest.mark.parametrize("prec", ["fp64", "mixed"])
 def test_wave_cpr_apply_and_fgmres(rs, ctx, orc, prec):
     """CPR on the block system: both of its ILU factors (the decoupled
