@@ -432,17 +432,27 @@ static int part_create(rs_ctx *ctx, const std::vector<int> &sbase, const std::ve
     const size_t fixed = PT_HDR + (size_t)tbytes + vbytes;
     if (groups > PT_MAX_GROUPS || fixed + (size_t)PT_MIN_SLOTS * slot > PT_SMEM) return RS_OK;
     // a second block per SM when there are more parts than SMs
-    int nslots = (int)std::min<size_t>((PT_SMEM - fixed) / slot, PT_MAX_SLOTS), per_sm = 1;
+    int nslots = (int)std::min<size_t>((PT_SMEM - fixed) / slot, PT_MAX_SLOTS);
     const size_t half = PT_SMEM / 2 - 1024;
-    if ((int)S.part.size() > ctx->num_sms && half >= fixed + (size_t)PT_MIN_SLOTS * slot) {
-        per_sm = 2;
+    if ((int)S.part.size() > ctx->num_sms && half >= fixed + (size_t)PT_MIN_SLOTS * slot)
         nslots = (int)std::min<size_t>((half - fixed) / slot, PT_MAX_SLOTS);
-    }
-    // The rule: a step of a block is about 0.6 us (FP32 0.4), a round of blocks
-    // 10 us besides; a segment level 1.6 us (FP32 1.0).
+    // The rule: both times in us, fitted to 52 applies of 1,920 to 524,288 rows in 1 to
+    // 450 boxes, ILU(0) to ILU(2) (within 10 % of nearly all).  Here a step costs
+    // its FP64 or FP32 chain of m entries, and blocks on one SM take turns.  A segment
+    // level costs the chain of a segment's rows or the hand-off between short
+    // segments (`line` rows each).  One block / segments, us: 24 x 20 x 17 in 1 x 2 x 2 boxes,
+    // ILU(1) 105 / 86 FP64, 47 / 52 FP32; in 2 x 2 x 2 87 / 92 and 39 / 59; 40 x 36 x 30 in
+    // 6 x 6 x 6 103 / 75 and 48 / 50; 100 x 90 x 50 in 90 159 / 245 and 71 / 185, in 450
+    // 271 / 254 and 119 / 196; one box of 24^3, ILU(0) 219 / 107 and 96 / 74.
     const bool dbl = sizeof(T) == 8;
-    const int waves = ((int)S.part.size() + per_sm * ctx->num_sms - 1) / (per_sm * ctx->num_sms);
-    const double mine = waves * (10.0 + PT_GROUP * groups * (dbl ? 0.6 : 0.4)), theirs = 8.0 + seg_levels * (dbl ? 1.6 : 1.0);
+    const int rounds = ((int)S.part.size() + ctx->num_sms - 1) / ctx->num_sms, steps = PT_GROUP * groups;
+    int64_t ent = 0;
+    for (const PtChunk &c : S.chunk) ent += c.wm >> 16;
+    const double m = (double)ent / S.chunk.size(), line = 2.0 * n / (f->SL.nseg + f->SU.nseg);
+    const double mine = rounds * (dbl ? 9.5 + 0.0046 * most + steps * (0.372 + 0.038 * m)
+                                      : 8.1 + 0.0032 * most + steps * (0.064 + 0.027 * m));
+    const double level = dbl ? std::max(0.2 + 0.21 * m, 1.5 - 0.02 * line) : std::max(0.3 + 0.085 * m, 0.95 - 0.01 * line);
+    const double theirs = 8.0 + seg_levels * level + n * (dbl ? 0.21e-3 : 0.15e-3);
     if (mine > theirs) return RS_OK;
     PartSweep *R = new PartSweep();
     R->ctx = ctx;

@@ -178,6 +178,28 @@ def test_ras_subdomains_in_one_block(rs, ctx, orc, shape, parts, overlap, level,
     assert rel(same.numpy(), want) <= tol
 
 
+# which sweeps the rule takes: a block per subdomain is one launch (levels of
+# more than 128 rows, rows of more than 8 entries per triangle, more subdomains
+# than SMs), the segment sweeps are four with the gather and the scatter
+@pytest.mark.parametrize("shape,parts,overlap,level,prec,launches", [
+    ((24, 20, 17), (2, 1, 1), 1, 1, "fp64", 1), ((24, 20, 17), (2, 2, 2), 1, 2, "fp64", 1),
+    ((24, 20, 17), (2, 2, 2), 1, 2, "mixed", 1), ((40, 36, 30), (3, 3, 3), 1, 0, "fp64", 1),
+    ((40, 36, 30), (6, 6, 6), 1, 1, "mixed", 1), ((40, 36, 30), (6, 6, 6), 1, 1, "fp64", 4),
+    ((24, 20, 17), (1, 2, 2), 1, 1, "fp64", 4), ((24, 24, 24), (1, 1, 1), 0, 0, "mixed", 4)])
+def test_ras_rule_for_the_sweeps(rs, ctx, orc, shape, parts, overlap, level, prec, launches):
+    g = synth.Grid(*shape)
+    d = synth.pressure_7pt(g, 58, kz_scale=0.1)
+    part, nparts = rs.box_partition(shape, parts), int(np.prod(parts))
+    M = rs.Precond(ctx, rs.Mat.csr(ctx, d), "ras", prec=prec, nparts=nparts, part=part, overlap=overlap, level=level)
+    r = np.random.default_rng(59).standard_normal(g.n)
+    z = rs.Vec.zeros(ctx, g.n)
+    n0 = ctx.launches()
+    M.apply(rs.Vec(ctx, r), z)
+    assert ctx.launches() - n0 == launches
+    want = orc.Ras(orc.Mat.csr(d), nparts, part=part, overlap=overlap, level=level).apply(r)
+    assert rel(z.numpy(), want) <= (1e-12 if prec == "fp64" else 1e-5)
+
+
 @pytest.mark.parametrize("prec", ["fp64", "mixed"])
 def test_ras_subdomains_in_one_block_report_every_wait_over_the_limit(rs, ctx, prec):
     """A limit of one cycle has run out when the first copy arrives, however
