@@ -121,7 +121,7 @@ struct rs_mat {
         int off[8];
         int64_t ld = 0;          // (block) rows, rounded up to 32
         double *val = nullptr;   // [nd][bs][bs][ld]: entry (r, c) of each row's block at offset k
-        unsigned char *mask = nullptr;   // [nrows] bit k: the row has an entry at offset k
+        unsigned char *mask = nullptr;   // [nrows] bit k: the row has an entry at offset k (part of val's allocation)
     } dia;
     struct {
         int nslice = 0;          // 0: no such layout

@@ -190,32 +190,31 @@ k_spmv_sell(int nslice, const int2 *__restrict__ rows, const int *__restrict__ s
 // ---------------------------------------------------------------------------
 // building the layouts
 // ---------------------------------------------------------------------------
-// values and masks; *bad |= 1 when an entry's offset is not among off[0..nd)
+// Every place of the layout (0 where a row has no entry) and the masks; *bad |= 1
+// when an entry's offset is not among off[0..nd).  A thread per scalar row,
+// threadIdx.y the row of the block; columns and offsets both ascend.
 template <int BS>
-__global__ void k_dia_fill(DiaArgs a, int nd, const int *__restrict__ ptr, const int *__restrict__ col,
-                           const double *__restrict__ src, double *__restrict__ val, unsigned char *__restrict__ mask,
-                           int *bad)
+__global__ void __launch_bounds__(256)
+k_dia_fill(DiaArgs a, int nd, const int *__restrict__ ptr, const int *__restrict__ col, const double *__restrict__ src,
+           double *__restrict__ val, unsigned char *__restrict__ mask, int *bad)
 {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (int64_t)a.n * BS) return;
-    const int I = (int)(i / BS), r = (int)(i - (int64_t)I * BS);
+    const int64_t I = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (I >= a.n) return;
+    const int r = threadIdx.y, p1 = ptr[I + 1];
+    int p = ptr[I];
     unsigned m = 0;
-    bool ok = true;
-    for (int p = ptr[I]; p < ptr[I + 1]; ++p) {
-        const int d = col[p] - I;
-        int k = 0;
-        while (k < nd && a.off[k] != d) ++k;
-        if (k == nd) {
-            ok = false;
-            continue;
-        }
-        m |= 1u << k;
+    for (int k = 0; k < nd; ++k) {
+        const bool in = p < p1 && col[p] - I == a.off[k];
 #pragma unroll
         for (int c = 0; c < BS; ++c)
-            val[(int64_t)(k * BS * BS + r * BS + c) * a.ld + I] = src[(int64_t)p * BS * BS + r * BS + c];
+            val[(int64_t)(k * BS * BS + r * BS + c) * a.ld + I] = in ? src[((int64_t)p * BS + r) * BS + c] : 0.0;
+        m |= (unsigned)in << k;
+        p += in;
     }
-    if (!ok) atomicOr(bad, 1);
-    if (r == 0) mask[I] = (unsigned char)m;
+    if (r == 0) {
+        mask[I] = (unsigned char)m;
+        if (p < p1) atomicOr(bad, 1);
+    }
 }
 
 constexpr int SELL_WIN = 512;       // rows sorted by length together
@@ -303,6 +302,8 @@ k_sell_fill(int nslice, const int2 *__restrict__ rows, const int *__restrict__ s
     }
 }
 
+int dia_grid(const rs_mat *A, int rows) { return (int)(((int64_t)A->nrows + rows - 1) / rows); }
+
 // The offsets of a few sample rows (on the host: a caller's pattern), the
 // candidates of a stencil layout, or those of a matrix of the same pattern;
 // 0 when there are too many or the layout would be too empty.
@@ -334,28 +335,25 @@ int dia_build(rs_mat *A, int nd, const int (&off)[DIA_MAX])
 {
     rs_ctx *ctx = A->ctx;
     const int64_t ld = ((int64_t)A->nrows + 31) / 32 * 32;
-    const size_t bytes = sizeof(double) * nd * BS * BS * (size_t)ld;
-    int *bad = nullptr;
-    int st = rs_alloc(ctx, (void **)&A->dia.val, bytes);
-    st = st ? st : rs_alloc(ctx, (void **)&A->dia.mask, A->nrows);
-    st = st ? st : rs_alloc(ctx, (void **)&bad, sizeof(int));
-    int hbad = 1;
-    if (!st && (cudaMemsetAsync(A->dia.val, 0, bytes, ctx->stream) != cudaSuccess ||
-                cudaMemsetAsync(bad, 0, sizeof(int), ctx->stream) != cudaSuccess))
-        st = RS_ERR_CUDA;
+    const size_t places = (size_t)nd * BS * BS * ld;
+    int *hbad = (int *)(ctx->h_pinned + 40);
+    // one allocation: values, masks, the flag
+    RS_TRY(rs_alloc(ctx, (void **)&A->dia.val, sizeof(double) * places + ld + sizeof(int)));
+    A->dia.mask = (unsigned char *)(A->dia.val + places);
+    int *bad = (int *)(A->dia.mask + ld);
+    A->dia.ld = ld;
+    std::copy(off, off + nd, A->dia.off);
+    A->dia.nd = nd;
+    int st = cudaMemsetAsync(bad, 0, sizeof(int), ctx->stream) == cudaSuccess ? RS_OK : RS_ERR_CUDA;
     if (!st) {
-        A->dia.ld = ld;
-        std::copy(off, off + nd, A->dia.off);
-        A->dia.nd = nd;
-        k_dia_fill<BS><<<(int)(((int64_t)A->n + 255) / 256), 256, 0, ctx->stream>>>(dia_args(A), nd, A->ptr, A->col, A->val,
-                                                                          A->dia.val, A->dia.mask, bad);
+        k_dia_fill<BS><<<dia_grid(A, 64), dim3(64, BS), 0, ctx->stream>>>(dia_args(A), nd, A->ptr, A->col, A->val,
+                                                                                  A->dia.val, A->dia.mask, bad);
         st = rs_check_launch(ctx);
     }
-    if (!st && (cudaMemcpyAsync(&hbad, bad, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream) != cudaSuccess ||
+    if (!st && (cudaMemcpyAsync(hbad, bad, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream) != cudaSuccess ||
                 cudaStreamSynchronize(ctx->stream) != cudaSuccess))
         st = RS_ERR_CUDA;
-    rs_free(ctx, bad);
-    if (st || hbad) rs_spmv_layout_free(A);
+    if (st || *hbad) rs_spmv_layout_free(A);
     return st;
 }
 
@@ -420,8 +418,6 @@ int dia_dispatch(const rs_mat *A, F launch)
     return rs_check_launch(A->ctx);
 }
 
-int dia_grid(const rs_mat *A, int rows) { return (int)(((int64_t)A->nrows + rows - 1) / rows); }
-
 template <int BS>
 int dia_launch(const rs_mat *A, const double *x, double alpha, double beta, const double *bvec, double *y,
                const int *skip, const double *dinv)
@@ -452,7 +448,6 @@ void rs_spmv_layout_free(rs_mat *A)
 {
     rs_ctx *ctx = A->ctx;
     rs_free(ctx, A->dia.val);
-    rs_free(ctx, A->dia.mask);
     rs_free(ctx, A->sell.rows);
     rs_free(ctx, A->sell.sptr);
     rs_free(ctx, A->sell.col);
