@@ -950,37 +950,40 @@ void cfg_of(int fp32, int *G, int *rl, int *ru)
 bool rs_wave_detect(int n, const std::vector<int> &ptr, const std::vector<int> &col, int *gx, int *gy, int *gz)
 {
     if (n < 2) return false;
-    std::vector<int> offs;
+    int offs[3], no = 0;                      // distinct distances to the diagonal
     for (int i = 0; i < n; ++i)
         for (int q = ptr[i]; q < ptr[i + 1]; ++q) {
             const int d = std::abs(col[q] - i);
-            if (d == 0 || std::find(offs.begin(), offs.end(), d) != offs.end()) continue;
-            offs.push_back(d);
-            if (offs.size() > 3) return false;
+            int k = 0;
+            while (k < no && offs[k] != d) ++k;
+            if (d == 0 || k < no) continue;
+            if (no == 3) return false;
+            offs[no++] = d;
         }
-    if (offs.empty()) return false;
-    std::sort(offs.begin(), offs.end());
+    if (no == 0) return false;
+    std::sort(offs, offs + no);
     int nx, nxy;
     if (offs[0] == 1) {
-        nx = offs.size() >= 2 ? offs[1] : n;
-        nxy = offs.size() == 3 ? offs[2] : n;
+        nx = no >= 2 ? offs[1] : n;
+        nxy = no == 3 ? offs[2] : n;
     } else {
-        if (offs.size() == 3) return false;
+        if (no == 3) return false;
         nx = offs[0];
-        nxy = offs.size() == 2 ? offs[1] : n;
+        nxy = no == 2 ? offs[1] : n;
     }
     if (nx < 2 || nxy % nx != 0 || n % nxy != 0) return false;
     const int ny = nxy / nx, nz = n / nxy;
     if (nx > RS_WAVE_MAX_NX || (int64_t)ny * nz < 2) return false;
-    for (int i = 0; i < n; ++i) {
-        const int x = i % nx, y = (i / nx) % ny, z = i / nxy;
-        for (int q = ptr[i]; q < ptr[i + 1]; ++q) {
-            const int d = col[q] - i;
-            const bool ok = d == 0 || (d == -1 && x > 0) || (d == 1 && x < nx - 1) || (d == -nx && y > 0) ||
-                            (d == nx && y < ny - 1) || (d == -nxy && z > 0) || (d == nxy && z < nz - 1);
-            if (!ok) return false;
-        }
-    }
+    int i = 0;
+    for (int z = 0; z < nz; ++z)
+        for (int y = 0; y < ny; ++y)
+            for (int x = 0; x < nx; ++x, ++i)
+                for (int q = ptr[i]; q < ptr[i + 1]; ++q) {
+                    const int d = col[q] - i;
+                    const bool ok = d == 0 || (d == -1 && x > 0) || (d == 1 && x < nx - 1) || (d == -nx && y > 0) ||
+                                    (d == nx && y < ny - 1) || (d == -nxy && z > 0) || (d == nxy && z < nz - 1);
+                    if (!ok) return false;
+                }
     *gx = nx;
     *gy = ny;
     *gz = nz;
