@@ -428,6 +428,22 @@ def test_small_system_arnoldi(rs, ctx, orc, shape, restart, solver):
     assert rel(x.numpy(), xo) <= 1e-6
 
 
+@pytest.mark.parametrize("shape,per_step", [((24, 16, 16), 2), ((25, 16, 16), 5)])
+def test_arnoldi_step_rule(rs, ctx, shape, per_step):
+    """6144 rows take the step in one launch beside the product, 6400 in three
+    passes and the scaling."""
+    d = synth.pressure_7pt(synth.Grid(*shape), 21, kz_scale=0.1)
+    A = rs.Mat.csr(ctx, d)
+    b, x = vec(rs, ctx, np.ones(A.n)), rs.Vec.zeros(ctx, A.n)
+    counts = []
+    for steps in (10, 20):
+        rs.vec_set_value(x, 0.0)
+        n0 = ctx.launches()
+        rs.solve_gmres(A, None, b, x, restart=30, rtol=0.0, maxit=steps)
+        counts.append(ctx.launches() - n0)
+    assert counts[1] - counts[0] == 10 * per_step
+
+
 def test_unpreconditioned_and_edge_cases(rs, ctx, orc):
     g = synth.Grid(8, 7, 6)
     d = synth.pressure_7pt(g, 3, accum=0.5)     # well conditioned: short, smooth convergence
