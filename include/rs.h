@@ -124,11 +124,14 @@ typedef struct {
     /* Triangular sweeps of every ILU(0) / block ILU(0) factor of this
      * preconditioner (Eq. 3).  0 [0]: the library's choice, at present the
      * same as 2 (measured faster than the segment sweeps on every grid
-     * workload); 1: the segment sweeps; 2: the wavefront sweeps, taken when
+     * workload); 1: the segment sweeps; 2: the sweeps by wavefronts, taken when
      * the pattern is (a subset of) the 7-point stencil of a structured grid
      * in natural order (x fastest; the grid is read off the pattern), else
-     * the segment sweeps.  RAS local factors always take the segment
-     * sweeps. */
+     * the segment sweeps.  Wavefronts of a small grid are solved in one thread
+     * block and one launch, of a larger one by tiles in many blocks, whichever is
+     * estimated to be faster.  RAS local factors do not look at this field:
+     * scalar subdomains that fit in shared memory take a thread block each
+     * where that is estimated to be faster, all others the segment sweeps. */
     int32_t sweep;
     /* Segment sweeps: the longest run of segments one warp carries, > 0 (1:
      * no runs).  0 [0]: no limit for FP64 scalar factors, no runs for FP32
@@ -241,7 +244,15 @@ int rs_vec_mdot_noalloc(const double *V, int32_t ld, int32_t n, int32_t k, const
 /* ---- matrices (Sec. 2.3) ---------------------------------------------- */
 
 /* MatCreate/MatAssemble (Figs. 16-19) for an n x n CSR matrix:
- * rowptr[n+1], col[nnz], val[nnz] (FP64), host or device per `mem`. */
+ * rowptr[n+1], col[nnz], val[nnz] (FP64), host or device per `mem`.
+ *
+ * The library keeps its own copy, and for its products a second one where
+ * the (block) entries lie at no more than 8 distances from the diagonal, at
+ * least 0.7 of them present (blocks up to 3 x 3), or a scalar matrix has
+ * 32,768 rows or more: 145 instead of 88 bytes a row with seven points, 1041
+ * instead of 536 a row of 3 x 3 blocks.  Without room for it the matrix is
+ * as usable as with it.  Creation waits for the stream (about 20 us more than
+ * without the second copy for a small matrix, 3 to 6 % for a large one). */
 int rs_mat_create_csr(rs_ctx *ctx, int32_t n, const int32_t *rowptr, const int32_t *col,
                       const double *val, int mem, rs_mat **A);
 /* A block matrix of nb x nb blocks of size bs x bs (bs = 3 for the
@@ -323,12 +334,14 @@ int rs_precond_get_ras(const rs_pc *M, int32_t *gidx, int32_t *ptr, int32_t *col
  * row by row in dependency order).  Wavefront sweeps (a structured 7-point
  * pattern on an nx x ny x nz grid): the cells on the longest dependency
  * chain, nx + ny + nz - 2, each one step of the wavefront.  Which sweeps a
- * factor takes: rs_precond_sweep_kind.  RS_ERR_INVALID_ARG for RS_PC_NONE
- * or NULL arguments. */
+ * factor takes: rs_precond_sweep_kind.  RS_PC_RAS: the segment levels of the
+ * stacked subdomains, also where a thread block per subdomain solves them.
+ * RS_ERR_INVALID_ARG for RS_PC_NONE or NULL arguments. */
 int rs_precond_sweep_levels(const rs_pc *M, int32_t *levels_l, int32_t *levels_u);
 /* The sweeps the full-system factor takes: *kind = 0 segment sweeps, 1
- * wavefront sweeps; for wavefronts (nx, ny, nz) is the grid read off the
- * pattern (else 0, 0, 0).  Any output but kind may be NULL. */
+ * sweeps by wavefronts (in one thread block or in many); for wavefronts
+ * (nx, ny, nz) is the grid read off the pattern (else 0, 0, 0).  RS_PC_RAS: 0.
+ * Any output but kind may be NULL. */
 int rs_precond_sweep_kind(const rs_pc *M, int32_t *kind, int32_t *nx, int32_t *ny, int32_t *nz);
 /* Runs of the same sweeps: a run is a sequence of segments that one warp
  * solves in turn, each segment reading the one before it from the warp's
@@ -337,7 +350,9 @@ int rs_precond_sweep_kind(const rs_pc *M, int32_t *kind, int32_t *nx, int32_t *n
  * the warps take; longest_l / longest_u: the segments of the longest run.
  * The number of runs never exceeds the number of segments.  Runs change the
  * schedule, not the arithmetic: results are those of one segment per run.
- * RS_ERR_INVALID_ARG for RS_PC_NONE or NULL arguments. */
+ * RS_PC_RAS: the runs of the stacked subdomains' segment sweeps, whether or
+ * not they are the ones taken.  RS_ERR_INVALID_ARG for RS_PC_NONE or NULL
+ * arguments. */
 int rs_precond_sweep_runs(const rs_pc *M, int32_t *runs_l, int32_t *runs_u, int32_t *longest_l,
                           int32_t *longest_u);
 /* The schedule of one triangular sweep of a pattern, computed on the host

@@ -180,8 +180,9 @@ void rs_amg_destroy(AmgData *M)
     delete M;
 }
 
-int rs_amg_create(rs_ctx *ctx, int n, int64_t nnz, const int *d_ptr, const int *d_col, const double *d_val, const rs_mat *A0,
-                  const rs_mat *like,                  double theta, int max_levels, int max_coarse, int nu, int smoother, AmgData **out)
+int rs_amg_create(rs_ctx *ctx, int n, int64_t nnz, const int *d_ptr, const int *d_col, const double *d_val,
+                  const rs_mat *A0, const rs_mat *like, double theta, int max_levels, int max_coarse, int nu,
+                  int smoother, AmgData **out)
 {
     *out = nullptr;
     if (n < 1 || max_levels < 1 || max_levels > RS_AMG_MAXLEV || max_coarse < 1 || nu < 1 || !(theta >= 0.0) ||

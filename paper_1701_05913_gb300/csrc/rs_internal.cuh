@@ -404,9 +404,9 @@ int rs_ras_apply(RasData *R, const double *r, double *z, const int *skip);
 void rs_ras_destroy(RasData *R);
 // A0: the level-0 matrix when the caller has one as an rs_mat (else built
 // from the arrays; like: a block matrix of that pattern)
-int rs_amg_create(rs_ctx *ctx, int n, int64_t nnz, const int *d_ptr, const int *d_col, const double *d_val, const rs_mat *A0,
-                  const rs_mat *like,
-                  double theta, int max_levels, int max_coarse, int nu, int smoother, AmgData **out);
+int rs_amg_create(rs_ctx *ctx, int n, int64_t nnz, const int *d_ptr, const int *d_col, const double *d_val,
+                  const rs_mat *A0, const rs_mat *like, double theta, int max_levels, int max_coarse, int nu,
+                  int smoother, AmgData **out);
 // the hierarchy of Alg. 3 on the device (rs_amg_setup.cu): from M->A[0]
 int rs_amg_setup_device(AmgData *M, double theta, int max_levels, int max_coarse);
 int rs_amg_apply(AmgData *M, const double *r, double *z, const int *skip);

@@ -220,11 +220,6 @@ struct CgsCfg {
     static constexpr size_t SMEM = (size_t)S * STAGE * sizeof(double) + 2 * S * sizeof(unsigned long long);
 };
 
-// NC: columns of the ring and of the reduction (a power of two); NCC: the
-// unrolled bound of the multiply-add loops (nc rounded down to 4); the last
-// nc - NCC (0 to 3) columns take a warp-uniform branch, so that no FP64
-// multiply-add is issued for a column that does not exist (predicated-off
-// FP64 instructions still occupy the FP64 pipe on this GPU).
 // The Givens rotations on the new Hessenberg column h[0..nc) with
 // h_{nc,nc-1} = hnext (h[nc] is set to 0), the rotated residual, the
 // convergence and happy-breakdown tests and the next vector's scale.  cs, sn:
@@ -287,6 +282,11 @@ __device__ __forceinline__ void givens_update(GmresDev *d, int nc, double *h, co
     d->hdiv = hinv;            // v_{i+1} = w / h_{i+1,i}
 }
 
+// NC: columns of the ring and of the reduction (a power of two); NCC: the
+// unrolled bound of the multiply-add loops (nc rounded down to 4); the last
+// nc - NCC (0 to 3) columns take a warp-uniform branch, so that no FP64
+// multiply-add is issued for a column that does not exist (predicated-off
+// FP64 instructions still occupy the FP64 pipe on this GPU).
 template <int NC, int NCC, int MODE>
 __global__ void __launch_bounds__(CgsCfg<NC>::THREADS)
 k_cgs_pass(int n, int ld, int nc, const double *__restrict__ V, double *w, double *partials, unsigned *ticket,
@@ -426,7 +426,11 @@ k_cgs_pass(int n, int ld, int nc, const double *__restrict__ V, double *w, doubl
 // ---------------------------------------------------------------------------
 #define CS_CTAS 8
 #define CS_THREADS 256
-#define CS_MAX_ROWS 6144                            // beyond, the passes' more SMs win
+// Beyond, the passes' more SMs win.  A GMRES(30) cycle with ILU(0), us, in one
+// launch a step / in passes: 960 rows 1242 / 1611, 1920 1521 / 1813, 3072 1866 /
+// 2159, 4096 2118 / 2334, 6144 2314 / 2420; 7168 rows (24 columns fit) 2428 / 2452,
+// 9216 (19 columns) 2923 / 2853.
+#define CS_MAX_ROWS 6144
 #define CS_SMEM (190 * 1024)
 
 // rows of a block: even, so that a column's rows are whole 16-byte copies

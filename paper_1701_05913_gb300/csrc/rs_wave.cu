@@ -316,7 +316,13 @@ k_wave_sweep(WaveArgs g, const T *__restrict__ rec, const T *__restrict__ rhs, T
             const T *grec = rec + base * RB;
             const T *grhs = rhs + base * BS;
             int qb = 0, qstep = rs_wave_chunk_step(0, nch, R, G);    // next chunk to copy, and the step that frees its slot
-            // steps the compute warp has left
+            // Steps the compute warp has left.  Neither this load nor st_cons
+            // orders memory.  Relied on: the reads of what is freed were done before
+            // the counter was stored (see st_cons), and what overwrites it here,
+            // stores into the ring and bulk copies into slots, is issued after a
+            // branch on the counter's value, and stores are not issued ahead of their
+            // branch.  (With an acquire here 128 x 128 x 64 takes 240.7 instead
+            // of 239.3 us in FP64, 130.6 instead of 129.6 in FP32.)
             auto cons_now = [&]() -> int { return __shfl_sync(FULL, *(volatile int *)&hd->cons, 0); };
             auto issue_ready = [&](int c) {
                 while (c >= qstep) {
