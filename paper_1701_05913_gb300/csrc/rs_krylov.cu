@@ -673,7 +673,6 @@ static int launch_cgs_pass(rs_ctx *ctx, int n, int ld, int nc, double *V, GmresD
                           : MODE == CGS_UPDATE_DOTS ? RS_PROF_CGS_UPDATE_DOTS : RS_PROF_CGS_UPDATE_NORM);
     rs_pdl(k_cgs_pass<NC, NCC, MODE>, red_grid(ctx, n, C::TILE), C::THREADS, C::SMEM, ctx)(
         n, ld, nc, V, V + (size_t)nc * ld, ctx->red_partials, ctx->red_ticket, d, ctx->d_err, ctx->spin_limit);
-    ctx->launches++;
     return rs_check_launch(ctx);
 }
 
