@@ -336,7 +336,7 @@ int dia_build(rs_mat *A, int nd, const int (&off)[DIA_MAX])
     rs_ctx *ctx = A->ctx;
     const int64_t ld = ((int64_t)A->nrows + 31) / 32 * 32;
     const size_t places = (size_t)nd * BS * BS * ld;
-    int *hbad = (int *)(ctx->h_pinned + 40);
+    int hbad = 1;
     // one allocation: values, masks, the flag
     RS_TRY(rs_alloc(ctx, (void **)&A->dia.val, sizeof(double) * places + ld + sizeof(int)));
     A->dia.mask = (unsigned char *)(A->dia.val + places);
@@ -350,10 +350,10 @@ int dia_build(rs_mat *A, int nd, const int (&off)[DIA_MAX])
                                                                                   A->dia.val, A->dia.mask, bad);
         st = rs_check_launch(ctx);
     }
-    if (!st && (cudaMemcpyAsync(hbad, bad, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream) != cudaSuccess ||
+    if (!st && (cudaMemcpyAsync(&hbad, bad, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream) != cudaSuccess ||
                 cudaStreamSynchronize(ctx->stream) != cudaSuccess))
         st = RS_ERR_CUDA;
-    if (st || *hbad) rs_spmv_layout_free(A);
+    if (st || hbad) rs_spmv_layout_free(A);
     return st;
 }
 
