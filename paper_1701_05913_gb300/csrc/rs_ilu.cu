@@ -1580,15 +1580,19 @@ static int apply_seg(IluFactor *f, const double *r, double *z, const double *sca
     {
         RsProfScope prof(ctx, BS == 1 ? RS_PROF_LSWEEP : RS_PROF_BLSWEEP);
         const SegArgs a = seg_args(ctx, f->SL, f->nrows, f->state, skip);
-        // Blocks that carry runs are one warp each, about as many as SMs: those of a
-        // programmatic launch start beside the gather or update before and are
-        // spread unevenly.  ILU(0) of 8 row ranges of 100 x 100 x 50: 220 us programmatic,
-        // 201 plain; the whole grid, after its own U sweep: 331 and 337.
+        // Blocks of a programmatic launch start beside the gather or update before and
+        // are spread unevenly, which costs sweeps that are bound by their SM's FP64
+        // unit or have about a block per SM: those with runs (one warp a block) and of
+        // FP64 blocks are launched plainly.  Programmatic / plain: ILU(0) of 8 row
+        // ranges of 100 x 100 x 50 220 / 201 us an apply, the whole grid after its own U
+        // sweep 331 / 337; 20 FGMRES steps with block ILU(0) at 64^3 26.5 / 23.4 ms, with
+        // RAS of blocks at 100 x 100 x 40 13.1 / 12.3, at 12 x 10 x 9 2.30 / 2.33.
+        constexpr bool fp64_blocks = BS > 1 && sizeof(T) == 8;
         if (rl)
             rs_pdl(k_lsolve_seg<BS, T, BS == 1>, gl, 32 * wl, sl, ctx, true)(
                 a, (const T *)f->SL.val, (const T *)f->SL.mul, r, scale, y, zt);
         else
-            rs_pdl(k_lsolve_seg<BS, T, false>, gl, 32 * wl, sl, ctx)(
+            rs_pdl(k_lsolve_seg<BS, T, false>, gl, 32 * wl, sl, ctx, fp64_blocks)(
                 a, (const T *)f->SL.val, (const T *)f->SL.mul, r, scale, y, zt);
     }
     RS_TRY(rs_check_launch(ctx));

@@ -895,12 +895,12 @@ int wave_apply_t(IluFactor *f, const double *r, double *z, const double *scale, 
     RS_TRY((raise_sweep_smem<BS, T, false>(ctx)));
     // FP64 block units are bound by their SM's FP64 unit, so two on one SM beside an
     // idle SM double the pace that all wait for.  Blocks of a programmatic launch start
-    // beside the kernel before and are placed so; with about one or two units per
+    // beside the kernel before and are placed so; with half a unit to two units per
     // SM the sweeps are launched without.  Programmatic / plain, both sweeps in us,
     // 152 SMs, 3 x 3 blocks: 84 units 269 / 273, 112 324 / 309, 128 374 / 328, 160
     // 417 / 382, 216 473 / 462, 260 508 / 505, 384 593 / 602; 4 x 4: 72 440 / 444, 128
-    // 768 / 552, 160 810 / 705.
-    const bool plain = C::NCW > 1 && 3 * W.nunits >= 2 * ctx->num_sms && W.nunits < 2 * ctx->num_sms;
+    // 768 / 552, 160 810 / 705; in 8 BiCGSTAB steps: 28 units 3.03 / 3.08 ms, 90 5.51 / 5.26.
+    const bool plain = C::NCW > 1 && 2 * W.nunits >= ctx->num_sms && W.nunits < 2 * ctx->num_sms;
     {
         RsProfScope prof(ctx, BS == 1 ? RS_PROF_LSWEEP : RS_PROF_BLSWEEP);
         rs_pdl(k_wave_in<BS, T>, gp, WAVE_PERM_THREADS, 0, ctx)(g, r, scale, (T *)W.rw, (T *)W.zw);
